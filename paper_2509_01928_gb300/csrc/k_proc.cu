@@ -342,7 +342,12 @@ int stream_blocks(const ising_context *c, int64_t count) {
 constexpr int kSR = 4;             // rows per thread
 constexpr int kSTR = kSR * kPT;    // rows per row tile
 constexpr int kSTC = 256;          // columns per column tile
-constexpr int kSUnit = 64;         // column tiles per work unit
+// Column tiles per work unit: as many as give every CTA slot (two per SM) about kSWaves units,
+// so that the last wave is a small share, at most kSUnit. A unit's start (five phases per row, the
+// row sums' atomics) costs about 2 % of one tile. 64 tiles per unit at every n left 195 units for
+// 304 slots at n = 60,000: 2.04 ms per product, 0.80 ms now; n = 10^6 keeps 64.
+constexpr int kSUnit = 64;
+constexpr int kSWaves = 8;
 
 // lane l returns the sum over the warp's lanes of v[l] (v[b]: column b of a 32-column chunk)
 __device__ __forceinline__ float reduce_scatter32(float (&v)[32]) {
@@ -386,8 +391,8 @@ __device__ __forceinline__ void sym_unit(const XT *__restrict__ x, unsigned long
     __shared__ __align__(16) float xs[kSTC];
     __shared__ float red[kPT / 32][kSTC];
     const int64_t r0 = static_cast<int64_t>(un.x) * kSTR;
-    const int64_t c_begin = DIAG ? r0 : static_cast<int64_t>(un.y) * kSTC;
-    const int ntile = DIAG ? static_cast<int>((min(n, r0 + kSTR) - r0 + kSTC - 1) / kSTC) : un.z;
+    const int64_t c_begin = static_cast<int64_t>(un.y) * kSTC;
+    const int ntile = un.z;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float xr[kSR];
     uint64_t P[kSR], D32[kSR];  // phase at the next 32-column chunk, its advance per chunk
@@ -552,21 +557,24 @@ ising_status_t sym_setup(ising_context *c) {
     if (c->proc_units_count > 0) return ISING_OK;
     const int64_t n = c->n;
     const int64_t rt = (n + kSTR - 1) / kSTR, ct = (n + kSTC - 1) / kSTC;
-    int64_t total = rt;  // counted before anything is allocated
+    int64_t tiles = 0;  // off-diagonal column tiles
+    for (int64_t I = 0; I < rt; ++I) tiles += std::max<int64_t>(0, ct - (I + 1) * (kSTR / kSTC));
+    const int64_t per = std::max<int64_t>(1, std::min<int64_t>(kSUnit, tiles / (2LL * kSWaves * c->num_sms)));
+    int64_t total = 0;  // counted before anything is allocated
     for (int64_t I = 0; I < rt; ++I) {
-        const int64_t first = (I + 1) * (kSTR / kSTC);
-        if (first < ct) total += (ct - first + kSUnit - 1) / kSUnit;
+        const int64_t first = I * (kSTR / kSTC), next = std::min(ct, first + kSTR / kSTC);
+        total += (next - first + per - 1) / per + (ct - next + per - 1) / per;
     }
     if (total > 0x7FFFFFFF) return fail(ISING_ERR_UNSUPPORTED, "procedural product: too many work units");
     std::vector<int4> u;
     u.reserve(static_cast<size_t>(total));
-    for (int64_t I = 0; I < rt; ++I) u.push_back(make_int4(static_cast<int>(I), 0, 0, 1));
-    for (int64_t I = 0; I < rt; ++I) {
-        const int64_t first = (I + 1) * (kSTR / kSTC);
-        for (int64_t t = first; t < ct; t += kSUnit)
-            u.push_back(make_int4(static_cast<int>(I), static_cast<int>(t),
-                                  static_cast<int>(std::min<int64_t>(kSUnit, ct - t)), 0));
-    }
+    for (int diag = 1; diag >= 0; --diag)
+        for (int64_t I = 0; I < rt; ++I) {
+            const int64_t first = I * (kSTR / kSTC), next = std::min(ct, first + kSTR / kSTC);
+            for (int64_t t = diag ? first : next; t < (diag ? next : ct); t += per)
+                u.push_back(make_int4(static_cast<int>(I), static_cast<int>(t),
+                                      static_cast<int>(std::min<int64_t>(per, (diag ? next : ct) - t)), diag));
+        }
     DOCH_CHECK(c->proc_units.ensure(sizeof(int4) * u.size()));
     DOCH_CUDA(cudaMemcpy(c->proc_units.ptr, u.data(), sizeof(int4) * u.size(), cudaMemcpyHostToDevice));
     DOCH_CHECK(c->proc_acc.ensure(sizeof(unsigned long long) * n + 256));
