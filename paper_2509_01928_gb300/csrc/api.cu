@@ -439,6 +439,7 @@ void destroy_ctx(ising_context *c) {
     cudaFree(c->val);
     cudaFree(c->right);
     cudaFree(c->down);
+    c->edge.release();
     cudaFree(c->dense);
     cudaFree(c->h_f32);
     cudaFree(c->h_f64);
@@ -681,7 +682,7 @@ ising_status_t step(ising_context *c, const void *xi, void *xo, int xtype, int R
         const double a = alpha_h[p.alpha_len == 1 ? 0 : k];
         if (xtype == ISING_F32)
             return torus_step_f32(c, static_cast<const float *>(xi), static_cast<float *>(xo), R,
-                                  static_cast<float>(a), 1.0 / beta_h[0], st);
+                                  a, 1.0 / beta_h[0], st);
         return torus_step_f64(c, static_cast<const double *>(xi), static_cast<double *>(xo), R, a,
                               beta_h[0], st);
     }
@@ -1201,9 +1202,13 @@ ising_status_t ising_iterate(ising_handle_t h, void *x, int32_t xtype, int32_t R
         if (!done && iters > 0) {
             DOCH_CHECK(c->ping.ensure(xbytes));
             void *cur = xd, *nxt = c->ping.ptr;
-            const bool pairs_ok = !Hd && c->format == ISING_FMT_TORUS2D && xtype == ISING_F32 &&
-                                  !(c->flags & ISING_FLAG_SINGLE_STEP) &&
-                                  torus_pair_ok(c, static_cast<const float *>(cur), static_cast<const float *>(nxt), R);
+            const bool fused_ok = !Hd && c->format == ISING_FMT_TORUS2D && xtype == ISING_F32 &&
+                                  !(c->flags & ISING_FLAG_SINGLE_STEP);
+            const bool pairs_ok = fused_ok && torus_pair_ok(c, static_cast<const float *>(cur),
+                                                            static_cast<const float *>(nxt), R);
+            // the other lattices (several replicas, ragged widths, odd alignments) take the general walk
+            const bool walk_ok = fused_ok && !torus_vec4_ok(c, static_cast<const float *>(cur),
+                                                            static_cast<const float *>(nxt), R);
             // steps per lattice pass: at most 3 (default) or ISING_LATTICE_PASS = 1, 2 or 3
             int per_pass = 3;
             if (const char *env = std::getenv("ISING_LATTICE_PASS")) {
@@ -1212,6 +1217,16 @@ ising_status_t ising_iterate(ising_handle_t h, void *x, int32_t xtype, int32_t R
             }
             const bool triples_ok = pairs_ok && per_pass >= 3 && c->l_rows >= 6;
             for (int k = 0; k < iters;) {
+                const int ts = std::min(per_pass, iters - k);
+                if (walk_ok && ts > 1) {
+                    const double a[3] = {alpha_h[alpha_len == 1 ? 0 : k], alpha_h[alpha_len == 1 ? 0 : k + 1],
+                                         alpha_h[alpha_len == 1 ? 0 : k + ts - 1]};
+                    DOCH_CHECK(torus_walk_f32(c, static_cast<const float *>(cur), static_cast<float *>(nxt), R, a, ts,
+                                              1.0 / beta_h[0], st));
+                    std::swap(cur, nxt);
+                    k += ts;
+                    continue;
+                }
                 if (triples_ok && k + 2 < iters) {  // three steps in one pass over the lattice
                     const double a1 = alpha_h[alpha_len == 1 ? 0 : k], a2 = alpha_h[alpha_len == 1 ? 0 : k + 1],
                                  a3 = alpha_h[alpha_len == 1 ? 0 : k + 2];

@@ -120,6 +120,7 @@ struct ising_context {
     // TORUS2D
     int64_t l_rows = 0, l_cols = 0;
     int8_t *right = nullptr, *down = nullptr;
+    doch::DevBuf edge;  // the four couplings of each site as one word (built on first use, k_torus_walk.cu)
     // DENSE: integer couplings held as BF16 (exact for |J| <= 256) in the
     // tensor-core tile order [ceil(n/128)][dense_ld/64][128][64], 128-byte
     // swizzled; dense_ld = n rounded up to 64 (zero padded)
@@ -189,13 +190,18 @@ namespace doch {
 // ---------------------------------------------------------------------------
 
 // TORUS2D, one DOCH step, x_out = T(x_in) (Eq. FPE). XT = float or double.
-ising_status_t torus_step_f32(const ising_context *c, const float *x_in, float *x_out, int R,
-                              float alpha, double inv_beta, cudaStream_t st);
-ising_status_t torus_step_f64(const ising_context *c, const double *x_in, double *x_out, int R,
+ising_status_t torus_step_f32(ising_context *c, const float *x_in, float *x_out, int R,
+                              double alpha, double inv_beta, cudaStream_t st);
+ising_status_t torus_step_f64(ising_context *c, const double *x_in, double *x_out, int R,
                               double alpha, double beta, cudaStream_t st);
+// TORUS2D, ts = 1, 2 or 3 DOCH steps in one pass (alpha[0 .. ts - 1]), FP32, any R, width and alignment.
+ising_status_t torus_walk_f32(ising_context *c, const float *x_in, float *x_out, int R, const double *alpha, int ts,
+                              double inv_beta, cudaStream_t st);
 // TORUS2D, two DOCH steps in one pass (alpha1 then alpha2), FP32, R = 1; only
 // when torus_pair_ok() holds.
 bool torus_pair_ok(const ising_context *c, const float *x_in, const float *x_out, int R);
+// R = 1, width a multiple of 4, 16-byte aligned: the lattices of k_torus.cu's kernels
+bool torus_vec4_ok(const ising_context *c, const float *x_in, const float *x_out, int R);
 ising_status_t torus_pair_f32(const ising_context *c, const float *x_in, float *x_out, float alpha1,
                               float alpha2, double inv_beta, cudaStream_t st);
 // TORUS2D, three DOCH steps in one pass (alpha1, alpha2, alpha3), same conditions
@@ -221,6 +227,17 @@ struct ParamTabs {
 // CSR, one DOCH step for all instances (alpha of step k), xtype F32 or F64.
 ising_status_t csr_step(const ising_context *c, const void *x_in, void *x_out, int xtype, int R,
                         const ParamTabs &p, int k, cudaStream_t st);
+// Steps k0 .. k0 + iters - 1 of instances that fit in shared memory, in one launch (k_csr_small.cu):
+// x_out (may equal x_in, may be NULL) receives the last iterate; with rec, the iterate after every
+// rec.every-th step of the run goes to rec.base, rec.base + rec.stride, ... ISING_ERR_UNSUPPORTED
+// when an instance does not fit.
+struct SmallRecord {
+    void *base = nullptr;
+    size_t stride = 0;
+    int every = 1;
+};
+ising_status_t csr_small_run(const ising_context *c, const void *x_in, void *x_out, int xtype, int R,
+                             const ParamTabs &p, int k0, int iters, const SmallRecord &rec, cudaStream_t st);
 // The same step with the H monitor fused (one instance): H(x^(k)) of Eq. Hamilton
 // per replica into H_out [R] (device), alpha_k and beta of the step.
 // ISING_ERR_UNSUPPORTED when the fused form does not apply (batched instances,

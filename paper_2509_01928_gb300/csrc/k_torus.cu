@@ -496,33 +496,6 @@ torus_f32_r1_vec4_t3(const float *__restrict__ xi, float *__restrict__ xo,
     cp_async_wait<0>();
 }
 
-// Any R, float or double, any alignment: one thread per (site, replica).
-template <typename T>
-__global__ void torus_generic(const T *__restrict__ xi, T *__restrict__ xo,
-                              const int8_t *__restrict__ right, const int8_t *__restrict__ down,
-                              int64_t Lr, int64_t Lc, int R, T alpha, T beta) {
-    const int64_t total = Lr * Lc * R;
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < total;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t site = t / R;
-        const int rep = static_cast<int>(t - site * R);
-        const int64_t rr = site / Lc, cc = site - rr * Lc;
-        const int64_t s_l = rr * Lc + (cc == 0 ? Lc - 1 : cc - 1);
-        const int64_t s_r = rr * Lc + (cc + 1 == Lc ? 0 : cc + 1);
-        const int64_t s_u = (rr == 0 ? Lr - 1 : rr - 1) * Lc + cc;
-        const int64_t s_d = (rr + 1 == Lr ? 0 : rr + 1) * Lc + cc;
-        const T u = static_cast<T>(right[site]) * xi[s_r * R + rep] +
-                    static_cast<T>(right[s_l]) * xi[s_l * R + rep] +
-                    static_cast<T>(down[site]) * xi[s_d * R + rep] +
-                    static_cast<T>(down[s_u]) * xi[s_u * R + rep];
-        const T z = (u + alpha * xi[t]);
-        if constexpr (sizeof(T) == 4)
-            xo[t] = cbrtf(z * beta);  // beta holds 1/beta for float
-        else
-            xo[t] = cbrt(z / beta);
-    }
-}
-
 // ring depth of the two-step kernel: rows staged ahead of the one in use
 constexpr int kT2Depth = 4;
 constexpr size_t kT2Smem = sizeof(T2Ring<kT2Depth>);
@@ -605,25 +578,19 @@ ising_status_t torus_step_f32_traced(ising_context *c, const float *x_in, float 
     return ham_fused_finish_launch(c->partials.as<double>(), static_cast<int>(v.blocks()), 1, alpha_k, beta, H_out, st);
 }
 
-ising_status_t torus_step_f32(const ising_context *c, const float *x_in, float *x_out, int R,
-                              float alpha, double inv_beta, cudaStream_t st) {
-    const int64_t Lr = c->l_rows, Lc = c->l_cols;
-    if (vec4_ok(c, x_in, x_out, R)) {
-        const Vec4Shape v = vec4_shape(c);
-        const float c3 = lattice_c3(inv_beta);
-        torus_f32_r1_vec4<false><<<static_cast<unsigned>(v.blocks()), kThreads, 0, st>>>(
-            x_in, x_out, c->right, c->down, static_cast<int>(Lr), static_cast<int>(Lc), v.tiles,
-            static_cast<int>(v.bpt), alpha, c3, nullptr);
-    } else {
-        const int64_t total = Lr * Lc * R;
-        int64_t blocks = (total + 255) / 256;
-        const int64_t cap = static_cast<int64_t>(c->num_sms) * 16;
-        if (blocks > cap) blocks = cap;
-        torus_generic<float><<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-            x_in, x_out, c->right, c->down, Lr, Lc, R, alpha, static_cast<float>(inv_beta));
-    }
+ising_status_t torus_step_f32(ising_context *c, const float *x_in, float *x_out, int R,
+                              double alpha, double inv_beta, cudaStream_t st) {
+    if (!vec4_ok(c, x_in, x_out, R)) return torus_walk_f32(c, x_in, x_out, R, &alpha, 1, inv_beta, st);
+    const Vec4Shape v = vec4_shape(c);
+    torus_f32_r1_vec4<false><<<static_cast<unsigned>(v.blocks()), kThreads, 0, st>>>(
+        x_in, x_out, c->right, c->down, static_cast<int>(c->l_rows), static_cast<int>(c->l_cols), v.tiles,
+        static_cast<int>(v.bpt), static_cast<float>(alpha), lattice_c3(inv_beta), nullptr);
     DOCH_CUDA(cudaGetLastError());
     return ISING_OK;
+}
+
+bool torus_vec4_ok(const ising_context *c, const float *x_in, const float *x_out, int R) {
+    return vec4_ok(c, x_in, x_out, R);
 }
 
 bool torus_pair_ok(const ising_context *c, const float *x_in, const float *x_out, int R) {
@@ -670,18 +637,6 @@ ising_status_t torus_triple_f32(const ising_context *c, const float *x_in, float
     torus_f32_r1_vec4_t3<kT2Depth><<<static_cast<unsigned>(blocks), kThreads, kT2Smem, st>>>(
         x_in, x_out, c->right, c->down, static_cast<int>(Lr), static_cast<int>(Lc), static_cast<int>(segs),
         static_cast<int>(bpt), alpha1, alpha2, alpha3, c3);
-    DOCH_CUDA(cudaGetLastError());
-    return ISING_OK;
-}
-
-ising_status_t torus_step_f64(const ising_context *c, const double *x_in, double *x_out, int R,
-                              double alpha, double beta, cudaStream_t st) {
-    const int64_t total = c->l_rows * c->l_cols * R;
-    int64_t blocks = (total + 255) / 256;
-    const int64_t cap = static_cast<int64_t>(c->num_sms) * 16;
-    if (blocks > cap) blocks = cap;
-    torus_generic<double><<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-        x_in, x_out, c->right, c->down, c->l_rows, c->l_cols, R, alpha, beta);
     DOCH_CUDA(cudaGetLastError());
     return ISING_OK;
 }

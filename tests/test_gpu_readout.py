@@ -38,7 +38,7 @@ def _shifted(a, skip):
 @pytest.mark.parametrize("kind", ["torus", "torus_odd", "er", "hub"])
 def test_integer_energies(kind, R):
     J = {"torus": lambda: I.torus_pm1(6, 8, seed=1), "torus_odd": lambda: I.torus_pm1(2, 517, seed=2),
-         "er": lambda: I.erdos_renyi_pm1(97, 0.3, seed=3), "hub": lambda: short_rows_mixed(531, seed=4)}[kind]()
+         "er": lambda: I.erdos_renyi_pm1(97, 0.3, seed=3), "hub": lambda: short_rows_mixed(530, seed=4)}[kind]()
     x = I.x0_uniform(J.n, R, seed=5)
     x[::31] = -0.0
     s = O.sign(x.astype(np.float64))
@@ -56,7 +56,7 @@ def test_integer_energies(kind, R):
 
 @pytest.mark.parametrize("R", [1, 6, 16])
 def test_real_energies_of_uneven_instances(R):
-    sizes, degs = [5, 1000, 64, 3], [2, 12, 9, 2]
+    sizes, degs = [6, 1000, 64, 8], [2, 12, 9, 2]
     gs = [I.regular_gauss(n, d, seed=10 + n) for n, d in zip(sizes, degs)]
     hs = [I.field_gauss(n, 0.1, seed=20 + n) for n in sizes]
     off = np.cumsum([0] + sizes).astype(np.int64)
