@@ -14,10 +14,7 @@
 // thread's loads are pipelined across its rows (csr_pipe.cuh); the sums are the
 // ones csr_step forms, in the same order.
 //
-// csr_fused: the whole iteration in one launch for instances that fit in
-// shared memory. One CTA per (instance, replica) keeps that replica's
-// iterate in two shared-memory buffers and separates the steps with
-// __syncthreads(); the CSR arrays stream through L1/L2.
+// Instances that fit in shared memory run all their steps in one launch (k_csr_small.cu).
 #include <algorithm>
 
 #include "cbrt.cuh"
@@ -27,12 +24,6 @@
 
 namespace doch {
 namespace {
-
-template <typename T>
-__device__ __forceinline__ T dcbrt(T z) {
-    if constexpr (sizeof(T) == 4) return cbrtf(z);
-    else return cbrt(z);
-}
 
 // The update of the step kernels, x = cbrt(z / beta) for z = (J x + alpha x + h)_i:
 // FP32 through the prescaled power-of-two cube root (cbrt.cuh; zs = 2^(3k) / beta,
@@ -270,112 +261,6 @@ csr_step_pipe_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64
     }
 }
 
-// One CTA per (instance b = blockIdx.y, replica r = blockIdx.x); shared
-// memory holds two copies of that instance's iterate for replica r.
-template <typename XT, typename VT>
-__global__ void __launch_bounds__(1024)
-csr_fused_kernel(XT *__restrict__ x, const int64_t *__restrict__ row_ptr,
-                 const int32_t *__restrict__ col, const VT *__restrict__ val,
-                 const XT *__restrict__ h, const int64_t *__restrict__ inst_off, int64_t n, int R,
-                 const double *__restrict__ alpha_tab, int alpha_len,
-                 const double *__restrict__ beta_tab, int iters) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    XT *buf = reinterpret_cast<XT *>(smem_raw);
-    const int b = blockIdx.y, r = blockIdx.x;
-    const int64_t lo = inst_off ? inst_off[b] : 0;
-    const int64_t hi = inst_off ? inst_off[b + 1] : n;
-    const int nb = static_cast<int>(hi - lo);
-    XT *cur = buf, *nxt = buf + nb;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = x[(lo + i) * R + r];
-    const XT bb = static_cast<XT>(beta_tab[b]);
-    __syncthreads();
-    for (int k = 0; k < iters; ++k) {
-        const XT a = static_cast<XT>(alpha_tab[static_cast<int64_t>(b) * alpha_len +
-                                               (alpha_len == 1 ? 0 : k)]);
-        for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-            const int64_t row = lo + i;
-            XT acc = XT(0);
-            const int64_t e1 = __ldg(row_ptr + row + 1);
-            for (int64_t e = __ldg(row_ptr + row); e < e1; ++e)
-                acc += static_cast<XT>(__ldg(val + e)) * cur[__ldg(col + e) - lo];
-            const XT hv = h ? h[row] : XT(0);
-            nxt[i] = dcbrt((acc + a * cur[i] + hv) / bb);
-        }
-        __syncthreads();
-        XT *t = cur; cur = nxt; nxt = t;
-    }
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) x[(lo + i) * R + r] = cur[i];
-}
-
-// Small instances over a cluster of K CTAs per (instance b = blockIdx.y, replica r = blockIdx.x / K):
-// every CTA keeps both copies of the pair's whole iterate, computes the rows of its share
-// [q c, (q+1) c) (c = ceil(n_b / K), q its rank in the cluster) with the arithmetic of
-// csr_fused_kernel, and stores each new value into the next copy of all K CTAs (distributed
-// shared memory); a cluster barrier ends each step. The same iterates as one CTA per pair, with
-// the FP64 arithmetic of a pair spread over K SMs.
-__device__ __forceinline__ uint32_t cl_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cl_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t cl_map(const void *p, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-                 : "=r"(r)
-                 : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void cl_store(uint32_t a, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
-}
-__device__ __forceinline__ void cl_store(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-
-template <typename XT, typename VT>
-__global__ void __launch_bounds__(1024)
-csr_fused_cluster(XT *__restrict__ x, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                  const VT *__restrict__ val, const XT *__restrict__ h, const int64_t *__restrict__ inst_off,
-                  int64_t n, int R, const double *__restrict__ alpha_tab, int alpha_len,
-                  const double *__restrict__ beta_tab, int iters, int K) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    XT *buf = reinterpret_cast<XT *>(smem_raw);
-    const uint32_t q = cl_rank();
-    const int b = blockIdx.y, r = blockIdx.x / K;
-    const int64_t lo = inst_off ? inst_off[b] : 0;
-    const int64_t hi = inst_off ? inst_off[b + 1] : n;
-    const int nb = static_cast<int>(hi - lo);
-    const int chunk = (nb + K - 1) / K;
-    const int i0 = min(nb, static_cast<int>(q) * chunk), i1 = min(nb, i0 + chunk);
-    XT *cur = buf, *nxt = buf + nb;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = x[(lo + i) * R + r];
-    const XT bb = static_cast<XT>(beta_tab[b]);
-    cl_sync();  // every CTA of the cluster runs, and has loaded, before the first remote store
-    for (int k = 0; k < iters; ++k) {
-        const XT a = static_cast<XT>(alpha_tab[static_cast<int64_t>(b) * alpha_len + (alpha_len == 1 ? 0 : k)]);
-        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-            const int64_t row = lo + i;
-            XT acc = XT(0);
-            const int64_t e1 = __ldg(row_ptr + row + 1);
-            for (int64_t e = __ldg(row_ptr + row); e < e1; ++e)
-                acc += static_cast<XT>(__ldg(val + e)) * cur[__ldg(col + e) - lo];
-            const XT hv = h ? h[row] : XT(0);
-            const XT v = dcbrt((acc + a * cur[i] + hv) / bb);
-            nxt[i] = v;
-            for (int t = 0; t < K; ++t)
-                if (t != static_cast<int>(q)) cl_store(cl_map(nxt + i, static_cast<uint32_t>(t)), v);
-        }
-        cl_sync();  // the new values of every share are in every CTA; the old copy is free
-        XT *t = cur;
-        cur = nxt;
-        nxt = t;
-    }
-    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) x[(lo + i) * R + r] = cur[i];
-}
-
 int step_blocks(const ising_context *c, int C) {
     const int rows_per_block = C <= 256 ? 256 / C : 1;
     int64_t blocks = (c->n + rows_per_block - 1) / rows_per_block;
@@ -450,87 +335,6 @@ ising_status_t dispatch_val(const ising_context *c, const XT *xi, XT *xo, int R,
     return ISING_OK;
 }
 
-// the cluster size for the fused kernel: the largest K in {16, 8, 4, 2} (16 is a non-portable size)
-// that leaves each CTA at least 32 rows and keeps all pairs' clusters within the SMs; 1 when none does
-int fused_cluster_k(const ising_context *c, int R, int kmax) {
-    for (int K = kmax; K >= 2; K >>= 1)
-        if (static_cast<int64_t>(c->n_inst) * R * K <= c->num_sms && c->max_inst_n >= 32LL * K) return K;
-    return 1;
-}
-
-template <typename XT, typename VT>
-ising_status_t launch_fused_cluster(const ising_context *c, XT *x, int R, const XT *h, const ParamTabs &p,
-                                    int iters, int K, cudaStream_t st) {
-    const size_t smem = 2 * static_cast<size_t>(c->max_inst_n) * sizeof(XT);
-    auto kern = csr_fused_cluster<XT, VT>;
-    DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    if (K > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return ISING_ERR_UNSUPPORTED;
-    }
-    const int64_t chunk = (c->max_inst_n + K - 1) / K;
-    int threads = static_cast<int>(std::min<int64_t>(1024, (chunk + 31) / 32 * 32));
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(K);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(static_cast<unsigned>(R * K), static_cast<unsigned>(c->n_inst));
-    cfg.blockDim = dim3(static_cast<unsigned>(threads));
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) != cudaSuccess || nclusters < 1) {
-        cudaGetLastError();
-        return ISING_ERR_UNSUPPORTED;
-    }
-    DOCH_CUDA(cudaLaunchKernelEx(&cfg, kern, x, static_cast<const int64_t *>(c->row_ptr),
-                                 static_cast<const int32_t *>(c->col), static_cast<const VT *>(c->val), h,
-                                 static_cast<const int64_t *>(c->n_inst > 1 ? c->inst_off : nullptr), c->n, R,
-                                 p.alpha_d, p.alpha_len, p.beta_d, iters, K));
-    return ISING_OK;
-}
-
-template <typename XT, typename VT>
-ising_status_t launch_fused(const ising_context *c, XT *x, int R, const XT *h,
-                            const ParamTabs &p, int iters, cudaStream_t st) {
-    for (int kmax = 16; kmax >= 2; kmax >>= 1) {
-        const int K = fused_cluster_k(c, R, kmax);
-        if (K < 2) break;
-        const ising_status_t s = launch_fused_cluster<XT, VT>(c, x, R, h, p, iters, K, st);
-        if (s != ISING_ERR_UNSUPPORTED) return s;
-        kmax = K;  // this size is not available: try the next smaller one
-    }
-    const size_t smem = 2 * static_cast<size_t>(c->max_inst_n) * sizeof(XT);
-    auto kern = csr_fused_kernel<XT, VT>;
-    DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(smem)));
-    int threads = 1024;
-    if (c->max_inst_n < 1024) threads = static_cast<int>(((c->max_inst_n + 31) / 32) * 32);
-    if (threads < 32) threads = 32;
-    dim3 grid(static_cast<unsigned>(R), static_cast<unsigned>(c->n_inst));
-    kern<<<grid, threads, smem, st>>>(x, c->row_ptr, c->col, static_cast<const VT *>(c->val), h,
-                                      c->n_inst > 1 ? c->inst_off : nullptr, c->n, R, p.alpha_d,
-                                      p.alpha_len, p.beta_d, iters);
-    DOCH_CUDA(cudaGetLastError());
-    return ISING_OK;
-}
-
-template <typename XT>
-ising_status_t fused_dispatch(const ising_context *c, XT *x, int R, const XT *h,
-                              const ParamTabs &p, int iters, cudaStream_t st) {
-    switch (c->jtype) {
-        case ISING_I8: return launch_fused<XT, int8_t>(c, x, R, h, p, iters, st);
-        case ISING_I32: return launch_fused<XT, int32_t>(c, x, R, h, p, iters, st);
-        case ISING_F32: return launch_fused<XT, float>(c, x, R, h, p, iters, st);
-        case ISING_F64: return launch_fused<XT, double>(c, x, R, h, p, iters, st);
-        default: return fail(ISING_ERR_UNSUPPORTED, "CSR value type not supported on the device");
-    }
-}
-
 }  // namespace
 
 size_t csr_fused_max_spins(int xtype) {
@@ -588,17 +392,6 @@ ising_status_t csr_step_traced(ising_context *c, const void *xi, void *xo, int x
     const ising_status_t s = csr_step_impl(c, xi, xo, xtype, R, p, k, c->partials.as<double>(), &blocks, st);
     if (s != ISING_OK) return s;
     return ham_fused_finish_launch(c->partials.as<double>(), blocks, R, alpha_k, beta, H_out, st);
-}
-
-ising_status_t csr_fused(const ising_context *c, void *x, int xtype, int R, const ParamTabs &p,
-                         int iters, cudaStream_t st) {
-    if (static_cast<size_t>(c->max_inst_n) > csr_fused_max_spins(xtype))
-        return ISING_ERR_UNSUPPORTED;
-    if (xtype == ISING_F64)
-        return fused_dispatch<double>(c, static_cast<double *>(x), R, c->h_f64, p, iters, st);
-    if (xtype == ISING_F32)
-        return fused_dispatch<float>(c, static_cast<float *>(x), R, c->h_f32, p, iters, st);
-    return ISING_ERR_UNSUPPORTED;
 }
 
 }  // namespace doch
