@@ -1647,7 +1647,8 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
         auto al = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
         const size_t A = al(static_cast<size_t>(c->n) * R * xel);        // one iterate
         const size_t G = al(static_cast<size_t>(c->n) * R * sizeof(float)); // one adjoint state
-        const size_t part_b = al(sizeof(double) * static_cast<size_t>(iters) * grid);
+        const size_t part_b = al(sizeof(double) * static_cast<size_t>(iters) *
+                                 static_cast<size_t>(std::max(grid, adjoint_small_blocks(c, R))));
         const size_t lpart_b = al(sizeof(double) * grid);
         const size_t out_b = al(sizeof(double) * (static_cast<size_t>(iters) + 1) + 8);
         const size_t wide_b = xtype == ISING_F64 ? A : 0;                   // FP64 copy of dL/dx0
@@ -1673,19 +1674,46 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
             if (m == seg_len(sg_i) && sg_i + 1 < S) return ck(sg_i + 1);
             return sg(m - 1);
         };
+        // instances that fit in shared memory: the forward pass, and each segment's recomputation, in one launch
+        bool small = backward_small(c, xtype, R);
+        auto run_small = [&](int k0, int steps, int every, void *to) {
+            return csr_small_run(c, ck(k0 / C), nullptr, xtype, R, p, k0, steps, SmallRecord{to, A, every}, st);
+        };
+        if (small) {
+            ising_status_t fs = S > 1 ? run_small(0, (S - 1) * C, C, ck(1)) : ISING_OK;
+            if (fs == ISING_OK) fs = run_small((S - 1) * C, seg_len(S - 1), 1, sg(0));
+            if (fs != ISING_OK && fs != ISING_ERR_UNSUPPORTED) return fs;
+            small = fs == ISING_OK;
+        }
         // forward: all segments, storing the checkpoints
-        for (int sg_i = 0; sg_i < S; ++sg_i)
+        for (int sg_i = 0; !small && sg_i < S; ++sg_i)
             for (int m = 1; m <= seg_len(sg_i); ++m)
                 DOCH_CHECK(csr_step(c, xs(sg_i, m - 1), xs(sg_i, m), xtype, R, p, sg_i * C + m - 1, st));
         // loss and g^N (x^N is the last iterate of the last segment)
         int gc = 0;
         DOCH_CHECK(csr_loss_w(c, xs(S - 1, seg_len(S - 1)), xtype, gbuf[gc], R, V, grid, lpart, zeros_d, st));
         const float inv_beta = static_cast<float>(1.0 / beta);
+        bool small_adjoint = small;
+        int pblocks = grid;  // partial sums per step in `part`
         for (int sg_i = S - 1; sg_i >= 0; --sg_i) {
             const int len = seg_len(sg_i);
-            if (sg_i < S - 1)  // the last segment's iterates are still in place from the forward pass
-                for (int m = 1; m < len; ++m)
-                    DOCH_CHECK(csr_step(c, xs(sg_i, m - 1), xs(sg_i, m), xtype, R, p, sg_i * C + m - 1, st));
+            if (sg_i < S - 1 && len > 1) {  // the last segment's iterates are still in place from the forward pass
+                if (small) DOCH_CHECK(run_small(sg_i * C, len - 1, 1, sg(0)));
+                else
+                    for (int m = 1; m < len; ++m)
+                        DOCH_CHECK(csr_step(c, xs(sg_i, m - 1), xs(sg_i, m), xtype, R, p, sg_i * C + m - 1, st));
+            }
+            if (small_adjoint) {
+                const AdjointSegment as{gbuf[gc], gbuf[1 - gc], ck(sg_i), sg(0), A, sg_i * C, len, part, zeros_d};
+                const ising_status_t rs = adjoint_small_run(c, as, xtype, R, p, &pblocks, st);
+                if (rs == ISING_OK) {
+                    gc = 1 - gc;
+                    continue;
+                }
+                if (rs != ISING_ERR_UNSUPPORTED || sg_i < S - 1) return rs;
+                small_adjoint = false;  // refused at the first segment: single steps for all of them
+                pblocks = grid;
+            }
             for (int m = len - 1; m >= 0; --m) {
                 const int k = sg_i * C + m;
                 DOCH_CHECK(csr_adjoint_step(c, gbuf[gc], xs(sg_i, m), xtype, gbuf[1 - gc], R, V,
@@ -1694,7 +1722,7 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
                 gc = 1 - gc;
             }
         }
-        DOCH_CHECK(adjoint_finish_launch(part, iters, grid, beta, lpart, grid, R, ga_d, loss_d, st));
+        DOCH_CHECK(adjoint_finish_launch(part, iters, pblocks, beta, lpart, grid, R, ga_d, loss_d, st));
         bool must_sync = false;
         auto put = [&](void *dst, const void *src, size_t bytes) -> ising_status_t {
             if (!dst) return ISING_OK;

@@ -40,6 +40,7 @@
 #include "csr_pipe.cuh"
 #include "hamsum.cuh"
 #include "internal.cuh"
+#include "root.cuh"
 
 namespace doch {
 namespace {
@@ -84,14 +85,6 @@ __device__ __forceinline__ void st(float *p, const float (&v)[V]) {
 #pragma unroll
     for (int k = 0; k < V; ++k) q[k] = v[k];
     *reinterpret_cast<T *>(p) = w;
-}
-
-// w = g / (3 x^2), 0 where x = 0: the fast division (within 2 ulp) for a normal
-// denominator below 2^126, the IEEE division for the rest
-__device__ __forceinline__ float dcbrt_weight(float g, float x) {
-    const float d = 3.0f * x * x;
-    if (d >= 0x1p-126f && d < 0x1p126f) return __fdividef(g, d);
-    return x == 0.0f ? 0.0f : g / d;
 }
 
 __device__ __forceinline__ double block_sum(double v) {

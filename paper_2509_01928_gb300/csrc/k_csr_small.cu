@@ -2,22 +2,26 @@
 // run in one launch,
 //   x'[i][r] = cbrt( ( sum_e val[e] x[col[e]][r] + alpha_b x[i][r] + h_i ) / beta_b ).
 //
-// One cluster of K CTAs (K = 16, 8, 4, 2 or 1) per (instance, replica). Every CTA keeps both
+// One cluster of K <= 16 CTAs per (instance, replica). Every CTA keeps both
 // copies of the pair's whole iterate, forms the rows of its share [q c, (q + 1) c), c = ceil(n_b / K),
-// and stores each new value into the next copy of all K CTAs (distributed shared memory); a
-// cluster barrier (about 400 clocks) ends each step. P threads share a row: each adds every P-th
+// and sends each new value to the next copy of all K CTAs (distributed shared memory), each of which
+// counts the bytes that arrive (about 650 clocks per step). P threads share a row: each adds every P-th
 // entry, a shuffle tree adds the P sums, and then one thread per row takes the cube root, in
 // whole warps. The couplings of a CTA's rows are copied to shared memory once per launch, already
-// in the iterate's type.
+// in the iterate's type (FP64 iterates and 8-bit couplings: the upper words of the FP64 values,
+// whose lower words are zero, 6 instead of 10 bytes an entry).
 //
-// Bound by FP64 arithmetic (2 lanes per clock and SM; an integer -> FP64 conversion costs as much
-// as an FP64 FMA): one FMA per entry and replica, the tree and nine operations per cube root. 800
-// spins, 38,000 entries, R = 8, FP64: 10.0 us per step with one thread per row, the couplings
-// converted at every use and CUDA's cbrt of a quotient, 3.7 us per step now; the arithmetic
-// alone takes about 0.9 us on the 128 SMs used.
+// Bound by FP64 arithmetic (half a lane per clock and SM partition, about 150 clocks from one operation
+// to the next that needs it; an integer -> FP64 conversion costs as much as an FMA): one FMA per entry
+// and replica, the tree and nine operations per cube root. 800 spins, 38,000 entries, R = 8, FP64, per
+// step: 10.0 us with one thread per row, the couplings converted at every use and CUDA's cbrt of a
+// quotient; 3.7 us per step with the couplings held in FP64; the arithmetic alone takes about 0.9 us on
+// the 128 SMs used. Of 7000 clocks the products take 4700, the update 1600 and the exchange 650.
 #include <algorithm>
 
+#include "hamsum.cuh"
 #include "internal.cuh"
+#include "mbar.cuh"
 #include "root.cuh"
 
 namespace doch {
@@ -38,21 +42,80 @@ __device__ __forceinline__ uint32_t cl_map(const void *p, uint32_t rank) {
                  : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void cl_store(uint32_t a, double v) {
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+// a value into a peer's shared memory; its bytes count on the peer's mbarrier when they are there
+__device__ __forceinline__ void cl_send(uint32_t a, double v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(a),
+                 "l"(__double_as_longlong(v)), "r"(bar)
+                 : "memory");
 }
-__device__ __forceinline__ void cl_store(uint32_t a, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+__device__ __forceinline__ void cl_send(uint32_t a, float v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a),
+                 "r"(__float_as_uint(v)), "r"(bar)
+                 : "memory");
 }
 
+// The exchange of a cluster's shares. Every CTA counts the bytes its peers send for step k on one of
+// two mbarriers (k even / odd). A peer sends step k + 1 only after this CTA's step k reached it whole,
+// which this CTA sends after it has received step k - 1: so two mbarriers, and two copies of the
+// iterate, are enough, and no cluster-wide barrier is needed. Waits are bounded (1 s): on expiry the
+// error word is set and the kernel ends at its closing cluster barrier.
+struct Exchange {
+    unsigned long long bar[2];
+    int abort_flag;
+};
+constexpr int kStaticSmem = 1024;  // at least the kernels' static shared memory
+
+__device__ __forceinline__ void exchange_init(Exchange &x) {  // before the opening cluster barrier
+    if (threadIdx.x == 0) {
+        mbar_init(&x.bar[0], 1);
+        mbar_init(&x.bar[1], 1);
+        x.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+}
+// step s (from 0): arm for `bytes` from the peers
+__device__ __forceinline__ void exchange_expect(Exchange &x, int s, uint32_t bytes) {
+    if (threadIdx.x == 0) mbar_expect_tx(&x.bar[s & 1], bytes);
+}
+template <typename T>
+__device__ __forceinline__ void exchange_send(Exchange &x, int s, T *slot, T v, int q, int K) {
+    for (int t = 1; t < K; ++t) {
+        const uint32_t to = static_cast<uint32_t>(q + t < K ? q + t : q + t - K);
+        cl_send(cl_map(slot, to), v, cl_map(&x.bar[s & 1], to));
+    }
+}
+// all threads: this CTA's own share is written and the peers' have arrived
+__device__ __forceinline__ bool exchange_wait(Exchange &x, int s, int K, int *err) {
+    if (K == 1) {
+        __syncthreads();
+        return true;
+    }
+    const bool ok = mbar_wait(&x.bar[s & 1], (s >> 1) & 1, err, &x.abort_flag);
+    return !__syncthreads_or(!ok);
+}
+
+// a coupling as held in shared memory
+template <typename XT, typename VT>
+struct Held {
+    using type = XT;
+    static __device__ __forceinline__ XT pack(VT v) { return static_cast<XT>(v); }
+    static __device__ __forceinline__ XT value(XT v) { return v; }
+};
+template <>
+struct Held<double, int8_t> {
+    using type = int;
+    static __device__ __forceinline__ int pack(int8_t v) { return __double2hiint(static_cast<double>(v)); }
+    static __device__ __forceinline__ double value(int v) { return __hiloint2double(v, 0); }
+};
+
 // Shared memory: cur | nxt (XT [nb] each) | z (XT [rows], P > 1 only), then, as far as there is room
-// for at least the shares it fits, val (XT [cap]) | row ranges (int [rows + 1]) | col (uint16 [cap])
+// for at least the shares it fits, val (Held [cap]) | row ranges (int [rows + 1]) | col (uint16 [cap])
 template <typename XT, int P>
 constexpr int64_t state_bytes(int64_t nb, int64_t rows) {
     return static_cast<int64_t>(sizeof(XT)) * (2 * nb + (P > 1 ? rows : 0)) + 16;
 }
-template <typename XT>
-constexpr int64_t entry_bytes() { return sizeof(XT) + sizeof(uint16_t); }
+template <typename XT, typename VT>
+constexpr int64_t entry_bytes() { return sizeof(typename Held<XT, VT>::type) + sizeof(uint16_t); }
 
 template <typename XT, typename VT, int P>
 __global__ void __launch_bounds__(1024)
@@ -60,8 +123,9 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
           const int32_t *__restrict__ col, const VT *__restrict__ val, const XT *__restrict__ h,
           const int64_t *__restrict__ inst_off, int64_t n, int R, const double *__restrict__ alpha_tab, int alpha_len,
           const double *__restrict__ beta_tab, int k0, int iters, int K, int rows_cap, int cap,
-          unsigned char *rec, size_t rec_stride, int rec_every) {
+          unsigned char *rec, size_t rec_stride, int rec_every, int *__restrict__ err) {
     extern __shared__ __align__(16) unsigned char small_smem[];
+    __shared__ Exchange ex;
     const int q = static_cast<int>(cl_rank());
     const int b = blockIdx.y, r = blockIdx.x / K;
     const int64_t lo = inst_off ? inst_off[b] : 0;
@@ -71,7 +135,8 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     const int i0 = min(nb, q * chunk), i1 = min(nb, i0 + chunk), rows = i1 - i0;
     XT *cur = reinterpret_cast<XT *>(small_smem), *nxt = cur + nb;
     XT *z = nxt + nb;
-    XT *lv = P > 1 ? z + rows_cap : z;
+    using Hd = Held<XT, VT>;
+    typename Hd::type *lv = reinterpret_cast<typename Hd::type *>(P > 1 ? z + rows_cap : z);
     int *lr = reinterpret_cast<int *>(lv + cap);
     uint16_t *lc = reinterpret_cast<uint16_t *>(lr + rows_cap + 1);
     for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = x_in[(lo + i) * R + r];
@@ -81,7 +146,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     if (local) {
         const int cnt = static_cast<int>(row_ptr[lo + i1] - e0);
         for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-            lv[e] = static_cast<XT>(val[e0 + e]);
+            lv[e] = Hd::pack(val[e0 + e]);
             lc[e] = static_cast<uint16_t>(col[e0 + e] - lo);
         }
     }
@@ -90,11 +155,13 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     const int sub = threadIdx.x % P;
     const int rl = threadIdx.x / P, rstep = blockDim.x / P;
     const int top = (rows + rstep - 1) / rstep * rstep;  // whole warps take part in the shuffles
+    exchange_init(ex);
     // every CTA of the cluster runs, and has loaded, before the first remote store
     if (K > 1) cl_sync();
     else __syncthreads();
     for (int k = 0; k < iters; ++k) {
         const XT a = static_cast<XT>(arow[alpha_len == 1 ? 0 : k0 + k]);
+        if (K > 1) exchange_expect(ex, k, static_cast<uint32_t>((nb - rows) * sizeof(XT)));
         const bool keep = rec && (k + 1) % rec_every == 0;
         XT *rp = reinterpret_cast<XT *>(rec + (keep ? static_cast<size_t>((k + 1) / rec_every - 1) : 0) * rec_stride);
         auto update = [&](int i, XT u) {  // row i of the share: the new value into every CTA's next copy
@@ -102,10 +169,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
             const XT hv = h ? __ldg(h + row) : XT(0);
             const XT v = root_newton(u + a * cur[i0 + i] + hv, root);
             nxt[i0 + i] = v;
-            for (int t = 1; t < K; ++t) {
-                const int to = q + t < K ? q + t : q + t - K;
-                cl_store(cl_map(nxt + i0 + i, static_cast<uint32_t>(to)), v);
-            }
+            exchange_send(ex, k, nxt + i0 + i, v, q, K);
             if (keep) rp[row * R + r] = v;
         };
         for (int i = rl; i < top; i += rstep) {
@@ -114,7 +178,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
                 if (local) {
                     const int f1 = lr[i + 1];
 #pragma unroll 4
-                    for (int e = lr[i] + sub; e < f1; e += P) acc += lv[e] * cur[lc[e]];
+                    for (int e = lr[i] + sub; e < f1; e += P) acc += Hd::value(lv[e]) * cur[lc[e]];
                 } else {
                     const int64_t f1 = __ldg(row_ptr + lo + i0 + i + 1);
                     for (int64_t e = __ldg(row_ptr + lo + i0 + i) + sub; e < f1; e += P)
@@ -133,22 +197,116 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
             __syncthreads();
             for (int i = threadIdx.x; i < rows; i += blockDim.x) update(i, z[i]);
         }
-        if (K > 1) cl_sync();  // the new values of every share are in every CTA; the old copy is free
-        else __syncthreads();
+        if (!exchange_wait(ex, k, K, err)) break;
         XT *t = cur;
         cur = nxt;
         nxt = t;
     }
     if (x_out)
         for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) x_out[(lo + i) * R + r] = cur[i];
+    if (K > 1) cl_sync();  // no CTA leaves while a peer may still send to it
 }
 
-// the cluster size: the largest K in {16, 8, 4, 2} (16 is a non-portable size) that leaves each CTA
-// at least 32 rows and keeps all pairs' clusters within the SMs; 1 when none does
-int cluster_k(const ising_context *c, int R, int kmax) {
-    for (int K = kmax; K >= 2; K >>= 1)
-        if (static_cast<int64_t>(c->n_inst) * R * K <= c->num_sms && c->max_inst_n >= 32LL * K) return K;
-    return 1;
+// Adjoint steps k0 + len - 1 .. k0 of one instance that fits in shared memory, in one launch: with
+// the adjoint state w^k (FP32) held as csr_small holds its iterate, a cluster per replica,
+//   g^k = (J w^k + alpha_k w^k) / beta,   w^(k-1) = g^k / (3 (x^k)^2)  (g^0 itself when k = 0),
+// and the partial sums of dL/dalpha_k = sum w^k x^k / beta of every CTA into part[k][gridDim.x]
+// (per thread FP64 for FP64 iterates, a compensated FP32 sum of split products for FP32 ones; FP64
+// across threads). x^(k0) is x_first and x^(k0 + m) = x_seg + (m - 1) stride. The next step's own x
+// is loaded, and the block's sum formed, before the wait for the peers' shares.
+template <typename XT, typename VT>
+__global__ void __launch_bounds__(1024)
+adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, const unsigned char *__restrict__ x_seg,
+              size_t stride, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+              const VT *__restrict__ val, int n, int R, const float *__restrict__ alpha_tab,
+              const float *__restrict__ inv_beta_tab, int k0, int len, int K, int rows_cap, int cap,
+              double *__restrict__ part, unsigned long long *__restrict__ zeros, int *__restrict__ err) {
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    __shared__ Exchange ex;
+    __shared__ double red[2][32];  // by the step's parity: thread 0 reads one while the next step fills the other
+    const int q = static_cast<int>(cl_rank());
+    const int r = blockIdx.x / K;
+    const int i0 = min(n, q * rows_cap), rows = min(n, i0 + rows_cap) - i0;
+    float *cur = reinterpret_cast<float *>(small_smem), *nxt = cur + n, *lv = nxt + n;
+    int *lr = reinterpret_cast<int *>(lv + cap);
+    uint16_t *lc = reinterpret_cast<uint16_t *>(lr + rows_cap + 1);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) cur[i] = w_in[static_cast<int64_t>(i) * R + r];
+    const int64_t e0 = row_ptr[i0];
+    const int cnt = static_cast<int>(row_ptr[i0 + rows] - e0);  // <= cap
+    for (int i = threadIdx.x; i <= rows; i += blockDim.x) lr[i] = static_cast<int>(row_ptr[i0 + i] - e0);
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+        lv[e] = static_cast<float>(val[e0 + e]);
+        lc[e] = static_cast<uint16_t>(col[e0 + e]);
+    }
+    const float inv_beta = inv_beta_tab[0];
+    auto iterate = [&](int m) {
+        return m == 0 ? x_first : reinterpret_cast<const XT *>(x_seg + static_cast<size_t>(m - 1) * stride);
+    };
+    const int64_t at = static_cast<int64_t>(i0 + threadIdx.x) * R + r;  // the thread's first row
+    const bool has = threadIdx.x < rows;
+    XT x_own = has ? iterate(len - 1)[at] : XT(0);
+    unsigned nz = 0;
+    exchange_init(ex);
+    if (K > 1) cl_sync();
+    else __syncthreads();
+    for (int m = len - 1; m >= 0; --m) {
+        const int k = k0 + m;
+        const float a = __ldg(alpha_tab + k);
+        const XT *xm = iterate(m);
+        const int s = len - 1 - m;
+        if (K > 1 && m > 0) exchange_expect(ex, s, static_cast<uint32_t>((n - rows) * sizeof(float)));
+        double ga = 0.0;
+        DotSum32 ga32;
+        for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+            const int64_t row = static_cast<int64_t>(i0 + i) * R + r;
+            const XT xc = i < static_cast<int>(blockDim.x) ? x_own : xm[row];
+            const int f1 = lr[i + 1];
+            float acc = 0.f;
+#pragma unroll 4
+            for (int e = lr[i]; e < f1; ++e) acc += lv[e] * cur[lc[e]];
+            const float wi = cur[i0 + i];
+            if constexpr (sizeof(XT) == 8) ga += static_cast<double>(wi) * xc;
+            else ga32.add(wi, xc);
+            const float g = (acc + a * wi) * inv_beta;
+            float out = g;
+            if (k > 0) {
+                nz += xc == XT(0);
+                out = dcbrt_weight(g, static_cast<float>(xc));
+            }
+            if (m == 0) {
+                w_out[row] = out;
+                continue;
+            }
+            nxt[i0 + i] = out;
+            exchange_send(ex, s, nxt + i0 + i, out, q, K);
+        }
+        if (has && m > 0) x_own = iterate(m - 1)[at];
+        if constexpr (sizeof(XT) == 4) ga = ga32.value();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+        if (threadIdx.x % 32 == 0) red[m & 1][threadIdx.x / 32] = ga;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int w = 0; w < static_cast<int>(blockDim.x / 32); ++w) t += red[m & 1][w];
+            part[static_cast<int64_t>(k) * gridDim.x + blockIdx.x] = t;
+        }
+        if (m > 0 && !exchange_wait(ex, s, K, err)) break;
+        float *t = cur;
+        cur = nxt;
+        nxt = t;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nz += __shfl_xor_sync(0xffffffffu, nz, o);
+    if (threadIdx.x % 32 == 0 && nz) atomicAdd(zeros, static_cast<unsigned long long>(nz));
+    if (K > 1) cl_sync();  // no CTA leaves while a peer may still send to it
+}
+
+// the largest cluster size worth trying: each CTA keeps at least 32 rows and all pairs' clusters have
+// an SM per CTA
+int cluster_max(const ising_context *c, int R) {
+    const int64_t pairs = static_cast<int64_t>(c->n_inst) * R;
+    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({16, c->num_sms / pairs, c->max_inst_n / 32})));
 }
 
 template <typename XT, typename VT, int P>
@@ -159,8 +317,8 @@ ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R
     if (state > optin) return ISING_ERR_UNSUPPORTED;
     // room for the couplings of the fullest share, as far as it goes (shares that need more read the CSR arrays)
     const int64_t left = optin - state - static_cast<int64_t>(sizeof(int)) * (chunk + 1);
-    const int64_t cap = left <= 0 ? -1 : std::min(left / entry_bytes<XT>(), std::min(c->max_row_nnz * chunk, c->nnz)) / 4 * 4;
-    const int smem = static_cast<int>(cap < 0 ? state : optin - left + cap * entry_bytes<XT>());
+    const int64_t cap = left <= 0 ? -1 : std::min(left / entry_bytes<XT, VT>(), std::min(c->max_row_nnz * chunk, c->nnz)) / 4 * 4;
+    const int smem = static_cast<int>(cap < 0 ? state : optin - left + cap * entry_bytes<XT, VT>());
     auto kern = csr_small<XT, VT, P>;
     DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     if (K > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
@@ -182,7 +340,7 @@ ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R
     cfg.numAttrs = 1;
     if (K > 1) {
         int nclusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) != cudaSuccess || nclusters < 1) {
+        if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) != cudaSuccess || nclusters < R * c->n_inst) {
             cudaGetLastError();
             return ISING_ERR_UNSUPPORTED;
         }
@@ -192,8 +350,63 @@ ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R
                                  static_cast<const int64_t *>(c->n_inst > 1 ? c->inst_off : nullptr), c->n, R,
                                  p.alpha_d, p.alpha_len, p.beta_d, k0, iters, K, static_cast<int>(chunk),
                                  static_cast<int>(cap), static_cast<unsigned char *>(rec.base), rec.stride,
-                                 rec.every));
+                                 rec.every, c->err_word));
     return ISING_OK;
+}
+
+// The adjoint in clusters of K CTAs; ISING_ERR_UNSUPPORTED where the state, or the couplings of the
+// fullest share, do not fit, or the clusters of all replicas do not run at once.
+template <typename XT, typename VT>
+ising_status_t launch_adjoint_k(const ising_context *c, const AdjointSegment &s, int R, const ParamTabs &p, int K,
+                                int64_t optin, cudaStream_t st) {
+    const int n = static_cast<int>(c->n), chunk = (n + K - 1) / K;
+    int64_t most = std::min(c->max_row_nnz * chunk, c->nnz);
+    most = (most + 3) / 4 * 4;
+    const int64_t smem = 8LL * n + 4 * (chunk + 1) + most * static_cast<int64_t>(sizeof(float) + sizeof(uint16_t));
+    if (smem > optin) return ISING_ERR_UNSUPPORTED;
+    auto kern = adjoint_small<XT, VT>;
+    DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    if (K > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return ISING_ERR_UNSUPPORTED;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(K);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(static_cast<unsigned>(R * K));
+    cfg.blockDim = dim3(static_cast<unsigned>(std::min(1024, (chunk + 31) / 32 * 32)));
+    cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (K > 1) {
+        int nclusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) != cudaSuccess || nclusters < R) {
+            cudaGetLastError();
+            return ISING_ERR_UNSUPPORTED;
+        }
+    }
+    DOCH_CUDA(cudaLaunchKernelEx(&cfg, kern, s.w_in, s.w_out, static_cast<const XT *>(s.x_first),
+                                 static_cast<const unsigned char *>(s.x_seg), s.stride,
+                                 static_cast<const int64_t *>(c->row_ptr), static_cast<const int32_t *>(c->col),
+                                 static_cast<const VT *>(c->val), n, R, p.alpha_f, p.inv_beta_f, s.k0, s.len, K, chunk,
+                                 static_cast<int>(most), s.part, s.zeros, c->err_word));
+    return ISING_OK;
+}
+
+template <typename XT>
+ising_status_t adjoint_dispatch_k(const ising_context *c, const AdjointSegment &s, int R, const ParamTabs &p, int K,
+                                  int64_t optin, cudaStream_t st) {
+    switch (c->jtype) {
+        case ISING_I8: return launch_adjoint_k<XT, int8_t>(c, s, R, p, K, optin, st);
+        case ISING_I32: return launch_adjoint_k<XT, int32_t>(c, s, R, p, K, optin, st);
+        case ISING_F32: return launch_adjoint_k<XT, float>(c, s, R, p, K, optin, st);
+        case ISING_F64: return launch_adjoint_k<XT, double>(c, s, R, p, K, optin, st);
+        default: return fail(ISING_ERR_UNSUPPORTED, "backward: coupling type");
+    }
 }
 
 template <typename XT, typename VT>
@@ -202,8 +415,11 @@ ising_status_t launch_small(const ising_context *c, const XT *x_in, XT *x_out, i
     int dev = 0, optin = 0;
     DOCH_CUDA(cudaGetDevice(&dev));
     DOCH_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    for (int kmax = 16;; kmax >>= 1) {
-        const int K = cluster_k(c, R, kmax);
+    optin -= kStaticSmem;
+    // the largest cluster whose copies for all pairs run at once (a cluster lies within one GPU processing
+    // cluster, so sizes that fill those badly drop out): 1500 spins at density 0.08, R = 20, FP64: 6 CTAs
+    // per pair
+    for (int K = cluster_max(c, R);; --K) {
         const int64_t chunk = (c->max_inst_n + K - 1) / K;
         // threads per row: four or two where a share is small and its rows are long enough to split (more
         // would spend as many FP64 additions on the tree as they take from the rows)
@@ -213,7 +429,6 @@ ising_status_t launch_small(const ising_context *c, const XT *x_in, XT *x_out, i
             : split && chunk <= 512 ? launch_k<XT, VT, 2>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st)
                                     : launch_k<XT, VT, 1>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st);
         if (s != ISING_ERR_UNSUPPORTED || K == 1) return s;
-        kmax = K;  // this size is not available: try the next smaller one
     }
 }
 
@@ -240,6 +455,36 @@ ising_status_t csr_small_run(const ising_context *c, const void *x_in, void *x_o
     if (xtype == ISING_F32)
         return dispatch_small<float>(c, static_cast<const float *>(x_in), static_cast<float *>(x_out), R, c->h_f32, p,
                                      k0, iters, rec, st);
+    return ISING_ERR_UNSUPPORTED;
+}
+
+// The adjoint's forward steps and adjoint steps run here for small instances with at least four CTAs
+// per replica. FP64: every instance that fits (bound by FP64 arithmetic on either path; single steps
+// add two launch latencies and 8 us of row latency each): 2000 spins, R = 8, 100 steps: 2.56 -> 1.35 ms;
+// 10,000 spins of degree 6, R = 16, 60 steps: 2.78 -> 2.18 ms. FP32: up to 6144 spins, past which the
+// stores of every new value into all CTAs (13 clocks a warp) cost more than single steps: 60 steps,
+// R = 4, 1000 spins: 1.21 -> 0.78 ms; R = 8, 6000 spins: 1.25 -> 1.13 ms; R = 16, 10,000 spins would go
+// from 1.26 to 1.56 ms.
+bool backward_small(const ising_context *c, int xtype, int R) {
+    return c->n_inst == 1 && c->n <= (xtype == ISING_F64 ? 65536 : 6144) &&
+           static_cast<size_t>(c->n) <= csr_fused_max_spins(xtype) && cluster_max(c, R) >= 4;
+}
+
+int adjoint_small_blocks(const ising_context *c, int R) { return R * cluster_max(c, R); }
+
+ising_status_t adjoint_small_run(const ising_context *c, const AdjointSegment &s, int xtype, int R, const ParamTabs &p,
+                                 int *blocks, cudaStream_t st) {
+    int dev = 0, optin = 0;
+    DOCH_CUDA(cudaGetDevice(&dev));
+    DOCH_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    optin -= kStaticSmem;
+    if (c->n_inst != 1 || c->n > 65536) return ISING_ERR_UNSUPPORTED;
+    for (int K = cluster_max(c, R); K >= 1; --K) {
+        const ising_status_t e = xtype == ISING_F64 ? adjoint_dispatch_k<double>(c, s, R, p, K, optin, st)
+                                                    : adjoint_dispatch_k<float>(c, s, R, p, K, optin, st);
+        *blocks = R * K;
+        if (e != ISING_ERR_UNSUPPORTED) return e;
+    }
     return ISING_ERR_UNSUPPORTED;
 }
 

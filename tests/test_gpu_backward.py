@@ -99,6 +99,28 @@ def test_adjoint_short_rows_mixed_degrees(R):
     assert _rel(gx, gx_r) <= 1e-3 and np.abs(gx - gx_r).max() <= 1e-3 * np.abs(gx_r).max()
 
 
+@pytest.mark.parametrize("n, R, iters, ckpt", [(36, 3, 5, 2), (130, 1, 9, 1), (1000, 2, 12, 50), (1003, 38, 6, 4),
+                                               (1003, 39, 6, 4), (6001, 5, 7, 3), (14400, 2, 4, 3)])
+def test_adjoint_of_small_instances(n, R, iters, ckpt):
+    """Instances whose iterate fits in shared memory run whole segments per launch: one CTA or a
+    cluster per replica, shares that do not divide n, segments of one step, more replicas than
+    clusters of four fit (single steps), and the largest FP64 iterates."""
+    g = I.regular_pm1(n + n % 2, 3, seed=n) if n > 6000 else short_rows_mixed(n + 200 + n % 2, seed=n)
+    x0 = I.x0_uniform(g.n, R, seed=87, dtype=np.float64)
+    a0, beta = O.alpha_beta(g, eta=1.0, method="wigner")
+    alpha = a0 * (1.0 + 0.1 * np.cos(np.arange(iters) / 3.0))
+    ga_r, gx_r, loss_r, z_r = O.backward(O.Problem(g), x0, alpha, beta, iters)
+    h = N.ising_create(N.Problem(g))
+    try:
+        ga, gx, loss, ze = _gpu_backward(h, x0, alpha, beta, iters, ckpt)
+    finally:
+        N.ising_destroy(h)
+    assert ze == z_r
+    assert loss == pytest.approx(loss_r, rel=1e-5)
+    assert _rel(ga, ga_r) <= 1e-3 and np.abs(ga - ga_r).max() <= 1e-3 * np.abs(ga_r).max()
+    assert _rel(gx, gx_r) <= 1e-3 and np.abs(gx - gx_r).max() <= 1e-3 * np.abs(gx_r).max()
+
+
 def test_adjoint_with_field_and_gaussian_couplings():
     g = I.regular_gauss(2000, 5, seed=82)
     hf = I.field_gauss(g.n, 0.1, seed=83)
