@@ -447,6 +447,8 @@ void destroy_ctx(ising_context *c) {
     cudaFree(c->err_word);
     if (c->err_host) cudaFreeHost(c->err_host);
     if (c->count_host) cudaFreeHost(c->count_host);
+    for (cudaEvent_t e : c->count_event)
+        if (e) cudaEventDestroy(e);
     cudaFree(c->batch_order);
     cudaFree(c->ell_col);
     cudaFree(c->ell_val);
@@ -1397,9 +1399,12 @@ ising_status_t ising_iterate_until(ising_handle_t h, void *x, int32_t xtype, int
             xd = c->stage_x.ptr;
             DOCH_CUDA(cudaMemcpyAsync(xd, x, xbytes, cudaMemcpyHostToDevice, st));
         }
+        const bool one_launch = until_ok(c, xd, xtype, R);  // a launch per step
+        if (one_launch) DOCH_CHECK(c->ping.ensure(xbytes));
         // work: result | partials | running | steps | stopped_now | n_running (256-byte aligned)
         auto al = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
-        const size_t o1 = al(xbytes), o2 = o1 + al(stop_partials_bytes(c, R)), o3 = o2 + al(sizeof(int) * pairs),
+        const size_t o1 = one_launch ? 0 : al(xbytes),
+                     o2 = o1 + al(one_launch ? until_partials_bytes(c, R) : stop_partials_bytes(c, R)), o3 = o2 + al(sizeof(int) * pairs),
                      o4 = o3 + al(sizeof(int32_t) * pairs), o5 = o4 + al(sizeof(int) * pairs), tot = o5 + 256;
         DOCH_CHECK(c->work.ensure(tot));
         unsigned char *wb = c->work.as<unsigned char>();
@@ -1410,7 +1415,9 @@ ising_status_t ising_iterate_until(ising_handle_t h, void *x, int32_t xtype, int
         s.steps = reinterpret_cast<int32_t *>(wb + o3);
         s.stopped_now = reinterpret_cast<int *>(wb + o4);
         s.n_running = reinterpret_cast<int *>(wb + o5);
-        {
+        if (one_launch) {
+            DOCH_CHECK(until_init(pairs, max_iters, s, st));
+        } else {
             std::vector<int> ones(pairs, 1), st0(pairs, max_iters);
             DOCH_CUDA(cudaMemcpyAsync(s.running, ones.data(), sizeof(int) * pairs, cudaMemcpyHostToDevice, st));
             DOCH_CUDA(cudaMemcpyAsync(s.steps, st0.data(), sizeof(int32_t) * pairs, cudaMemcpyHostToDevice, st));
@@ -1430,8 +1437,28 @@ ising_status_t ising_iterate_until(ising_handle_t h, void *x, int32_t xtype, int
                                              static_cast<float>(eps), s.steps);
         }
         if (rs != ISING_OK && rs != ISING_ERR_UNSUPPORTED) return rs;
-        if (rs == ISING_ERR_UNSUPPORTED) {
-            if (!c->count_host) DOCH_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->count_host), sizeof(int), 0));
+        if (one_launch) {
+            if (!c->count_host) DOCH_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->count_host), 2 * sizeof(int), 0));
+            for (cudaEvent_t &e : c->count_event)
+                if (!e) DOCH_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            void *buf[2] = {xd, c->ping.ptr};
+            constexpr int kPoll = 8;  // steps per copy of the running-pair count, read while the next steps run
+            int k = 0;
+            while (k < max_iters) {
+                const int chunk = k / kPoll;
+                for (const int end = std::min(max_iters, k + kPoll); k < end; ++k)
+                    DOCH_CHECK(until_step(c, buf[k & 1], buf[1 - (k & 1)], xtype, R, p, eps, k, s, st));
+                if (k == max_iters) break;
+                DOCH_CUDA(cudaMemcpyAsync(c->count_host + (chunk & 1), s.n_running, sizeof(int), cudaMemcpyDeviceToHost, st));
+                DOCH_CUDA(cudaEventRecord(c->count_event[chunk & 1], st));
+                if (chunk > 0) {
+                    DOCH_CUDA(cudaEventSynchronize(c->count_event[1 - (chunk & 1)]));
+                    if (c->count_host[1 - (chunk & 1)] == 0) break;
+                }
+            }
+            DOCH_CHECK(until_finish(c, xd, c->ping.ptr, xtype, R, eps, k, s, st));
+        } else if (rs == ISING_ERR_UNSUPPORTED) {
+            if (!c->count_host) DOCH_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->count_host), 2 * sizeof(int), 0));
             DOCH_CHECK(c->ping.ensure(xbytes));
             void *cur = xd, *nxt = c->ping.ptr;
             constexpr int kPoll = 8;  // steps between host checks of the running-pair count

@@ -3,9 +3,13 @@
 // of the row after it in flight while the current row's neighbours are gathered,
 // so a row waits for one round of memory latency instead of three
 // (row_ptr -> col -> gather).
+//
+// Also here: the vector loads and stores and the update of the CSR step kernels.
 #pragma once
 
 #include <cstdint>
+
+#include "cbrt.cuh"
 
 namespace doch {
 
@@ -33,6 +37,51 @@ __device__ __forceinline__ void pipe_first_batch(const int32_t *__restrict__ col
         js[t] = t < m ? __ldg(c + t) : 0;
         ws[t] = t < m ? static_cast<AT>(__ldg(v + t)) : AT(0);
     }
+}
+
+// The update of the step kernels, x = cbrt(z / beta) for z = (J x + alpha x + h)_i:
+// FP32 through the prescaled power-of-two cube root (cbrt.cuh; zs = 2^(3k) / beta,
+// xsc = 2^-k per instance), FP64 through cbrt(z / beta).
+template <typename T>
+__device__ __forceinline__ T step_update(T z, T beta, float zs, float xsc) {
+    if constexpr (sizeof(T) == 4) return cbrt_pow2(z * zs) * xsc;
+    else return cbrt(z / beta);
+}
+
+template <typename T, int V> struct VecOf;
+template <> struct VecOf<float, 1> { using type = float; };
+template <> struct VecOf<float, 2> { using type = float2; };
+template <> struct VecOf<float, 4> { using type = float4; };
+template <> struct VecOf<double, 1> { using type = double; };
+template <> struct VecOf<double, 2> { using type = double2; };
+
+template <typename T, int V>
+__device__ __forceinline__ void ldv(const T *p, T (&v)[V]) {
+    using VT = typename VecOf<T, V>::type;
+    const VT w = __ldg(reinterpret_cast<const VT *>(p));
+    const T *q = reinterpret_cast<const T *>(&w);
+#pragma unroll
+    for (int k = 0; k < V; ++k) v[k] = q[k];
+}
+
+// the same past L1: values that the kernel before this one wrote while this one was starting
+template <typename T, int V>
+__device__ __forceinline__ void ldv_cg(const T *p, T (&v)[V]) {
+    using VT = typename VecOf<T, V>::type;
+    const VT w = __ldcg(reinterpret_cast<const VT *>(p));
+    const T *q = reinterpret_cast<const T *>(&w);
+#pragma unroll
+    for (int k = 0; k < V; ++k) v[k] = q[k];
+}
+
+template <typename T, int V>
+__device__ __forceinline__ void stv(T *p, const T (&v)[V]) {
+    using VT = typename VecOf<T, V>::type;
+    VT w;
+    T *q = reinterpret_cast<T *>(&w);
+#pragma unroll
+    for (int k = 0; k < V; ++k) q[k] = v[k];
+    *reinterpret_cast<VT *>(p) = w;
 }
 
 }  // namespace doch

@@ -45,6 +45,16 @@ struct DotSum32 {
         c = ((t - s) - y) - e;
         s = t;
     }
+    // another sum: the rounding of s + o.s is recovered exactly and joins the low parts, whose own
+    // rounding is 2^-48 of the sum
+    __device__ __forceinline__ void merge(float os, float oc) {
+        const float t = s + os;
+        const float z = t - s;
+        const float e = (s - (t - z)) + (os - z);
+        const float lo = e - (c + oc);
+        s = t + lo;
+        c = (s - t) - lo;
+    }
     __device__ __forceinline__ double value() const { return static_cast<double>(s) - static_cast<double>(c); }
 };
 

@@ -25,15 +25,6 @@
 namespace doch {
 namespace {
 
-// The update of the step kernels, x = cbrt(z / beta) for z = (J x + alpha x + h)_i:
-// FP32 through the prescaled power-of-two cube root (cbrt.cuh; zs = 2^(3k) / beta,
-// xsc = 2^-k per instance), FP64 through cbrt(z / beta).
-template <typename T>
-__device__ __forceinline__ T step_update(T z, T beta, float zs, float xsc) {
-    if constexpr (sizeof(T) == 4) return cbrt_pow2(z * zs) * xsc;
-    else return cbrt(z / beta);
-}
-
 __device__ __forceinline__ int find_inst(const int64_t *__restrict__ off, int n_inst, int64_t i) {
     int lo = 0, hi = n_inst - 1;
     while (lo < hi) {
@@ -41,32 +32,6 @@ __device__ __forceinline__ int find_inst(const int64_t *__restrict__ off, int n_
         if (__ldg(off + mid) <= i) lo = mid; else hi = mid - 1;
     }
     return lo;
-}
-
-template <typename T, int V> struct VecOf;
-template <> struct VecOf<float, 1> { using type = float; };
-template <> struct VecOf<float, 2> { using type = float2; };
-template <> struct VecOf<float, 4> { using type = float4; };
-template <> struct VecOf<double, 1> { using type = double; };
-template <> struct VecOf<double, 2> { using type = double2; };
-
-template <typename T, int V>
-__device__ __forceinline__ void ldv(const T *p, T (&v)[V]) {
-    using VT = typename VecOf<T, V>::type;
-    const VT w = __ldg(reinterpret_cast<const VT *>(p));
-    const T *q = reinterpret_cast<const T *>(&w);
-#pragma unroll
-    for (int k = 0; k < V; ++k) v[k] = q[k];
-}
-
-template <typename T, int V>
-__device__ __forceinline__ void stv(T *p, const T (&v)[V]) {
-    using VT = typename VecOf<T, V>::type;
-    VT w;
-    T *q = reinterpret_cast<T *>(&w);
-#pragma unroll
-    for (int k = 0; k < V; ++k) q[k] = v[k];
-    *reinterpret_cast<VT *>(p) = w;
 }
 
 constexpr int kCsrBatch = 8;  // entries whose loads are issued together

@@ -1,0 +1,401 @@
+// DOCH steps with the stopping rule of Remark S2 for one CSR instance with short rows:
+//   x^(k+1) = T(x^k),  r^(k) = ||x^(k+1) - x^k||_2 / ||x^k||_2 per replica; a replica stops at the
+//   first k with r^(k) < eps and keeps x^(k+1).
+//
+// One launch per step. Its row blocks form x^(k+1) as csr_step_pipe_kernel does (the same sums in the
+// same order) and the sums of r^(k) from the values they hold; its first blocks decide r^(k-1) from
+// the sums that launch k - 1 left, one warp per replica, so that no launch waits for a reduction.
+// A stopped replica is no longer written. The decision of step k - 1 falls while launch k writes
+// x^(k+1) over x^(k-1), in the buffer that does not hold x^k: a replica that stops there keeps x^k in
+// buffer k mod 2, and later launches leave it alone. until_finish collects the buffers.
+//
+// Sums: per thread compensated FP32 of split products for FP32 iterates, merged across a block's
+// threads with the rounding of every merge kept (relative error below 2^-44 of these positive sums; an
+// FP64 operation holds an SM partition for 64 clocks a warp, and widening each warp's eight sums took
+// as long as the step), FP64 across blocks; FP64 throughout for FP64 iterates.
+//
+// Bound by the latency of the gathers, as the step. 100,000 spins of degree 3, R = 8, FP32, 200 steps:
+// 5.5 ms with four launches per step (step, norms, decision, copy), 2.4 ms so; 2000 spins of degree 8,
+// R = 3: 2.1 -> 0.8 ms.
+#include <algorithm>
+#include <cmath>
+
+#include "csr_pipe.cuh"
+#include "hamsum.cuh"
+#include "internal.cuh"
+
+namespace doch {
+namespace {
+
+constexpr int kUThreads = 256;
+constexpr int kUWarps = kUThreads / 32;
+constexpr int kUBatch = 4;  // entries of a row's first batch, loaded one row ahead
+
+// resident blocks per SM that the kernel is compiled for: FP32 sums take 16 registers more than the step
+// (four blocks: 2.40 -> 3.38 ms for the 192 steps above), FP64 steps gain from a third block (0.95 -> 0.86 ms
+// for 12,000 spins, R = 16)
+constexpr int kUBlocksPerSm = 3;
+
+// r < eps for r = sqrt(d) / sqrt(s), without the roots where the squares already tell
+__device__ __forceinline__ bool below(double d, double s, double eps) {
+    const double lim = eps * eps * s;
+    if (lim > 1e-290 && lim < 1e290) {
+        if (d > 1.0001 * lim) return false;
+        if (d < 0.9999 * lim) return true;
+    }
+    return sqrt(d) / sqrt(s) < eps;
+}
+
+// step k of pair t, whole warp: part[2 t + m][blocks] added in a fixed order
+__device__ void until_decide(const double *__restrict__ part, int blocks, double eps, int k, int t, int *running,
+                             int32_t *__restrict__ steps, int *n_running) {
+    const int lane = threadIdx.x & 31;
+    const double *p = part + static_cast<int64_t>(t) * 2 * blocks;
+    double d = 0.0, s = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < blocks; b += 32) {
+        d += p[b];
+        s += p[blocks + b];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        d += __shfl_xor_sync(0xffffffffu, d, o);
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    if (lane != 0 || !running[t] || !below(d, s, eps)) return;
+    steps[t] = k + 1;
+    __stcg(running + t, 0);
+    atomicSub(n_running, 1);
+}
+
+// grid: dblocks deciding blocks, then row blocks
+template <typename XT, typename VT, int V>
+__global__ void __launch_bounds__(kUThreads, kUBlocksPerSm)
+until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__restrict__ row_ptr,
+             const int32_t *__restrict__ col, const VT *__restrict__ val, const XT *__restrict__ h, int n, int R,
+             const XT *__restrict__ alpha_tab, const XT *__restrict__ beta_tab, const float *__restrict__ zs_tab,
+             const float *__restrict__ xs_tab, int dblocks, double eps, int k, double *__restrict__ part,
+             const double *__restrict__ part_before, int *running, int32_t *__restrict__ steps, int *n_running) {
+    const int blocks = static_cast<int>(gridDim.x) - dblocks, blk = static_cast<int>(blockIdx.x) - dblocks;
+    if (blk < 0) {
+        pdl_wait();
+        pdl_trigger();
+        const int t = static_cast<int>(blockIdx.x) * kUWarps + (threadIdx.x >> 5);
+        if (k > 0 && t < R) until_decide(part_before, blocks, eps, k - 1, t, running, steps, n_running);
+        return;
+    }
+    const int C = R / V;
+    const int rows_per_block = kUThreads / C;
+    const int ch = threadIdx.x % C;
+    const int rl = threadIdx.x / C;
+    const int S = blocks * rows_per_block;
+    int i = rl < rows_per_block ? blk * rows_per_block + rl : n;
+    int e0, e1, f0, f1;  // entry ranges of rows i and i + S
+    int32_t js[kUBatch];
+    XT ws[kUBatch];
+    pipe_row_range(row_ptr, i, n, e0, e1);
+    pipe_row_range(row_ptr, i + S, n, f0, f1);
+    pipe_first_batch<kUBatch>(col, val, e0, e1, js, ws);
+    pdl_wait();  // the couplings above are never written
+    pdl_trigger();
+    if (!__syncthreads_or(threadIdx.x == 0 && __ldcg(n_running) != 0)) return;  // every result is in place
+    const XT a = alpha_tab[0];
+    const XT bb = beta_tab[0];
+    float zs = 1.f, xsc = 1.f;
+    if constexpr (sizeof(XT) == 4) {
+        zs = zs_tab[0];
+        xsc = xs_tab[0];
+    }
+    // a flag lowered during this launch may or may not be seen: this launch's writes miss x^k either way
+    bool run[V], all = true, any = false;
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        run[q] = __ldcg(running + ch * V + q) != 0;
+        all = all && run[q];
+        any = any || run[q];
+    }
+    if (!any) i = n;
+    DotSum32 d32[V], s32[V];
+    double d64[V], s64[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) d64[q] = s64[q] = 0.0;
+    for (; i < n; i += S) {
+        const int cnt = e1 - e0 < kUBatch ? e1 - e0 : kUBatch;
+        XT xv[kUBatch][V];
+#pragma unroll
+        for (int t = 0; t < kUBatch; ++t)
+            if (t < cnt) ldv_cg<XT, V>(xi + static_cast<int64_t>(js[t]) * R + ch * V, xv[t]);
+        XT xs[V];
+        ldv_cg<XT, V>(xi + static_cast<int64_t>(i) * R + ch * V, xs);
+        const XT hi = h ? h[i] : XT(0);
+        // the next row's first batch and the range of the row after it
+        int32_t js2[kUBatch];
+        XT ws2[kUBatch];
+        pipe_first_batch<kUBatch>(col, val, f0, f1, js2, ws2);
+        int g0, g1;
+        pipe_row_range(row_ptr, i + 2 * S, n, g0, g1);
+        XT acc[V];
+#pragma unroll
+        for (int q = 0; q < V; ++q) acc[q] = XT(0);
+#pragma unroll
+        for (int t = 0; t < kUBatch; ++t)
+            if (t < cnt) {
+#pragma unroll
+                for (int q = 0; q < V; ++q) acc[q] += ws[t] * xv[t][q];
+            }
+#pragma unroll 4
+        for (int e = e0 + kUBatch; e < e1; ++e) {  // entries past the first batch, in entry order
+            const int64_t j = __ldg(col + e);
+            const XT w = static_cast<XT>(__ldg(val + e));
+            XT xr[V];
+            ldv_cg<XT, V>(xi + j * R + ch * V, xr);
+#pragma unroll
+            for (int q = 0; q < V; ++q) acc[q] += w * xr[q];
+        }
+        XT out[V];
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            out[q] = step_update(acc[q] + a * xs[q] + hi, bb, zs, xsc);
+            const XT e = out[q] - xs[q];
+            if constexpr (sizeof(XT) == 4) {
+                d32[q].add(e, e);
+                s32[q].add(xs[q], xs[q]);
+            } else {
+                d64[q] += e * e;
+                s64[q] += xs[q] * xs[q];
+            }
+        }
+        XT *to = xo + static_cast<int64_t>(i) * R + ch * V;
+        if (all) {
+            stv<XT, V>(to, out);
+        } else {
+#pragma unroll
+            for (int q = 0; q < V; ++q)
+                if (run[q]) to[q] = out[q];
+        }
+        e0 = f0;
+        e1 = f1;
+        f0 = g0;
+        f1 = g1;
+#pragma unroll
+        for (int t = 0; t < kUBatch; ++t) {
+            js[t] = js2[t];
+            ws[t] = ws2[t];
+        }
+    }
+    // the block's sums into part[2 (ch V + q) + m][blk]
+    __shared__ double red[8 * kUThreads];
+    if (C <= 32 && (C & (C - 1)) == 0) {  // a warp's lanes of one chunk are C apart
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = 2 * C * V;  // per <= 256
+        if constexpr (sizeof(XT) == 4) {
+            float2 *part32 = reinterpret_cast<float2 *>(red);  // [warp][ch V + q][m]
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                for (int o = 16; o >= C; o >>= 1) {
+                    d32[q].merge(__shfl_xor_sync(0xffffffffu, d32[q].s, o), __shfl_xor_sync(0xffffffffu, d32[q].c, o));
+                    s32[q].merge(__shfl_xor_sync(0xffffffffu, s32[q].s, o), __shfl_xor_sync(0xffffffffu, s32[q].c, o));
+                }
+                if (lane < C) {
+                    part32[warp * per + (lane * V + q) * 2] = make_float2(d32[q].s, d32[q].c);
+                    part32[warp * per + (lane * V + q) * 2 + 1] = make_float2(s32[q].s, s32[q].c);
+                }
+            }
+            __syncthreads();
+            if (static_cast<int>(threadIdx.x) < per) {
+                DotSum32 v;
+#pragma unroll
+                for (int w = 0; w < kUWarps; ++w) {
+                    const float2 u = part32[w * per + threadIdx.x];
+                    v.merge(u.x, u.y);
+                }
+                part[static_cast<int64_t>(threadIdx.x) * blocks + blk] = v.value();
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < V; ++q) {
+                for (int o = 16; o >= C; o >>= 1) {
+                    d64[q] += __shfl_xor_sync(0xffffffffu, d64[q], o);
+                    s64[q] += __shfl_xor_sync(0xffffffffu, s64[q], o);
+                }
+                if (lane < C) {
+                    red[warp * per + (lane * V + q) * 2] = d64[q];
+                    red[warp * per + (lane * V + q) * 2 + 1] = s64[q];
+                }
+            }
+            __syncthreads();
+            if (static_cast<int>(threadIdx.x) < per) {
+                double v[kUWarps];
+#pragma unroll
+                for (int w = 0; w < kUWarps; ++w) v[w] = red[w * per + threadIdx.x];
+                part[static_cast<int64_t>(threadIdx.x) * blocks + blk] =
+                    ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+            }
+        }
+        return;
+    }
+    for (int q = 0; q < V; ++q) {  // any C: a tree over the block's rows
+        double d = 0.0, s = 0.0;
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (j == q) {
+                if constexpr (sizeof(XT) == 4) {
+                    d = d32[j].value();
+                    s = s32[j].value();
+                } else {
+                    d = d64[j];
+                    s = s64[j];
+                }
+            }
+        red[threadIdx.x] = d;
+        red[kUThreads + threadIdx.x] = s;
+        __syncthreads();
+        int rows = rows_per_block;
+        while (rows > 1) {
+            const int half = (rows + 1) / 2;
+            if (rl + half < rows) {
+                red[threadIdx.x] += red[threadIdx.x + half * C];
+                red[kUThreads + threadIdx.x] += red[kUThreads + threadIdx.x + half * C];
+            }
+            __syncthreads();
+            rows = half;
+        }
+        if (rl == 0) {
+            part[static_cast<int64_t>((ch * V + q) * 2) * blocks + blk] = red[ch];
+            part[static_cast<int64_t>((ch * V + q) * 2 + 1) * blocks + blk] = red[kUThreads + ch];
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void until_init_kernel(int pairs, int max_iters, int *running, int32_t *steps, int *n_running) {
+    for (int t = threadIdx.x; t < pairs; t += blockDim.x) {
+        running[t] = 1;
+        steps[t] = max_iters;
+    }
+    if (threadIdx.x == 0) *n_running = pairs;
+}
+
+__global__ void __launch_bounds__(kUThreads)
+until_last_kernel(const double *__restrict__ part, int blocks, double eps, int k, int R, int *running,
+                  int32_t *__restrict__ steps, int *n_running) {
+    const int t = static_cast<int>(blockIdx.x) * kUWarps + (threadIdx.x >> 5);
+    if (t < R) until_decide(part, blocks, eps, k, t, running, steps, n_running);
+}
+
+// x^(steps) of the replicas that ended in the other buffer
+template <typename XT>
+__global__ void __launch_bounds__(kUThreads)
+until_collect(XT *__restrict__ xa, const XT *__restrict__ xb, int64_t count, int R, const int32_t *__restrict__ steps) {
+    for (int64_t t = static_cast<int64_t>(blockIdx.x) * kUThreads + threadIdx.x; t < count;
+         t += static_cast<int64_t>(gridDim.x) * kUThreads)
+        if (steps[t % R] & 1) xa[t] = xb[t];
+}
+
+// (the other buffer is an allocation of its own)
+int vec_width(const void *x, int xtype, int R) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(x);
+    if (xtype == ISING_F64) return R % 2 == 0 && a % 16 == 0 ? 2 : 1;
+    return R % 4 == 0 && a % 16 == 0 ? 4 : R % 2 == 0 && a % 8 == 0 ? 2 : 1;
+}
+
+int until_blocks(const ising_context *c, int C) {
+    const int64_t rows_per_block = kUThreads / C;
+    const int64_t cap = static_cast<int64_t>(c->num_sms) * kUBlocksPerSm;
+    return static_cast<int>(std::max<int64_t>(1, std::min((c->n + rows_per_block - 1) / rows_per_block, cap)));
+}
+
+double *partials_of(const ising_context *c, int R, int k, StopState &s) {
+    return s.partials + (k & 1) * (until_partials_bytes(c, R) / (2 * sizeof(double)));
+}
+
+template <typename XT, typename VT, int V>
+ising_status_t launch_until(const ising_context *c, const XT *xi, XT *xo, int R, const XT *h, const ParamTabs &p,
+                            double eps, int k, StopState &s, cudaStream_t st) {
+    const int C = R / V;
+    const int blocks = until_blocks(c, C);
+    const int dblocks = (R + kUWarps - 1) / kUWarps;
+    const XT *alpha = nullptr, *beta = nullptr;
+    if constexpr (sizeof(XT) == 8) {
+        alpha = p.alpha_d;
+        beta = p.beta_d;
+    } else {
+        alpha = p.alpha_f;
+        beta = p.inv_beta_f;
+    }
+    DOCH_CUDA(launch_chained(until_kernel<XT, VT, V>, dim3(static_cast<unsigned>(dblocks + blocks)), dim3(kUThreads), st,
+                             xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, static_cast<int>(c->n), R,
+                             alpha, beta, p.zscale_f, p.xscale_f, dblocks, eps, k, partials_of(c, R, k, s),
+                             partials_of(c, R, k + 1, s), s.running, s.steps, s.n_running));
+    return ISING_OK;
+}
+
+template <typename XT, int V>
+ising_status_t until_typed(const ising_context *c, const XT *xi, XT *xo, int R, const XT *h, const ParamTabs &p,
+                           double eps, int k, StopState &s, cudaStream_t st) {
+    switch (c->jtype) {
+        case ISING_I8: return launch_until<XT, int8_t, V>(c, xi, xo, R, h, p, eps, k, s, st);
+        case ISING_I32: return launch_until<XT, int32_t, V>(c, xi, xo, R, h, p, eps, k, s, st);
+        case ISING_F32: return launch_until<XT, float, V>(c, xi, xo, R, h, p, eps, k, s, st);
+        case ISING_F64: return launch_until<XT, double, V>(c, xi, xo, R, h, p, eps, k, s, st);
+        default: return fail(ISING_ERR_UNSUPPORTED, "CSR value type not supported on the device");
+    }
+}
+
+}  // namespace
+
+// the rows that csr_step_pipe_kernel takes, with a block per row chunk at least
+bool until_ok(const ising_context *c, const void *x, int xtype, int R) {
+    return c->format == ISING_FMT_CSR && c->n_inst == 1 && (xtype == ISING_F32 || xtype == ISING_F64) &&
+           R / vec_width(x, xtype, R) <= kUThreads && c->nnz <= static_cast<int64_t>(kPipeAvgDeg) * c->n &&
+           c->n < (int64_t(1) << 30) && c->nnz < (int64_t(1) << 30);
+}
+
+size_t until_partials_bytes(const ising_context *c, int R) {
+    return 2 * sizeof(double) * 2 * static_cast<size_t>(R) * static_cast<size_t>(c->num_sms) * kUBlocksPerSm;
+}
+
+ising_status_t until_init(int pairs, int max_iters, StopState &s, cudaStream_t st) {
+    until_init_kernel<<<1, 256, 0, st>>>(pairs, max_iters, s.running, s.steps, s.n_running);
+    DOCH_CUDA(cudaGetLastError());
+    return ISING_OK;
+}
+
+ising_status_t until_step(const ising_context *c, const void *cur, void *nxt, int xtype, int R, const ParamTabs &p,
+                          double eps, int k, StopState &s, cudaStream_t st) {
+    const int V = vec_width(k % 2 == 0 ? cur : nxt, xtype, R);
+    if (xtype == ISING_F64) {
+        const double *xi = static_cast<const double *>(cur);
+        double *xo = static_cast<double *>(nxt);
+        return V == 2 ? until_typed<double, 2>(c, xi, xo, R, c->h_f64, p, eps, k, s, st)
+                      : until_typed<double, 1>(c, xi, xo, R, c->h_f64, p, eps, k, s, st);
+    }
+    const float *xi = static_cast<const float *>(cur);
+    float *xo = static_cast<float *>(nxt);
+    return V == 4   ? until_typed<float, 4>(c, xi, xo, R, c->h_f32, p, eps, k, s, st)
+           : V == 2 ? until_typed<float, 2>(c, xi, xo, R, c->h_f32, p, eps, k, s, st)
+                    : until_typed<float, 1>(c, xi, xo, R, c->h_f32, p, eps, k, s, st);
+}
+
+ising_status_t until_finish(const ising_context *c, void *xa, const void *xb, int xtype, int R, double eps,
+                            int launched, StopState &s, cudaStream_t st) {
+    const int C = R / vec_width(xa, xtype, R);
+    if (launched > 0) {
+        until_last_kernel<<<(R + kUWarps - 1) / kUWarps, kUThreads, 0, st>>>(
+            partials_of(c, R, launched - 1, s), until_blocks(c, C), eps, launched - 1, R, s.running, s.steps,
+            s.n_running);
+        DOCH_CUDA(cudaGetLastError());
+    }
+    const int64_t count = c->n * R;
+    const unsigned blocks = static_cast<unsigned>(
+        std::max<int64_t>(1, std::min<int64_t>((count + kUThreads - 1) / kUThreads, 16LL * c->num_sms)));
+    if (xtype == ISING_F64)
+        until_collect<<<blocks, kUThreads, 0, st>>>(static_cast<double *>(xa), static_cast<const double *>(xb), count, R,
+                                                   s.steps);
+    else
+        until_collect<<<blocks, kUThreads, 0, st>>>(static_cast<float *>(xa), static_cast<const float *>(xb), count, R,
+                                                   s.steps);
+    DOCH_CUDA(cudaGetLastError());
+    return ISING_OK;
+}
+
+}  // namespace doch

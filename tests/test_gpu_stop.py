@@ -14,6 +14,7 @@ import oracle as O
 from paper_2509_01928_gb300 import _native as N
 from paper_2509_01928_gb300 import build as B
 from paper_2509_01928_gb300 import inputs as I
+from short_rows import short_rows_mixed
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -91,6 +92,55 @@ def test_stop_fp32_matches_oracle():
     x, steps = _run(J, x0, [alpha], [beta], 300, 1e-4, h=h)
     compared, _ = _compare(O.Problem(J, h), x0, alpha, beta, 300, 1e-4, x, steps, 1e-3, 1e-5)
     assert compared >= R - 1
+
+
+@pytest.mark.parametrize("n, R", [(30, 1), (300, 2), (1000, 3), (1002, 20), (5000, 64), (300, 130), (400, 256)])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_stop_one_launch_per_step(n, R, dtype):
+    """Short-row instances: replicas that stop at different steps, groups of lanes and of any other
+    number of threads per row, rows of every length, up to 256 threads a row."""
+    J = I.regular_gauss(n + n % 2, 3, seed=n + R) if n < 1000 else short_rows_mixed(n, seed=n)
+    f64 = dtype == "f64"
+    if J.val.dtype == np.float64 and not f64:
+        J.val = J.val.astype(np.float32)
+    x0 = I.x0_uniform(J.n, R, seed=315, dtype=np.float64 if f64 else np.float32)
+    alpha, beta = O.alpha_beta(J, eta=1.0, method="wigner")
+    eps = 1e-3
+    x, steps = _run(J, x0, [alpha], [beta], 60, eps)
+    _, ksteps, rtr = O.doch_until(O.Problem(J), x0.astype(np.float64), alpha, beta, 60, eps)
+    clear = np.array([np.all(np.abs(rtr[:ksteps[r], r] / eps - 1.0) > (1e-9 if f64 else 1e-2)) for r in range(R)])
+    assert clear.sum() >= R // 2 and np.array_equal(steps[clear], ksteps[clear])
+    # every replica holds the iterate of its own step count
+    hd = N.ising_create(N.Problem(J))
+    try:
+        for k in np.unique(steps):
+            xk = torch.from_numpy(x0.copy()).cuda()
+            N.ising_iterate(hd, xk, [alpha], [beta], int(k))
+            sel = steps == k
+            err = _rel(x[:, sel], xk.cpu().numpy()[:, sel].astype(np.float64))
+            if f64:
+                assert err.max() <= 1e-10
+            else:  # two FP32 kernels: components near zero take either sign now and then
+                assert np.median(err) <= 1e-5 and err.max() <= 0.1
+    finally:
+        N.ising_destroy(hd)
+
+
+def test_stop_one_launch_equals_steps():
+    """Where ising_iterate takes single steps too, the iterates agree bit for bit, in both buffers."""
+    J = short_rows_mixed(40010, seed=71)
+    x0 = I.x0_uniform(J.n, 12, seed=316)
+    alpha, beta = O.alpha_beta(J, eta=1.0, method="wigner")
+    x, steps = _run(J, x0, [alpha], [beta], 60, 2e-2)
+    assert len(np.unique(steps)) > 1
+    hd = N.ising_create(N.Problem(J))
+    try:
+        for k in np.unique(steps):
+            xk = torch.from_numpy(x0.copy()).cuda()
+            N.ising_iterate(hd, xk, [alpha], [beta], int(k))
+            assert np.array_equal(x[:, steps == k], xk.cpu().numpy()[:, steps == k])
+    finally:
+        N.ising_destroy(hd)
 
 
 def test_stop_batched_host_buffers_and_extremes():
