@@ -10,8 +10,18 @@
 #include <cstdint>
 
 #include "cbrt.cuh"
+#include "root.cuh"
 
 namespace doch {
+
+// a coupling in the arithmetic's type; 8-bit couplings reach FP64 through FP32 and a move of its fields
+// (root.cuh), an FP64 conversion costs as much as an FMA
+template <typename AT, typename VT>
+__device__ __forceinline__ AT coupling(VT v) { return static_cast<AT>(v); }
+template <>
+__device__ __forceinline__ double coupling<double, int8_t>(int8_t v) {
+    return v ? widen_normal(static_cast<float>(v)) : 0.0;
+}
 
 // entry range [e0, e1) of row i (empty past the last row), in the kernel's index type IT
 // (32-bit where the rows and entries allow it: fewer registers, more resident warps)
@@ -35,18 +45,29 @@ __device__ __forceinline__ void pipe_first_batch(const int32_t *__restrict__ col
 #pragma unroll
     for (int t = 0; t < B; ++t) {
         js[t] = t < m ? __ldg(c + t) : 0;
-        ws[t] = t < m ? static_cast<AT>(__ldg(v + t)) : AT(0);
+        ws[t] = t < m ? coupling<AT, VT>(__ldg(v + t)) : AT(0);
     }
 }
 
-// The update of the step kernels, x = cbrt(z / beta) for z = (J x + alpha x + h)_i:
-// FP32 through the prescaled power-of-two cube root (cbrt.cuh; zs = 2^(3k) / beta,
-// xsc = 2^-k per instance), FP64 through cbrt(z / beta).
+// The update of the step kernels, x = cbrt(z / beta) for z = (J x + alpha x + h)_i: FP32 through the
+// prescaled power-of-two cube root (cbrt.cuh; zs = 2^(3k) / beta, xsc = 2^-k per instance), FP64
+// through two Newton steps (root.cuh: 11 FP64 operations, against about 50 for z / beta and cbrt).
 template <typename T>
-__device__ __forceinline__ T step_update(T z, T beta, float zs, float xsc) {
-    if constexpr (sizeof(T) == 4) return cbrt_pow2(z * zs) * xsc;
-    else return cbrt(z / beta);
-}
+struct StepRoot;
+template <>
+struct StepRoot<float> {
+    float zs, xsc;
+    __device__ __forceinline__ StepRoot(const float *, const float *zs_tab, const float *xs_tab, int b)
+        : zs(__ldg(zs_tab + b)), xsc(__ldg(xs_tab + b)) {}
+    __device__ __forceinline__ float operator()(float z) const { return cbrt_pow2(z * zs) * xsc; }
+};
+template <>
+struct StepRoot<double> {
+    RootF64 p;
+    __device__ __forceinline__ StepRoot(const double *beta_tab, const float *, const float *, int b)
+        : p(make_root<double>(__ldg(beta_tab + b))) {}
+    __device__ __forceinline__ double operator()(double z) const { return root_newton(z, p); }
+};
 
 template <typename T, int V> struct VecOf;
 template <> struct VecOf<float, 1> { using type = float; };

@@ -77,6 +77,29 @@ __device__ __forceinline__ void ld(const double *p, double (&v)[V]) {
     }
 }
 
+// the same past L1 (values that the kernel before this one wrote while this one was starting)
+template <int V>
+__device__ __forceinline__ void ld_cg(const float *p, float (&v)[V]) {
+    using T = typename F4<V>::type;
+    const T w = __ldcg(reinterpret_cast<const T *>(p));
+    const float *q = reinterpret_cast<const float *>(&w);
+#pragma unroll
+    for (int k = 0; k < V; ++k) v[k] = q[k];
+}
+template <int V>
+__device__ __forceinline__ void ld_cg(const double *p, double (&v)[V]) {
+    if constexpr (V == 4) {
+        const double2 a = __ldcg(reinterpret_cast<const double2 *>(p));
+        const double2 b = __ldcg(reinterpret_cast<const double2 *>(p) + 1);
+        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    } else if constexpr (V == 2) {
+        const double2 a = __ldcg(reinterpret_cast<const double2 *>(p));
+        v[0] = a.x; v[1] = a.y;
+    } else {
+        v[0] = __ldcg(p);
+    }
+}
+
 template <int V>
 __device__ __forceinline__ void st(float *p, const float (&v)[V]) {
     using T = typename F4<V>::type;
@@ -200,16 +223,18 @@ adjoint_step_kernel(const float *__restrict__ w_in, const XT *__restrict__ x_cur
     pipe_row_range(row_ptr, i, n, e0, e1);
     pipe_row_range(row_ptr, i + S, n, f0, f1);
     pipe_first_batch<kBatchB>(col, val, e0, e1, js, ws);
+    pdl_wait();  // the couplings above are never written
+    pdl_trigger();
     for (; i < n; i += S) {
         const int cnt = e1 - e0 < kBatchB ? static_cast<int>(e1 - e0) : kBatchB;
         float wj[kBatchB][V];
 #pragma unroll
         for (int t = 0; t < kBatchB; ++t)
-            if (t < cnt) ld<V>(w_in + static_cast<int64_t>(js[t]) * R + ch * V, wj[t]);
+            if (t < cnt) ld_cg<V>(w_in + static_cast<int64_t>(js[t]) * R + ch * V, wj[t]);
         float wi[V];
         XT xc[V];
-        ld<V>(w_in + static_cast<int64_t>(i) * R + ch * V, wi);
-        ld<V>(x_cur + static_cast<int64_t>(i) * R + ch * V, xc);
+        ld_cg<V>(w_in + static_cast<int64_t>(i) * R + ch * V, wi);
+        ld_cg<V>(x_cur + static_cast<int64_t>(i) * R + ch * V, xc);
         // the next row's first batch and the range of the row after it
         int32_t js2[kBatchB];
         float ws2[kBatchB];
@@ -231,7 +256,7 @@ adjoint_step_kernel(const float *__restrict__ w_in, const XT *__restrict__ x_cur
             const int64_t j = __ldg(col + e);
             const float wv = static_cast<float>(__ldg(val + e));
             float wr[V];
-            ld<V>(w_in + j * R + ch * V, wr);
+            ld_cg<V>(w_in + j * R + ch * V, wr);
 #pragma unroll
             for (int q = 0; q < V; ++q) acc[q] += wv * wr[q];
         }
@@ -310,16 +335,15 @@ void launch_loss(const ising_context *c, const XT *x, float *w, int R, int grid,
 }
 
 template <typename XT, typename VT, int V>
-void launch_adj(const ising_context *c, const float *wi, const XT *xc, float *wo, int R, float a, float ib,
+cudaError_t launch_adj(const ising_context *c, const float *wi, const XT *xc, float *wo, int R, float a, float ib,
                 int final_step, int grid, double *part, unsigned long long *zeros, cudaStream_t st) {
     if (c->n < (int64_t(1) << 30) && c->nnz < (int64_t(1) << 30))  // 32-bit rows and entry offsets
-        adjoint_step_kernel<XT, VT, V, int><<<grid, kBThreads, 0, st>>>(
-            wi, xc, wo, c->row_ptr, c->col, static_cast<const VT *>(c->val), static_cast<int>(c->n), R, a, ib,
-            final_step, part, zeros);
-    else
-        adjoint_step_kernel<XT, VT, V, int64_t><<<grid, kBThreads, 0, st>>>(
-            wi, xc, wo, c->row_ptr, c->col, static_cast<const VT *>(c->val), c->n, R, a, ib, final_step, part,
-            zeros);
+        return launch_chained(adjoint_step_kernel<XT, VT, V, int>, dim3(static_cast<unsigned>(grid)), dim3(kBThreads), st,
+                              wi, xc, wo, c->row_ptr, c->col, static_cast<const VT *>(c->val), static_cast<int>(c->n), R,
+                              a, ib, final_step, part, zeros);
+    return launch_chained(adjoint_step_kernel<XT, VT, V, int64_t>, dim3(static_cast<unsigned>(grid)), dim3(kBThreads), st,
+                          wi, xc, wo, c->row_ptr, c->col, static_cast<const VT *>(c->val), c->n, R, a, ib, final_step,
+                          part, zeros);
 }
 
 template <typename XT, typename VT>
@@ -335,10 +359,9 @@ ising_status_t loss_v(const ising_context *c, const XT *x, float *w, int R, int 
 template <typename XT, typename VT>
 ising_status_t adj_v(const ising_context *c, const float *wi, const XT *xc, float *wo, int R, int V, float a,
                      float ib, int final_step, int grid, double *part, unsigned long long *zeros, cudaStream_t st) {
-    if (V == 4) launch_adj<XT, VT, 4>(c, wi, xc, wo, R, a, ib, final_step, grid, part, zeros, st);
-    else if (V == 2) launch_adj<XT, VT, 2>(c, wi, xc, wo, R, a, ib, final_step, grid, part, zeros, st);
-    else launch_adj<XT, VT, 1>(c, wi, xc, wo, R, a, ib, final_step, grid, part, zeros, st);
-    DOCH_CUDA(cudaGetLastError());
+    if (V == 4) DOCH_CUDA((launch_adj<XT, VT, 4>(c, wi, xc, wo, R, a, ib, final_step, grid, part, zeros, st)));
+    else if (V == 2) DOCH_CUDA((launch_adj<XT, VT, 2>(c, wi, xc, wo, R, a, ib, final_step, grid, part, zeros, st)));
+    else DOCH_CUDA((launch_adj<XT, VT, 1>(c, wi, xc, wo, R, a, ib, final_step, grid, part, zeros, st)));
     return ISING_OK;
 }
 

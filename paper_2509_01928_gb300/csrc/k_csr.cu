@@ -7,12 +7,17 @@
 // consecutive replicas of each neighbour x[j][*] (coalesced) and share the
 // row's col/val entries. FP32 steps take the cube root as the prescaled
 // power-of-two form of cbrt.cuh (the lattice, batched and dense kernels use the
-// same form), FP64 steps cbrt.
+// same form), FP64 steps two Newton steps (root.cuh): bound by FP64 arithmetic,
+// 100,000 spins of degree 8, R = 16, 200 steps with the stopping rule 21.9 -> 14.3 ms
+// against a quotient and cbrt.
 //
 // csr_step_pipe: the same step for short rows (at most kPipeAvgDeg entries per
 // row on average, one instance, no monitor). The grid is one resident wave and a
 // thread's loads are pipelined across its rows (csr_pipe.cuh); the sums are the
-// ones csr_step forms, in the same order.
+// ones csr_step forms, in the same order. A launch starts, and loads its first
+// couplings, while the one before it ends: a gradient of 20,000 spins of degree 3,
+// R = 8, FP32, 60 steps (170 short launches) 1.25 -> 0.93 ms, of 100,000 spins,
+// R = 64, 100 steps 5.53 -> 4.95 ms.
 //
 // Instances that fit in shared memory run all their steps in one launch (k_csr_small.cu).
 #include <algorithm>
@@ -57,23 +62,14 @@ csr_step_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *_
     const int ch = threadIdx.x % C;
     const int rl = threadIdx.x / C;
     HamSum<XT> hs[TRACE ? V : 1][4];
-    // the cube root's prescale (FP32): one instance's values are loaded once per thread -- two
-    // loads per row cost the S5 workload 2.5 % -- batched instances look theirs up per row
-    float zs0 = 1.f, xsc0 = 1.f;
-    if constexpr (sizeof(XT) == 4) {
-        zs0 = __ldg(zs_tab);
-        xsc0 = __ldg(xs_tab);
-    }
+    // the cube root's constants: one instance's are loaded once per thread -- two loads per row cost the
+    // S5 workload 2.5 % -- batched instances look theirs up per row
+    const StepRoot<XT> root0(beta_tab, zs_tab, xs_tab, 0);
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * rows_per_block + rl; rl < rows_per_block && i < n;
          i += static_cast<int64_t>(gridDim.x) * rows_per_block) {
         const int b = n_inst > 1 ? find_inst(inst_off, n_inst, i) : 0;
         const XT a = alpha_tab[static_cast<int64_t>(b) * alpha_len + ak];
-        const XT bb = beta_tab[b];
-        float zs = zs0, xsc = xsc0;
-        if (sizeof(XT) == 4 && n_inst > 1) {
-            zs = __ldg(zs_tab + b);
-            xsc = __ldg(xs_tab + b);
-        }
+        const StepRoot<XT> root = n_inst > 1 ? StepRoot<XT>(beta_tab, zs_tab, xs_tab, b) : root0;
         XT acc[V];
 #pragma unroll
         for (int q = 0; q < V; ++q) acc[q] = XT(0);
@@ -87,7 +83,7 @@ csr_step_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *_
 #pragma unroll
             for (int t = 0; t < kCsrBatch; ++t) {
                 js[t] = __ldg(col + e + t);
-                ws[t] = static_cast<XT>(__ldg(val + e + t));
+                ws[t] = coupling<XT, VT>(__ldg(val + e + t));
             }
             XT xv[kCsrBatch][V];
 #pragma unroll
@@ -99,7 +95,7 @@ csr_step_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *_
         }
         for (; e < e1; ++e) {
             const int64_t j = __ldg(col + e);
-            const XT w = static_cast<XT>(__ldg(val + e));
+            const XT w = coupling<XT, VT>(__ldg(val + e));
             XT xv[V];
             ldv<XT, V>(xi + j * R + ch * V, xv);
 #pragma unroll
@@ -109,7 +105,7 @@ csr_step_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *_
         ldv<XT, V>(xi + i * R + ch * V, xs);
         const XT hi = h ? h[i] : XT(0);
 #pragma unroll
-        for (int q = 0; q < V; ++q) out[q] = step_update(acc[q] + a * xs[q] + hi, bb, zs, xsc);
+        for (int q = 0; q < V; ++q) out[q] = root(acc[q] + a * xs[q] + hi);
         stv<XT, V>(xo + i * R + ch * V, out);
         if constexpr (TRACE) {
 #pragma unroll
@@ -159,12 +155,7 @@ csr_step_pipe_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64
                      const float *__restrict__ xs_tab) {
     const int C = R / V;
     const XT a = alpha_tab[alpha_len == 1 ? 0 : k];
-    const XT bb = beta_tab[0];
-    float zs = 1.f, xsc = 1.f;
-    if constexpr (sizeof(XT) == 4) {
-        zs = zs_tab[0];
-        xsc = xs_tab[0];
-    }
+    const StepRoot<XT> root(beta_tab, zs_tab, xs_tab, 0);
     const int rows_per_block = blockDim.x / C;
     const int ch = threadIdx.x % C;
     const int rl = threadIdx.x / C;
@@ -176,14 +167,16 @@ csr_step_pipe_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64
     pipe_row_range(row_ptr, i, n, e0, e1);
     pipe_row_range(row_ptr, i + S, n, f0, f1);
     pipe_first_batch<kPipeB>(col, val, e0, e1, js, ws);
+    pdl_wait();  // the couplings above are never written
+    pdl_trigger();
     for (; i < n; i += S) {
         const int cnt = e1 - e0 < kPipeB ? static_cast<int>(e1 - e0) : kPipeB;
         XT xv[kPipeB][V];
 #pragma unroll
         for (int t = 0; t < kPipeB; ++t)
-            if (t < cnt) ldv<XT, V>(xi + static_cast<int64_t>(js[t]) * R + ch * V, xv[t]);
+            if (t < cnt) ldv_cg<XT, V>(xi + static_cast<int64_t>(js[t]) * R + ch * V, xv[t]);
         XT xs[V];
-        ldv<XT, V>(xi + static_cast<int64_t>(i) * R + ch * V, xs);
+        ldv_cg<XT, V>(xi + static_cast<int64_t>(i) * R + ch * V, xs);
         const XT hi = h ? h[i] : XT(0);
         // the next row's first batch and the range of the row after it
         int32_t js2[kPipeB];
@@ -204,15 +197,15 @@ csr_step_pipe_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64
 #pragma unroll 4
         for (int e = e0 + kPipeB; e < e1; ++e) {
             const int64_t j = __ldg(col + e);
-            const XT w = static_cast<XT>(__ldg(val + e));
+            const XT w = coupling<XT, VT>(__ldg(val + e));
             XT xr[V];
-            ldv<XT, V>(xi + j * R + ch * V, xr);
+            ldv_cg<XT, V>(xi + j * R + ch * V, xr);
 #pragma unroll
             for (int q = 0; q < V; ++q) acc[q] += w * xr[q];
         }
         XT out[V];
 #pragma unroll
-        for (int q = 0; q < V; ++q) out[q] = step_update(acc[q] + a * xs[q] + hi, bb, zs, xsc);
+        for (int q = 0; q < V; ++q) out[q] = root(acc[q] + a * xs[q] + hi);
         stv<XT, V>(xo + static_cast<int64_t>(i) * R + ch * V, out);
         e0 = f0;
         e1 = f1;
@@ -263,14 +256,13 @@ struct StepTabs {
 };
 
 template <typename XT, typename VT, int V>
-void launch_step(const ising_context *c, const XT *xi, XT *xo, int R, const XT *h, const StepTabs<XT> &t, int k,
+cudaError_t launch_step(const ising_context *c, const XT *xi, XT *xo, int R, const XT *h, const StepTabs<XT> &t, int k,
                  double *hpart, cudaStream_t st) {
     const int C = R / V;
     if (use_pipe(c, C, hpart != nullptr)) {
-        csr_step_pipe_kernel<XT, VT, V><<<static_cast<unsigned>(pipe_blocks<XT>(c, C)), 256, 0, st>>>(
-            xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, static_cast<int>(c->n), R, t.alpha,
-            t.alpha_len, k, t.beta, t.zs, t.xsc);
-        return;
+        return launch_chained(csr_step_pipe_kernel<XT, VT, V>, dim3(static_cast<unsigned>(pipe_blocks<XT>(c, C))),
+                              dim3(256), st, xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h,
+                              static_cast<int>(c->n), R, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc);
     }
     const int blocks = step_blocks(c, C);
     const int threads = C <= 256 ? 256 : ((C + 31) / 32) * 32;
@@ -282,6 +274,7 @@ void launch_step(const ising_context *c, const XT *xi, XT *xo, int R, const XT *
         csr_step_kernel<XT, VT, V, false><<<static_cast<unsigned>(blocks), threads, 0, st>>>(
             xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, c->inst_off, c->n_inst,
             c->n, R, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc, nullptr);
+    return cudaGetLastError();
 }
 
 template <typename XT, int V>
@@ -290,13 +283,12 @@ ising_status_t dispatch_val(const ising_context *c, const XT *xi, XT *xo, int R,
     if (R / V > 1024) return fail(ISING_ERR_UNSUPPORTED, "CSR step: R / vector width must be <= 1024");
     if (hpart && R / V > 256) return ISING_ERR_UNSUPPORTED;  // the fused monitor needs one row per 256 threads
     switch (c->jtype) {
-        case ISING_I8: launch_step<XT, int8_t, V>(c, xi, xo, R, h, t, k, hpart, st); break;
-        case ISING_I32: launch_step<XT, int32_t, V>(c, xi, xo, R, h, t, k, hpart, st); break;
-        case ISING_F32: launch_step<XT, float, V>(c, xi, xo, R, h, t, k, hpart, st); break;
-        case ISING_F64: launch_step<XT, double, V>(c, xi, xo, R, h, t, k, hpart, st); break;
+        case ISING_I8: DOCH_CUDA((launch_step<XT, int8_t, V>(c, xi, xo, R, h, t, k, hpart, st))); break;
+        case ISING_I32: DOCH_CUDA((launch_step<XT, int32_t, V>(c, xi, xo, R, h, t, k, hpart, st))); break;
+        case ISING_F32: DOCH_CUDA((launch_step<XT, float, V>(c, xi, xo, R, h, t, k, hpart, st))); break;
+        case ISING_F64: DOCH_CUDA((launch_step<XT, double, V>(c, xi, xo, R, h, t, k, hpart, st))); break;
         default: return fail(ISING_ERR_UNSUPPORTED, "CSR value type not supported on the device");
     }
-    DOCH_CUDA(cudaGetLastError());
     return ISING_OK;
 }
 

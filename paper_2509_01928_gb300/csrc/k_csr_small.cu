@@ -210,16 +210,18 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
 // Adjoint steps k0 + len - 1 .. k0 of one instance that fits in shared memory, in one launch: with
 // the adjoint state w^k (FP32) held as csr_small holds its iterate, a cluster per replica,
 //   g^k = (J w^k + alpha_k w^k) / beta,   w^(k-1) = g^k / (3 (x^k)^2)  (g^0 itself when k = 0),
-// and the partial sums of dL/dalpha_k = sum w^k x^k / beta of every CTA into part[k][gridDim.x]
-// (per thread FP64 for FP64 iterates, a compensated FP32 sum of split products for FP32 ones; FP64
-// across threads). x^(k0) is x_first and x^(k0 + m) = x_seg + (m - 1) stride. The next step's own x
-// is loaded, and the block's sum formed, before the wait for the peers' shares.
+// and the partial sums of dL/dalpha_k = sum w^k x^k / beta of every CTA into part[k][gridDim.x]. A
+// row's products are summed with compensation (relative error of grad_x0 over twelve seeds of 2000 spins, R = 8,
+// FP64, 100 steps: 1.5e-6 on average, single steps 1.7e-6); the partial sums are per thread FP64 for FP64
+// iterates, compensated FP32 of split products for FP32 ones, and FP64 across threads. x^(k0) is
+// x_first and x^(k0 + m) = x_seg + (m - 1) stride. The next step's own x is loaded, and the block's sum
+// formed, before the wait for the peers' shares.
 template <typename XT, typename VT>
 __global__ void __launch_bounds__(1024)
 adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, const unsigned char *__restrict__ x_seg,
               size_t stride, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-              const VT *__restrict__ val, int n, int R, const float *__restrict__ alpha_tab,
-              const float *__restrict__ inv_beta_tab, int k0, int len, int K, int rows_cap, int cap,
+              const VT *__restrict__ val, int n, int R, const double *__restrict__ alpha_tab,
+              const double *__restrict__ beta_tab, int k0, int len, int K, int rows_cap, int cap,
               double *__restrict__ part, unsigned long long *__restrict__ zeros, int *__restrict__ err) {
     extern __shared__ __align__(16) unsigned char small_smem[];
     __shared__ Exchange ex;
@@ -238,7 +240,9 @@ adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, c
         lv[e] = static_cast<float>(val[e0 + e]);
         lc[e] = static_cast<uint16_t>(col[e0 + e]);
     }
-    const float inv_beta = inv_beta_tab[0];
+    // alpha and 1 / beta as a float and its remainder: their rounding would be the same at every step
+    const double ib = 1.0 / beta_tab[0];
+    const float ib_hi = static_cast<float>(ib), ib_lo = static_cast<float>(ib - ib_hi);
     auto iterate = [&](int m) {
         return m == 0 ? x_first : reinterpret_cast<const XT *>(x_seg + static_cast<size_t>(m - 1) * stride);
     };
@@ -251,7 +255,8 @@ adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, c
     else __syncthreads();
     for (int m = len - 1; m >= 0; --m) {
         const int k = k0 + m;
-        const float a = __ldg(alpha_tab + k);
+        const double ad = __ldg(alpha_tab + k);
+        const float a_hi = static_cast<float>(ad), a_lo = static_cast<float>(ad - a_hi);
         const XT *xm = iterate(m);
         const int s = len - 1 - m;
         if (K > 1 && m > 0) exchange_expect(ex, s, static_cast<uint32_t>((n - rows) * sizeof(float)));
@@ -261,17 +266,21 @@ adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, c
             const int64_t row = static_cast<int64_t>(i0 + i) * R + r;
             const XT xc = i < static_cast<int>(blockDim.x) ? x_own : xm[row];
             const int f1 = lr[i + 1];
-            float acc = 0.f;
-#pragma unroll 4
-            for (int e = lr[i]; e < f1; ++e) acc += lv[e] * cur[lc[e]];
             const float wi = cur[i0 + i];
+            DotSum32 acc;
+            acc.add(a_lo * wi);
+            acc.add(a_hi, wi);
+#pragma unroll 4
+            for (int e = lr[i]; e < f1; ++e) acc.add(lv[e], cur[lc[e]]);
             if constexpr (sizeof(XT) == 8) ga += static_cast<double>(wi) * xc;
             else ga32.add(wi, xc);
-            const float g = (acc + a * wi) * inv_beta;
+            const float z = acc.s - acc.c;
+            const float g = fmaf(z, ib_lo, z * ib_hi);
             float out = g;
             if (k > 0) {
                 nz += xc == XT(0);
-                out = dcbrt_weight(g, static_cast<float>(xc));
+                const float xf = static_cast<float>(xc);
+                out = xf == 0.0f ? 0.0f : g / (3.0f * xf * xf);
             }
             if (m == 0) {
                 w_out[row] = out;
@@ -392,7 +401,7 @@ ising_status_t launch_adjoint_k(const ising_context *c, const AdjointSegment &s,
     DOCH_CUDA(cudaLaunchKernelEx(&cfg, kern, s.w_in, s.w_out, static_cast<const XT *>(s.x_first),
                                  static_cast<const unsigned char *>(s.x_seg), s.stride,
                                  static_cast<const int64_t *>(c->row_ptr), static_cast<const int32_t *>(c->col),
-                                 static_cast<const VT *>(c->val), n, R, p.alpha_f, p.inv_beta_f, s.k0, s.len, K, chunk,
+                                 static_cast<const VT *>(c->val), n, R, p.alpha_d, p.beta_d, s.k0, s.len, K, chunk,
                                  static_cast<int>(most), s.part, s.zeros, c->err_word));
     return ISING_OK;
 }
@@ -458,16 +467,14 @@ ising_status_t csr_small_run(const ising_context *c, const void *x_in, void *x_o
     return ISING_ERR_UNSUPPORTED;
 }
 
-// The adjoint's forward steps and adjoint steps run here for small instances with at least four CTAs
-// per replica. FP64: every instance that fits (bound by FP64 arithmetic on either path; single steps
-// add two launch latencies and 8 us of row latency each): 2000 spins, R = 8, 100 steps: 2.56 -> 1.35 ms;
-// 10,000 spins of degree 6, R = 16, 60 steps: 2.78 -> 2.18 ms. FP32: up to 6144 spins, past which the
-// stores of every new value into all CTAs (13 clocks a warp) cost more than single steps: 60 steps,
-// R = 4, 1000 spins: 1.21 -> 0.78 ms; R = 8, 6000 spins: 1.25 -> 1.13 ms; R = 16, 10,000 spins would go
-// from 1.26 to 1.56 ms.
+// The adjoint's forward steps and adjoint steps run here for instances of at most 2048 spins with at
+// least four CTAs per replica; larger ones take single steps, whose launches overlap. Shared memory
+// against single steps, ms per gradient: FP64, 2000 spins, R = 8, 100 steps 1.37 / 1.49; 4000 spins, R = 4,
+// 60 steps 1.15 / 1.14, R = 16 1.44 / 1.22; FP32, 60 steps, 1000 spins, R = 16 0.75 / 0.87, 2000 spins, R = 8
+// 0.85 / 0.86, 6000 spins 1.10 / 0.88 (every new value is stored into all CTAs, 13 clocks a warp).
 bool backward_small(const ising_context *c, int xtype, int R) {
-    return c->n_inst == 1 && c->n <= (xtype == ISING_F64 ? 65536 : 6144) &&
-           static_cast<size_t>(c->n) <= csr_fused_max_spins(xtype) && cluster_max(c, R) >= 4;
+    return c->n_inst == 1 && c->n <= 2048 && static_cast<size_t>(c->n) <= csr_fused_max_spins(xtype) &&
+           cluster_max(c, R) >= 4;
 }
 
 int adjoint_small_blocks(const ising_context *c, int R) { return R * cluster_max(c, R); }

@@ -100,12 +100,7 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
     pdl_trigger();
     if (!__syncthreads_or(threadIdx.x == 0 && __ldcg(n_running) != 0)) return;  // every result is in place
     const XT a = alpha_tab[0];
-    const XT bb = beta_tab[0];
-    float zs = 1.f, xsc = 1.f;
-    if constexpr (sizeof(XT) == 4) {
-        zs = zs_tab[0];
-        xsc = xs_tab[0];
-    }
+    const StepRoot<XT> root(beta_tab, zs_tab, xs_tab, 0);
     // a flag lowered during this launch may or may not be seen: this launch's writes miss x^k either way
     bool run[V], all = true, any = false;
 #pragma unroll
@@ -146,7 +141,7 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
 #pragma unroll 4
         for (int e = e0 + kUBatch; e < e1; ++e) {  // entries past the first batch, in entry order
             const int64_t j = __ldg(col + e);
-            const XT w = static_cast<XT>(__ldg(val + e));
+            const XT w = coupling<XT, VT>(__ldg(val + e));
             XT xr[V];
             ldv_cg<XT, V>(xi + j * R + ch * V, xr);
 #pragma unroll
@@ -155,7 +150,7 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
         XT out[V];
 #pragma unroll
         for (int q = 0; q < V; ++q) {
-            out[q] = step_update(acc[q] + a * xs[q] + hi, bb, zs, xsc);
+            out[q] = root(acc[q] + a * xs[q] + hi);
             const XT e = out[q] - xs[q];
             if constexpr (sizeof(XT) == 4) {
                 d32[q].add(e, e);

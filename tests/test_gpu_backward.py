@@ -100,12 +100,12 @@ def test_adjoint_short_rows_mixed_degrees(R):
 
 
 @pytest.mark.parametrize("n, R, iters, ckpt", [(36, 3, 5, 2), (130, 1, 9, 1), (1000, 2, 12, 50), (1003, 38, 6, 4),
-                                               (1003, 39, 6, 4), (6001, 5, 7, 3), (14400, 2, 4, 3)])
+                                               (1003, 39, 6, 4), (1848, 5, 7, 3), (1850, 2, 4, 3)])
 def test_adjoint_of_small_instances(n, R, iters, ckpt):
     """Instances whose iterate fits in shared memory run whole segments per launch: one CTA or a
     cluster per replica, shares that do not divide n, segments of one step, more replicas than
-    clusters of four fit (single steps), and the largest FP64 iterates."""
-    g = I.regular_pm1(n + n % 2, 3, seed=n) if n > 6000 else short_rows_mixed(n + 200 + n % 2, seed=n)
+    clusters of four fit (single steps), and both sides of 2048 spins."""
+    g = short_rows_mixed(n + 200 + n % 2, seed=n)
     x0 = I.x0_uniform(g.n, R, seed=87, dtype=np.float64)
     a0, beta = O.alpha_beta(g, eta=1.0, method="wigner")
     alpha = a0 * (1.0 + 0.1 * np.cos(np.arange(iters) / 3.0))
