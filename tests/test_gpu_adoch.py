@@ -22,6 +22,7 @@ import oracle as O
 from paper_2509_01928_gb300 import _native as N
 from paper_2509_01928_gb300 import build as B
 from paper_2509_01928_gb300 import inputs as I
+from short_rows import short_rows_mixed
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -181,3 +182,41 @@ def test_adoch_rejects_dense():
             N.ising_iterate_adoch(hd, x, [1.0], [1.0], 3, 2)
     finally:
         N.ising_destroy(hd)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("graph, R", [("csr", 1), ("csr", 3), ("csr", 20), ("csr", 256), ("csr", 300), ("ragged", 1),
+                                      ("ragged", 4), ("two_rows", 2)])
+def test_adoch_any_replica_count(graph, R, dtype):
+    """The general step: threads over rows and replicas for any number of replicas, rows of every
+    length, ragged and degenerate lattices; x and every clear decision against the oracle on the
+    device's own decisions, the first and last H against Eq. Hamilton."""
+    h = None
+    if graph == "csr":
+        J = short_rows_mixed(402, seed=9)
+        h = I.field_gauss(J.n, 0.1, seed=10).astype(np.float32).astype(np.float64)
+    else:
+        J = I.torus_pm1(*((7, 13) if graph == "ragged" else (2, 9)), seed=11)
+    f64 = dtype == "f64"
+    x0 = I.x0_uniform(J.n, R, seed=12, dtype=np.float64 if f64 else np.float32)
+    alpha, beta = O.alpha_beta(J, eta=1.0, method="wigner")
+    iters = 7
+    hd = N.ising_create(N.Problem(J, h if h is None else h.astype(np.float32)))
+    try:
+        x = torch.from_numpy(x0.copy()).cuda()
+        acc = torch.zeros(iters, R, dtype=torch.int8, device="cuda")
+        H = torch.zeros(iters + 1, R, dtype=torch.float64, device="cuda")
+        N.ising_iterate_adoch(hd, x, [alpha], [beta], iters, 3, accepted=acc, H_trace=H)
+        x, acc, H = x.cpu().numpy().astype(np.float64), acc.cpu().numpy(), H.cpu().numpy()
+    finally:
+        N.ising_destroy(hd)
+    P = O.Problem(J, h)
+    ref, _, margin = O.adoch(P, x0.astype(np.float64), alpha, beta, iters, 3, decisions=acc, margins=True)
+    tie = 1e-10 if f64 else 1e-4
+    assert np.array_equal(acc[np.abs(margin) > tie], (margin >= 0).astype(np.int8)[np.abs(margin) > tie])
+    H0 = np.array([O.hamiltonian(P, x0[:, r:r + 1].astype(np.float64), alpha, beta)[0] for r in range(R)])
+    Hn = np.array([O.hamiltonian(P, x[:, r:r + 1], alpha, beta)[0] for r in range(R)])
+    assert np.allclose(H[0], H0, rtol=1e-10 if f64 else 1e-5) and np.allclose(H[-1], Hn, rtol=1e-10)
+    err = np.linalg.norm(x - ref, axis=0) / np.linalg.norm(ref, axis=0)
+    # FP32: seven steps of one rounding each, amplified where a component passes near zero
+    assert np.median(err) <= (1e-12 if f64 else 1e-5) and err.max() <= (1e-9 if f64 else 1e-2)
