@@ -17,7 +17,11 @@
 //   X  : replica-major [kblocks][R_pad][64] BF16 with the same swizzle, so
 //        the rows r0 .. r0+N-1 of one K block are one contiguous N x 128 B
 //        image; spins >= n are zero.
-// Tiles: one CTA per (128 rows of J) x (N = up to 256 replicas).
+// Tiles: one CTA per (128 rows of J) x (N = up to 256 replicas), or a cluster of S <= 8 CTAs that
+// share the tile's K blocks where the tiles alone leave SMs idle (split_of): each CTA puts its partial
+// accumulator in its shared memory, and CTA s adds the S partials of its share of the columns, in
+// order, through distributed shared memory and finishes them. 2000 spins, R = 100 (16 tiles): 21.5 us
+// per step with 16 CTAs, 13.7 us with clusters of 6.
 //
 // Pipeline per CTA (256 threads):
 //   warp 0, one lane: producer. K-block kb (64 columns of J = 64 spins of
@@ -41,6 +45,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -72,6 +77,7 @@ struct DenseSmem {
     alignas(8) unsigned long long conv[kS];             // ternary: A tile expanded
     alignas(8) unsigned long long jfull[kJStages];      // ternary: packed tile landed
     alignas(8) unsigned long long jempty[kJStages];     // ternary: packed tile read
+    alignas(16) int qsum[4][256];  // energy terms of the tile's four row groups per column
     alignas(8) unsigned long long acc_ready;
     uint32_t tmem_base;
     int abort_flag;
@@ -170,12 +176,25 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(bar)) : "memory");
 }
 
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a float at `own`'s offset in the shared memory of CTA `rank` of the cluster
+__device__ __forceinline__ float cluster_load(const float *own, uint32_t rank) {
+    uint32_t a;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr(own)), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
 // BF16 bits of a 2-bit ternary code: 0 -> 0, 1 -> +1, 2 -> -1 (3 unused -> 0)
 __device__ __forceinline__ uint32_t tern_bf16(uint32_t code) {
     return code == 1 ? 0x3F80u : (code == 2 ? 0xBF80u : 0u);
 }
 
-// MODE 0: DOCH step into Xt_out. MODE 1: energy partials q_r into q_out (int64).
+// MODE 0: DOCH step into Xt_out. MODE 1: energy partials q_r of every row tile into q_out [row tile][R] (int64).
 // TERN: J is stored as packed 2-bit codes (entries in {-1, 0, +1}); warps 4-7
 // expand each K block into BF16 and store it in tensor memory (columns a_col +
 // 32 s for stage s), from where the MMA reads A; shared memory then carries
@@ -184,7 +203,7 @@ template <int MODE, bool TERN>
 __global__ void __launch_bounds__(kThreadsTC, 1)
 dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ xt_in,
                 __nv_bfloat16 *__restrict__ xt_out, const float *__restrict__ h, int n, int kblocks, int R,
-                int R_pad, int n_tile, uint32_t tmem_cols, uint32_t a_col, float alpha, float zscale,
+                int R_pad, int n_tile, uint32_t tmem_cols, uint32_t a_col, int split, float alpha, float zscale,
                 float xscale,
                 long long *__restrict__ q_out, int *__restrict__ err) {
     extern __shared__ unsigned char smem_raw[];
@@ -194,12 +213,16 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     Smem &sm = *reinterpret_cast<Smem *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * kBM;
+    const int m_tile = blockIdx.x / split, rank = blockIdx.x % split;
+    const int m_tiles = gridDim.x / split;
+    const int m0 = m_tile * kBM;
+    // this CTA's K blocks: k_count from k_first
+    const int k_first = kblocks * rank / split, k_count = kblocks * (rank + 1) / split - k_first;
     const int r0 = blockIdx.y * n_tile;
     // bytes of J per K block: a BF16 tile, or a packed ternary tile expanded on chip
     constexpr uint32_t a_bytes = TERN ? kTernTile : kBM * kBK * 2;
     const uint32_t b_bytes = static_cast<uint32_t>(n_tile) * kBK * 2;
-    const unsigned char *a_src = static_cast<const unsigned char *>(jt) + static_cast<size_t>(blockIdx.x) * kblocks * a_bytes;
+    const unsigned char *a_src = static_cast<const unsigned char *>(jt) + static_cast<size_t>(m_tile) * kblocks * a_bytes;
     const __nv_bfloat16 *b_src = xt_in + static_cast<size_t>(r0) * kBK;
     volatile int *abort_flag = &sm.abort_flag;
 
@@ -235,12 +258,13 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     // any moment the CTAs stream different parts of J (equal 4 MB-aligned
     // offsets in lockstep would queue on the same DRAM channels) and read
     // different blocks of X from L2. Sum order only changes FP32 rounding.
-    const int kb0 = static_cast<int>(static_cast<int64_t>(blockIdx.x) * kblocks / gridDim.x);
+    const int kb0 = static_cast<int>(static_cast<int64_t>(m_tile) * k_count / m_tiles);
     if (warp == 0 && lane == 0) {
-        for (int it = 0; it < kblocks; ++it) {
+        for (int it = 0; it < k_count; ++it) {
             const int s = it % kStages;
             int kb = kb0 + it;
-            if (kb >= kblocks) kb -= kblocks;
+            if (kb >= k_count) kb -= k_count;
+            kb += k_first;
             if (it >= kStages && !mbar_wait(&sm.empty[s], ((it / kStages) - 1) & 1, err, abort_flag)) break;
             if (TERN) {
                 mbar_expect_tx(&sm.full[s], b_bytes);
@@ -254,7 +278,7 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     } else if (warp == 1 && lane == 0) {
         const uint32_t idesc = idesc_bf16(kBM, n_tile);
         bool ok = true;
-        for (int it = 0; it < kblocks; ++it) {
+        for (int it = 0; it < k_count; ++it) {
             const int s = it % kStages;
             // ternary: A is ready when the converters arrived on conv[s]; B when full[s] completed
             if ((TERN && !mbar_wait(&sm.conv[s], (it / kStages) & 1, err, abort_flag)) ||
@@ -282,10 +306,11 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
         }
     } else if (TERN && warp == 3 && lane == 0) {
         // producer of the packed ternary tiles (2 KB each), kJStages ahead
-        for (int it = 0; it < kblocks; ++it) {
+        for (int it = 0; it < k_count; ++it) {
             const int p = it % kJStages;
             int kb = kb0 + it;
-            if (kb >= kblocks) kb -= kblocks;
+            if (kb >= k_count) kb -= k_count;
+            kb += k_first;
             if (it >= kJStages && !mbar_wait(&sm.jempty[p], ((it / kJStages) - 1) & 1, err, abort_flag)) break;
             mbar_expect_tx(&sm.jfull[p], a_bytes);
             bulk_load(sm.jp[p], a_src + static_cast<size_t>(kb) * a_bytes, a_bytes, &sm.jfull[p]);
@@ -298,7 +323,7 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
         // waits are made warp-uniform: tcgen05.st is a .sync.aligned instruction.
         const int t = threadIdx.x - 128;
         const uint32_t a_lane = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + a_col;
-        for (int it = 0; it < kblocks; ++it) {
+        for (int it = 0; it < k_count; ++it) {
             const int s = it % kStages, p = it % kJStages;
             if (!__all_sync(0xffffffffu, mbar_wait(&sm.jfull[p], (it / kJStages) & 1, err, abort_flag))) break;
             const uint4 codes = *reinterpret_cast<const uint4 *>(sm.jp[p] + 16 * t);
@@ -324,42 +349,76 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
         const int row = m0 + 32 * q + lane;
         // warp-uniform decision: tcgen05.ld below is a .sync.aligned warp instruction
         const bool ok = __all_sync(0xffffffffu, mbar_wait_idle(&sm.acc_ready, 0, err, abort_flag) && !*abort_flag);
-        if (ok) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const float hv = (h && row < n) ? h[row] : 0.f;
-            for (int c0 = 32 * half; c0 < n_tile; c0 += 64) {
-                float acc[32];
-                tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, acc);
-                if (MODE == 0) {
-                    float xo[32];
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) {  // all loads first
-                        const int r = r0 + c0 + k;
-                        xo[k] = (row < n && r < R) ? __bfloat162float(xt_in[xs_index(r, row, R_pad)]) : 0.f;
-                    }
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) {
-                        const int r = r0 + c0 + k;
-                        if (row < n && r < R) {
-                            const float z = (acc[k] + alpha * xo[k] + hv) * zscale;
-                            xt_out[xs_index(r, row, R_pad)] = __float2bfloat16_rn(cbrt_pow2(z) * xscale);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) {
-                        const int r = r0 + c0 + k;
-                        long long contrib = 0;
-                        if (row < n && r < R) {
-                            const float s = __bfloat162float(xt_in[xs_index(r, row, R_pad)]);
-                            contrib = static_cast<long long>(s) * static_cast<long long>(acc[k]);
-                        }
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) contrib += __shfl_xor_sync(0xffffffffu, contrib, o);
-                        if (lane == 0 && r < R && contrib != 0) atomicAdd(reinterpret_cast<unsigned long long *>(q_out + r),
-                                                                      static_cast<unsigned long long>(contrib));
-                    }
+        const float hv = (h && row < n) ? h[row] : 0.f;
+        if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        // the product (J X)_(row, r) of column c = r - r0: the new iterate, or the energy term
+        auto finish = [&](int c, float u, float x) {
+            const int r = r0 + c;
+            if (MODE == 0) {
+                if (row < n && r < R) {
+                    const float z = (u + alpha * x + hv) * zscale;
+                    xt_out[xs_index(r, row, R_pad)] = __float2bfloat16_rn(cbrt_pow2(z) * xscale);
                 }
+            } else {  // |s u| < 2^24: a warp's 32 terms add in 32 bits
+                const int sum = __reduce_add_sync(0xffffffffu, row < n && r < R ? static_cast<int>(x * u) : 0);
+                if (lane == 0) sm.qsum[q][c] = sum;
+            }
+        };
+        auto state = [&](int c) {
+            const int r = r0 + c;
+            return row < n && r < R ? __bfloat162float(xt_in[xs_index(r, row, R_pad)]) : 0.f;
+        };
+        if (split == 1) {
+            if (ok)
+                for (int c0 = 32 * half; c0 < n_tile; c0 += 64) {
+                    float acc[32], xo[32];
+                    tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, acc);
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) xo[k] = state(c0 + k);  // all loads first
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) finish(c0 + k, acc[k], xo[k]);  // columns c < 256
+                }
+        } else {
+            // partial accumulators [column][128 rows] over the B ring, which every MMA has left
+            float *partial = reinterpret_cast<float *>(sm.b);
+            if (ok)
+                for (int c0 = 32 * half; c0 < n_tile; c0 += 64) {
+                    float acc[32];
+                    tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, acc);
+#pragma unroll
+                    for (int k = 0; k < 32; ++k)
+                        if (c0 + k < n_tile) partial[(c0 + k) * kBM + 32 * q + lane] = acc[k];
+                }
+            const int c1 = n_tile * (rank + 1) / split;
+            constexpr int kCols = 4;  // columns in flight per thread
+            cluster_sync();
+            for (int c = n_tile * rank / split + half; c < c1; c += 2 * kCols) {
+                float u[kCols], xo[kCols];
+#pragma unroll
+                for (int j = 0; j < kCols; ++j) {
+                    u[j] = 0.f;
+                    xo[j] = c + 2 * j < c1 ? state(c + 2 * j) : 0.f;
+                }
+                for (int t = 0; t < split; ++t)
+#pragma unroll
+                    for (int j = 0; j < kCols; ++j)
+                        if (c + 2 * j < c1) u[j] += cluster_load(partial + (c + 2 * j) * kBM + 32 * q + lane, t);
+#pragma unroll
+                for (int j = 0; j < kCols; ++j)
+                    if (c + 2 * j < c1) finish(c + 2 * j, u[j], xo[j]);
+            }
+            cluster_sync();  // no CTA leaves while a peer reads its partials
+        }
+        if (MODE == 1) {  // the tile's terms per replica: q_out[row tile][R]
+            __syncthreads();
+            const int r = r0 + threadIdx.x;
+            const bool mine = split == 1 || (static_cast<int>(threadIdx.x) >= n_tile * rank / split &&
+                                             static_cast<int>(threadIdx.x) < n_tile * (rank + 1) / split);
+            if (static_cast<int>(threadIdx.x) < n_tile && r < R && mine) {
+                long long t = 0;
+#pragma unroll
+                for (int w = 0; w < 4; ++w) t += sm.qsum[w][threadIdx.x];
+                q_out[static_cast<size_t>(m_tile) * R + r] = t;
             }
         }
     }
@@ -386,50 +445,55 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     }
 }
 
-// x [n][R] (caller layout, BF16) <-> the swizzled replica-major layout
-__global__ void to_replica_major(const __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ xt, int n,
-                                 int R, int R_pad) {
-    __shared__ __nv_bfloat16 tile[32][33];
-    const int i0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int i = i0 + k, r = r0 + threadIdx.x;
-        tile[k][threadIdx.x] = (i < n && r < R) ? x[static_cast<size_t>(i) * R + r] : __float2bfloat16_rn(0.f);
+// x [n][R] (caller layout, BF16) <-> the swizzled replica-major layout; a block takes one K block
+// (64 spins) x 32 replicas
+constexpr int kTR = 32;
+
+// SPIN: +1 / -1 of iterates of any supported type (sign(0) = +1); otherwise BF16 as it is. Padding
+// (spins >= n, replicas >= R) is written as zero. Grid (kblocks, ceil(R_pad / 32)).
+template <typename XT, bool SPIN>
+__global__ void __launch_bounds__(256)
+to_replica_major(const XT *__restrict__ x, __nv_bfloat16 *__restrict__ xt, int n, int R, int R_pad) {
+    __shared__ __nv_bfloat16 tile[kTR][kBK + 2];  // [replica][spin]
+    const int i0 = blockIdx.x * kBK, r0 = blockIdx.y * kTR;
+    for (int k = threadIdx.x; k < kBK * kTR; k += 256) {
+        const int i = i0 + k / kTR, r = r0 + k % kTR;
+        float v = 0.f;
+        if (i < n && r < R) {
+            const XT w = x[static_cast<size_t>(i) * R + r];
+            if constexpr (sizeof(XT) == 2) v = __bfloat162float(w);
+            else v = static_cast<float>(w);
+            if (SPIN) v = v >= 0.f ? 1.f : -1.f;
+        }
+        tile[k % kTR][k / kTR] = __float2bfloat16_rn(v);
     }
     __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int r = r0 + k, i = i0 + threadIdx.x;
-        if (r < R && i < n) xt[xs_index(r, i, R_pad)] = tile[threadIdx.x][k];
+    const int r = r0 + threadIdx.x / 8, c = threadIdx.x % 8;  // 16 bytes of a replica's 64 spins
+    if (r < R_pad) {
+        uint4 v;
+        unsigned *w = &v.x;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            w[e] = *reinterpret_cast<const unsigned *>(&tile[threadIdx.x / 8][8 * c + 2 * e]);
+        *reinterpret_cast<uint4 *>(xt + xs_index(r, i0 + 8 * c, R_pad)) = v;
     }
 }
 
-__global__ void from_replica_major(const __nv_bfloat16 *__restrict__ xt, __nv_bfloat16 *__restrict__ x, int n,
-                                   int R, int R_pad) {
-    __shared__ __nv_bfloat16 tile[32][33];
-    const int i0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int r = r0 + k, i = i0 + threadIdx.x;
-        tile[k][threadIdx.x] = (r < R && i < n) ? xt[xs_index(r, i, R_pad)] : __float2bfloat16_rn(0.f);
+__global__ void __launch_bounds__(256)
+from_replica_major(const __nv_bfloat16 *__restrict__ xt, __nv_bfloat16 *__restrict__ x, int n, int R, int R_pad) {
+    __shared__ __nv_bfloat16 tile[kTR][kBK + 2];
+    const int i0 = blockIdx.x * kBK, r0 = blockIdx.y * kTR;
+    const int r = r0 + threadIdx.x / 8, c = threadIdx.x % 8;
+    if (r < R_pad) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(xt + xs_index(r, i0 + 8 * c, R_pad));
+        const unsigned *w = &v.x;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) *reinterpret_cast<unsigned *>(&tile[threadIdx.x / 8][8 * c + 2 * e]) = w[e];
     }
     __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int i = i0 + k, r = r0 + threadIdx.x;
-        if (i < n && r < R) x[static_cast<size_t>(i) * R + r] = tile[threadIdx.x][k];
-    }
-}
-
-// spins (BF16 +1/-1, sign(0) = +1) of iterates of any supported type, replica-major
-template <typename XT>
-__global__ void spins_replica_major(const XT *__restrict__ x, __nv_bfloat16 *__restrict__ st, int n, int R,
-                                    int R_pad) {
-    const int64_t total = static_cast<int64_t>(n) * R;
-    for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < total;
-         t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t i = t / R;
-        const int r = static_cast<int>(t - i * R);
-        float v;
-        if constexpr (sizeof(XT) == 2) v = __bfloat162float(x[t]);
-        else v = static_cast<float>(x[t]);
-        st[xs_index(r, static_cast<int>(i), R_pad)] = __float2bfloat16_rn(v >= 0.f ? 1.f : -1.f);
+    for (int k = threadIdx.x; k < kBK * kTR; k += 256) {
+        const int i = i0 + k / kTR, q = r0 + k % kTR;
+        if (i < n && q < R) x[static_cast<size_t>(i) * R + q] = tile[k % kTR][k / kTR];
     }
 }
 
@@ -445,13 +509,19 @@ __global__ void field_dot_spins(const __nv_bfloat16 *__restrict__ st, const int6
                                                   static_cast<unsigned long long>(acc));
 }
 
-__global__ void dense_energy_finish(const long long *__restrict__ q, const long long *__restrict__ hs,
+// one warp per replica: the row tiles' terms
+__global__ void dense_energy_finish(const long long *__restrict__ q_tiles, int m_tiles, const long long *__restrict__ hs,
                                     long long j_sum, int R, int64_t *E_i, int64_t *cut_i, double *E_d,
                                     double *cut_d) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const long long E = -(q[r] / 2) - hs[r];
-    const long long cut = -((j_sum - q[r]) / 2);
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
+    if (r >= R) return;  // whole warps
+    long long q = 0;
+    for (int t = lane; t < m_tiles; t += 32) q += q_tiles[static_cast<size_t>(t) * R + r];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if (lane != 0) return;
+    const long long E = -(q / 2) - hs[r];
+    const long long cut = -((j_sum - q) / 2);
     if (E_i) E_i[r] = E;
     if (cut_i) cut_i[r] = cut;
     if (E_d) E_d[r] = static_cast<double>(E);
@@ -495,11 +565,30 @@ ising_status_t launch_dense(const ising_context *c, const DenseGeom &g, const __
     auto kern = c->dense_ternary ? dense_tc_kernel<MODE, true> : dense_tc_kernel<MODE, false>;
     const size_t smem = c->dense_ternary ? smem_bytes<true>() : smem_bytes<false>();
     DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    dim3 grid(static_cast<unsigned>(g.m_tiles), static_cast<unsigned>(g.r_tiles));
-    kern<<<grid, kThreadsTC, smem, st>>>(c->dense, xt_in, xt_out, h, g.n,
-                                                 g.kblocks, g.R, g.R_pad, g.n_tile, g.tmem_cols, g.a_col, alpha,
-                                                 zscale, xscale, q_out, c->err_word);
-    DOCH_CUDA(cudaGetLastError());
+    // K blocks shared by up to 8 CTAs (the portable cluster size) while all tiles' clusters run at once
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(kThreadsTC);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const int tiles = g.m_tiles * g.r_tiles;
+    int split = std::max(1, std::min({8, c->num_sms / tiles, g.kblocks}));
+    for (;; --split) {
+        attr[0].val.clusterDim.x = static_cast<unsigned>(split);
+        cfg.gridDim = dim3(static_cast<unsigned>(g.m_tiles * split), static_cast<unsigned>(g.r_tiles));
+        int clusters = 0;
+        if (split == 1) break;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= tiles) break;
+        cudaGetLastError();
+    }
+    DOCH_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<const void *>(c->dense), xt_in, xt_out, h, g.n, g.kblocks, g.R,
+                                 g.R_pad, g.n_tile, g.tmem_cols, g.a_col, split, alpha, zscale, xscale, q_out,
+                                 c->err_word));
     return ISING_OK;
 }
 
@@ -512,9 +601,10 @@ ising_status_t dense_iterate(ising_context *c, void *x, int R, const double *alp
     DOCH_CHECK(c->work.ensure(2 * xt_bytes));
     __nv_bfloat16 *xt[2] = {c->work.as<__nv_bfloat16>(),
                             reinterpret_cast<__nv_bfloat16 *>(c->work.as<unsigned char>() + xt_bytes)};
-    DOCH_CUDA(cudaMemsetAsync(c->work.ptr, 0, 2 * xt_bytes, st));
-    dim3 tb(32, 8), tg((g.n + 31) / 32, (R + 31) / 32);
-    to_replica_major<<<tg, tb, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), xt[0], g.n, R, g.R_pad);
+    if (g.n % kBK != 0 || R != g.R_pad)  // the steps write spins < n and replicas < R only
+        DOCH_CUDA(cudaMemsetAsync(xt[1], 0, xt_bytes, st));
+    const dim3 tg(static_cast<unsigned>(g.kblocks), static_cast<unsigned>((g.R_pad + kTR - 1) / kTR));
+    to_replica_major<__nv_bfloat16, false><<<tg, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), xt[0], g.n, R, g.R_pad);
     DOCH_CUDA(cudaGetLastError());
     // cube root on (z 2^(3k)) / beta, rescaled by 2^-k (exact powers of two, k from beta)
     const double inv_beta = 1.0 / beta;
@@ -527,7 +617,7 @@ ising_status_t dense_iterate(ising_context *c, void *x, int R, const double *alp
         DOCH_CHECK(launch_dense<0>(c, g, xt[cur], xt[1 - cur], c->h_f32, a, zscale, xscale, nullptr, st));
         cur = 1 - cur;
     }
-    from_replica_major<<<tg, tb, 0, st>>>(xt[cur], static_cast<__nv_bfloat16 *>(x), g.n, R, g.R_pad);
+    from_replica_major<<<tg, 256, 0, st>>>(xt[cur], static_cast<__nv_bfloat16 *>(x), g.n, R, g.R_pad);
     DOCH_CUDA(cudaGetLastError());
     return ISING_OK;
 }
@@ -536,19 +626,17 @@ ising_status_t dense_energy(ising_context *c, const void *x, int xtype, int R, i
                             double *E_d, double *cut_d, cudaStream_t st) {
     const DenseGeom g = geometry(c, R);
     const size_t st_bytes = static_cast<size_t>(g.R_pad) * g.kblocks * kBK * 2;
-    DOCH_CHECK(c->partials.ensure(st_bytes + 2 * sizeof(long long) * R + 256));
+    DOCH_CHECK(c->partials.ensure(st_bytes + sizeof(long long) * R * (static_cast<size_t>(g.m_tiles) + 1) + 256));
     __nv_bfloat16 *sp = c->partials.as<__nv_bfloat16>();
     long long *q = reinterpret_cast<long long *>(c->partials.as<unsigned char>() + ((st_bytes + 255) & ~size_t(255)));
-    long long *hs = q + R;
-    DOCH_CUDA(cudaMemsetAsync(c->partials.ptr, 0, c->partials.bytes, st));
-    const int64_t total = static_cast<int64_t>(g.n) * R;
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > 16LL * c->num_sms) blocks = 16LL * c->num_sms;
+    long long *hs = q + static_cast<size_t>(g.m_tiles) * R;
+    DOCH_CUDA(cudaMemsetAsync(hs, 0, sizeof(long long) * R, st));
+    const dim3 tg(static_cast<unsigned>(g.kblocks), static_cast<unsigned>((g.R_pad + kTR - 1) / kTR));
     switch (xtype) {
-        case ISING_BF16: spins_replica_major<<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), sp, g.n, R, g.R_pad); break;
-        case ISING_F32: spins_replica_major<<<blocks, 256, 0, st>>>(static_cast<const float *>(x), sp, g.n, R, g.R_pad); break;
-        case ISING_F64: spins_replica_major<<<blocks, 256, 0, st>>>(static_cast<const double *>(x), sp, g.n, R, g.R_pad); break;
-        case ISING_I8: spins_replica_major<<<blocks, 256, 0, st>>>(static_cast<const int8_t *>(x), sp, g.n, R, g.R_pad); break;
+        case ISING_BF16: to_replica_major<__nv_bfloat16, true><<<tg, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), sp, g.n, R, g.R_pad); break;
+        case ISING_F32: to_replica_major<float, true><<<tg, 256, 0, st>>>(static_cast<const float *>(x), sp, g.n, R, g.R_pad); break;
+        case ISING_F64: to_replica_major<double, true><<<tg, 256, 0, st>>>(static_cast<const double *>(x), sp, g.n, R, g.R_pad); break;
+        case ISING_I8: to_replica_major<int8_t, true><<<tg, 256, 0, st>>>(static_cast<const int8_t *>(x), sp, g.n, R, g.R_pad); break;
         default: return fail(ISING_ERR_INVALID_ARG, "dense energy: x type");
     }
     DOCH_CUDA(cudaGetLastError());
@@ -558,7 +646,7 @@ ising_status_t dense_energy(ising_context *c, const void *x, int xtype, int R, i
         field_dot_spins<<<fg, 256, 0, st>>>(sp, c->h_i64, g.n, g.R_pad, hs);
         DOCH_CUDA(cudaGetLastError());
     }
-    dense_energy_finish<<<(R + 127) / 128, 128, 0, st>>>(q, hs, c->dense_jsum, R, E_i, cut_i, E_d, cut_d);
+    dense_energy_finish<<<(R + 3) / 4, 128, 0, st>>>(q, g.m_tiles, hs, c->dense_jsum, R, E_i, cut_i, E_d, cut_d);
     DOCH_CUDA(cudaGetLastError());
     return ISING_OK;
 }

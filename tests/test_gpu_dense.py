@@ -101,6 +101,36 @@ def test_dense_iterates_bf16(n, R, kind):
         N.ising_destroy(h)
 
 
+@pytest.mark.parametrize("n, R, kind", [(65, 3, "pm1"), (1000, 256, "int"), (1100, 300, "pm1"), (2300, 100, "pm1"),
+                                        (2440, 33, "pm1_sparse"), (4100, 16, "pm1"), (4100, 5, "int")])
+def test_dense_shared_k_blocks(n, R, kind):
+    """Instances whose row tiles leave SMs idle: a tile's K blocks are shared by 2 to 8 CTAs (counts
+    that do not divide the blocks or the columns). One step within one BF16 ulp, energies exact."""
+    J = _jmat(kind, n, 96)
+    P = O.Problem(J)
+    alpha, beta = O.alpha_beta(J, eta=1.0, method="wigner")
+    xt, x0 = _bf16(I.x0_uniform(n, R, seed=97))
+    h = N.ising_create(N.Problem(J))
+    try:
+        x = xt.cuda()
+        N.ising_iterate(h, x, [alpha], [beta], 1)
+        ref = O.doch(P, x0, alpha, beta, 1)
+        ref_bf = torch.from_numpy(ref.astype(np.float32)).to(torch.bfloat16).float().numpy()
+        # z = (J x + alpha x)_i is an FP32 sum of n terms |J x| with partial sums of order sqrt(n): its rounding
+        # stays below n 2^-24 max|J|, which the root of a z near zero amplifies
+        z, dz = beta * ref ** 3, n * 2.0 ** -24 * np.abs(J).max()
+        amplified = np.maximum(np.abs(np.cbrt((z + dz) / beta) - ref), np.abs(np.cbrt((z - dz) / beta) - ref))
+        err = np.abs(x.float().cpu().numpy() - ref_bf)
+        assert np.all(err <= _bf16_ulp(ref) * 1.0001 + amplified)
+        assert np.mean(err <= _bf16_ulp(ref) * 1.0001) >= 0.9999  # such z are rare
+        E = np.zeros(R, np.int64)
+        N.ising_energy(h, xt.cuda(), E_int=E)
+        s = O.sign(x0).astype(np.int64)
+        assert np.array_equal(E, -((s * (J.astype(np.int64) @ s)).sum(0) // 2))
+    finally:
+        N.ising_destroy(h)
+
+
 @pytest.mark.parametrize("n, R, kind", [(300, 40, "pm1"), (128, 1, "pm1"), (520, 257, "pm1"),
                                         (300, 40, "int"), (520, 257, "int"), (300, 40, "pm1_sparse")])
 def test_dense_energy_exact(n, R, kind):
