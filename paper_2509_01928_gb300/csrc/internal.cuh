@@ -152,6 +152,9 @@ struct ising_context {
     doch::DevBuf stage_out; // staging of host outputs
     doch::DevBuf partials;  // reduction partials
     doch::DevBuf params;    // alpha/beta tables on the device
+    unsigned char *params_stage = nullptr;  // pinned staging of the tables
+    size_t params_stage_bytes = 0;
+    cudaEvent_t params_event = nullptr;     // its last copy
     doch::DevBuf ckpt;      // checkpoints of the adjoint
     doch::DevBuf work;      // misc. work space
     doch::DevBuf tune;      // eta tuning: the probe iterate and its energies
