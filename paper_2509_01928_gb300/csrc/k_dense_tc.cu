@@ -21,7 +21,7 @@
 // share the tile's K blocks where the tiles alone leave SMs idle (split_of): each CTA puts its partial
 // accumulator in its shared memory, and CTA s adds the S partials of its share of the columns, in
 // order, through distributed shared memory and finishes them. 2000 spins, R = 100 (16 tiles): 21.5 us
-// per step with 16 CTAs, 13.7 us with clusters of 6.
+// per step with 16 CTAs, 10.4 us with clusters of 6.
 //
 // Pipeline per CTA (256 threads):
 //   warp 0, one lane: producer. K-block kb (64 columns of J = 64 spins of
@@ -34,12 +34,11 @@
 //     it once the MMAs that read it complete). After the last block it
 //     commits the "accumulator ready" mbarrier.
 //   warp 2: allocates and frees the TMEM columns.
-//   epilogue, all eight warps once the accumulator is ready: warp w owns
-//     TMEM lanes (rows) 32 (w % 4) .. +31 and every other 32-column block
-//     from block w / 4; it reads 32 columns at a time (tcgen05.ld 32x32b.x32)
-//     and writes the new iterate (cube root as sign(z) 2^(log2|z|/3) with the
-//     hardware lg2/ex2 on a power-of-two prescaled z; BF16 output) or the
-//     energy partials.
+//   epilogue, all eight warps once the accumulator is ready: warp w moves TMEM
+//     lanes (rows) 32 (w % 4) .. +31 of every other 32-column block (tcgen05.ld
+//     32x32b.x32) into shared memory, then whole columns, four rows per lane, to
+//     the new iterate (cube root as sign(z) 2^(log2|z|/3) with the hardware
+//     lg2/ex2 on a power-of-two prescaled z; BF16 output) or the energy partials.
 // Every mbarrier wait is bounded (~1 s of %globaltimer); on expiry the CTA
 // sets the error word, drains its TMA copies (bounded), frees TMEM, returns.
 #include <cuda.h>
@@ -62,6 +61,7 @@ template <bool TERN> constexpr int kStagesOf = TERN ? 6 : 4;
 constexpr int kBM = 128;           // rows of J per tile (MMA M)
 constexpr int kBK = 64;            // K per stage: 64 BF16 = 128 bytes = one swizzle row
 constexpr int kThreadsTC = 256;
+constexpr int kMaxSplit = 8;       // CTAs that share a tile's K blocks (the portable cluster size)
 
 constexpr uint32_t kTernTile = kBM * kBK / 4;  // bytes of one packed ternary J tile (2 bits per entry)
 constexpr int kJStages = 8;                      // packed ternary tiles staged ahead
@@ -77,7 +77,7 @@ struct DenseSmem {
     alignas(8) unsigned long long conv[kS];             // ternary: A tile expanded
     alignas(8) unsigned long long jfull[kJStages];      // ternary: packed tile landed
     alignas(8) unsigned long long jempty[kJStages];     // ternary: packed tile read
-    alignas(16) int qsum[4][256];  // energy terms of the tile's four row groups per column
+    alignas(16) int qsum[256];     // energy terms of the tile per column
     alignas(8) unsigned long long acc_ready;
     uint32_t tmem_base;
     int abort_flag;
@@ -180,12 +180,15 @@ __device__ __forceinline__ void cluster_sync() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// a float at `own`'s offset in the shared memory of CTA `rank` of the cluster
-__device__ __forceinline__ float cluster_load(const float *own, uint32_t rank) {
+// four floats at `own`'s offset in the shared memory of CTA `rank` of the cluster
+__device__ __forceinline__ float4 cluster_load4(const float *own, uint32_t rank) {
     uint32_t a;
-    float v;
+    float4 v;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr(own)), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a)
+                 : "memory");
     return v;
 }
 
@@ -342,70 +345,93 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
         }
     }
     __syncwarp();
-    // Epilogue, all eight warps: warp w reads TMEM lanes 32 (w % 4) .. +31 (its
-    // 32 rows) and every other 32-column block starting at block w / 4.
+    // Epilogue, all eight warps: warp w moves TMEM lanes 32 (w % 4) .. +31 (its 32 rows) of every other
+    // 32-column block into shared memory, then takes whole columns, a lane per four rows: four spins
+    // of a replica are 8 bytes of X (2-byte accesses by row took 55 us per step at n = 9000, R = 256, two CTAs
+    // per tile; 40 so).
     {
         const int q = warp & 3, half = warp >> 2;
-        const int row = m0 + 32 * q + lane;
         // warp-uniform decision: tcgen05.ld below is a .sync.aligned warp instruction
         const bool ok = __all_sync(0xffffffffu, mbar_wait_idle(&sm.acc_ready, 0, err, abort_flag) && !*abort_flag);
-        const float hv = (h && row < n) ? h[row] : 0.f;
-        if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // the product (J X)_(row, r) of column c = r - r0: the new iterate, or the energy term
-        auto finish = [&](int c, float u, float x) {
-            const int r = r0 + c;
+        // accumulators [column][128 rows] over the B ring, which every MMA has left
+        float *partial = reinterpret_cast<float *>(sm.b);
+        if (ok) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int c0 = 32 * half; c0 < n_tile; c0 += 64) {
+                float acc[32];
+                tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, acc);
+#pragma unroll
+                for (int k = 0; k < 32; ++k)
+                    if (c0 + k < n_tile) partial[(c0 + k) * kBM + 32 * q + lane] = acc[k];
+            }
+        }
+        const int row4 = m0 + 4 * lane;
+        float h4[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) h4[e] = MODE == 0 && h && row4 + e < n ? h[row4 + e] : 0.f;
+        auto state = [&](int r) {  // spins past n are zero in X and stay so
+            return row4 < n ? *reinterpret_cast<const uint2 *>(xt_in + xs_index(r, row4, R_pad)) : make_uint2(0u, 0u);
+        };
+        // the product (J X) of rows row4 .. row4 + 3 and column c: the new iterate, or the energy terms
+        auto finish = [&](int c, float4 u4, uint2 xw) {
+            const float u[4] = {u4.x, u4.y, u4.z, u4.w};
+            const float x4[4] = {__uint_as_float(xw.x << 16), __uint_as_float(xw.x & 0xffff0000u),
+                                 __uint_as_float(xw.y << 16), __uint_as_float(xw.y & 0xffff0000u)};
             if (MODE == 0) {
-                if (row < n && r < R) {
-                    const float z = (u + alpha * x + hv) * zscale;
-                    xt_out[xs_index(r, row, R_pad)] = __float2bfloat16_rn(cbrt_pow2(z) * xscale);
+                uint32_t out[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float z = (u[e] + alpha * x4[e] + h4[e]) * zscale;
+                    const __nv_bfloat16 y = __float2bfloat16_rn(cbrt_pow2(z) * xscale);
+                    out[e] = row4 + e < n ? __bfloat16_as_ushort(y) : 0u;
                 }
-            } else {  // |s u| < 2^24: a warp's 32 terms add in 32 bits
-                const int sum = __reduce_add_sync(0xffffffffu, row < n && r < R ? static_cast<int>(x * u) : 0);
-                if (lane == 0) sm.qsum[q][c] = sum;
+                if (row4 < n)
+                    *reinterpret_cast<uint2 *>(xt_out + xs_index(r0 + c, row4, R_pad)) =
+                        make_uint2(out[0] | out[1] << 16, out[2] | out[3] << 16);
+            } else {  // |s u| < 2^24: 128 terms add in 32 bits
+                int term = 0;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) term += static_cast<int>(x4[e] * u[e]);
+                const int sum = __reduce_add_sync(0xffffffffu, term);
+                if (lane == 0) sm.qsum[c] = sum;
             }
         };
-        auto state = [&](int c) {
-            const int r = r0 + c;
-            return row < n && r < R ? __bfloat162float(xt_in[xs_index(r, row, R_pad)]) : 0.f;
-        };
+        constexpr int kW = kThreadsTC / 32;
         if (split == 1) {
-            if (ok)
-                for (int c0 = 32 * half; c0 < n_tile; c0 += 64) {
-                    float acc[32], xo[32];
-                    tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, acc);
+            __syncthreads();
+            const int cols = n_tile < R - r0 ? n_tile : R - r0;
+            constexpr int kAhead = 4;  // columns whose loads are issued together
+            for (int c = warp; ok && c < cols; c += kW * kAhead) {
+                uint2 xw[kAhead];
+                float4 u[kAhead];
 #pragma unroll
-                    for (int k = 0; k < 32; ++k) xo[k] = state(c0 + k);  // all loads first
+                for (int e = 0; e < kAhead; ++e)
+                    if (c + e * kW < cols) {
+                        xw[e] = state(r0 + c + e * kW);
+                        u[e] = *reinterpret_cast<const float4 *>(partial + (c + e * kW) * kBM + 4 * lane);
+                    }
 #pragma unroll
-                    for (int k = 0; k < 32; ++k) finish(c0 + k, acc[k], xo[k]);  // columns c < 256
-                }
+                for (int e = 0; e < kAhead; ++e)
+                    if (c + e * kW < cols) finish(c + e * kW, u[e], xw[e]);
+            }
         } else {
-            // partial accumulators [column][128 rows] over the B ring, which every MMA has left
-            float *partial = reinterpret_cast<float *>(sm.b);
-            if (ok)
-                for (int c0 = 32 * half; c0 < n_tile; c0 += 64) {
-                    float acc[32];
-                    tmem_ld32(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, acc);
-#pragma unroll
-                    for (int k = 0; k < 32; ++k)
-                        if (c0 + k < n_tile) partial[(c0 + k) * kBM + 32 * q + lane] = acc[k];
-                }
             const int c1 = n_tile * (rank + 1) / split;
-            constexpr int kCols = 4;  // columns in flight per thread
             cluster_sync();
-            for (int c = n_tile * rank / split + half; c < c1; c += 2 * kCols) {
-                float u[kCols], xo[kCols];
+            for (int c = n_tile * rank / split + warp; c < c1 && r0 + c < R; c += kW) {
+                float4 v[kMaxSplit];  // all partials of a column in flight
 #pragma unroll
-                for (int j = 0; j < kCols; ++j) {
-                    u[j] = 0.f;
-                    xo[j] = c + 2 * j < c1 ? state(c + 2 * j) : 0.f;
-                }
-                for (int t = 0; t < split; ++t)
+                for (int t = 0; t < kMaxSplit; ++t)
+                    if (t < split) v[t] = cluster_load4(partial + c * kBM + 4 * lane, t);
+                const uint2 xw = state(r0 + c);
 #pragma unroll
-                    for (int j = 0; j < kCols; ++j)
-                        if (c + 2 * j < c1) u[j] += cluster_load(partial + (c + 2 * j) * kBM + 32 * q + lane, t);
-#pragma unroll
-                for (int j = 0; j < kCols; ++j)
-                    if (c + 2 * j < c1) finish(c + 2 * j, u[j], xo[j]);
+                for (int t = 1; t < kMaxSplit; ++t)
+                    if (t < split) {
+                        v[0].x += v[t].x;
+                        v[0].y += v[t].y;
+                        v[0].z += v[t].z;
+                        v[0].w += v[t].w;
+                    }
+                finish(c, v[0], xw);
             }
             cluster_sync();  // no CTA leaves while a peer reads its partials
         }
@@ -415,10 +441,7 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
             const bool mine = split == 1 || (static_cast<int>(threadIdx.x) >= n_tile * rank / split &&
                                              static_cast<int>(threadIdx.x) < n_tile * (rank + 1) / split);
             if (static_cast<int>(threadIdx.x) < n_tile && r < R && mine) {
-                long long t = 0;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) t += sm.qsum[w][threadIdx.x];
-                q_out[static_cast<size_t>(m_tile) * R + r] = t;
+                q_out[static_cast<size_t>(m_tile) * R + r] = sm.qsum[threadIdx.x];
             }
         }
     }
@@ -577,7 +600,7 @@ ising_status_t launch_dense(const ising_context *c, const DenseGeom &g, const __
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const int tiles = g.m_tiles * g.r_tiles;
-    int split = std::max(1, std::min({8, c->num_sms / tiles, g.kblocks}));
+    int split = std::max(1, std::min({kMaxSplit, c->num_sms / tiles, g.kblocks}));
     for (;; --split) {
         attr[0].val.clusterDim.x = static_cast<unsigned>(split);
         cfg.gridDim = dim3(static_cast<unsigned>(g.m_tiles * split), static_cast<unsigned>(g.r_tiles));
