@@ -452,8 +452,7 @@ void destroy_ctx(ising_context *c) {
         cudaEventDestroy(c->params_event);
     }
     if (c->params_stage) cudaFreeHost(c->params_stage);
-    for (cudaEvent_t e : c->count_event)
-        if (e) cudaEventDestroy(e);
+    if (c->until_progress) cudaFreeHost(c->until_progress);
     cudaFree(c->batch_order);
     cudaFree(c->ell_col);
     cudaFree(c->ell_val);
@@ -1454,27 +1453,39 @@ ising_status_t ising_iterate_until(ising_handle_t h, void *x, int32_t xtype, int
         }
         if (rs != ISING_OK && rs != ISING_ERR_UNSUPPORTED) return rs;
         if (one_launch) {
-            if (!c->count_host) DOCH_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->count_host), 2 * sizeof(int), 0));
-            for (cudaEvent_t &e : c->count_event)
-                if (!e) DOCH_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            if (!c->until_progress) {
+                DOCH_CUDA(cudaHostAlloc(&c->until_progress, sizeof(UntilProgress), cudaHostAllocMapped));
+                std::memset(c->until_progress, 0, sizeof(UntilProgress));
+            }
+            void *progress_dev = nullptr;
+            DOCH_CUDA(cudaHostGetDevicePointer(&progress_dev, c->until_progress, 0));
+            s.progress = static_cast<UntilProgress *>(progress_dev);
+            s.call = c->until_calls = (c->until_calls + 1) & 0x3fffffff;
+            const unsigned mark = static_cast<unsigned>(s.call) << 1;
+            // the host stays kAhead launches ahead of the one that last reported (no copies or events in the stream)
+            constexpr int kAhead = 12;
+            auto reported = [&](bool *done) {  // launches of this call known to run
+                const uint64_t w = __atomic_load_n(static_cast<const uint64_t *>(c->until_progress), __ATOMIC_ACQUIRE);
+                const unsigned m = static_cast<unsigned>(w >> 32);
+                *done = m == (mark | 1u);
+                return (m & ~1u) == mark ? static_cast<int>(static_cast<unsigned>(w)) + 1 : 0;
+            };
             void *buf[2] = {xd, c->ping.ptr};
-            constexpr int kPoll = 8;  // steps per copy of the running-pair count, read while the next steps run
             int k = 0;
-            while (k < max_iters) {
-                const int chunk = k / kPoll;
-                for (const int end = std::min(max_iters, k + kPoll); k < end; ++k)
-                    DOCH_CHECK(until_step(c, buf[k & 1], buf[1 - (k & 1)], xtype, R, p, eps, k, s, st));
-                if (k == max_iters) break;
-                DOCH_CUDA(cudaMemcpyAsync(c->count_host + (chunk & 1), s.n_running, sizeof(int), cudaMemcpyDeviceToHost, st));
-                DOCH_CUDA(cudaEventRecord(c->count_event[chunk & 1], st));
-                if (chunk > 0) {
-                    DOCH_CUDA(cudaEventSynchronize(c->count_event[1 - (chunk & 1)]));
-                    if (c->count_host[1 - (chunk & 1)] == 0) break;
-                }
+            for (bool done = false; k < max_iters && !done; ++k) {
+                int spins = 0;
+                while (k - reported(&done) >= kAhead && !done)
+                    if (++spins % 4096 == 0) {  // a failed stream reports nothing; a finished one has run them all
+                        const cudaError_t e = cudaStreamQuery(st);
+                        if (e == cudaSuccess) break;
+                        if (e != cudaErrorNotReady) return cuda_fail(e, "stopping rule");
+                    }
+                if (done) break;
+                DOCH_CHECK(until_step(c, buf[k & 1], buf[1 - (k & 1)], xtype, R, p, eps, k, s, st));
             }
             DOCH_CHECK(until_finish(c, xd, c->ping.ptr, xtype, R, eps, k, s, st));
         } else if (rs == ISING_ERR_UNSUPPORTED) {
-            if (!c->count_host) DOCH_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->count_host), 2 * sizeof(int), 0));
+            if (!c->count_host) DOCH_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->count_host), sizeof(int), 0));
             DOCH_CHECK(c->ping.ensure(xbytes));
             void *cur = xd, *nxt = c->ping.ptr;
             constexpr int kPoll = 8;  // steps between host checks of the running-pair count

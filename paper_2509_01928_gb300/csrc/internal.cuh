@@ -160,8 +160,9 @@ struct ising_context {
     doch::DevBuf tune;      // eta tuning: the probe iterate and its energies
     int *err_word = nullptr;  // device error word
     int *err_host = nullptr;  // pinned mirror
-    int *count_host = nullptr;  // pinned [2]: running-pair counts of the stopping rule
-    cudaEvent_t count_event[2] = {nullptr, nullptr};  // their copies
+    int *count_host = nullptr;  // pinned: running-pair count of the stopping rule
+    void *until_progress = nullptr;  // pinned and mapped: UntilProgress of the calls
+    int until_calls = 0;
     // batched instances: longest-first queue order, queue counter, tuned shapes,
     // and the captured graph of the persistent launch with the key it was built for
     int32_t *batch_order = nullptr;
@@ -318,12 +319,18 @@ ising_status_t params_device(const ising_context *c, double eta, int method, dou
 
 // Stopping rule of Remark S2 (k_stop.cu): device state per (instance,
 // replica) pair and the kernels run after each step x^(k) -> x^(k+1).
+struct alignas(8) UntilProgress {
+    int k;          // a launch that runs
+    unsigned mark;  // call << 1 | (no pair runs any more)
+};
 struct StopState {
     double *partials = nullptr;    // [pair][chunk][2]: sums of (x^(k+1) - x^(k))^2 and (x^(k))^2
     int *running = nullptr;        // [pair] 1 while the pair runs
     int32_t *steps = nullptr;      // [pair] steps taken (max_iters for a pair that never stops)
     int *stopped_now = nullptr;    // [pair] 1 if the pair stopped at this step
     int *n_running = nullptr;      // pairs still running
+    UntilProgress *progress = nullptr;  // in mapped host memory (until_step)
+    int call = 0;                       // marks this call's reports
 };
 // Stopping rule of Remark S2 on one short-row CSR instance (k_until.cu): launch k forms x^(k+1)
 // from x^k, the sums of r^(k), and decides r^(k-1). Buffers cur / nxt alternate between launches; a

@@ -12,7 +12,7 @@
 // Sums: per thread compensated FP32 of split products for FP32 iterates, merged across a block's
 // threads with the rounding of every merge kept (relative error below 2^-44 of these positive sums; an
 // FP64 operation holds an SM partition for 64 clocks a warp, and widening each warp's eight sums took
-// as long as the step), FP64 across blocks; FP64 throughout for FP64 iterates.
+// as long as the step), and across blocks; FP64 throughout for FP64 iterates.
 //
 // Bound by the latency of the gathers, as the step. 100,000 spins of degree 3, R = 8, FP32, 200 steps:
 // 5.5 ms with four launches per step (step, norms, decision, copy), 2.4 ms so; 2000 spins of degree 8,
@@ -36,60 +36,140 @@ constexpr int kUBatch = 4;  // entries of a row's first batch, loaded one row ah
 // for 12,000 spins, R = 16)
 constexpr int kUBlocksPerSm = 3;
 
-// r < eps for r = sqrt(d) / sqrt(s), without the roots where the squares already tell
-__device__ __forceinline__ bool below(double d, double s, double eps) {
-    const double lim = eps * eps * s;
-    if (lim > 1e-290 && lim < 1e290) {
-        if (d > 1.0001 * lim) return false;
-        if (d < 0.9999 * lim) return true;
+// a block's sum as it is left for the next launch, and sums of them
+template <typename XT>
+struct UntilSum;
+template <>
+struct UntilSum<float> {
+    using Slot = float2;
+    DotSum32 v;
+    __device__ __forceinline__ void merge(Slot o) { v.merge(o.x, o.y); }
+    __device__ __forceinline__ void merge_lane(int o) { merge(from_lane(o)); }
+    __device__ __forceinline__ Slot from_lane(int o) const {
+        return make_float2(__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o));
     }
-    return sqrt(d) / sqrt(s) < eps;
+    __device__ __forceinline__ Slot slot() const { return make_float2(v.s, v.c); }
+    __device__ __forceinline__ float near() const { return v.s; }
+    __device__ __forceinline__ double value() const { return v.value(); }
+};
+template <>
+struct UntilSum<double> {
+    using Slot = double;
+    double v = 0.0;
+    __device__ __forceinline__ void merge(Slot o) { v += o; }
+    __device__ __forceinline__ void merge_lane(int o) { merge(from_lane(o)); }
+    __device__ __forceinline__ Slot from_lane(int o) const { return __shfl_xor_sync(0xffffffffu, v, o); }
+    __device__ __forceinline__ Slot slot() const { return v; }
+    __device__ __forceinline__ float near() const { return static_cast<float>(v); }
+    __device__ __forceinline__ double value() const { return v; }
+};
+
+// r < eps for r = sqrt(d) / sqrt(s), without FP64 where FP32 squares already tell (FP64 operations that
+// wait for one another take about 150 clocks each, and every step waits for the slowest block)
+template <typename XT>
+__device__ __forceinline__ bool below(const UntilSum<XT> &d, const UntilSum<XT> &s, double eps) {
+    const float e = static_cast<float>(eps), lim = e * e * s.near();
+    if (e > 1e-15f && lim > 1e-30f && lim < 1e30f) {
+        if (d.near() > 1.0001f * lim) return false;
+        if (d.near() < 0.9999f * lim) return true;
+    }
+    return sqrt(d.value()) / sqrt(s.value()) < eps;
 }
 
 // step k of pair t, whole warp: part[2 t + m][blocks] added in a fixed order
-__device__ void until_decide(const double *__restrict__ part, int blocks, double eps, int k, int t, int *running,
-                             int32_t *__restrict__ steps, int *n_running) {
+template <typename XT>
+__device__ void until_decide(const typename UntilSum<XT>::Slot *__restrict__ part, int blocks, double eps, int k, int t,
+                             int *running, int32_t *__restrict__ steps, int *n_running) {
     const int lane = threadIdx.x & 31;
-    const double *p = part + static_cast<int64_t>(t) * 2 * blocks;
-    double d = 0.0, s = 0.0;
-#pragma unroll 4
-    for (int b = lane; b < blocks; b += 32) {
-        d += p[b];
-        s += p[blocks + b];
+    const typename UntilSum<XT>::Slot *p = part + static_cast<int64_t>(t) * 2 * blocks;
+    UntilSum<XT> d, s;
+    constexpr int kAhead = 8;  // loads in flight
+    for (int b = lane; b < blocks; b += 32 * kAhead) {
+        typename UntilSum<XT>::Slot vd[kAhead], vs[kAhead];
+#pragma unroll
+        for (int e = 0; e < kAhead; ++e)
+            if (b + 32 * e < blocks) {
+                vd[e] = __ldcg(p + b + 32 * e);
+                vs[e] = __ldcg(p + blocks + b + 32 * e);
+            }
+#pragma unroll
+        for (int e = 0; e < kAhead; ++e)
+            if (b + 32 * e < blocks) {
+                d.merge(vd[e]);
+                s.merge(vs[e]);
+            }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        d += __shfl_xor_sync(0xffffffffu, d, o);
-        s += __shfl_xor_sync(0xffffffffu, s, o);
+        d.merge_lane(o);
+        s.merge_lane(o);
     }
-    if (lane != 0 || !running[t] || !below(d, s, eps)) return;
+    if (lane != 0 || !__ldcg(running + t) || !below<XT>(d, s, eps)) return;
     steps[t] = k + 1;
     __stcg(running + t, 0);
     atomicSub(n_running, 1);
 }
 
-// grid: dblocks deciding blocks, then row blocks
+__device__ __forceinline__ void until_report(UntilProgress *p, int k, int call, bool done) {
+    asm volatile("st.volatile.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(k), "r"(call << 1 | (done ? 1 : 0)) : "memory");
+}
+
+// ldv_cg that stays where it is written: before the test of the running flags
+template <typename T, int V>
+__device__ __forceinline__ void ldv_now(const T *p, T (&v)[V]) {
+    if constexpr (sizeof(T) * V == 16) {
+        uint32_t w[4];
+        asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                     : "l"(p));
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            if constexpr (sizeof(T) == 4) v[k] = __uint_as_float(w[k]);
+            else v[k] = __hiloint2double(static_cast<int>(w[2 * k + 1]), static_cast<int>(w[2 * k]));
+        }
+    } else if constexpr (sizeof(T) * V == 8) {
+        uint32_t w[2];
+        asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p));
+        if constexpr (V == 2) {
+            v[0] = __uint_as_float(w[0]);
+            v[1] = __uint_as_float(w[1]);
+        } else {
+            v[0] = __hiloint2double(static_cast<int>(w[1]), static_cast<int>(w[0]));
+        }
+    } else {
+        uint32_t w;
+        asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(w) : "l"(p));
+        v[0] = __uint_as_float(w);
+    }
+}
+
+// grid: dblocks deciding blocks, then row blocks. A row takes Cp threads: its C = R / V chunks, or C
+// rounded up to a power of two (spare lanes idle), so that shuffles add the rows of a warp.
 template <typename XT, typename VT, int V>
 __global__ void __launch_bounds__(kUThreads, kUBlocksPerSm)
 until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__restrict__ row_ptr,
              const int32_t *__restrict__ col, const VT *__restrict__ val, const XT *__restrict__ h, int n, int R,
              const XT *__restrict__ alpha_tab, const XT *__restrict__ beta_tab, const float *__restrict__ zs_tab,
-             const float *__restrict__ xs_tab, int dblocks, double eps, int k, double *__restrict__ part,
-             const double *__restrict__ part_before, int *running, int32_t *__restrict__ steps, int *n_running) {
+             const float *__restrict__ xs_tab, int Cp, int dblocks, double eps, int k, typename UntilSum<XT>::Slot *__restrict__ part,
+             const typename UntilSum<XT>::Slot *__restrict__ part_before, int *running, int32_t *__restrict__ steps,
+             int *n_running, UntilProgress *progress, int call) {
     const int blocks = static_cast<int>(gridDim.x) - dblocks, blk = static_cast<int>(blockIdx.x) - dblocks;
     if (blk < 0) {
         pdl_wait();
         pdl_trigger();
         const int t = static_cast<int>(blockIdx.x) * kUWarps + (threadIdx.x >> 5);
-        if (k > 0 && t < R) until_decide(part_before, blocks, eps, k - 1, t, running, steps, n_running);
+        if (k > 0 && t < R) until_decide<XT>(part_before, blocks, eps, k - 1, t, running, steps, n_running);
+        __syncthreads();
+        if (blockIdx.x == 0 && threadIdx.x == 0)  // for the host: launch k runs, and whether any replica still does
+            until_report(progress, k, call, __ldcg(n_running) == 0);
         return;
     }
     const int C = R / V;
-    const int rows_per_block = kUThreads / C;
-    const int ch = threadIdx.x % C;
-    const int rl = threadIdx.x / C;
+    const int rows_per_block = kUThreads / Cp;
+    const int ch = threadIdx.x % Cp;
+    const int rl = threadIdx.x / Cp;
     const int S = blocks * rows_per_block;
-    int i = rl < rows_per_block ? blk * rows_per_block + rl : n;
+    int i = rl < rows_per_block && ch < C ? blk * rows_per_block + rl : n;
     int e0, e1, f0, f1;  // entry ranges of rows i and i + S
     int32_t js[kUBatch];
     XT ws[kUBatch];
@@ -98,18 +178,16 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
     pipe_first_batch<kUBatch>(col, val, e0, e1, js, ws);
     pdl_wait();  // the couplings above are never written
     pdl_trigger();
-    if (!__syncthreads_or(threadIdx.x == 0 && __ldcg(n_running) != 0)) return;  // every result is in place
     const XT a = alpha_tab[0];
     const StepRoot<XT> root(beta_tab, zs_tab, xs_tab, 0);
     // a flag lowered during this launch may or may not be seen: this launch's writes miss x^k either way
     bool run[V], all = true, any = false;
 #pragma unroll
     for (int q = 0; q < V; ++q) {
-        run[q] = __ldcg(running + ch * V + q) != 0;
+        run[q] = ch < C && __ldcg(running + ch * V + q) != 0;
         all = all && run[q];
         any = any || run[q];
     }
-    if (!any) i = n;
     DotSum32 d32[V], s32[V];
     double d64[V], s64[V];
 #pragma unroll
@@ -119,9 +197,10 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
         XT xv[kUBatch][V];
 #pragma unroll
         for (int t = 0; t < kUBatch; ++t)
-            if (t < cnt) ldv_cg<XT, V>(xi + static_cast<int64_t>(js[t]) * R + ch * V, xv[t]);
+            if (t < cnt) ldv_now<XT, V>(xi + static_cast<int64_t>(js[t]) * R + ch * V, xv[t]);
         XT xs[V];
-        ldv_cg<XT, V>(xi + static_cast<int64_t>(i) * R + ch * V, xs);
+        ldv_now<XT, V>(xi + static_cast<int64_t>(i) * R + ch * V, xs);
+        if (!any) break;  // (the loads above do not wait for the flags)
         const XT hi = h ? h[i] : XT(0);
         // the next row's first batch and the range of the row after it
         int32_t js2[kUBatch];
@@ -143,7 +222,7 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
             const int64_t j = __ldg(col + e);
             const XT w = coupling<XT, VT>(__ldg(val + e));
             XT xr[V];
-            ldv_cg<XT, V>(xi + j * R + ch * V, xr);
+            ldv_now<XT, V>(xi + j * R + ch * V, xr);
 #pragma unroll
             for (int q = 0; q < V; ++q) acc[q] += w * xr[q];
         }
@@ -180,85 +259,91 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
     }
     // the block's sums into part[2 (ch V + q) + m][blk]
     __shared__ double red[8 * kUThreads];
-    if (C <= 32 && (C & (C - 1)) == 0) {  // a warp's lanes of one chunk are C apart
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = 2 * C * V;  // per <= 256
-        if constexpr (sizeof(XT) == 4) {
-            float2 *part32 = reinterpret_cast<float2 *>(red);  // [warp][ch V + q][m]
+    if (!__syncthreads_or(any)) return;  // every replica of the block stopped: no sums
+    if (Cp <= 32 && (Cp & (Cp - 1)) == 0) {  // a warp's lanes of one chunk are Cp apart
+        // the 2 V sums of a lane by halves: at each level a lane hands one half of its values to the lane
+        // `o` away and merges the other half with that lane's, then whole values once one is left (8
+        // merges instead of 32 for V = 4, Cp = 2)
+        UntilSum<XT> v[2 * V];
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                for (int o = 16; o >= C; o >>= 1) {
-                    d32[q].merge(__shfl_xor_sync(0xffffffffu, d32[q].s, o), __shfl_xor_sync(0xffffffffu, d32[q].c, o));
-                    s32[q].merge(__shfl_xor_sync(0xffffffffu, s32[q].s, o), __shfl_xor_sync(0xffffffffu, s32[q].c, o));
-                }
-                if (lane < C) {
-                    part32[warp * per + (lane * V + q) * 2] = make_float2(d32[q].s, d32[q].c);
-                    part32[warp * per + (lane * V + q) * 2 + 1] = make_float2(s32[q].s, s32[q].c);
+        for (int q = 0; q < V; ++q) {
+            if constexpr (sizeof(XT) == 4) {
+                v[2 * q].v = d32[q];
+                v[2 * q + 1].v = s32[q];
+            } else {
+                v[2 * q].v = d64[q];
+                v[2 * q + 1].v = s64[q];
+            }
+        }
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = 2 * V * Cp;  // per <= 256
+        int base = 0, held = 2 * V;  // this lane holds values base .. base + held - 1
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            const int o = 16 >> l;
+            constexpr int kAll = 2 * V;
+            const int cnt = kAll >> l > 1 ? kAll >> l : 1;
+            if (o >= Cp) {
+                if (cnt > 1) {
+                    const bool up = (lane & o) != 0;
+#pragma unroll
+                    for (int j = 0; j < cnt / 2; ++j) {
+                        UntilSum<XT> keep = up ? v[cnt / 2 + j] : v[j], send = up ? v[j] : v[cnt / 2 + j];
+                        keep.merge(send.from_lane(o));
+                        v[j] = keep;
+                    }
+                    base += up ? cnt / 2 : 0;
+                    held = cnt / 2;
+                } else {
+                    v[0].merge_lane(o);
                 }
             }
-            __syncthreads();
-            if (static_cast<int>(threadIdx.x) < per) {
-                DotSum32 v;
+        }
+        typename UntilSum<XT>::Slot *slots = reinterpret_cast<typename UntilSum<XT>::Slot *>(red);  // [warp][chunk][value]
+        if (lane % Cp < C) {
 #pragma unroll
-                for (int w = 0; w < kUWarps; ++w) {
-                    const float2 u = part32[w * per + threadIdx.x];
-                    v.merge(u.x, u.y);
-                }
-                part[static_cast<int64_t>(threadIdx.x) * blocks + blk] = v.value();
-            }
-        } else {
+            for (int j = 0; j < 2 * V; ++j)
+                if (j < held) slots[warp * per + (lane % Cp) * 2 * V + base + j] = v[j].slot();
+        }
+        __syncthreads();
+        if (static_cast<int>(threadIdx.x) < 2 * V * C) {
+            UntilSum<XT> t;
 #pragma unroll
-            for (int q = 0; q < V; ++q) {
-                for (int o = 16; o >= C; o >>= 1) {
-                    d64[q] += __shfl_xor_sync(0xffffffffu, d64[q], o);
-                    s64[q] += __shfl_xor_sync(0xffffffffu, s64[q], o);
-                }
-                if (lane < C) {
-                    red[warp * per + (lane * V + q) * 2] = d64[q];
-                    red[warp * per + (lane * V + q) * 2 + 1] = s64[q];
-                }
-            }
-            __syncthreads();
-            if (static_cast<int>(threadIdx.x) < per) {
-                double v[kUWarps];
-#pragma unroll
-                for (int w = 0; w < kUWarps; ++w) v[w] = red[w * per + threadIdx.x];
-                part[static_cast<int64_t>(threadIdx.x) * blocks + blk] =
-                    ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
-            }
+            for (int w = 0; w < kUWarps; ++w) t.merge(slots[w * per + threadIdx.x]);
+            part[static_cast<int64_t>(threadIdx.x) * blocks + blk] = t.slot();
         }
         return;
     }
-    for (int q = 0; q < V; ++q) {  // any C: a tree over the block's rows
-        double d = 0.0, s = 0.0;
+    // any C: a tree over the block's rows
+    typename UntilSum<XT>::Slot *slots = reinterpret_cast<typename UntilSum<XT>::Slot *>(red);  // [m][thread]
 #pragma unroll
-        for (int j = 0; j < V; ++j)
-            if (j == q) {
-                if constexpr (sizeof(XT) == 4) {
-                    d = d32[j].value();
-                    s = s32[j].value();
-                } else {
-                    d = d64[j];
-                    s = s64[j];
-                }
-            }
-        red[threadIdx.x] = d;
-        red[kUThreads + threadIdx.x] = s;
-        __syncthreads();
-        int rows = rows_per_block;
-        while (rows > 1) {
+    for (int q = 0; q < V; ++q) {
+        UntilSum<XT> d, s;
+        if constexpr (sizeof(XT) == 4) {
+            d.v = d32[q];
+            s.v = s32[q];
+        } else {
+            d.v = d64[q];
+            s.v = s64[q];
+        }
+        for (int rows = rows_per_block; rows > 1;) {
             const int half = (rows + 1) / 2;
+            if (rl >= half && rl < rows) {
+                slots[threadIdx.x] = d.slot();
+                slots[kUThreads + threadIdx.x] = s.slot();
+            }
+            __syncthreads();
             if (rl + half < rows) {
-                red[threadIdx.x] += red[threadIdx.x + half * C];
-                red[kUThreads + threadIdx.x] += red[kUThreads + threadIdx.x + half * C];
+                d.merge(slots[threadIdx.x + half * Cp]);
+                s.merge(slots[kUThreads + threadIdx.x + half * Cp]);
             }
             __syncthreads();
             rows = half;
         }
         if (rl == 0) {
-            part[static_cast<int64_t>((ch * V + q) * 2) * blocks + blk] = red[ch];
-            part[static_cast<int64_t>((ch * V + q) * 2 + 1) * blocks + blk] = red[kUThreads + ch];
+            typename UntilSum<XT>::Slot *to = part + static_cast<int64_t>((ch * V + q) * 2) * blocks + blk;
+            to[0] = d.slot();
+            to[blocks] = s.slot();
         }
-        __syncthreads();
     }
 }
 
@@ -270,11 +355,12 @@ __global__ void until_init_kernel(int pairs, int max_iters, int *running, int32_
     if (threadIdx.x == 0) *n_running = pairs;
 }
 
+template <typename XT>
 __global__ void __launch_bounds__(kUThreads)
-until_last_kernel(const double *__restrict__ part, int blocks, double eps, int k, int R, int *running,
+until_last_kernel(const typename UntilSum<XT>::Slot *__restrict__ part, int blocks, double eps, int k, int R, int *running,
                   int32_t *__restrict__ steps, int *n_running) {
     const int t = static_cast<int>(blockIdx.x) * kUWarps + (threadIdx.x >> 5);
-    if (t < R) until_decide(part, blocks, eps, k, t, running, steps, n_running);
+    if (t < R) until_decide<XT>(part, blocks, eps, k, t, running, steps, n_running);
 }
 
 // x^(steps) of the replicas that ended in the other buffer
@@ -293,14 +379,24 @@ int vec_width(const void *x, int xtype, int R) {
     return R % 4 == 0 && a % 16 == 0 ? 4 : R % 2 == 0 && a % 8 == 0 ? 2 : 1;
 }
 
+// threads per row: the chunks, rounded up to a power of two where at least 3 in 4 lanes stay busy
+int row_threads(int C) {
+    int p = 1;
+    while (p < C) p <<= 1;
+    return p <= 32 && 4 * C >= 3 * p ? p : C;
+}
+
 int until_blocks(const ising_context *c, int C) {
-    const int64_t rows_per_block = kUThreads / C;
+    const int64_t rows_per_block = kUThreads / row_threads(C);
     const int64_t cap = static_cast<int64_t>(c->num_sms) * kUBlocksPerSm;
     return static_cast<int>(std::max<int64_t>(1, std::min((c->n + rows_per_block - 1) / rows_per_block, cap)));
 }
 
-double *partials_of(const ising_context *c, int R, int k, StopState &s) {
-    return s.partials + (k & 1) * (until_partials_bytes(c, R) / (2 * sizeof(double)));
+template <typename XT>
+typename UntilSum<XT>::Slot *partials_of(const ising_context *c, int R, int k, StopState &s) {
+    static_assert(sizeof(typename UntilSum<XT>::Slot) == sizeof(double), "the halves hold either");
+    return reinterpret_cast<typename UntilSum<XT>::Slot *>(
+        s.partials + (k & 1) * (until_partials_bytes(c, R) / (2 * sizeof(double))));
 }
 
 template <typename XT, typename VT, int V>
@@ -319,8 +415,8 @@ ising_status_t launch_until(const ising_context *c, const XT *xi, XT *xo, int R,
     }
     DOCH_CUDA(launch_chained(until_kernel<XT, VT, V>, dim3(static_cast<unsigned>(dblocks + blocks)), dim3(kUThreads), st,
                              xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, static_cast<int>(c->n), R,
-                             alpha, beta, p.zscale_f, p.xscale_f, dblocks, eps, k, partials_of(c, R, k, s),
-                             partials_of(c, R, k + 1, s), s.running, s.steps, s.n_running));
+                             alpha, beta, p.zscale_f, p.xscale_f, row_threads(C), dblocks, eps, k, partials_of<XT>(c, R, k, s),
+                             partials_of<XT>(c, R, k + 1, s), s.running, s.steps, s.n_running, s.progress, s.call));
     return ISING_OK;
 }
 
@@ -375,9 +471,13 @@ ising_status_t until_finish(const ising_context *c, void *xa, const void *xb, in
                             int launched, StopState &s, cudaStream_t st) {
     const int C = R / vec_width(xa, xtype, R);
     if (launched > 0) {
-        until_last_kernel<<<(R + kUWarps - 1) / kUWarps, kUThreads, 0, st>>>(
-            partials_of(c, R, launched - 1, s), until_blocks(c, C), eps, launched - 1, R, s.running, s.steps,
-            s.n_running);
+        const unsigned grid = static_cast<unsigned>((R + kUWarps - 1) / kUWarps);
+        if (xtype == ISING_F64)
+            until_last_kernel<double><<<grid, kUThreads, 0, st>>>(partials_of<double>(c, R, launched - 1, s), until_blocks(c, C),
+                                                                  eps, launched - 1, R, s.running, s.steps, s.n_running);
+        else
+            until_last_kernel<float><<<grid, kUThreads, 0, st>>>(partials_of<float>(c, R, launched - 1, s), until_blocks(c, C),
+                                                                 eps, launched - 1, R, s.running, s.steps, s.n_running);
         DOCH_CUDA(cudaGetLastError());
     }
     const int64_t count = c->n * R;
