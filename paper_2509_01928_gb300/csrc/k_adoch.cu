@@ -174,9 +174,16 @@ adoch_step(Fn fn, Candidates<XT> x1, Candidates<XT> x0, XT *next_y, XT *next_x, 
     SiteSum<XT> acc[kTerms];
     pdl_wait();
     pdl_trigger();
+    // one load of the decisions per block: all blocks ask one L2 slice for these lines
+    __shared__ int dec[2][kAThreads];
+    if (active && rl == 0) {
+        dec[0][threadIdx.x] = __ldcg(dec1 + b * R + r);
+        dec[1][threadIdx.x] = __ldcg(dec0 + b * R + r);
+    }
+    __syncthreads();
     if (active) {
-        const XT *xk = __ldcg(dec1 + b * R + r) ? x1.accepted : x1.rejected;
-        const XT *xp = __ldcg(dec0 + b * R + r) ? x0.accepted : x0.rejected;
+        const XT *xk = dec[0][threadIdx.x - rl * Cb] ? x1.accepted : x1.rejected;
+        const XT *xp = dec[1][threadIdx.x - rl * Cb] ? x0.accepted : x0.rejected;
         // (row, column) of the site, advanced without division (lattice only)
         int64_t rr = 0, cc = 0, Lc = 1, dr = 0, dc = 0;
         if constexpr (Fn::kGrid) {

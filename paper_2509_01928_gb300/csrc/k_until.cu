@@ -15,8 +15,8 @@
 // as long as the step), and across blocks; FP64 throughout for FP64 iterates.
 //
 // Bound by the latency of the gathers, as the step. 100,000 spins of degree 3, R = 8, FP32, 200 steps:
-// 5.5 ms with four launches per step (step, norms, decision, copy), 2.4 ms so; 2000 spins of degree 8,
-// R = 3: 2.1 -> 0.8 ms.
+// 5.5 ms with four launches per step (step, norms, decision, copy), 1.5 ms so; 2000 spins of degree 8,
+// R = 3: 2.1 -> 0.54 ms.
 #include <algorithm>
 #include <cmath>
 
@@ -32,7 +32,7 @@ constexpr int kUWarps = kUThreads / 32;
 constexpr int kUBatch = 4;  // entries of a row's first batch, loaded one row ahead
 
 // resident blocks per SM that the kernel is compiled for: FP32 sums take 16 registers more than the step
-// (four blocks: 2.40 -> 3.38 ms for the 192 steps above), FP64 steps gain from a third block (0.95 -> 0.86 ms
+// (four blocks spill: 2.40 -> 3.38 ms for the steps above when measured), FP64 steps gain from a third block (0.95 -> 0.86 ms
 // for 12,000 spins, R = 16)
 constexpr int kUBlocksPerSm = 3;
 
@@ -182,9 +182,27 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
     const StepRoot<XT> root(beta_tab, zs_tab, xs_tab, 0);
     // a flag lowered during this launch may or may not be seen: this launch's writes miss x^k either way
     bool run[V], all = true, any = false;
+    int flag[V];  // one load: all warps of the grid ask one L2 slice for this line (V loads a warp: 2 us a step)
+#pragma unroll
+    for (int q = 0; q < V; ++q) flag[q] = 0;
+    if (ch < C) {
+        if constexpr (V == 4) {
+            const int4 w = __ldcg(reinterpret_cast<const int4 *>(running + ch * V));
+            flag[0] = w.x;
+            flag[1] = w.y;
+            flag[2] = w.z;
+            flag[3] = w.w;
+        } else if constexpr (V == 2) {
+            const int2 w = __ldcg(reinterpret_cast<const int2 *>(running + ch * V));
+            flag[0] = w.x;
+            flag[1] = w.y;
+        } else {
+            flag[0] = __ldcg(running + ch);
+        }
+    }
 #pragma unroll
     for (int q = 0; q < V; ++q) {
-        run[q] = ch < C && __ldcg(running + ch * V + q) != 0;
+        run[q] = flag[q] != 0;
         all = all && run[q];
         any = any || run[q];
     }
