@@ -12,12 +12,15 @@
 // whose lower words are zero, 6 instead of 10 bytes an entry).
 //
 // Bound by FP64 arithmetic (half a lane per clock and SM partition, about 150 clocks from one operation
-// to the next that needs it; an integer -> FP64 conversion costs as much as an FMA): one FMA per entry
-// and replica, the tree and nine operations per cube root. 800 spins, 38,000 entries, R = 8, FP64, per
-// step: 10.0 us with one thread per row, the couplings converted at every use and CUDA's cbrt of a
-// quotient; 3.7 us per step with the couplings held in FP64; the arithmetic alone takes about 0.9 us on
-// the 128 SMs used. Of 7000 clocks the products take 4700, the update 1600 and the exchange 650.
+// to the next that needs it; an integer -> FP64 conversion costs as much as an FMA) and the latency of
+// a step's chain: products, tree, cube root, exchange. FP64 iterates with 8-bit couplings take their
+// products in integers (fixed point, below): nine FP64 operations per cube root and five around it are left.
+// 800 spins, 38,000 entries, R = 8, FP64, per step: 10.0 us with one thread per row, the couplings
+// converted at every use and CUDA's cbrt of a quotient; 3.5 us with the couplings held in FP64 and four
+// threads per row (products 2.3, update 0.8, exchange 0.35); 2.6 us in fixed point with eight. The FP64
+// operations alone take about 0.25 us on the 128 SMs used.
 #include <algorithm>
+#include <type_traits>
 
 #include "hamsum.cuh"
 #include "internal.cuh"
@@ -102,18 +105,43 @@ struct Held {
     static __device__ __forceinline__ XT value(XT v) { return v; }
 };
 template <>
-struct Held<double, int8_t> {
+struct Held<double, int8_t> {  // the integer (fixed-point steps), or the FP64 value's upper word
     using type = int;
-    static __device__ __forceinline__ int pack(int8_t v) { return __double2hiint(static_cast<double>(v)); }
+    static __device__ __forceinline__ int pack(int8_t v) { return v; }
+    static __device__ __forceinline__ int upper(int v) { return v ? __double2hiint(static_cast<double>(v)) : 0; }
     static __device__ __forceinline__ double value(int v) { return __hiloint2double(v, 0); }
 };
 
-// Shared memory: cur | nxt (XT [nb] each) | z (XT [rows], P > 1 only), then, as far as there is room
+// Fixed-point steps (FP64 iterates, 8-bit couplings): every x_j is held as the integer round(x_j 2^s),
+// s from a bound M >= max |x_j| such that every row's sum of J_ij x_j stays below 2^62, so that J x is
+// summed exactly in integers, at integer rate, from terms with an absolute error of rowabs M 2^-62
+// (FP64 sums round by about M 2^-53 at every addition; relative error against plain FP64 arithmetic in
+// torch over 1000 steps of 800 spins, R = 8, six seeds: 4.41e-16 to 5.33e-16 in FP64, 4.40e-16 to 5.30e-16
+// in fixed point; 60 steps of 1500 spins, R = 4: 0.6e-15 to 4.0e-15 and 0.6e-15 to 3.1e-15). M of the next
+// iterate follows from |x'| <= cbrt((rowabs + |alpha|) M + max |h|) / beta), rounded up. x itself is
+// kept in FP64 where it is added (alpha x) and returned. Runs that record iterates keep FP64 sums: their
+// scales would depend on where a run starts.
+__device__ __forceinline__ float next_bound(float m, float rowabs, float alpha, float hmax, float inv_beta) {
+    const float z = ((rowabs + fabsf(alpha)) * m + hmax) * inv_beta;
+    return ex2_fast(lg2_fast(z) * (1.0f / 3.0f)) * 1.0001f;
+}
+__device__ __forceinline__ int fixed_shift(float m, float rowabs) {  // rowabs m 2^shift < 2^61
+    return 61 - (ilogbf(rowabs * m * 1.0001f) + 1);
+}
+__device__ __forceinline__ long long to_fixed(double v, int shift) {  // the shift in the exponent's field
+    return __double2ll_rn(__hiloint2double(__double2hiint(v) + (shift << 20), __double2loint(v)));
+}
+__device__ __forceinline__ double two_to(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// Shared memory: cur | nxt (XT [nb] each) | z (XT [rows], P > 1 only) | own (XT [rows], the share's x,
+// where fixed-point steps may run), then, as far as there is room
 // for at least the shares it fits, val (Held [cap]) | row ranges (int [rows + 1]) | col (uint16 [cap])
 template <typename XT, int P>
-constexpr int64_t state_bytes(int64_t nb, int64_t rows) {
-    return static_cast<int64_t>(sizeof(XT)) * (2 * nb + (P > 1 ? rows : 0)) + 16;
+constexpr int64_t state_bytes(int64_t nb, int64_t rows, bool own) {
+    return static_cast<int64_t>(sizeof(XT)) * (2 * nb + (P > 1 ? rows : 0) + (own ? rows : 0)) + 16;
 }
+template <typename XT, typename VT>
+constexpr bool can_fix() { return sizeof(XT) == 8 && sizeof(VT) == 1; }
 template <typename XT, typename VT>
 constexpr int64_t entry_bytes() { return sizeof(typename Held<XT, VT>::type) + sizeof(uint16_t); }
 
@@ -126,6 +154,9 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
           unsigned char *rec, size_t rec_stride, int rec_every, int *__restrict__ err) {
     extern __shared__ __align__(16) unsigned char small_smem[];
     __shared__ Exchange ex;
+    constexpr bool kFix = can_fix<XT, VT>();
+    __shared__ int rowabs_of[kFix ? 16 : 1];          // every CTA's largest row sum of |J| (INT_MAX: no fixed point)
+    __shared__ unsigned top_word[kFix ? 3 : 1];       // upper words of max |x|, max |h|; the share's rowabs
     const int q = static_cast<int>(cl_rank());
     const int b = blockIdx.y, r = blockIdx.x / K;
     const int64_t lo = inst_off ? inst_off[b] : 0;
@@ -136,10 +167,27 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     XT *cur = reinterpret_cast<XT *>(small_smem), *nxt = cur + nb;
     XT *z = nxt + nb;
     using Hd = Held<XT, VT>;
-    typename Hd::type *lv = reinterpret_cast<typename Hd::type *>(P > 1 ? z + rows_cap : z);
+    const bool with_own = kFix && K > 1;
+    XT *own = P > 1 ? z + rows_cap : z;
+    typename Hd::type *lv = reinterpret_cast<typename Hd::type *>(with_own ? own + rows_cap : own);
     int *lr = reinterpret_cast<int *>(lv + cap);
     uint16_t *lc = reinterpret_cast<uint16_t *>(lr + rows_cap + 1);
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = x_in[(lo + i) * R + r];
+    if constexpr (kFix) {
+        if (threadIdx.x < 3) top_word[threadIdx.x] = 0;
+        __syncthreads();
+        unsigned tx = 0, th = 0;
+        for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+            const XT v = x_in[(lo + i) * R + r];
+            cur[i] = v;
+            tx = max(tx, static_cast<unsigned>(__double2hiint(v)) & 0x7fffffffu);
+            if (h) th = max(th, static_cast<unsigned>(__double2hiint(__ldg(h + lo + i))) & 0x7fffffffu);
+            if (with_own && i >= i0 && i < i1) own[i - i0] = v;
+        }
+        atomicMax(&top_word[0], tx);
+        atomicMax(&top_word[1], th);
+    } else {
+        for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = x_in[(lo + i) * R + r];
+    }
     const int64_t e0 = row_ptr[lo + i0];
     const bool local = row_ptr[lo + i1] - e0 <= cap;  // uniform over the block
     for (int i = threadIdx.x; i <= rows && local; i += blockDim.x) lr[i] = static_cast<int>(row_ptr[lo + i0 + i] - e0);
@@ -148,6 +196,52 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
         for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
             lv[e] = Hd::pack(val[e0 + e]);
             lc[e] = static_cast<uint16_t>(col[e0 + e] - lo);
+        }
+    }
+    bool fixed = false;
+    float bound = 0.f, rowabs = 0.f, hmax = 0.f, inv_beta = 0.f;
+    int shift = 0;
+    if constexpr (kFix) {
+        __syncthreads();
+        int sum = 0;
+        for (int i = threadIdx.x; i < rows && local; i += blockDim.x) {
+            int t = 0;
+            for (int e = lr[i]; e < lr[i + 1]; ++e) t += abs(lv[e]);
+            sum = max(sum, t);
+        }
+        atomicMax(&top_word[2], static_cast<unsigned>(sum));
+        if (K > 1) cl_sync();  // every CTA of the cluster runs
+        else __syncthreads();
+        if (threadIdx.x < K) {
+            const int mine = local ? static_cast<int>(top_word[2]) : 0x7fffffff;
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cl_map(&rowabs_of[q], threadIdx.x)), "r"(mine) : "memory");
+        }
+        if (K > 1) cl_sync();
+        else __syncthreads();
+        int most = 1;
+        for (int t = 0; t < K; ++t) most = max(most, rowabs_of[t]);
+        // bounds just above the maxima; FP32 carries them, so their range and the scales' is checked, at
+        // the start and at the point that the bounds move towards
+        const double mx = __hiloint2double(static_cast<int>(top_word[0] + 1), 0);
+        const double mh = top_word[1] ? __hiloint2double(static_cast<int>(top_word[1] + 1), 0) : 0.0;
+        bound = __double2float_ru(mx);
+        hmax = __double2float_ru(mh);
+        rowabs = static_cast<float>(most) * 1.0001f;
+        inv_beta = static_cast<float>(1.0 / beta_tab[b]) * 1.0001f;
+        bool bad = !(with_own && !rec && top_word[0] < 0x7ff00000u && top_word[1] < 0x7ff00000u && most != 0x7fffffff &&
+                     bound > 1e-12f && bound < 1e10f && hmax < 1e12f && inv_beta > 1e-20f && inv_beta < 1e12f);
+        for (int k = threadIdx.x; k < (alpha_len == 1 ? 1 : iters); k += blockDim.x) {
+            const float ak = static_cast<float>(alpha_tab[static_cast<int64_t>(b) * alpha_len + (alpha_len == 1 ? 0 : k0 + k)]);
+            const float z = (rowabs + fabsf(ak)) * inv_beta;  // without a field the squared bound tends to z
+            bad = bad || !(z > 1e-20f && z < 1e12f);
+        }
+        fixed = !__syncthreads_or(bad);
+        if (fixed) {
+            shift = fixed_shift(bound, rowabs);
+            for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = __longlong_as_double(to_fixed(cur[i], shift));
+        } else if (local) {
+            const int cnt = lr[rows];
+            for (int e = threadIdx.x; e < cnt; e += blockDim.x) lv[e] = Hd::upper(lv[e]);
         }
     }
     const auto root = make_root<XT>(beta_tab[b]);
@@ -164,17 +258,48 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
         if (K > 1) exchange_expect(ex, k, static_cast<uint32_t>((nb - rows) * sizeof(XT)));
         const bool keep = rec && (k + 1) % rec_every == 0;
         XT *rp = reinterpret_cast<XT *>(rec + (keep ? static_cast<size_t>((k + 1) / rec_every - 1) : 0) * rec_stride);
+        const double unit = two_to(-shift);
+        if constexpr (kFix) {
+            if (fixed) {
+                bound = next_bound(bound, rowabs, static_cast<float>(a), hmax, inv_beta);
+                shift = fixed_shift(bound, rowabs);
+            }
+        }
         auto update = [&](int i, XT u) {  // row i of the share: the new value into every CTA's next copy
             const int64_t row = lo + i0 + i;
             const XT hv = h ? __ldg(h + row) : XT(0);
-            const XT v = root_newton(u + a * cur[i0 + i] + hv, root);
+            XT v;
+            if (kFix && fixed) {
+                if constexpr (kFix) {
+                    XT w = a * own[i];
+                    if (h) w += hv;
+                    const XT y = root_newton(fma(__ll2double_rn(__double_as_longlong(u)), unit, w), root);
+                    own[i] = y;
+                    v = __longlong_as_double(to_fixed(y, shift));
+                }
+            } else {
+                v = root_newton(u + a * cur[i0 + i] + hv, root);
+                if (keep) rp[row * R + r] = v;
+            }
             nxt[i0 + i] = v;
             exchange_send(ex, k, nxt + i0 + i, v, q, K);
-            if (keep) rp[row * R + r] = v;
         };
         for (int i = rl; i < top; i += rstep) {
             XT acc = XT(0);
-            if (i < rows) {
+            if (kFix && fixed) {
+                if constexpr (kFix) {
+                    const long long *fx = reinterpret_cast<const long long *>(cur);
+                    long long sum = 0;
+                    if (i < rows) {
+                        const int f1 = lr[i + 1];
+#pragma unroll 4
+                        for (int e = lr[i] + sub; e < f1; e += P) sum += static_cast<long long>(lv[e]) * fx[lc[e]];
+                    }
+#pragma unroll
+                    for (int o = P / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                    acc = __longlong_as_double(sum);
+                }
+            } else if (i < rows) {
                 if (local) {
                     const int f1 = lr[i + 1];
 #pragma unroll 4
@@ -185,8 +310,10 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
                         acc += static_cast<XT>(__ldg(val + e)) * cur[__ldg(col + e) - lo];
                 }
             }
+            if (!(kFix && fixed)) {
 #pragma unroll
-            for (int o = P / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                for (int o = P / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            }
             if (P == 1) {
                 if (i < rows) update(i, acc);
             } else if (sub == 0 && i < rows) {
@@ -203,7 +330,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
         nxt = t;
     }
     if (x_out)
-        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) x_out[(lo + i) * R + r] = cur[i];
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) x_out[(lo + i) * R + r] = kFix && fixed ? own[i - i0] : cur[i];
     if (K > 1) cl_sync();  // no CTA leaves while a peer may still send to it
 }
 
@@ -322,7 +449,7 @@ template <typename XT, typename VT, int P>
 ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R, const XT *h, const ParamTabs &p,
                         int k0, int iters, int K, const SmallRecord &rec, int64_t optin, cudaStream_t st) {
     const int64_t chunk = (c->max_inst_n + K - 1) / K;
-    const int64_t state = state_bytes<XT, P>(c->max_inst_n, chunk);
+    const int64_t state = state_bytes<XT, P>(c->max_inst_n, chunk, can_fix<XT, VT>() && K > 1);
     if (state > optin) return ISING_ERR_UNSUPPORTED;
     // room for the couplings of the fullest share, as far as it goes (shares that need more read the CSR arrays)
     const int64_t left = optin - state - static_cast<int64_t>(sizeof(int)) * (chunk + 1);
@@ -431,12 +558,23 @@ ising_status_t launch_small(const ising_context *c, const XT *x_in, XT *x_out, i
     for (int K = cluster_max(c, R);; --K) {
         const int64_t chunk = (c->max_inst_n + K - 1) / K;
         // threads per row: four or two where a share is small and its rows are long enough to split (more
-        // would spend as many FP64 additions on the tree as they take from the rows)
+        // would spend as many FP64 additions on the tree as they take from the rows); eight or four where
+        // the products are integers (1000 spins at density 0.05, R = 20, shares of 143 rows, 300 steps: 1.63 ms
+        // with two, 1.42 with four, 1.24 with eight; 800 spins at 0.06, R = 8, shares of 50, 1000 steps: 2.72 ms with
+        // four, 2.59 with eight, 2.87 with sixteen)
         const bool split = c->nnz >= 8 * c->n;
-        const ising_status_t s =
-            split && chunk <= 128   ? launch_k<XT, VT, 4>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st)
-            : split && chunk <= 512 ? launch_k<XT, VT, 2>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st)
-                                    : launch_k<XT, VT, 1>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st);
+        auto run = [&](auto p_threads) {
+            return launch_k<XT, VT, decltype(p_threads)::value>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st);
+        };
+        ising_status_t s;
+        if constexpr (can_fix<XT, VT>())
+            s = split && chunk <= 256   ? run(std::integral_constant<int, 8>())
+                : split && chunk <= 512 ? run(std::integral_constant<int, 4>())
+                                        : run(std::integral_constant<int, 1>());
+        else
+            s = split && chunk <= 128   ? run(std::integral_constant<int, 4>())
+                : split && chunk <= 512 ? run(std::integral_constant<int, 2>())
+                                        : run(std::integral_constant<int, 1>());
         if (s != ISING_ERR_UNSUPPORTED || K == 1) return s;
     }
 }

@@ -579,3 +579,44 @@ def test_fused_hamiltonian_monitor(kind):
     assert np.all(np.abs(fused - exact) <= 1e-5 * np.abs(exact).max()), np.abs(fused - exact).max()
     _, Href = O.doch(O.Problem(J), x0, alpha, beta, 1, trace=True)
     np.testing.assert_allclose(fused[0], Href[0], rtol=1e-5)
+
+
+@pytest.mark.parametrize("n, R, density, jmax", [(40, 2, 0.5, 1), (300, 8, 0.02, 1), (801, 8, 0.06, 1), (801, 1, 0.06, 127),
+                                                 (1500, 20, 0.08, 3), (700, 40, 0.05, 1), (600, 100, 0.05, 1)])
+@pytest.mark.parametrize("start", ["uniform", "wide", "tiny", "huge", "zero"])
+def test_small_fp64_int8_steps(n, R, density, jmax, start):
+    """FP64 iterates of small instances with 8-bit couplings take J x in fixed point; starts outside its
+    range (and one CTA per replica) take FP64 sums. Components over many orders of magnitude, a field and
+    a schedule of alpha included; 1e-12 against the oracle at every size of share and cluster."""
+    rng = np.random.default_rng(n + R)
+    keep = np.triu(rng.random((n, n)) < density, 1)
+    i, j = keep.nonzero()
+    v = rng.integers(1, jmax + 1, i.size) * rng.choice([-1, 1], i.size)
+    g = I.csr_from_upper(n, i, j, v.astype(np.int8))
+    h = rng.normal(size=n) * 0.3 if start in ("uniform", "tiny") else None
+    x0 = rng.uniform(-1, 1, (n, R))
+    if start == "wide":
+        x0 *= 10.0 ** rng.uniform(-9, 0, (n, R))
+    elif start == "tiny":
+        x0 *= 1e-200
+    elif start == "huge":  # all components: one alone makes its neighbours equal, whose sums cancel to their rounding
+        x0 *= 1e200
+    elif start == "zero":
+        x0[::2] = 0.0
+    a0, beta = O.alpha_beta(g, eta=1.0, method="wigner")
+    iters = 6
+    alpha = np.full(iters, a0) if start == "uniform" else np.array([a0])
+    if start == "uniform":
+        alpha *= 1.0 + 0.2 * np.sin(np.arange(iters))
+    P = O.Problem(g, h)
+    ref = x0
+    for k in range(iters):
+        ref = O.doch(P, ref, float(alpha[k if alpha.size > 1 else 0]), beta, 1)
+    hd = N.ising_create(N.Problem(g, h))
+    try:
+        x = torch.from_numpy(x0.copy()).cuda()
+        N.ising_iterate(hd, x, alpha, [beta], iters)
+        x = x.cpu().numpy()
+    finally:
+        N.ising_destroy(hd)
+    assert np.all(np.linalg.norm(x - ref, axis=0) <= 1e-12 * np.linalg.norm(ref, axis=0))
