@@ -1702,7 +1702,7 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
         const size_t A = al(static_cast<size_t>(c->n) * R * xel);        // one iterate
         const size_t G = al(static_cast<size_t>(c->n) * R * sizeof(float)); // one adjoint state
         const size_t part_b = al(sizeof(double) * static_cast<size_t>(iters) *
-                                 static_cast<size_t>(std::max(grid, adjoint_small_blocks(c, R))));
+                                 static_cast<size_t>(std::max(grid, backward_small(c, xtype, R) ? adjoint_small_parts(c, R) : 0)));
         const size_t lpart_b = al(sizeof(double) * grid);
         const size_t out_b = al(sizeof(double) * (static_cast<size_t>(iters) + 1) + 8);
         const size_t wide_b = xtype == ISING_F64 ? A : 0;                   // FP64 copy of dL/dx0

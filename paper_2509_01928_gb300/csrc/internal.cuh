@@ -410,8 +410,8 @@ ising_status_t csr_adjoint_step(const ising_context *c, const float *w_in, const
                                 int grid, double *part, unsigned long long *zeros, cudaStream_t st);
 // Adjoint steps k0 + len - 1 .. k0 in one launch for an instance that fits in shared memory
 // (k_csr_small.cu): w_in = w^(k0 + len - 1), w_out = w^(k0 - 1) or g^0; x_first = x^(k0),
-// x^(k0 + m) = x_seg + (m - 1) stride; part [iters][blocks] with the number of blocks returned
-// (the same for every segment, at most adjoint_small_blocks). ISING_ERR_UNSUPPORTED when it does not fit.
+// x^(k0 + m) = x_seg + (m - 1) stride; part [iters][blocks] with the number of partial sums per step returned
+// (the same for every segment, at most adjoint_small_parts). ISING_ERR_UNSUPPORTED when it does not fit.
 struct AdjointSegment {
     const float *w_in;
     float *w_out;
@@ -423,7 +423,7 @@ struct AdjointSegment {
     unsigned long long *zeros;
 };
 bool backward_small(const ising_context *c, int xtype, int R);
-int adjoint_small_blocks(const ising_context *c, int R);
+int adjoint_small_parts(const ising_context *c, int R);
 ising_status_t adjoint_small_run(const ising_context *c, const AdjointSegment &s, int xtype, int R, const ParamTabs &p,
                                  int *blocks, cudaStream_t st);
 ising_status_t widen_f32_to_f64(const float *a, double *b, int64_t count, int num_sms, cudaStream_t st);

@@ -335,28 +335,95 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
 }
 
 // Adjoint steps k0 + len - 1 .. k0 of one instance that fits in shared memory, in one launch: with
-// the adjoint state w^k (FP32) held as csr_small holds its iterate, a cluster per replica,
+// the adjoint state w^k held as csr_small holds its iterate, a cluster per replica and a thread per row,
 //   g^k = (J w^k + alpha_k w^k) / beta,   w^(k-1) = g^k / (3 (x^k)^2)  (g^0 itself when k = 0),
-// and the partial sums of dL/dalpha_k = sum w^k x^k / beta of every CTA into part[k][gridDim.x]. A
-// row's products are summed with compensation (relative error of grad_x0 over twelve seeds of 2000 spins, R = 8,
-// FP64, 100 steps: 1.5e-6 on average, single steps 1.7e-6); the partial sums are per thread FP64 for FP64
-// iterates, compensated FP32 of split products for FP32 ones, and FP64 across threads. x^(k0) is
-// x_first and x^(k0 + m) = x_seg + (m - 1) stride. The next step's own x is loaded, and the block's sum
-// formed, before the wait for the peers' shares.
+// and the partial sums of dL/dalpha_k = sum w^k x^k / beta of every CTA into part[k][CTA]. Within a
+// run the state has the iterate's type: FP64 for FP64 iterates (few rows per CTA, so the latency of the
+// chain counts and not the FP64 rate; the factor 1 / (3 beta x^2) is formed before the wait for the
+// peers' shares); FP32 with compensated row sums for FP32 ones. w_in and w_out are FP32. The products
+// w x (FP64, or FP32 split exactly) stay in shared memory for up to `hold` steps, and are then added in FP64,
+// a warp per step: added at every step they were a third of it. x^(k0) is x_first and
+// x^(k0 + m) = x_seg + (m - 1) stride, each loaded a step ahead.
+template <typename XT>
+struct AdjointRow;
+template <>
+struct AdjointRow<float> {
+    float ib_hi, ib_lo, x;  // 1 / beta as a float and its remainder: its rounding would be the same at every step
+    __device__ __forceinline__ explicit AdjointRow(double beta) : x(0.f) {
+        const double ib = 1.0 / beta;
+        ib_hi = static_cast<float>(ib);
+        ib_lo = static_cast<float>(ib - ib_hi);
+    }
+    __device__ __forceinline__ void set(float x_) { x = x_; }
+    template <typename F>
+    __device__ __forceinline__ float sum(double alpha, float w, int e0, int e1, F &&term) const {
+        const float a_hi = static_cast<float>(alpha), a_lo = static_cast<float>(alpha - a_hi);
+        DotSum32 acc;
+        acc.add(a_lo * w);
+        acc.add(a_hi, w);
+#pragma unroll 4
+        for (int e = e0; e < e1; ++e) term(e, [&](float v, float wj) { acc.add(v, wj); });
+        const float z = acc.s - acc.c;
+        return fmaf(z, ib_lo, z * ib_hi);
+    }
+    using Product = float2;  // rounded product and its error
+    static __device__ __forceinline__ float2 product(float a, float b) {
+        const float p = __fmul_rn(a, b);
+        return make_float2(p, fmaf(a, b, -p));
+    }
+    static __device__ __forceinline__ double value(float2 p) { return static_cast<double>(p.x) + static_cast<double>(p.y); }
+    __device__ __forceinline__ float weigh(float g) const { return x == 0.0f ? 0.0f : g / (3.0f * x * x); }
+};
+template <>
+struct AdjointRow<double> {
+    double ib, factor;  // factor = 1 / (3 x^2)
+    __device__ __forceinline__ explicit AdjointRow(double beta) : ib(1.0 / beta), factor(0.0) {}
+    __device__ __forceinline__ void set(double x) {
+        const double d = 3.0 * x * x;
+        const float df = static_cast<float>(d);
+        if (df > 1e-30f && df < 1e30f) {  // two Newton steps from the FP32 reciprocal
+            double r = static_cast<double>(1.0f / df);
+            r = fma(r, fma(-d, r, 1.0), r);
+            factor = r;
+        } else {
+            factor = d == 0.0 ? 0.0 : 1.0 / d;
+        }
+    }
+    template <typename F>
+    __device__ __forceinline__ double sum(double alpha, double w, int e0, int e1, F &&term) const {
+        double acc = alpha * w;
+#pragma unroll 4
+        for (int e = e0; e < e1; ++e) term(e, [&](double v, double wj) { acc += v * wj; });
+        return acc * ib;
+    }
+    using Product = double;
+    static __device__ __forceinline__ double product(double a, double b) { return a * b; }
+    static __device__ __forceinline__ double value(double p) { return p; }
+    __device__ __forceinline__ double weigh(double g) const { return g * factor; }
+};
+
+// bytes before the held products: cur | nxt (XT [n] each) | couplings (XT [cap]) | row ranges (int [rows + 1]) |
+// columns (uint16 [cap])
+template <typename XT>
+constexpr int64_t adjoint_held_at(int64_t n, int64_t rows, int64_t cap) {
+    return (static_cast<int64_t>(sizeof(XT)) * (2 * n + cap) + 4 * (rows + 1) + 2 * cap + 15) / 16 * 16;
+}
+
 template <typename XT, typename VT>
 __global__ void __launch_bounds__(1024)
 adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, const unsigned char *__restrict__ x_seg,
               size_t stride, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
               const VT *__restrict__ val, int n, int R, const double *__restrict__ alpha_tab,
-              const double *__restrict__ beta_tab, int k0, int len, int K, int rows_cap, int cap,
+              const double *__restrict__ beta_tab, int k0, int len, int K, int rows_cap, int cap, int hold,
               double *__restrict__ part, unsigned long long *__restrict__ zeros, int *__restrict__ err) {
     extern __shared__ __align__(16) unsigned char small_smem[];
     __shared__ Exchange ex;
-    __shared__ double red[2][32];  // by the step's parity: thread 0 reads one while the next step fills the other
     const int q = static_cast<int>(cl_rank());
     const int r = blockIdx.x / K;
     const int i0 = min(n, q * rows_cap), rows = min(n, i0 + rows_cap) - i0;
-    float *cur = reinterpret_cast<float *>(small_smem), *nxt = cur + n, *lv = nxt + n;
+    XT *cur = reinterpret_cast<XT *>(small_smem), *nxt = cur + n, *lv = nxt + n;
+    using Product = typename AdjointRow<XT>::Product;
+    Product *held = reinterpret_cast<Product *>(small_smem + adjoint_held_at<XT>(n, rows_cap, cap));
     int *lr = reinterpret_cast<int *>(lv + cap);
     uint16_t *lc = reinterpret_cast<uint16_t *>(lr + rows_cap + 1);
     for (int i = threadIdx.x; i < n; i += blockDim.x) cur[i] = w_in[static_cast<int64_t>(i) * R + r];
@@ -364,18 +431,18 @@ adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, c
     const int cnt = static_cast<int>(row_ptr[i0 + rows] - e0);  // <= cap
     for (int i = threadIdx.x; i <= rows; i += blockDim.x) lr[i] = static_cast<int>(row_ptr[i0 + i] - e0);
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-        lv[e] = static_cast<float>(val[e0 + e]);
+        lv[e] = static_cast<XT>(val[e0 + e]);
         lc[e] = static_cast<uint16_t>(col[e0 + e]);
     }
-    // alpha and 1 / beta as a float and its remainder: their rounding would be the same at every step
-    const double ib = 1.0 / beta_tab[0];
-    const float ib_hi = static_cast<float>(ib), ib_lo = static_cast<float>(ib - ib_hi);
     auto iterate = [&](int m) {
         return m == 0 ? x_first : reinterpret_cast<const XT *>(x_seg + static_cast<size_t>(m - 1) * stride);
     };
-    const int64_t at = static_cast<int64_t>(i0 + threadIdx.x) * R + r;  // the thread's first row
+    const int64_t at = static_cast<int64_t>(i0 + threadIdx.x) * R + r;  // the thread's row (rows <= blockDim.x)
     const bool has = threadIdx.x < rows;
-    XT x_own = has ? iterate(len - 1)[at] : XT(0);
+    const int own = i0 + static_cast<int>(threadIdx.x);
+    XT x_own = has ? iterate(len - 1)[at] : XT(0), x_next = has && len > 1 ? iterate(len - 2)[at] : XT(0);
+    AdjointRow<XT> row(beta_tab[0]);
+    row.set(x_own);
     unsigned nz = 0;
     exchange_init(ex);
     if (K > 1) cl_sync();
@@ -383,52 +450,42 @@ adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, c
     for (int m = len - 1; m >= 0; --m) {
         const int k = k0 + m;
         const double ad = __ldg(alpha_tab + k);
-        const float a_hi = static_cast<float>(ad), a_lo = static_cast<float>(ad - a_hi);
-        const XT *xm = iterate(m);
         const int s = len - 1 - m;
-        if (K > 1 && m > 0) exchange_expect(ex, s, static_cast<uint32_t>((n - rows) * sizeof(float)));
-        double ga = 0.0;
-        DotSum32 ga32;
-        for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-            const int64_t row = static_cast<int64_t>(i0 + i) * R + r;
-            const XT xc = i < static_cast<int>(blockDim.x) ? x_own : xm[row];
-            const int f1 = lr[i + 1];
-            const float wi = cur[i0 + i];
-            DotSum32 acc;
-            acc.add(a_lo * wi);
-            acc.add(a_hi, wi);
-#pragma unroll 4
-            for (int e = lr[i]; e < f1; ++e) acc.add(lv[e], cur[lc[e]]);
-            if constexpr (sizeof(XT) == 8) ga += static_cast<double>(wi) * xc;
-            else ga32.add(wi, xc);
-            const float z = acc.s - acc.c;
-            const float g = fmaf(z, ib_lo, z * ib_hi);
-            float out = g;
+        if (K > 1 && m > 0) exchange_expect(ex, s, static_cast<uint32_t>((n - rows) * sizeof(XT)));
+        if (has) {
+            const XT wi = cur[own];
+            const XT g = row.sum(ad, wi, lr[threadIdx.x], lr[threadIdx.x + 1],
+                                 [&](int e, auto &&add) { add(lv[e], cur[lc[e]]); });
+            XT out = g;
             if (k > 0) {
-                nz += xc == XT(0);
-                const float xf = static_cast<float>(xc);
-                out = xf == 0.0f ? 0.0f : g / (3.0f * xf * xf);
+                nz += x_own == XT(0);
+                out = row.weigh(g);
             }
             if (m == 0) {
-                w_out[row] = out;
-                continue;
+                w_out[at] = static_cast<float>(out);
+            } else {
+                nxt[own] = out;
+                exchange_send(ex, s, nxt + own, out, q, K);
             }
-            nxt[i0 + i] = out;
-            exchange_send(ex, s, nxt + i0 + i, out, q, K);
+            held[(s % hold) * rows_cap + threadIdx.x] = AdjointRow<XT>::product(wi, x_own);
         }
-        if (has && m > 0) x_own = iterate(m - 1)[at];
-        if constexpr (sizeof(XT) == 4) ga = ga32.value();
+        x_own = x_next;
+        row.set(x_own);
+        if (has && m > 1) x_next = iterate(m - 2)[at];
+        if (s % hold == hold - 1 || m == 0) {  // the held steps' sums: k + (s % hold) .. k
+            __syncthreads();
+            for (int t = threadIdx.x / 32; t <= s % hold; t += blockDim.x / 32) {
+                double ga = 0.0;
+                for (int i = threadIdx.x % 32; i < rows; i += 32) ga += AdjointRow<XT>::value(held[t * rows_cap + i]);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        if (threadIdx.x % 32 == 0) red[m & 1][threadIdx.x / 32] = ga;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t = 0.0;
-            for (int w = 0; w < static_cast<int>(blockDim.x / 32); ++w) t += red[m & 1][w];
-            part[static_cast<int64_t>(k) * gridDim.x + blockIdx.x] = t;
+                for (int o = 16; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+                if (threadIdx.x % 32 == 0)
+                    part[static_cast<int64_t>(k + s % hold - t) * gridDim.x + blockIdx.x] = ga;
+            }
+            __syncthreads();
         }
         if (m > 0 && !exchange_wait(ex, s, K, err)) break;
-        float *t = cur;
+        XT *t = cur;
         cur = nxt;
         nxt = t;
     }
@@ -498,8 +555,10 @@ ising_status_t launch_adjoint_k(const ising_context *c, const AdjointSegment &s,
     const int n = static_cast<int>(c->n), chunk = (n + K - 1) / K;
     int64_t most = std::min(c->max_row_nnz * chunk, c->nnz);
     most = (most + 3) / 4 * 4;
-    const int64_t smem = 8LL * n + 4 * (chunk + 1) + most * static_cast<int64_t>(sizeof(float) + sizeof(uint16_t));
-    if (smem > optin) return ISING_ERR_UNSUPPORTED;
+    const int64_t fixed_part = adjoint_held_at<XT>(n, chunk, most), step = 8LL * chunk;
+    if (fixed_part + step > optin || chunk > 1024) return ISING_ERR_UNSUPPORTED;
+    const int hold = static_cast<int>(std::min<int64_t>({s.len, 32, (optin - fixed_part) / step}));
+    const int64_t smem = fixed_part + hold * step;
     auto kern = adjoint_small<XT, VT>;
     DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
     if (K > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
@@ -529,7 +588,7 @@ ising_status_t launch_adjoint_k(const ising_context *c, const AdjointSegment &s,
                                  static_cast<const unsigned char *>(s.x_seg), s.stride,
                                  static_cast<const int64_t *>(c->row_ptr), static_cast<const int32_t *>(c->col),
                                  static_cast<const VT *>(c->val), n, R, p.alpha_d, p.beta_d, s.k0, s.len, K, chunk,
-                                 static_cast<int>(most), s.part, s.zeros, c->err_word));
+                                 static_cast<int>(most), hold, s.part, s.zeros, c->err_word));
     return ISING_OK;
 }
 
@@ -607,15 +666,16 @@ ising_status_t csr_small_run(const ising_context *c, const void *x_in, void *x_o
 
 // The adjoint's forward steps and adjoint steps run here for instances of at most 2048 spins with at
 // least four CTAs per replica; larger ones take single steps, whose launches overlap. Shared memory
-// against single steps, ms per gradient: FP64, 2000 spins, R = 8, 100 steps 1.37 / 1.49; 4000 spins, R = 4,
-// 60 steps 1.15 / 1.14, R = 16 1.44 / 1.22; FP32, 60 steps, 1000 spins, R = 16 0.75 / 0.87, 2000 spins, R = 8
-// 0.85 / 0.86, 6000 spins 1.10 / 0.88 (every new value is stored into all CTAs, 13 clocks a warp).
+// against single steps, ms per gradient: FP64, 2000 spins, R = 8, 100 steps 1.43 / 1.49 (relative error of
+// grad_x0 over twelve seeds 0.03 to 0.21 e-6 against 0.46 to 3.9 e-6); 1000 spins, R = 1, 60 steps 0.87 / 0.94;
+// 4000 spins, R = 16, with an FP32 state 1.44 / 1.22; FP32, 60 steps, 1000 spins, R = 16 0.76 / 0.87, 2000 spins,
+// R = 8 0.87 / 0.86, 6000 spins 1.10 / 0.88 (every new value is stored into all CTAs, 13 clocks a warp).
 bool backward_small(const ising_context *c, int xtype, int R) {
     return c->n_inst == 1 && c->n <= 2048 && static_cast<size_t>(c->n) <= csr_fused_max_spins(xtype) &&
            cluster_max(c, R) >= 4;
 }
 
-int adjoint_small_blocks(const ising_context *c, int R) { return R * cluster_max(c, R); }
+int adjoint_small_parts(const ising_context *c, int R) { return R * cluster_max(c, R); }
 
 ising_status_t adjoint_small_run(const ising_context *c, const AdjointSegment &s, int xtype, int R, const ParamTabs &p,
                                  int *blocks, cudaStream_t st) {
