@@ -620,3 +620,22 @@ def test_small_fp64_int8_steps(n, R, density, jmax, start):
     finally:
         N.ising_destroy(hd)
     assert np.all(np.linalg.norm(x - ref, axis=0) <= 1e-12 * np.linalg.norm(ref, axis=0))
+
+
+@pytest.mark.parametrize("n, per_row, R", [(2000, 110, 1), (2000, 110, 16), (5000, 60, 3), (5000, 110, 16)])
+def test_shares_that_do_not_fit_take_single_steps(n, per_row, R):
+    """Long integer rows around the size where a share's couplings no longer fit shared memory: both
+    routes against the oracle (FP32, three steps: reading of the conditioned bound)."""
+    hd = N.ising_create_s5(n, round(100.0 * per_row / n, 4), 5)
+    try:
+        g = N.ising_csr_export(hd)
+        J = I.CSR(n, g[0], g[1], g[2])
+        alpha, beta = O.alpha_beta(J, eta=1.0, method="wigner")
+        x0 = I.x0_uniform(n, R, seed=6)
+        x = torch.from_numpy(x0.copy()).cuda()
+        N.ising_iterate(hd, x, [alpha], [beta], 3)
+        ref = O.doch(O.Problem(J), x0.astype(np.float64), alpha, beta, 3)
+        err = np.linalg.norm(x.cpu().numpy() - ref, axis=0) / np.linalg.norm(ref, axis=0)
+        assert err.max() <= 1e-4 and np.median(err) <= 1e-5
+    finally:
+        N.ising_destroy(hd)
