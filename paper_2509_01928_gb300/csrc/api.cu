@@ -635,6 +635,13 @@ ising_status_t build_context(const HostProblem &hp, int flags, ising_context *c)
 size_t xtype_size(int t) { return dtype_size(t); }
 
 // upload the per-instance parameter tables and return views of them
+struct ParamBlob {
+    alignas(8) unsigned char bytes[3840];
+};
+__global__ void write_params(const __grid_constant__ ParamBlob blob, uint32_t *__restrict__ to, int words) {
+    for (int i = threadIdx.x; i < words; i += blockDim.x) to[i] = reinterpret_cast<const uint32_t *>(blob.bytes)[i];
+}
+
 ising_status_t upload_params(ising_context *c, const double *alpha, int alpha_len, const double *beta,
                              ParamTabs &out, cudaStream_t st) {
     const int ni = c->n_inst;
@@ -654,9 +661,12 @@ ising_status_t upload_params(ising_context *c, const double *alpha, int alpha_le
     auto al = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
     const size_t o1 = al(na * 8), o2 = o1 + al(ni * 8), o3 = o2 + al(na * 4), o4 = o3 + al(ni * 4),
                  o5 = o4 + al(ni * 4), tot = o5 + al(ni * 4);
-    // pinned staging, reused once its copy has read it: the call goes on to its kernels without waiting
-    // (a pageable copy and a synchronisation held the host 7.5 us and the stream behind its earlier work)
-    if (c->params_stage_bytes < tot) {
+    // small tables travel as a kernel's argument; larger ones through pinned staging, reused once its copy has
+    // read it: the call goes on to its kernels without waiting (a pageable copy and a synchronisation held
+    // the host 7.5 us; a copy engine's turn in the stream is a few us longer than a kernel's)
+    ParamBlob blob;
+    const bool small = tot <= sizeof(blob.bytes);
+    if (!small && c->params_stage_bytes < tot) {
         if (c->params_event) DOCH_CUDA(cudaEventSynchronize(c->params_event));
         if (c->params_stage) DOCH_CUDA(cudaFreeHost(c->params_stage));
         c->params_stage = nullptr;
@@ -664,9 +674,11 @@ ising_status_t upload_params(ising_context *c, const double *alpha, int alpha_le
         DOCH_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&c->params_stage), tot, cudaHostAllocDefault));
         c->params_stage_bytes = tot;
     }
-    if (!c->params_event) DOCH_CUDA(cudaEventCreateWithFlags(&c->params_event, cudaEventDisableTiming));
-    DOCH_CUDA(cudaEventSynchronize(c->params_event));
-    unsigned char *host = c->params_stage;
+    if (!small) {
+        if (!c->params_event) DOCH_CUDA(cudaEventCreateWithFlags(&c->params_event, cudaEventDisableTiming));
+        DOCH_CUDA(cudaEventSynchronize(c->params_event));
+    }
+    unsigned char *host = small ? blob.bytes : c->params_stage;
     std::memcpy(host, a.data(), na * 8);
     std::memcpy(host + o1, b.data(), ni * 8);
     for (size_t i = 0; i < na; ++i) reinterpret_cast<float *>(host + o2)[i] = static_cast<float>(a[i]);
@@ -678,8 +690,13 @@ ising_status_t upload_params(ising_context *c, const double *alpha, int alpha_le
         reinterpret_cast<float *>(host + o5)[i] = std::ldexp(1.0f, -k);
     }
     DOCH_CHECK(c->params.ensure(tot));
-    DOCH_CUDA(cudaMemcpyAsync(c->params.ptr, host, tot, cudaMemcpyHostToDevice, st));
-    DOCH_CUDA(cudaEventRecord(c->params_event, st));
+    if (small) {
+        write_params<<<1, 256, 0, st>>>(blob, c->params.as<uint32_t>(), static_cast<int>(tot / 4));
+        DOCH_CUDA(cudaGetLastError());
+    } else {
+        DOCH_CUDA(cudaMemcpyAsync(c->params.ptr, host, tot, cudaMemcpyHostToDevice, st));
+        DOCH_CUDA(cudaEventRecord(c->params_event, st));
+    }
     unsigned char *base = c->params.as<unsigned char>();
     out.alpha_d = reinterpret_cast<const double *>(base);
     out.beta_d = reinterpret_cast<const double *>(base + o1);

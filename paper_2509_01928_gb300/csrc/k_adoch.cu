@@ -169,11 +169,11 @@ adoch_step(Fn fn, Candidates<XT> x1, Candidates<XT> x0, XT *next_y, XT *next_x, 
     const int64_t hi = inst_off ? inst_off[b + 1] : n;
     const int64_t len = hi - lo;
     const int64_t s0 = lo + len * ch / chunks, s1 = lo + len * (ch + 1) / chunks;
-    const XT a = alpha_tab[b];
-    const AdochRoot<XT> root(beta_tab[b]);
     SiteSum<XT> acc[kTerms];
     pdl_wait();
     pdl_trigger();
+    const XT a = alpha_tab[b];
+    const AdochRoot<XT> root(beta_tab[b]);
     // one load of the decisions per block: all blocks ask one L2 slice for these lines
     __shared__ int dec[2][kAThreads];
     if (active && rl == 0) {
@@ -264,10 +264,10 @@ adoch_decide(const typename SiteSum<XT>::Slot *__restrict__ partials, int n_inst
     const int b = t / R;
     const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __shared__ double red[kTerms];
-    const double a = alpha_tab[b], be = beta_tab[b];
     double *ht = hist + static_cast<int64_t>(t) * (q + 1);
     pdl_wait();
     pdl_trigger();
+    const double a = alpha_tab[b], be = beta_tab[b];
     const typename SiteSum<XT>::Slot *p = partials + (static_cast<int64_t>(t) * kTerms + j) * chunks;
     SiteSum<XT> s;
     constexpr int kAhead = 8;  // loads in flight
