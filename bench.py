@@ -238,7 +238,7 @@ class Torus:
         self.units = float(self.n) * self.R * self.iters
         # three steps per lattice launch (the rest in one two-step or one single-step launch)
         self.dominant_launches = self.iters // STEPS_PER_LAUNCH + (1 if self.iters % STEPS_PER_LAUNCH else 0)
-        self.launches = self.dominant_launches + 3
+        self.launches = self.dominant_launches + 4
         self.config = {"workload": f"torus2d {self.L}x{self.L} +-1 int8 couplings, FP32 iterates, R=1, "
                                    f"{self.iters} DOCH iterations + sign + int64 energy/cut + best replica",
                        "n": self.n, "replicas": 1, "iters": self.iters,
@@ -342,7 +342,7 @@ class Dense:
         self.best = torch.zeros(1, dtype=torch.int32, device="cuda")
         self.units = float(self.n) * self.R * self.iters
         self.dominant_launches = self.iters
-        self.launches = self.iters + 2 + 4
+        self.launches = self.iters + 2 + 5
         self.config = {"workload": f"dense {self.n}x{self.n} +-1 (BF16, exact), R={self.R} BF16 replicas, "
                                    f"{self.iters} DOCH iterations on tcgen05 + exact int64 energy/cut",
                        "n": self.n, "replicas": self.R, "iters": self.iters,
@@ -432,7 +432,7 @@ class Precision:
         self.E = torch.zeros(self.R, dtype=torch.int64, device="cuda")
         self.units = float(self.n) * self.R * self.iters
         self.dominant_launches = self.iters
-        self.launches = self.iters + 2 + 4
+        self.launches = self.iters + 2 + 5
         self.stride, self.tol = args.precision_stride, args.precision_tol
         self.config = {"workload": f"dense {self.n}x{self.n} +-1, R={self.R}: BF16 tensor-core form "
                                    f"({self.iters} DOCH iterations + exact energy, timed) against the plain "
@@ -645,7 +645,7 @@ class Backward:
         self.loss = torch.zeros(1, dtype=torch.float64, device="cuda")
         self.units = float(self.n) * self.R * self.iters
         self.dominant_launches = self.iters
-        self.launches = 3 * self.iters + 4
+        self.launches = 3 * self.iters + 5
         self.config = {"workload": f"adjoint: random 3-regular n=1e5 +-1, R=64, {self.iters} FP32 iterations, "
                                    f"checkpoint every {self.ckpt}: loss + dL/dalpha[200] + dL/dx0",
                        "n": self.n, "replicas": self.R, "iters": self.iters,
@@ -812,7 +812,7 @@ class Adoch:
         self.dominant_launches = self.iters  # one ADOCH step = pass + decide + update
         # step 0: pass + decide; steps 1..N-1: one pass (update and next terms) + boundary edges +
         # decide; the last step: update only; readout: row_reduce + energy_finish
-        self.launches = 3 * self.iters + 2
+        self.launches = 3 * self.iters + 3
         self.config = {"workload": f"ADOCH (Algorithm 2) on the torus2d {self.L}x{self.L} +-1 int8 lattice, FP32, "
                                    f"R=1, q={self.q}, {self.iters} steps + sign + int64 energy",
                        "n": self.n, "replicas": 1, "iters": self.iters, "q": self.q,
@@ -895,7 +895,7 @@ class S5:
         self.E = torch.zeros(self.R, dtype=torch.int64, device="cuda")
         self.units = float(self.n) * self.R * self.iters
         self.dominant_launches = self.iters
-        self.launches = self.iters + 3
+        self.launches = self.iters + 4
         self.config = {"workload": f"Algorithm S5 n={self.n} p={self.p}% (9-bit couplings, {self.nnz} stored "
                                    f"entries) generated on the device, Wigner parameters on the device, R={self.R} "
                                    f"FP32, {self.iters} DOCH steps + sign + int64 energy",
@@ -978,7 +978,7 @@ class Proc:
         self.units = float(self.n) * self.R * self.iters
         self.dominant_launches = self.iters
         # per DOCH step: max |x|, symmetric product, finish; readout: spins, product, quadratic form
-        self.launches = 3 * self.iters + 3
+        self.launches = 3 * self.iters + 4
         self.config = {"workload": f"procedural dense J_ij = sin(ij + 100), n={self.n} (n^2 = {self.n ** 2:.1e} "
                                    f"couplings generated per product), R={self.R}, FP32, {self.iters} DOCH steps "
                                    f"+ sign + FP64 energy",

@@ -167,7 +167,7 @@ csr_step_pipe_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64
     pipe_first_batch<kPipeB>(col, val, e0, e1, js, ws);
     pdl_wait();  // the couplings above are never written
     pdl_trigger();
-    const XT a = __ldcg(alpha_tab + (alpha_len == 1 ? 0 : k));
+    const XT a = __ldg(alpha_tab + (alpha_len == 1 ? 0 : k));
     const StepRoot<XT> root(beta_tab, zs_tab, xs_tab, 0);
     for (; i < n; i += S) {
         const int cnt = e1 - e0 < kPipeB ? static_cast<int>(e1 - e0) : kPipeB;

@@ -8,8 +8,8 @@
 // counts the bytes that arrive (about 650 clocks per step). P threads share a row: each adds every P-th
 // entry, a shuffle tree adds the P sums, and then one thread per row takes the cube root, in
 // whole warps. The couplings of a CTA's rows are copied to shared memory once per launch, already
-// in the iterate's type (FP64 iterates and 8-bit couplings: the upper words of the FP64 values,
-// whose lower words are zero, 6 instead of 10 bytes an entry).
+// in the iterate's type (FP64 iterates and 8-bit couplings: the integers, or the upper words of the
+// FP64 values, whose lower words are zero: 6 instead of 10 bytes an entry).
 //
 // Bound by FP64 arithmetic (half a lane per clock and SM partition, about 150 clocks from one operation
 // to the next that needs it; an integer -> FP64 conversion costs as much as an FMA) and the latency of
@@ -118,7 +118,7 @@ struct Held<double, int8_t> {  // the integer (fixed-point steps), or the FP64 v
 // (FP64 sums round by about M 2^-53 at every addition; relative error against plain FP64 arithmetic in
 // torch over 1000 steps of 800 spins, R = 8, six seeds: 4.41e-16 to 5.33e-16 in FP64, 4.40e-16 to 5.30e-16
 // in fixed point; 60 steps of 1500 spins, R = 4: 0.6e-15 to 4.0e-15 and 0.6e-15 to 3.1e-15). M of the next
-// iterate follows from |x'| <= cbrt((rowabs + |alpha|) M + max |h|) / beta), rounded up. x itself is
+// iterate follows from |x'| <= cbrt(((rowabs + |alpha|) M + max |h|) / beta), rounded up. x itself is
 // kept in FP64 where it is added (alpha x) and returned. Runs that record iterates keep FP64 sums: their
 // scales would depend on where a run starts.
 __device__ __forceinline__ float next_bound(float m, float rowabs, float alpha, float hmax, float inv_beta) {

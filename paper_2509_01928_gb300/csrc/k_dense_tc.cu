@@ -656,10 +656,18 @@ ising_status_t dense_energy(ising_context *c, const void *x, int xtype, int R, i
     DOCH_CUDA(cudaMemsetAsync(hs, 0, sizeof(long long) * R, st));
     const dim3 tg(static_cast<unsigned>(g.kblocks), static_cast<unsigned>((g.R_pad + kTR - 1) / kTR));
     switch (xtype) {
-        case ISING_BF16: to_replica_major<__nv_bfloat16, true><<<tg, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), sp, g.n, R, g.R_pad); break;
-        case ISING_F32: to_replica_major<float, true><<<tg, 256, 0, st>>>(static_cast<const float *>(x), sp, g.n, R, g.R_pad); break;
-        case ISING_F64: to_replica_major<double, true><<<tg, 256, 0, st>>>(static_cast<const double *>(x), sp, g.n, R, g.R_pad); break;
-        case ISING_I8: to_replica_major<int8_t, true><<<tg, 256, 0, st>>>(static_cast<const int8_t *>(x), sp, g.n, R, g.R_pad); break;
+        case ISING_BF16:
+            to_replica_major<__nv_bfloat16, true><<<tg, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), sp, g.n, R, g.R_pad);
+            break;
+        case ISING_F32:
+            to_replica_major<float, true><<<tg, 256, 0, st>>>(static_cast<const float *>(x), sp, g.n, R, g.R_pad);
+            break;
+        case ISING_F64:
+            to_replica_major<double, true><<<tg, 256, 0, st>>>(static_cast<const double *>(x), sp, g.n, R, g.R_pad);
+            break;
+        case ISING_I8:
+            to_replica_major<int8_t, true><<<tg, 256, 0, st>>>(static_cast<const int8_t *>(x), sp, g.n, R, g.R_pad);
+            break;
         default: return fail(ISING_ERR_INVALID_ARG, "dense energy: x type");
     }
     DOCH_CUDA(cudaGetLastError());

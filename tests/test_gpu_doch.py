@@ -625,7 +625,8 @@ def test_small_fp64_int8_steps(n, R, density, jmax, start):
 @pytest.mark.parametrize("n, per_row, R", [(2000, 110, 1), (2000, 110, 16), (5000, 60, 3), (5000, 110, 16)])
 def test_shares_that_do_not_fit_take_single_steps(n, per_row, R):
     """Long integer rows around the size where a share's couplings no longer fit shared memory: both
-    routes against the oracle (FP32, three steps: reading of the conditioned bound)."""
+    routes against the oracle. FP32, three steps of sums of about 100 terms: 1e-5 for the median replica,
+    1e-4 where a component passes near zero."""
     hd = N.ising_create_s5(n, round(100.0 * per_row / n, 4), 5)
     try:
         g = N.ising_csr_export(hd)
