@@ -730,7 +730,7 @@ class Er800:
         self.best = torch.zeros(1, dtype=torch.int32, device="cuda")
         self.units = float(self.n) * self.R * self.iters
         self.dominant_launches = 1
-        self.launches = 1 + 3
+        self.launches = 1 + 4
         self.config = {"workload": "plain method FP64: Erdos-Renyi n=800 p=0.06 +-1, R=8, 1000 iterations "
                                    "(one launch, iterate in shared memory) + int64 energy/cut + best replica",
                        "n": self.n, "replicas": self.R, "iters": self.iters, "l2": "on-chip problem"}
