@@ -1764,8 +1764,15 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
         int gc = 0;
         DOCH_CHECK(csr_loss_w(c, xs(S - 1, seg_len(S - 1)), xtype, gbuf[gc], R, V, grid, lpart, zeros_d, st));
         const float inv_beta = static_cast<float>(1.0 / beta);
+        // one plan for all segments, whatever their lengths: it also lays out `part`
+        AdjointPlan plan;
         bool small_adjoint = small;
-        int pblocks = grid;  // partial sums per step in `part`
+        if (small_adjoint) {
+            const ising_status_t ps = adjoint_small_plan(c, xtype, R, iters, plan);
+            if (ps != ISING_OK && ps != ISING_ERR_UNSUPPORTED) return ps;
+            small_adjoint = ps == ISING_OK;
+        }
+        const int pblocks = small_adjoint ? plan.parts : grid;  // partial sums per step
         for (int sg_i = S - 1; sg_i >= 0; --sg_i) {
             const int len = seg_len(sg_i);
             if (sg_i < S - 1 && len > 1) {  // the last segment's iterates are still in place from the forward pass
@@ -1776,14 +1783,9 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
             }
             if (small_adjoint) {
                 const AdjointSegment as{gbuf[gc], gbuf[1 - gc], ck(sg_i), sg(0), A, sg_i * C, len, part, zeros_d};
-                const ising_status_t rs = adjoint_small_run(c, as, xtype, R, p, &pblocks, st);
-                if (rs == ISING_OK) {
-                    gc = 1 - gc;
-                    continue;
-                }
-                if (rs != ISING_ERR_UNSUPPORTED || sg_i < S - 1) return rs;
-                small_adjoint = false;  // refused at the first segment: single steps for all of them
-                pblocks = grid;
+                DOCH_CHECK(adjoint_small_run(c, plan, as, xtype, R, p, st));
+                gc = 1 - gc;
+                continue;
             }
             for (int m = len - 1; m >= 0; --m) {
                 const int k = sg_i * C + m;

@@ -410,8 +410,14 @@ ising_status_t csr_adjoint_step(const ising_context *c, const float *w_in, const
                                 int grid, double *part, unsigned long long *zeros, cudaStream_t st);
 // Adjoint steps k0 + len - 1 .. k0 in one launch for an instance that fits in shared memory
 // (k_csr_small.cu): w_in = w^(k0 + len - 1), w_out = w^(k0 - 1) or g^0; x_first = x^(k0),
-// x^(k0 + m) = x_seg + (m - 1) stride; part [iters][blocks] with the number of partial sums per step returned
-// (the same for every segment, at most adjoint_small_parts). ISING_ERR_UNSUPPORTED when it does not fit.
+// x^(k0 + m) = x_seg + (m - 1) stride; part [iters][parts]. The plan, and with it the number of partial
+// sums per step, is one for all segments of a gradient and the same for every checkpoint interval: made by
+// adjoint_small_plan from the gradient's steps (ISING_ERR_UNSUPPORTED when the instance does not fit).
+struct AdjointPlan {
+    int K = 0;      // CTAs per replica
+    int hold = 0;   // steps whose products are held before they are added
+    int parts = 0;  // partial sums per step, R K <= adjoint_small_parts
+};
 struct AdjointSegment {
     const float *w_in;
     float *w_out;
@@ -424,8 +430,9 @@ struct AdjointSegment {
 };
 bool backward_small(const ising_context *c, int xtype, int R);
 int adjoint_small_parts(const ising_context *c, int R);
-ising_status_t adjoint_small_run(const ising_context *c, const AdjointSegment &s, int xtype, int R, const ParamTabs &p,
-                                 int *blocks, cudaStream_t st);
+ising_status_t adjoint_small_plan(const ising_context *c, int xtype, int R, int iters, AdjointPlan &plan);
+ising_status_t adjoint_small_run(const ising_context *c, const AdjointPlan &plan, const AdjointSegment &s, int xtype,
+                                 int R, const ParamTabs &p, cudaStream_t st);
 ising_status_t widen_f32_to_f64(const float *a, double *b, int64_t count, int num_sms, cudaStream_t st);
 ising_status_t adjoint_finish_launch(const double *part, int iters, int blocks, double beta,
                                      const double *lpart, int lblocks, int R, double *grad_alpha,

@@ -550,61 +550,87 @@ ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R
     return ISING_OK;
 }
 
-// The adjoint in clusters of K CTAs; ISING_ERR_UNSUPPORTED where the state, or the couplings of the
-// fullest share, do not fit, or the clusters of all replicas do not run at once.
+// room for the couplings of the fullest share of a cluster of K CTAs
+int64_t adjoint_cap(const ising_context *c, int K) {
+    const int64_t chunk = (c->n + K - 1) / K;
+    return (std::min(c->max_row_nnz * chunk, c->nnz) + 3) / 4 * 4;
+}
+
 template <typename XT, typename VT>
-ising_status_t launch_adjoint_k(const ising_context *c, const AdjointSegment &s, int R, const ParamTabs &p, int K,
-                                int64_t optin, cudaStream_t st) {
-    const int n = static_cast<int>(c->n), chunk = (n + K - 1) / K;
-    int64_t most = std::min(c->max_row_nnz * chunk, c->nnz);
-    most = (most + 3) / 4 * 4;
-    const int64_t fixed_part = adjoint_held_at<XT>(n, chunk, most), step = 8LL * chunk;
-    if (fixed_part + step > optin || chunk > 1024) return ISING_ERR_UNSUPPORTED;
-    const int hold = static_cast<int>(std::min<int64_t>({s.len, 32, (optin - fixed_part) / step}));
-    const int64_t smem = fixed_part + hold * step;
+ising_status_t adjoint_config(const ising_context *c, int R, const AdjointPlan &plan, cudaLaunchConfig_t &cfg,
+                              cudaLaunchAttribute *attr) {
+    const int n = static_cast<int>(c->n), chunk = (n + plan.K - 1) / plan.K;
+    const int64_t smem = adjoint_held_at<XT>(n, chunk, adjoint_cap(c, plan.K)) + plan.hold * 8LL * chunk;
     auto kern = adjoint_small<XT, VT>;
     DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    if (K > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (plan.K > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
         return ISING_ERR_UNSUPPORTED;
     }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(K);
+    attr[0].val.clusterDim.x = static_cast<unsigned>(plan.K);
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(static_cast<unsigned>(R * K));
+    cfg.gridDim = dim3(static_cast<unsigned>(R * plan.K));
     cfg.blockDim = dim3(static_cast<unsigned>(std::min(1024, (chunk + 31) / 32 * 32)));
     cfg.dynamicSmemBytes = static_cast<size_t>(smem);
-    cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (K > 1) {
-        int nclusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg) != cudaSuccess || nclusters < R) {
-            cudaGetLastError();
-            return ISING_ERR_UNSUPPORTED;
-        }
-    }
-    DOCH_CUDA(cudaLaunchKernelEx(&cfg, kern, s.w_in, s.w_out, static_cast<const XT *>(s.x_first),
-                                 static_cast<const unsigned char *>(s.x_seg), s.stride,
-                                 static_cast<const int64_t *>(c->row_ptr), static_cast<const int32_t *>(c->col),
-                                 static_cast<const VT *>(c->val), n, R, p.alpha_d, p.beta_d, s.k0, s.len, K, chunk,
-                                 static_cast<int>(most), hold, s.part, s.zeros, c->err_word));
     return ISING_OK;
 }
 
-template <typename XT>
-ising_status_t adjoint_dispatch_k(const ising_context *c, const AdjointSegment &s, int R, const ParamTabs &p, int K,
-                                  int64_t optin, cudaStream_t st) {
-    switch (c->jtype) {
-        case ISING_I8: return launch_adjoint_k<XT, int8_t>(c, s, R, p, K, optin, st);
-        case ISING_I32: return launch_adjoint_k<XT, int32_t>(c, s, R, p, K, optin, st);
-        case ISING_F32: return launch_adjoint_k<XT, float>(c, s, R, p, K, optin, st);
-        case ISING_F64: return launch_adjoint_k<XT, double>(c, s, R, p, K, optin, st);
-        default: return fail(ISING_ERR_UNSUPPORTED, "backward: coupling type");
+// The largest cluster whose shares fit and whose copies for all replicas run at once
+template <typename XT, typename VT>
+ising_status_t adjoint_plan(const ising_context *c, int R, int iters, int64_t optin, AdjointPlan &plan) {
+    for (plan.K = cluster_max(c, R); plan.K >= 1; --plan.K) {
+        const int n = static_cast<int>(c->n), chunk = (n + plan.K - 1) / plan.K;
+        const int64_t left = optin - adjoint_held_at<XT>(n, chunk, adjoint_cap(c, plan.K)), step = 8LL * chunk;
+        if (left < step || chunk > 1024) continue;
+        plan.hold = static_cast<int>(std::min<int64_t>({iters, 32, left / step}));
+        plan.parts = R * plan.K;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        const ising_status_t s = adjoint_config<XT, VT>(c, R, plan, cfg, attr);
+        if (s == ISING_ERR_UNSUPPORTED) continue;
+        DOCH_CHECK(s);
+        if (plan.K == 1) return ISING_OK;
+        int nclusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&nclusters, adjoint_small<XT, VT>, &cfg) == cudaSuccess && nclusters >= R)
+            return ISING_OK;
+        cudaGetLastError();
     }
+    return ISING_ERR_UNSUPPORTED;
+}
+
+template <typename XT, typename VT>
+ising_status_t launch_adjoint(const ising_context *c, const AdjointPlan &plan, const AdjointSegment &s, int R,
+                              const ParamTabs &p, cudaStream_t st) {
+    const int n = static_cast<int>(c->n), chunk = (n + plan.K - 1) / plan.K;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    DOCH_CHECK((adjoint_config<XT, VT>(c, R, plan, cfg, attr)));
+    cfg.stream = st;
+    DOCH_CUDA(cudaLaunchKernelEx(&cfg, adjoint_small<XT, VT>, s.w_in, s.w_out, static_cast<const XT *>(s.x_first),
+                                 static_cast<const unsigned char *>(s.x_seg), s.stride,
+                                 static_cast<const int64_t *>(c->row_ptr), static_cast<const int32_t *>(c->col),
+                                 static_cast<const VT *>(c->val), n, R, p.alpha_d, p.beta_d, s.k0, s.len, plan.K, chunk,
+                                 static_cast<int>(adjoint_cap(c, plan.K)), plan.hold, s.part, s.zeros, c->err_word));
+    return ISING_OK;
+}
+
+// f(XT(), VT()) for the types of the iterates and the couplings
+template <typename F>
+ising_status_t adjoint_types(const ising_context *c, int xtype, F &&f) {
+    auto couplings = [&](auto x) -> ising_status_t {
+        switch (c->jtype) {
+            case ISING_I8: return f(x, int8_t());
+            case ISING_I32: return f(x, int32_t());
+            case ISING_F32: return f(x, float());
+            case ISING_F64: return f(x, double());
+            default: return fail(ISING_ERR_UNSUPPORTED, "backward: coupling type");
+        }
+    };
+    return xtype == ISING_F64 ? couplings(double()) : couplings(float());
 }
 
 template <typename XT, typename VT>
@@ -680,20 +706,22 @@ bool backward_small(const ising_context *c, int xtype, int R) {
 
 int adjoint_small_parts(const ising_context *c, int R) { return R * cluster_max(c, R); }
 
-ising_status_t adjoint_small_run(const ising_context *c, const AdjointSegment &s, int xtype, int R, const ParamTabs &p,
-                                 int *blocks, cudaStream_t st) {
+ising_status_t adjoint_small_plan(const ising_context *c, int xtype, int R, int iters, AdjointPlan &plan) {
     int dev = 0, optin = 0;
     DOCH_CUDA(cudaGetDevice(&dev));
     DOCH_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     optin -= kStaticSmem;
     if (c->n_inst != 1 || c->n > 65536) return ISING_ERR_UNSUPPORTED;
-    for (int K = cluster_max(c, R); K >= 1; --K) {
-        const ising_status_t e = xtype == ISING_F64 ? adjoint_dispatch_k<double>(c, s, R, p, K, optin, st)
-                                                    : adjoint_dispatch_k<float>(c, s, R, p, K, optin, st);
-        *blocks = R * K;
-        if (e != ISING_ERR_UNSUPPORTED) return e;
-    }
-    return ISING_ERR_UNSUPPORTED;
+    return adjoint_types(c, xtype, [&](auto x, auto v) {
+        return adjoint_plan<decltype(x), decltype(v)>(c, R, iters, optin, plan);
+    });
+}
+
+ising_status_t adjoint_small_run(const ising_context *c, const AdjointPlan &plan, const AdjointSegment &s, int xtype,
+                                 int R, const ParamTabs &p, cudaStream_t st) {
+    return adjoint_types(c, xtype, [&](auto x, auto v) {
+        return launch_adjoint<decltype(x), decltype(v)>(c, plan, s, R, p, st);
+    });
 }
 
 ising_status_t csr_fused(const ising_context *c, void *x, int xtype, int R, const ParamTabs &p, int iters,

@@ -121,6 +121,42 @@ def test_adjoint_of_small_instances(n, R, iters, ckpt):
     assert _rel(gx, gx_r) <= 1e-3 and np.abs(gx - gx_r).max() <= 1e-3 * np.abs(gx_r).max()
 
 
+@pytest.mark.parametrize("per_row, R, iters, ckpt", [(35, 10, 65, 32), (30, 10, 65, 32), (55, 11, 42, 20), (70, 10, 33, 32),
+                                                     (40, 14, 65, 32), (55, 16, 21, 20)])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_adjoint_of_long_rows_with_a_short_last_segment(per_row, R, iters, ckpt, dtype):
+    """Segments of different lengths need different shared memory, which decides how many CTAs a
+    replica can have: every dL/dalpha_k must come from the same layout of partial sums. FP64 gradients
+    are compared entry by entry, FP32 ones by norm within what the rounding of their trajectory moves
+    (about 2e-2 at most, as above) and bit by bit between checkpoint intervals."""
+    g = I.erdos_renyi_pm1(2000, per_row / 2000, seed=89)
+    P = O.Problem(g)
+    a0, beta = O.alpha_beta(g, eta=1.0, method="wigner")
+    alpha = a0 * (1.0 + 0.1 * np.cos(np.arange(iters) / 3.0))
+    x0 = O.doch(P, I.x0_uniform(g.n, R, seed=90, dtype=np.float64), a0, beta, 300).astype(dtype)
+    ga_r, gx_r, loss_r, z_r = O.backward(P, x0, alpha, beta, iters)
+    h = N.ising_create(N.Problem(g))
+    try:
+        ga, gx, loss, ze = _gpu_backward(h, x0, alpha, beta, iters, ckpt)
+        ga1, gx1, loss1, _ = _gpu_backward(h, x0, alpha, beta, iters, 1)
+        gan, gxn, lossn, _ = _gpu_backward(h, x0, alpha, beta, iters, iters)
+    finally:
+        N.ising_destroy(h)
+    assert ze == z_r
+    assert loss == loss1 == lossn == pytest.approx(loss_r, rel=1e-5)
+    if dtype == np.float32:
+        assert _rel(ga, ga_r) <= 2e-2
+        for o_ga, o_gx in ((ga1, gx1), (gan, gxn)):
+            assert np.array_equal(o_ga, ga) and np.array_equal(o_gx, gx)
+        return
+    # each entry against the size of its own step's neighbours: the gradients of early steps are small
+    near = np.maximum.reduce([np.abs(np.roll(ga_r, k)) for k in (-2, -1, 0, 1, 2)])
+    assert np.all(np.abs(ga - ga_r) <= 1e-3 * near)
+    assert _rel(gx, gx_r) <= 1e-3
+    for o_ga, o_gx in ((ga1, gx1), (gan, gxn)):  # between segments the state is rounded to FP32
+        assert _rel(o_ga, ga) <= 1e-5 and _rel(o_gx, gx) <= 1e-5
+
+
 def test_adjoint_with_field_and_gaussian_couplings():
     g = I.regular_gauss(2000, 5, seed=82)
     hf = I.field_gauss(g.n, 0.1, seed=83)
