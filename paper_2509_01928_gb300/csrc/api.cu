@@ -1717,7 +1717,8 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
         // layout of the handle's checkpoint buffer
         auto al = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
         const size_t A = al(static_cast<size_t>(c->n) * R * xel);        // one iterate
-        const size_t G = al(static_cast<size_t>(c->n) * R * sizeof(float)); // one adjoint state
+        // one adjoint state: FP32, or the iterate's type where the small path may run
+        const size_t G = backward_small(c, xtype, R) ? A : al(static_cast<size_t>(c->n) * R * sizeof(float));
         const size_t part_b = al(sizeof(double) * static_cast<size_t>(iters) *
                                  static_cast<size_t>(std::max(grid, backward_small(c, xtype, R) ? adjoint_small_parts(c, R) : 0)));
         const size_t lpart_b = al(sizeof(double) * grid);
@@ -1773,6 +1774,11 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
             small_adjoint = ps == ISING_OK;
         }
         const int pblocks = small_adjoint ? plan.parts : grid;  // partial sums per step
+        const bool state64 = small_adjoint && xtype == ISING_F64;
+        if (state64) {
+            DOCH_CHECK(widen_f32_to_f64(gbuf[gc], reinterpret_cast<double *>(gbuf[1 - gc]), c->n * R, c->num_sms, st));
+            gc = 1 - gc;
+        }
         for (int sg_i = S - 1; sg_i >= 0; --sg_i) {
             const int len = seg_len(sg_i);
             if (sg_i < S - 1 && len > 1) {  // the last segment's iterates are still in place from the forward pass
@@ -1803,7 +1809,7 @@ ising_status_t ising_backward(ising_handle_t h, const void *x0, int32_t xtype, i
             DOCH_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, st));
             return ISING_OK;
         };
-        if (xtype == ISING_F64) {
+        if (xtype == ISING_F64 && !state64) {
             DOCH_CHECK(widen_f32_to_f64(gbuf[gc], wide, c->n * R, c->num_sms, st));
             DOCH_CHECK(put(grad_x0, wide, xbytes));
         } else {

@@ -409,7 +409,7 @@ ising_status_t csr_adjoint_step(const ising_context *c, const float *w_in, const
                                 float *w_out, int R, int V, float alpha_k, float inv_beta, bool final_step,
                                 int grid, double *part, unsigned long long *zeros, cudaStream_t st);
 // Adjoint steps k0 + len - 1 .. k0 in one launch for an instance that fits in shared memory
-// (k_csr_small.cu): w_in = w^(k0 + len - 1), w_out = w^(k0 - 1) or g^0; x_first = x^(k0),
+// (k_csr_small.cu): w_in = w^(k0 + len - 1), w_out = w^(k0 - 1) or g^0, both in the iterate's type; x_first = x^(k0),
 // x^(k0 + m) = x_seg + (m - 1) stride; part [iters][parts]. The plan, and with it the number of partial
 // sums per step, is one for all segments of a gradient and the same for every checkpoint interval: made by
 // adjoint_small_plan from the gradient's steps (ISING_ERR_UNSUPPORTED when the instance does not fit).
@@ -419,8 +419,8 @@ struct AdjointPlan {
     int parts = 0;  // partial sums per step, R K <= adjoint_small_parts
 };
 struct AdjointSegment {
-    const float *w_in;
-    float *w_out;
+    const void *w_in;  // the iterate's type
+    void *w_out;
     const void *x_first;
     const void *x_seg;
     size_t stride;

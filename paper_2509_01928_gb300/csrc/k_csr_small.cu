@@ -338,9 +338,10 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
 // the adjoint state w^k held as csr_small holds its iterate, a cluster per replica and a thread per row,
 //   g^k = (J w^k + alpha_k w^k) / beta,   w^(k-1) = g^k / (3 (x^k)^2)  (g^0 itself when k = 0),
 // and the partial sums of dL/dalpha_k = sum w^k x^k / beta of every CTA into part[k][CTA]. Within a
-// run the state has the iterate's type: FP64 for FP64 iterates (few rows per CTA, so the latency of the
+// gradient the state has the iterate's type, between segments too (the result does not depend on the
+// checkpoint interval): FP64 for FP64 iterates (few rows per CTA, so the latency of the
 // chain counts and not the FP64 rate; the factor 1 / (3 beta x^2) is formed before the wait for the
-// peers' shares); FP32 with compensated row sums for FP32 ones. w_in and w_out are FP32. The products
+// peers' shares); FP32 with compensated row sums for FP32 ones. The products
 // w x (FP64, or FP32 split exactly) stay in shared memory for up to `hold` steps, and are then added in FP64,
 // a warp per step: added at every step they were a third of it. x^(k0) is x_first and
 // x^(k0 + m) = x_seg + (m - 1) stride, each loaded a step ahead.
@@ -411,7 +412,7 @@ constexpr int64_t adjoint_held_at(int64_t n, int64_t rows, int64_t cap) {
 
 template <typename XT, typename VT>
 __global__ void __launch_bounds__(1024)
-adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, const unsigned char *__restrict__ x_seg,
+adjoint_small(const XT *w_in, XT *w_out, const XT *__restrict__ x_first, const unsigned char *__restrict__ x_seg,
               size_t stride, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
               const VT *__restrict__ val, int n, int R, const double *__restrict__ alpha_tab,
               const double *__restrict__ beta_tab, int k0, int len, int K, int rows_cap, int cap, int hold,
@@ -462,7 +463,7 @@ adjoint_small(const float *w_in, float *w_out, const XT *__restrict__ x_first, c
                 out = row.weigh(g);
             }
             if (m == 0) {
-                w_out[at] = static_cast<float>(out);
+                w_out[at] = out;
             } else {
                 nxt[own] = out;
                 exchange_send(ex, s, nxt + own, out, q, K);
@@ -610,8 +611,8 @@ ising_status_t launch_adjoint(const ising_context *c, const AdjointPlan &plan, c
     cudaLaunchAttribute attr[1];
     DOCH_CHECK((adjoint_config<XT, VT>(c, R, plan, cfg, attr)));
     cfg.stream = st;
-    DOCH_CUDA(cudaLaunchKernelEx(&cfg, adjoint_small<XT, VT>, s.w_in, s.w_out, static_cast<const XT *>(s.x_first),
-                                 static_cast<const unsigned char *>(s.x_seg), s.stride,
+    DOCH_CUDA(cudaLaunchKernelEx(&cfg, adjoint_small<XT, VT>, static_cast<const XT *>(s.w_in), static_cast<XT *>(s.w_out),
+                                 static_cast<const XT *>(s.x_first), static_cast<const unsigned char *>(s.x_seg), s.stride,
                                  static_cast<const int64_t *>(c->row_ptr), static_cast<const int32_t *>(c->col),
                                  static_cast<const VT *>(c->val), n, R, p.alpha_d, p.beta_d, s.k0, s.len, plan.K, chunk,
                                  static_cast<int>(adjoint_cap(c, plan.K)), plan.hold, s.part, s.zeros, c->err_word));
