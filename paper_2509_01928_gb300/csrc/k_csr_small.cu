@@ -60,8 +60,10 @@ __device__ __forceinline__ void cl_send(uint32_t a, float v, uint32_t bar) {
 // The exchange of a cluster's shares. Every CTA counts the bytes its peers send for step k on one of
 // two mbarriers (k even / odd). A peer sends step k + 1 only after this CTA's step k reached it whole,
 // which this CTA sends after it has received step k - 1: so two mbarriers, and two copies of the
-// iterate, are enough, and no cluster-wide barrier is needed. Waits are bounded (1 s): on expiry the
-// error word is set and the kernel ends at its closing cluster barrier.
+// iterate, are enough, and no cluster-wide barrier is needed. This holds among the CTAs that own rows,
+// the first `owners` of the cluster. One without rows (a short instance beside a long one, whose size
+// sets the cluster's) holds nobody up: it takes no part, and nothing is sent to it. Waits are bounded
+// (1 s): on expiry the error word is set and the kernel ends at its closing cluster barrier.
 struct Exchange {
     unsigned long long bar[2];
     int abort_flag;
@@ -81,15 +83,15 @@ __device__ __forceinline__ void exchange_expect(Exchange &x, int s, uint32_t byt
     if (threadIdx.x == 0) mbar_expect_tx(&x.bar[s & 1], bytes);
 }
 template <typename T>
-__device__ __forceinline__ void exchange_send(Exchange &x, int s, T *slot, T v, int q, int K) {
-    for (int t = 1; t < K; ++t) {
-        const uint32_t to = static_cast<uint32_t>(q + t < K ? q + t : q + t - K);
+__device__ __forceinline__ void exchange_send(Exchange &x, int s, T *slot, T v, int q, int owners) {
+    for (int t = 1; t < owners; ++t) {
+        const uint32_t to = static_cast<uint32_t>(q + t < owners ? q + t : q + t - owners);
         cl_send(cl_map(slot, to), v, cl_map(&x.bar[s & 1], to));
     }
 }
 // all threads: this CTA's own share is written and the peers' have arrived
-__device__ __forceinline__ bool exchange_wait(Exchange &x, int s, int K, int *err) {
-    if (K == 1) {
+__device__ __forceinline__ bool exchange_wait(Exchange &x, int s, int owners, int *err) {
+    if (owners == 1) {
         __syncthreads();
         return true;
     }
@@ -164,6 +166,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     const int nb = static_cast<int>(hi - lo);
     const int chunk = (nb + K - 1) / K;  // <= rows_cap
     const int i0 = min(nb, q * chunk), i1 = min(nb, i0 + chunk), rows = i1 - i0;
+    const int owners = (nb + chunk - 1) / chunk;  // CTAs with rows: 0 .. owners - 1
     XT *cur = reinterpret_cast<XT *>(small_smem), *nxt = cur + nb;
     XT *z = nxt + nb;
     using Hd = Held<XT, VT>;
@@ -253,9 +256,9 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     // every CTA of the cluster runs, and has loaded, before the first remote store
     if (K > 1) cl_sync();
     else __syncthreads();
-    for (int k = 0; k < iters; ++k) {
+    for (int k = 0; k < iters && rows > 0; ++k) {
         const XT a = static_cast<XT>(arow[alpha_len == 1 ? 0 : k0 + k]);
-        if (K > 1) exchange_expect(ex, k, static_cast<uint32_t>((nb - rows) * sizeof(XT)));
+        if (owners > 1) exchange_expect(ex, k, static_cast<uint32_t>((nb - rows) * sizeof(XT)));
         const bool keep = rec && (k + 1) % rec_every == 0;
         XT *rp = reinterpret_cast<XT *>(rec + (keep ? static_cast<size_t>((k + 1) / rec_every - 1) : 0) * rec_stride);
         const double unit = two_to(-shift);
@@ -282,7 +285,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
                 if (keep) rp[row * R + r] = v;
             }
             nxt[i0 + i] = v;
-            exchange_send(ex, k, nxt + i0 + i, v, q, K);
+            exchange_send(ex, k, nxt + i0 + i, v, q, owners);
         };
         for (int i = rl; i < top; i += rstep) {
             XT acc = XT(0);
@@ -324,7 +327,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
             __syncthreads();
             for (int i = threadIdx.x; i < rows; i += blockDim.x) update(i, z[i]);
         }
-        if (!exchange_wait(ex, k, K, err)) break;
+        if (!exchange_wait(ex, k, owners, err)) break;
         XT *t = cur;
         cur = nxt;
         nxt = t;
@@ -344,7 +347,8 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
 // peers' shares); FP32 with compensated row sums for FP32 ones. The products
 // w x (FP64, or FP32 split exactly) stay in shared memory for up to `hold` steps, and are then added in FP64,
 // a warp per step: added at every step they were a third of it. x^(k0) is x_first and
-// x^(k0 + m) = x_seg + (m - 1) stride, each loaded a step ahead.
+// x^(k0 + m) = x_seg + (m - 1) stride, each loaded a step ahead. Every CTA of a cluster owns rows here:
+// K <= 16 and n >= 32 K (cluster_max) leave the last share at least 17.
 template <typename XT>
 struct AdjointRow;
 template <>

@@ -622,6 +622,29 @@ def test_small_fp64_int8_steps(n, R, density, jmax, start):
     assert np.all(np.linalg.norm(x - ref, axis=0) <= 1e-12 * np.linalg.norm(ref, axis=0))
 
 
+@pytest.mark.parametrize("sizes", [[1000, 17], [1000, 40, 10, 1], [600, 1, 33, 599]])
+@pytest.mark.parametrize("jdtype", [np.int8, np.float64])
+def test_small_fp64_batches_with_short_instances(sizes, jdtype):
+    """A short instance beside a long one: the cluster's size is set by the longest, so a short one
+    leaves CTAs without rows. Enough steps for CTAs of a cluster to drift apart."""
+    R, iters = 2, 300
+    gs = [I.erdos_renyi_pm1(n, min(1.0, 8.0 / n), seed=30 + k) if n > 1 else
+          I.csr_from_upper(1, np.zeros(0, np.int64), np.zeros(0, np.int64), np.zeros(0, np.int8))
+          for k, n in enumerate(sizes)]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    rp = np.concatenate([[0]] + [g.row_ptr[1:] + sum(int(q.row_ptr[-1]) for q in gs[:b]) for b, g in enumerate(gs)])
+    col = np.concatenate([g.col.astype(np.int64) + off[b] for b, g in enumerate(gs)])
+    J = I.CSR(int(off[-1]), rp.astype(np.int64), col.astype(np.int32), np.concatenate([g.val for g in gs]).astype(jdtype))
+    alphas, betas = zip(*[O.alpha_beta(g, eta=1.0, method="wigner") if g.n > 1 else (1.5, 7.0) for g in gs])
+    x0 = I.x0_uniform(J.n, R, seed=31, dtype=np.float64)
+    with Handle(J, None, off) as hd:
+        x = _dev(x0)
+        N.ising_iterate(hd, x, list(alphas), list(betas), iters, n_instances=len(sizes))
+        xg = x.cpu().numpy()
+    for b, g in enumerate(gs):
+        _close(xg[off[b]:off[b + 1]], O.doch(O.Problem(g), x0[off[b]:off[b + 1]], alphas[b], betas[b], iters), TOL64)
+
+
 @pytest.mark.parametrize("n, per_row, R", [(2000, 110, 1), (2000, 110, 16), (5000, 60, 3), (5000, 110, 16)])
 def test_shares_that_do_not_fit_take_single_steps(n, per_row, R):
     """Long integer rows around the size where a share's couplings no longer fit shared memory: both
