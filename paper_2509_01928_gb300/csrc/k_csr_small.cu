@@ -16,8 +16,8 @@
 // a step's chain: products, tree, cube root, exchange. FP64 iterates with 8-bit couplings take their
 // products in integers (fixed point, below): nine FP64 operations per cube root and five around it are left.
 // 800 spins, 38,000 entries, R = 8, FP64, per step: 10.0 us with one thread per row, the couplings
-// converted at every use and CUDA's cbrt of a quotient; 3.5 us with the couplings held in FP64 and four
-// threads per row (products 2.3, update 0.8, exchange 0.35); 2.6 us in fixed point with eight. The FP64
+// converted at every use and CUDA's cbrt of a quotient; 3.4 us with the couplings held in FP64 and four
+// threads per row (products 2.3, update 0.8, exchange 0.35); 2.75 us in fixed point with eight. The FP64
 // operations alone take about 0.25 us on the 128 SMs used.
 #include <algorithm>
 #include <type_traits>
@@ -114,36 +114,59 @@ struct Held<double, int8_t> {  // the integer (fixed-point steps), or the FP64 v
     static __device__ __forceinline__ double value(int v) { return __hiloint2double(v, 0); }
 };
 
-// Fixed-point steps (FP64 iterates, 8-bit couplings): every x_j is held as the integer round(x_j 2^s),
-// s from a bound M >= max |x_j| such that every row's sum of J_ij x_j stays below 2^62, so that J x is
-// summed exactly in integers, at integer rate, from terms with an absolute error of rowabs M 2^-62
-// (FP64 sums round by about M 2^-53 at every addition; relative error against plain FP64 arithmetic in
-// torch over 1000 steps of 800 spins, R = 8, six seeds: 4.41e-16 to 5.33e-16 in FP64, 4.40e-16 to 5.30e-16
-// in fixed point; 60 steps of 1500 spins, R = 4: 0.6e-15 to 4.0e-15 and 0.6e-15 to 3.1e-15). M of the next
-// iterate follows from |x'| <= cbrt(((rowabs + |alpha|) M + max |h|) / beta), rounded up. x itself is
-// kept in FP64 where it is added (alpha x) and returned. Runs that record iterates keep FP64 sums: their
-// scales would depend on where a run starts.
+// Fixed-point steps (FP64 iterates, 8-bit couplings). The iterate is held and exchanged in FP64; at the
+// start of a step every CTA also forms the integers round(x_j 2^s) of all of it, s from a bound M >= max |x_j|
+// such that every row's sum of |J_ij x_j| stays below 2^63. J x is then summed in integers, at integer
+// rate, with an error of at most rowabs_i 2^-s / 2 in row i (rowabs_i = sum_j |J_ij|).
+// A row takes that sum where it is no less exact than FP64 sums: where sum_j |J_ij x_j| >= rowabs_i 2^52 2^-s, so
+// that the error is within 2^-53 of the sum of the terms' magnitudes, one FP64 rounding. Every row tests
+// this at every step, from the upper words of its terms (`mag`, in units of 2^(32 - s)), and sums in FP64
+// otherwise: rows whose neighbours are small beside the largest component (starts over many orders of
+// magnitude, a spin pinned by a strong field, hubs). Where a row sum of |J| reaches kRowLimit most rows
+// would fail (rowabs M 2^-63 2^52 against a mean |x_j|), and such instances take FP64 sums throughout.
+// Error of the row sums that pass, relative to the terms' magnitudes, rms over all rows (FP64 in four partial
+// sums / fixed point): 800 spins of 48 entries 2.4e-17 / 0.9e-17, 1500 of 120 2.1e-17 / 0.5e-17, 1200 of 24
+// 2.6e-17 / 1.1e-17; x after 1000 steps of 800 spins, six seeds: within 4.4e-16 to 5.3e-16 of 64-bit torch in both.
+// M of the next iterate follows from |x'| <= cbrt(((rowabs + |alpha|) M + max |h|) / beta), rounded up. Runs
+// that record iterates keep FP64 sums: the bounds, and so the rounding, would depend on where a run starts.
+constexpr int kRowLimit = 256;
 __device__ __forceinline__ float next_bound(float m, float rowabs, float alpha, float hmax, float inv_beta) {
     const float z = ((rowabs + fabsf(alpha)) * m + hmax) * inv_beta;
     return ex2_fast(lg2_fast(z) * (1.0f / 3.0f)) * 1.0001f;
 }
-__device__ __forceinline__ int fixed_shift(float m, float rowabs) {  // rowabs m 2^shift < 2^61
-    return 61 - (ilogbf(rowabs * m * 1.0001f) + 1);
+__device__ __forceinline__ int fixed_shift(float m, float rowabs) {  // rowabs m 2^shift < 2^63 / 1.0001
+    return 63 - (ilogbf(rowabs * m * 1.0001f) + 1);
 }
-__device__ __forceinline__ long long to_fixed(double v, int shift) {  // the shift in the exponent's field
-    return __double2ll_rn(__hiloint2double(__double2hiint(v) + (shift << 20), __double2loint(v)));
+// round(v 2^shift), |v 2^shift| < 2^63, by integer shifts (an FP64 conversion costs as much as an FMA)
+__device__ __forceinline__ long long to_fixed(double v, int shift) {
+    const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+    const unsigned long long m = static_cast<unsigned long long>((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32 |
+                                 static_cast<unsigned>(__double2loint(v));
+    const int s = (e ? e : 1) + shift - 1075;  // |v| 2^shift = m 2^s
+    unsigned long long r = 0;
+    if (s >= 0) r = m << s;
+    else if (s > -55) r = ((m >> (-s - 1)) + 1) >> 1;
+    return hi < 0 ? -static_cast<long long>(r) : static_cast<long long>(r);
 }
 __device__ __forceinline__ double two_to(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// Shared memory: cur | nxt (XT [nb] each) | z (XT [rows], P > 1 only) | own (XT [rows], the share's x,
-// where fixed-point steps may run), then, as far as there is room
+// Shared memory: cur | nxt (XT [nb] each) | z (XT [rows], P > 1 only) | where fixed-point steps may run
+// integers (int64 [nb]) | rowabs (int [rows]), then, as far as there is room
 // for at least the shares it fits, val (Held [cap]) | row ranges (int [rows + 1]) | col (uint16 [cap])
 template <typename XT, int P>
-constexpr int64_t state_bytes(int64_t nb, int64_t rows, bool own) {
-    return static_cast<int64_t>(sizeof(XT)) * (2 * nb + (P > 1 ? rows : 0) + (own ? rows : 0)) + 16;
+constexpr int64_t state_bytes(int64_t nb, int64_t rows, bool fix) {
+    return static_cast<int64_t>(sizeof(XT)) * (2 * nb + (P > 1 ? rows : 0)) + (fix ? 8 * nb + 4 * rows : 0) + 16;
 }
 template <typename XT, typename VT>
 constexpr bool can_fix() { return sizeof(XT) == 8 && sizeof(VT) == 1; }
+// where a launch may take fixed-point steps: rows long enough to repay the integers of the whole iterate
+// (us per step, fixed point / FP64 sums: 300 spins of 3 entries, R = 8 1.93 / 1.49; 400 of 20, R = 1 1.88 / 1.69;
+// 1500 of 30, R = 8 3.21 / 4.18; 800 of 48, R = 8 2.75 / 3.41; 1000 of 50, R = 20 4.24 / 6.44; 1500 of 120, R = 20
+// 8.1 / 11.0)
+template <typename XT, typename VT>
+bool fixed_point(const ising_context *c, const SmallRecord &rec, int K) {
+    return can_fix<XT, VT>() && K > 1 && !rec.base && c->nnz >= 24 * c->n;
+}
 template <typename XT, typename VT>
 constexpr int64_t entry_bytes() { return sizeof(typename Held<XT, VT>::type) + sizeof(uint16_t); }
 
@@ -153,7 +176,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
           const int32_t *__restrict__ col, const VT *__restrict__ val, const XT *__restrict__ h,
           const int64_t *__restrict__ inst_off, int64_t n, int R, const double *__restrict__ alpha_tab, int alpha_len,
           const double *__restrict__ beta_tab, int k0, int iters, int K, int rows_cap, int cap,
-          unsigned char *rec, size_t rec_stride, int rec_every, int *__restrict__ err) {
+          int fix, unsigned char *rec, size_t rec_stride, int rec_every, int *__restrict__ err) {
     extern __shared__ __align__(16) unsigned char small_smem[];
     __shared__ Exchange ex;
     constexpr bool kFix = can_fix<XT, VT>();
@@ -170,9 +193,11 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     XT *cur = reinterpret_cast<XT *>(small_smem), *nxt = cur + nb;
     XT *z = nxt + nb;
     using Hd = Held<XT, VT>;
-    const bool with_own = kFix && K > 1;
-    XT *own = P > 1 ? z + rows_cap : z;
-    typename Hd::type *lv = reinterpret_cast<typename Hd::type *>(with_own ? own + rows_cap : own);
+    const bool may_fix = kFix && fix;
+    long long *fx = reinterpret_cast<long long *>(P > 1 ? z + rows_cap : z);
+    int *limit = reinterpret_cast<int *>(fx + nb);  // of a row: rowabs_i, negative while its sum is an FP64 one
+    typename Hd::type *lv = may_fix ? reinterpret_cast<typename Hd::type *>(limit + rows_cap)
+                                    : reinterpret_cast<typename Hd::type *>(fx);
     int *lr = reinterpret_cast<int *>(lv + cap);
     uint16_t *lc = reinterpret_cast<uint16_t *>(lr + rows_cap + 1);
     if constexpr (kFix) {
@@ -184,7 +209,6 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
             cur[i] = v;
             tx = max(tx, static_cast<unsigned>(__double2hiint(v)) & 0x7fffffffu);
             if (h) th = max(th, static_cast<unsigned>(__double2hiint(__ldg(h + lo + i))) & 0x7fffffffu);
-            if (with_own && i >= i0 && i < i1) own[i - i0] = v;
         }
         atomicMax(&top_word[0], tx);
         atomicMax(&top_word[1], th);
@@ -203,13 +227,13 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
     }
     bool fixed = false;
     float bound = 0.f, rowabs = 0.f, hmax = 0.f, inv_beta = 0.f;
-    int shift = 0;
     if constexpr (kFix) {
         __syncthreads();
         int sum = 0;
         for (int i = threadIdx.x; i < rows && local; i += blockDim.x) {
             int t = 0;
             for (int e = lr[i]; e < lr[i + 1]; ++e) t += abs(lv[e]);
+            if (may_fix) limit[i] = t;
             sum = max(sum, t);
         }
         atomicMax(&top_word[2], static_cast<unsigned>(sum));
@@ -231,7 +255,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
         hmax = __double2float_ru(mh);
         rowabs = static_cast<float>(most) * 1.0001f;
         inv_beta = static_cast<float>(1.0 / beta_tab[b]) * 1.0001f;
-        bool bad = !(with_own && !rec && top_word[0] < 0x7ff00000u && top_word[1] < 0x7ff00000u && most != 0x7fffffff &&
+        bool bad = !(may_fix && top_word[0] < 0x7ff00000u && top_word[1] < 0x7ff00000u && most < kRowLimit &&
                      bound > 1e-12f && bound < 1e10f && hmax < 1e12f && inv_beta > 1e-20f && inv_beta < 1e12f);
         for (int k = threadIdx.x; k < (alpha_len == 1 ? 1 : iters); k += blockDim.x) {
             const float ak = static_cast<float>(alpha_tab[static_cast<int64_t>(b) * alpha_len + (alpha_len == 1 ? 0 : k0 + k)]);
@@ -239,10 +263,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
             bad = bad || !(z > 1e-20f && z < 1e12f);
         }
         fixed = !__syncthreads_or(bad);
-        if (fixed) {
-            shift = fixed_shift(bound, rowabs);
-            for (int i = threadIdx.x; i < nb; i += blockDim.x) cur[i] = __longlong_as_double(to_fixed(cur[i], shift));
-        } else if (local) {
+        if (!fixed && local) {
             const int cnt = lr[rows];
             for (int e = threadIdx.x; e < cnt; e += blockDim.x) lv[e] = Hd::upper(lv[e]);
         }
@@ -261,24 +282,26 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
         if (owners > 1) exchange_expect(ex, k, static_cast<uint32_t>((nb - rows) * sizeof(XT)));
         const bool keep = rec && (k + 1) % rec_every == 0;
         XT *rp = reinterpret_cast<XT *>(rec + (keep ? static_cast<size_t>((k + 1) / rec_every - 1) : 0) * rec_stride);
-        const double unit = two_to(-shift);
+        double unit = 0.0;
         if constexpr (kFix) {
             if (fixed) {
+                const int shift = fixed_shift(bound, rowabs);
+                unit = two_to(-shift);
                 bound = next_bound(bound, rowabs, static_cast<float>(a), hmax, inv_beta);
-                shift = fixed_shift(bound, rowabs);
+                for (int i = threadIdx.x; i < nb; i += blockDim.x) fx[i] = to_fixed(cur[i], shift);
+                __syncthreads();
             }
         }
-        auto update = [&](int i, XT u) {  // row i of the share: the new value into every CTA's next copy
+        // row i of the share: the new value into every CTA's next copy; u is J x, as the integer's bits (in_fixed) or FP64
+        auto update = [&](int i, XT u, bool in_fixed) {
             const int64_t row = lo + i0 + i;
             const XT hv = h ? __ldg(h + row) : XT(0);
             XT v;
-            if (kFix && fixed) {
+            if (kFix && in_fixed) {
                 if constexpr (kFix) {
-                    XT w = a * own[i];
+                    XT w = a * cur[i0 + i];
                     if (h) w += hv;
-                    const XT y = root_newton(fma(__ll2double_rn(__double_as_longlong(u)), unit, w), root);
-                    own[i] = y;
-                    v = __longlong_as_double(to_fixed(y, shift));
+                    v = root_newton(fma(__ll2double_rn(__double_as_longlong(u)), unit, w), root);
                 }
             } else {
                 v = root_newton(u + a * cur[i0 + i] + hv, root);
@@ -289,18 +312,38 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
         };
         for (int i = rl; i < top; i += rstep) {
             XT acc = XT(0);
+            bool in_fixed = false;
             if (kFix && fixed) {
                 if constexpr (kFix) {
-                    const long long *fx = reinterpret_cast<const long long *>(cur);
                     long long sum = 0;
+                    unsigned mag = 0;  // sum of |J_ij| |upper word of x_j|, above the true magnitudes by at most rowabs_i
+                    int f0 = 0, f1 = 0, most = 0;
                     if (i < rows) {
-                        const int f1 = lr[i + 1];
+                        f0 = lr[i] + sub;
+                        f1 = lr[i + 1];
+                        most = limit[i];
 #pragma unroll 4
-                        for (int e = lr[i] + sub; e < f1; e += P) sum += static_cast<long long>(lv[e]) * fx[lc[e]];
+                        for (int e = f0; e < f1; e += P) {
+                            const int w = lv[e];
+                            const long long x = fx[lc[e]];
+                            sum += static_cast<long long>(w) * x;
+                            mag += static_cast<unsigned>(abs(w * static_cast<int>(x >> 32)));
+                        }
                     }
 #pragma unroll
-                    for (int o = P / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                    acc = __longlong_as_double(sum);
+                    for (int o = P / 2; o > 0; o >>= 1) {
+                        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                        mag += __shfl_xor_sync(0xffffffffu, mag, o);
+                    }
+                    in_fixed = most == 0 || (mag >> 20) > static_cast<unsigned>(most);
+                    if (__any_sync(0xffffffffu, !in_fixed)) {  // the rows that fail, in FP64
+                        if (!in_fixed)
+                            for (int e = f0; e < f1; e += P) acc += static_cast<double>(lv[e]) * cur[lc[e]];
+#pragma unroll
+                        for (int o = P / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                        if (P > 1 && !in_fixed && sub == 0) limit[i] = -most;
+                    }
+                    if (in_fixed) acc = __longlong_as_double(sum);
                 }
             } else if (i < rows) {
                 if (local) {
@@ -318,14 +361,21 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
                 for (int o = P / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             }
             if (P == 1) {
-                if (i < rows) update(i, acc);
+                if (i < rows) update(i, acc, in_fixed);
             } else if (sub == 0 && i < rows) {
                 z[i] = acc;
             }
         }
         if (P > 1) {
             __syncthreads();
-            for (int i = threadIdx.x; i < rows; i += blockDim.x) update(i, z[i]);
+            for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+                bool in_fixed = kFix && fixed;
+                if (in_fixed && limit[i] < 0) {
+                    in_fixed = false;
+                    limit[i] = -limit[i];
+                }
+                update(i, z[i], in_fixed);
+            }
         }
         if (!exchange_wait(ex, k, owners, err)) break;
         XT *t = cur;
@@ -333,7 +383,7 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
         nxt = t;
     }
     if (x_out)
-        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) x_out[(lo + i) * R + r] = kFix && fixed ? own[i - i0] : cur[i];
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) x_out[(lo + i) * R + r] = cur[i];
     if (K > 1) cl_sync();  // no CTA leaves while a peer may still send to it
 }
 
@@ -511,7 +561,8 @@ template <typename XT, typename VT, int P>
 ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R, const XT *h, const ParamTabs &p,
                         int k0, int iters, int K, const SmallRecord &rec, int64_t optin, cudaStream_t st) {
     const int64_t chunk = (c->max_inst_n + K - 1) / K;
-    const int64_t state = state_bytes<XT, P>(c->max_inst_n, chunk, can_fix<XT, VT>() && K > 1);
+    const bool fix = fixed_point<XT, VT>(c, rec, K);
+    const int64_t state = state_bytes<XT, P>(c->max_inst_n, chunk, fix);
     if (state > optin) return ISING_ERR_UNSUPPORTED;
     // room for the couplings of the fullest share, as far as it goes (shares that need more read the CSR arrays)
     const int64_t left = optin - state - static_cast<int64_t>(sizeof(int)) * (chunk + 1);
@@ -550,7 +601,7 @@ ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R
                                  static_cast<const int32_t *>(c->col), static_cast<const VT *>(c->val), h,
                                  static_cast<const int64_t *>(c->n_inst > 1 ? c->inst_off : nullptr), c->n, R,
                                  p.alpha_d, p.alpha_len, p.beta_d, k0, iters, K, static_cast<int>(chunk),
-                                 static_cast<int>(cap), static_cast<unsigned char *>(rec.base), rec.stride,
+                                 static_cast<int>(cap), fix ? 1 : 0, static_cast<unsigned char *>(rec.base), rec.stride,
                                  rec.every, c->err_word));
     return ISING_OK;
 }
@@ -652,15 +703,14 @@ ising_status_t launch_small(const ising_context *c, const XT *x_in, XT *x_out, i
         const int64_t chunk = (c->max_inst_n + K - 1) / K;
         // threads per row: four or two where a share is small and its rows are long enough to split (more
         // would spend as many FP64 additions on the tree as they take from the rows); eight or four where
-        // the products are integers (1000 spins at density 0.05, R = 20, shares of 143 rows, 300 steps: 1.63 ms
-        // with two, 1.42 with four, 1.24 with eight; 800 spins at 0.06, R = 8, shares of 50, 1000 steps: 2.72 ms with
-        // four, 2.59 with eight, 2.87 with sixteen)
+        // the products are integers (us per step with four / eight / sixteen: 1000 spins at density 0.05, R = 20,
+        // shares of 143 rows 4.7 / 4.2 / 4.7; 800 spins at 0.06, R = 8, shares of 50 3.0 / 2.7 / 3.4)
         const bool split = c->nnz >= 8 * c->n;
         auto run = [&](auto p_threads) {
             return launch_k<XT, VT, decltype(p_threads)::value>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st);
         };
         ising_status_t s;
-        if constexpr (can_fix<XT, VT>())
+        if (fixed_point<XT, VT>(c, rec, K))
             s = split && chunk <= 256   ? run(std::integral_constant<int, 8>())
                 : split && chunk <= 512 ? run(std::integral_constant<int, 4>())
                                         : run(std::integral_constant<int, 1>());

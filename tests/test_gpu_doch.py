@@ -622,6 +622,53 @@ def test_small_fp64_int8_steps(n, R, density, jmax, start):
     assert np.all(np.linalg.norm(x - ref, axis=0) <= 1e-12 * np.linalg.norm(ref, axis=0))
 
 
+@pytest.mark.parametrize("n, R, density, jmax", [(800, 8, 0.06, 1), (300, 8, 0.02, 1), (801, 3, 0.06, 127), (1500, 20, 0.08, 1),
+                                                 (700, 30, 0.05, 3), (64, 1, 0.3, 1)])
+@pytest.mark.parametrize("case", ["uniform", "one", "wide", "pinned", "parts", "hub"])
+def test_small_fp64_int8_components(n, R, density, jmax, case):
+    """One step of FP64 iterates with 8-bit couplings, component by component, at components of very
+    different sizes: one of 1e6 or spread over nine orders, a spin pinned by a field of 1e11, two parts of a
+    graph at 1e9 and 1e-9, a hub row. z_i = sum_j J_ij x_j + alpha x_i + h_i may differ from the oracle's by the
+    rounding of two FP64 sums of its terms, (terms + 2) 2^-52 sum |terms|; a root adds 4 ulp."""
+    rng = np.random.default_rng(7 * n + R)
+    keep = np.triu(rng.random((n, n)) < density, 1)
+    if case == "parts":
+        keep[:n // 2, n // 2:] = False
+    if case == "hub":
+        keep[0, 1:] = True
+    i, j = keep.nonzero()
+    g = I.csr_from_upper(n, i, j, (rng.integers(1, jmax + 1, i.size) * rng.choice([-1, 1], i.size)).astype(np.int8))
+    h = np.zeros(n)
+    x0 = rng.uniform(-1, 1, (n, R))
+    if case == "one":
+        x0[n // 3] = 1e6
+    elif case == "wide":
+        x0 *= 10.0 ** rng.uniform(-9, 0, (n, R))
+    elif case == "pinned":
+        h[n // 3] = 1e11
+    elif case == "parts":
+        x0[:n // 2] *= 1e9
+        x0[n // 2:] *= 1e-9
+    alpha, beta = O.alpha_beta(g, eta=1.0, method="wigner")
+    P = O.Problem(g, h if case == "pinned" else None)
+    rows = np.repeat(np.arange(n), np.diff(g.row_ptr))
+    hd = N.ising_create(N.Problem(g, h if case == "pinned" else None))
+    try:
+        for before in (0, 1, 4):
+            x_in = O.doch(P, x0, alpha, beta, before) if before else x0
+            ref = O.doch(P, x_in, alpha, beta, 1)
+            x = torch.from_numpy(x_in.copy()).cuda()
+            N.ising_iterate(hd, x, [alpha], [beta], 1)
+            size = np.abs(alpha * x_in) + np.abs(h)[:, None]
+            np.add.at(size, rows, np.abs(g.val.astype(np.float64))[:, None] * np.abs(x_in[g.col]))
+            dz = (np.diff(g.row_ptr) + 2)[:, None] * 2.0 ** -52 * size / beta
+            z = ref ** 3
+            room = np.maximum(np.abs(np.cbrt(z + dz) - np.cbrt(z)), np.abs(np.cbrt(z - dz) - np.cbrt(z)))
+            assert np.all(np.abs(x.cpu().numpy() - ref) <= room + 4 * 2.0 ** -52 * np.abs(ref)), before
+    finally:
+        N.ising_destroy(hd)
+
+
 @pytest.mark.parametrize("sizes", [[1000, 17], [1000, 40, 10, 1], [600, 1, 33, 599]])
 @pytest.mark.parametrize("jdtype", [np.int8, np.float64])
 def test_small_fp64_batches_with_short_instances(sizes, jdtype):
