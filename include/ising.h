@@ -430,6 +430,14 @@ ISING_API ising_status_t ising_selftest_cbrt(const float *z, float *ours, float 
 ISING_API ising_status_t ising_selftest_cbrt_log(const float *z, float *out, int64_t n, float c3, void *stream);
 
 /*
+ * Diagnostic: the 64-bit warp sum of the dense energy (row tiles whose s_i (J s)_i
+ * add up to 2^31 or more, as |J_ij| = 256 gives past n = 65536), on `warps` groups
+ * of 32 32-bit terms. terms and out are device arrays of 32 * warps and warps
+ * elements. Synchronises the stream.
+ */
+ISING_API ising_status_t ising_selftest_warp_sum(const int32_t *terms, int64_t *out, int32_t warps, void *stream);
+
+/*
  * Diagnostic: the procedural couplings J_ij = sin(i j + c) (1-based i, j;
  * J_ii = 0) for rows row0 .. row0 + rows - 1 and columns col0 .. col0 + cols - 1
  * (0-based indices), evaluated on the device exactly as the product kernels of

@@ -51,6 +51,7 @@
 #include "cbrt.cuh"
 #include "internal.cuh"
 #include "mbar.cuh"
+#include "warpsum.cuh"
 
 namespace doch {
 namespace {
@@ -77,7 +78,7 @@ struct DenseSmem {
     alignas(8) unsigned long long conv[kS];             // ternary: A tile expanded
     alignas(8) unsigned long long jfull[kJStages];      // ternary: packed tile landed
     alignas(8) unsigned long long jempty[kJStages];     // ternary: packed tile read
-    alignas(16) int qsum[256];     // energy terms of the tile per column
+    alignas(16) long long qsum[256];  // energy terms of the tile per column
     alignas(8) unsigned long long acc_ready;
     uint32_t tmem_base;
     int abort_flag;
@@ -388,11 +389,11 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
                 if (row4 < n)
                     *reinterpret_cast<uint2 *>(xt_out + xs_index(r0 + c, row4, R_pad)) =
                         make_uint2(out[0] | out[1] << 16, out[2] | out[3] << 16);
-            } else {  // |s u| < 2^24: 128 terms add in 32 bits
+            } else {  // |s u| <= 256 n: four terms add in 32 bits (n < 2^21: J would take 8 TB), 128 do not
                 int term = 0;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) term += static_cast<int>(x4[e] * u[e]);
-                const int sum = __reduce_add_sync(0xffffffffu, term);
+                const long long sum = warp_sum_wide(term);
                 if (lane == 0) sm.qsum[c] = sum;
             }
         };

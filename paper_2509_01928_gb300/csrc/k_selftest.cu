@@ -1,10 +1,12 @@
 // Diagnostic entry points: the device cube root cbrt_pow2 next to
 // CUDA's cbrtf on the same inputs (see ising_selftest_cbrt in ising.h), and the
-// lattice kernels' cube root with its log-domain offset (ising_selftest_cbrt_log).
+// lattice kernels' cube root with its log-domain offset (ising_selftest_cbrt_log),
+// and the warp sum of the dense energy's terms (ising_selftest_warp_sum).
 #include <cmath>
 
 #include "cbrt.cuh"
 #include "internal.cuh"
+#include "warpsum.cuh"
 
 namespace doch {
 namespace {
@@ -39,6 +41,27 @@ extern "C" ising_status_t ising_selftest_cbrt_log(const float *z, float *out, in
         int64_t blocks = (n + 255) / 256;
         if (blocks > 8LL * sms) blocks = 8LL * sms;
         cbrt_log_kernel<<<static_cast<unsigned>(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(z, out, n, c3);
+        DOCH_CUDA(cudaGetLastError());
+        DOCH_CUDA(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
+        return ISING_OK;
+    });
+}
+
+namespace doch {
+namespace {
+__global__ void warp_sum_kernel(const int32_t *__restrict__ terms, int64_t *__restrict__ out) {
+    const long long s = warp_sum_wide(terms[blockIdx.x * 32LL + threadIdx.x]);
+    if (threadIdx.x == 0) out[blockIdx.x] = s;
+}
+}  // namespace
+}  // namespace doch
+
+extern "C" ising_status_t ising_selftest_warp_sum(const int32_t *terms, int64_t *out, int32_t warps, void *stream) {
+    return doch::guarded([&]() -> ising_status_t {
+        using namespace doch;
+        if (!terms || !out || warps < 0) return fail(ISING_ERR_INVALID_ARG, "selftest_warp_sum: bad argument");
+        if (warps == 0) return ISING_OK;
+        warp_sum_kernel<<<static_cast<unsigned>(warps), 32, 0, static_cast<cudaStream_t>(stream)>>>(terms, out);
         DOCH_CUDA(cudaGetLastError());
         DOCH_CUDA(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
         return ISING_OK;

@@ -154,6 +154,19 @@ def test_dense_energy_exact(n, R, kind):
         N.ising_destroy(h)
 
 
+def test_dense_energy_terms_add_in_64_bits():
+    """The 128 terms s_i (J s)_i of a row tile reach 2^31 past n = 65536 at |J| = 256 (a matrix too large
+    for a test): the warp sum of its lanes' terms (four rows each, up to 2^26 and beyond) on its own."""
+    rng = np.random.default_rng(5)
+    t = rng.integers(-2 ** 31, 2 ** 31, (200, 32))
+    t[0], t[1], t[2] = 4 * 256 * 70000, -4 * 256 * 70000, 2 ** 31 - 1
+    t[3], t[4], t[5] = -2 ** 31, 0, -1
+    td = torch.from_numpy(t.astype(np.int32)).cuda()
+    out = torch.empty(len(t), dtype=torch.int64, device="cuda")
+    assert N.load().ising_selftest_warp_sum(N._ptr(td), N._ptr(out), len(t), None) == 0
+    assert np.array_equal(out.cpu().numpy(), t.sum(1))
+
+
 def test_dense_full_size_16384x256_sampled():
     """n = 16384 dense +-1, R = 256 BF16 replicas: all replicas run on the GPU,
     two sampled replicas are recomputed by the oracle (iterates after 1 and 5
