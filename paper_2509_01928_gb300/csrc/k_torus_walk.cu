@@ -95,7 +95,7 @@ struct WalkSmem {
 
 template <typename T, int V, int TS>
 __global__ void __launch_bounds__(kWT, sizeof(T) == 8 ? 3 : 2)
-torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restrict__ edge, int Lr, int Lc, int R,
+torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restrict__ edge, int64_t Lr, int64_t Lc, int R,
            int G, int groups, int nwin, int wout, int strips, Alphas<T, TS> alpha,
            typename RootOf<T>::type root) {
     extern __shared__ __align__(16) unsigned char walk_smem[];
@@ -103,31 +103,31 @@ torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restr
     const int t = threadIdx.x;
     const int grp = blockIdx.x % groups, rest = blockIdx.x / groups;
     const int win = rest % nwin, strip = rest / nwin;
-    const int r0 = static_cast<int>(static_cast<int64_t>(Lr) * strip / strips);
-    const int r1 = static_cast<int>(static_cast<int64_t>(Lr) * (strip + 1) / strips);
+    const int64_t r0 = Lr * strip / strips;
+    const int rows = static_cast<int>(Lr * (strip + 1) / strips - r0);  // (launch_walk)
     const int sites = blockDim.x / G;          // columns of the window, halo included
     const int s = min(t / G, sites - 1);       // threads past the last whole site repeat it
     const int g = t % G;
     const int tl = s * G + g;                  // this thread's slot (repeated ones write the same values)
     const int left = s > 0 ? tl - G : tl, right = s + 1 < sites ? tl + G : tl;
-    const int off = win * wout + s - TS;       // column, not wrapped
-    int col = off % Lc;
+    const int64_t off = static_cast<int64_t>(win) * wout + s - TS;  // column, not wrapped
+    int64_t col = off % Lc;
     if (col < 0) col += Lc;
     const bool writes = s >= TS && s < TS + wout && off < Lc && t / G < sites;
-    const int64_t W = static_cast<int64_t>(Lc) * R;
-    const int64_t at = static_cast<int64_t>(col) * R + (static_cast<int64_t>(grp) * G + g) * V;
+    const int64_t W = Lc * R;
+    const int64_t at = col * R + (static_cast<int64_t>(grp) * G + g) * V;
     const T *xc = xi + at;
     const uint32_t *ec = edge + col;
     T *oc = xo + at;
 
     // ring row k holds lattice row r0 - TS + k (wrapped); rows 0 .. nk - 1 are needed
-    const int nk = r1 - r0 + 2 * TS;
-    int rk = (r0 - TS) % Lr;  // lattice row of the next ring row to stage
+    const int nk = rows + 2 * TS;
+    int64_t rk = (r0 - TS) % Lr;  // lattice row of the next ring row to stage
     if (rk < 0) rk += Lr;
     auto stage = [&](int k, int slot) {
         if (k < nk) {
             copy_async<sizeof(T) * V>(&sm.x[slot][tl], xc + rk * W);
-            if (g == 0) copy_async<4>(&sm.e[slot][s], ec + static_cast<int64_t>(rk) * Lc);
+            if (g == 0) copy_async<4>(&sm.e[slot][s], ec + rk * Lc);
             rk = rk + 1 == Lr ? 0 : rk + 1;
         }
         commit_async();
@@ -146,8 +146,8 @@ torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restr
 #pragma unroll
         for (int q = 0; q < 4; ++q) w[l][q] = T(0);
     }
-    T *op = oc + static_cast<int64_t>(r0) * W;
-    const int iters = r1 - r0 + 2 * (TS - 1);
+    T *op = oc + r0 * W;
+    const int iters = rows + 2 * (TS - 1);
     int s0 = 0;  // ring slot of row i
     for (int i = 0; i < iters; ++i) {
         const int s1 = s0 + 1 == kWD ? 0 : s0 + 1, s2 = s1 + 1 == kWD ? 0 : s1 + 1;
@@ -232,9 +232,10 @@ ising_status_t launch_walk(const ising_context *c, const T *xi, T *xo, int R, co
     const int64_t slots = static_cast<int64_t>(c->num_sms) * occ;
     const int64_t strips = std::max<int64_t>(1, std::min<int64_t>(Lr, slots / (nwin * groups)));
     const int64_t blocks = strips * nwin * groups;
-    if (blocks > INT32_MAX) return fail(ISING_ERR_UNSUPPORTED, "lattice too large");
-    kern<<<static_cast<unsigned>(blocks), threads, smem, st>>>(xi, xo, c->edge.as<uint32_t>(), static_cast<int>(Lr),
-                                                               static_cast<int>(Lc), R, G, groups,
+    // (sides of 2^31 and more fit the memory; a block's rows stay below 2^31: strips fill the slots unless the
+    // windows and groups do, and then 2^31 rows of them do not fit)
+    if (blocks > INT32_MAX || Lr / strips > INT32_MAX - 16) return fail(ISING_ERR_UNSUPPORTED, "lattice too large");
+    kern<<<static_cast<unsigned>(blocks), threads, smem, st>>>(xi, xo, c->edge.as<uint32_t>(), Lr, Lc, R, G, groups,
                                                                static_cast<int>(nwin), wout,
                                                                static_cast<int>(strips), a, root);
     DOCH_CUDA(cudaGetLastError());
