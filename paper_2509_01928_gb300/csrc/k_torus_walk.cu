@@ -64,11 +64,12 @@ __device__ __forceinline__ void unpack(uint32_t w, double (&f)[4]) {
     for (int k = 0; k < 4; ++k) f[k] = g[k] == 0.f ? 0.0 : widen_normal(g[k]);
 }
 
-// one row of a thread's V values: the four neighbours in the order right, left, down, up
-template <typename T, int V, typename P>
+// one row of a thread's V values: the four neighbours in the order right, left, down, up. NEAR (FP32): the
+// roots without the test of their range, which `far` collects (root.cuh).
+template <typename T, int V, bool NEAR, typename P>
 __device__ __forceinline__ Vec<T, V> row_new(const Vec<T, V> &m, const Vec<T, V> &l, const Vec<T, V> &r,
                                              const Vec<T, V> &u, const Vec<T, V> &d, const T (&w)[4], T alpha,
-                                             const P &p) {
+                                             const P &p, float &far) {
     Vec<T, V> o;
 #pragma unroll
     for (int q = 0; q < V; ++q) {
@@ -76,7 +77,9 @@ __device__ __forceinline__ Vec<T, V> row_new(const Vec<T, V> &m, const Vec<T, V>
         z = fma(w[1], l.v[q], z);
         z = fma(w[2], d.v[q], z);
         z = fma(w[3], u.v[q], z);
-        o.v[q] = root_newton(fma(alpha, m.v[q], z), p);
+        z = fma(alpha, m.v[q], z);
+        if constexpr (NEAR) o.v[q] = root_near(z, p, far);
+        else o.v[q] = root_newton(z, p);
     }
     return o;
 }
@@ -93,33 +96,13 @@ struct WalkSmem {
     Vec<T, V> y[TS > 1 ? TS - 1 : 1][2][TS > 1 ? kWT : 1];
 };
 
-template <typename T, int V, int TS>
-__global__ void __launch_bounds__(kWT, sizeof(T) == 8 ? 3 : 2)
-torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restrict__ edge, int64_t Lr, int64_t Lc, int R,
-           int G, int groups, int nwin, int wout, int strips, Alphas<T, TS> alpha,
-           typename RootOf<T>::type root) {
-    extern __shared__ __align__(16) unsigned char walk_smem[];
-    WalkSmem<T, V, TS> &sm = *reinterpret_cast<WalkSmem<T, V, TS> *>(walk_smem);
-    const int t = threadIdx.x;
-    const int grp = blockIdx.x % groups, rest = blockIdx.x / groups;
-    const int win = rest % nwin, strip = rest / nwin;
-    const int64_t r0 = Lr * strip / strips;
-    const int rows = static_cast<int>(Lr * (strip + 1) / strips - r0);  // (launch_walk)
-    const int sites = blockDim.x / G;          // columns of the window, halo included
-    const int s = min(t / G, sites - 1);       // threads past the last whole site repeat it
-    const int g = t % G;
-    const int tl = s * G + g;                  // this thread's slot (repeated ones write the same values)
-    const int left = s > 0 ? tl - G : tl, right = s + 1 < sites ? tl + G : tl;
-    const int64_t off = static_cast<int64_t>(win) * wout + s - TS;  // column, not wrapped
-    int64_t col = off % Lc;
-    if (col < 0) col += Lc;
-    const bool writes = s >= TS && s < TS + wout && off < Lc && t / G < sites;
-    const int64_t W = Lc * R;
-    const int64_t at = col * R + (static_cast<int64_t>(grp) * G + g) * V;
-    const T *xc = xi + at;
-    const uint32_t *ec = edge + col;
-    T *oc = xo + at;
-
+// one block's strip of rows; returns the largest |log2| of its roots (NEAR)
+template <typename T, int V, int TS, bool NEAR>
+__device__ __forceinline__ float walk_strip(WalkSmem<T, V, TS> &sm, const T *xc, T *oc, const uint32_t *ec, int64_t Lr,
+                                            int64_t Lc, int64_t W, int64_t r0, int rows, int s, int g, int tl, int left,
+                                            int right, bool writes, const Alphas<T, TS> &alpha,
+                                            const typename RootOf<T>::type &root) {
+    float far = 0.f;
     // ring row k holds lattice row r0 - TS + k (wrapped); rows 0 .. nk - 1 are needed
     const int nk = rows + 2 * TS;
     int64_t rk = (r0 - TS) % Lr;  // lattice row of the next ring row to stage
@@ -158,7 +141,7 @@ torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restr
             for (int q = 0; q < 4; ++q) w[l][q] = w[l - 1][q];
         unpack(sm.e[s1][s], w[0]);
         const Vec<T, V> xd = sm.x[s2][tl];
-        Vec<T, V> y = row_new<T, V>(xm, sm.x[s1][left], sm.x[s1][right], xu, xd, w[0], alpha.a[0], root);
+        Vec<T, V> y = row_new<T, V, NEAR>(xm, sm.x[s1][left], sm.x[s1][right], xu, xd, w[0], alpha.a[0], root, far);
         xu = xm;
         xm = xd;
 #pragma unroll
@@ -167,8 +150,8 @@ torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restr
             sm.y[l - 1][i & 1][tl] = y;
             Vec<T, V> yn = y;
             if (i >= 2 * l)
-                yn = row_new<T, V>(yb[l], sm.y[l - 1][(i & 1) ^ 1][left], sm.y[l - 1][(i & 1) ^ 1][right], ya[l], y,
-                                   w[l], alpha.a[l], root);
+                yn = row_new<T, V, NEAR>(yb[l], sm.y[l - 1][(i & 1) ^ 1][left], sm.y[l - 1][(i & 1) ^ 1][right], ya[l], y,
+                                         w[l], alpha.a[l], root, far);
             ya[l] = yb[l];
             yb[l] = y;
             y = yn;
@@ -182,6 +165,50 @@ torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restr
         s0 = s1;
     }
     wait_async<0>();
+    return far;
+}
+
+// the strip again, each root with its test: out of line, so that the strip before it keeps its registers
+template <int V, int TS>
+__device__ __noinline__ void walk_again(WalkSmem<float, V, TS> *sm, const float *xc, float *oc, const uint32_t *ec,
+                                        int64_t Lr, int64_t Lc, int64_t W, int64_t r0, int rows, int s, int g, int tl,
+                                        int left, int right, bool writes, Alphas<float, TS> alpha, RootF32 root) {
+    walk_strip<float, V, TS, false>(*sm, xc, oc, ec, Lr, Lc, W, r0, rows, s, g, tl, left, right, writes, alpha, root);
+}
+
+template <typename T, int V, int TS>
+__global__ void __launch_bounds__(kWT, sizeof(T) == 8 ? 3 : 2)
+torus_walk(const T *__restrict__ xi, T *__restrict__ xo, const uint32_t *__restrict__ edge, int64_t Lr, int64_t Lc, int R,
+           int G, int groups, int nwin, int wout, int strips, Alphas<T, TS> alpha,
+           typename RootOf<T>::type root) {
+    extern __shared__ __align__(16) unsigned char walk_smem[];
+    WalkSmem<T, V, TS> &sm = *reinterpret_cast<WalkSmem<T, V, TS> *>(walk_smem);
+    const int t = threadIdx.x;
+    const int grp = blockIdx.x % groups, rest = blockIdx.x / groups;
+    const int win = rest % nwin, strip = rest / nwin;
+    const int64_t r0 = Lr * strip / strips;
+    const int rows = static_cast<int>(Lr * (strip + 1) / strips - r0);  // (launch_walk)
+    const int sites = blockDim.x / G;          // columns of the window, halo included
+    const int s = min(t / G, sites - 1);       // threads past the last whole site repeat it
+    const int g = t % G;
+    const int tl = s * G + g;                  // this thread's slot (repeated ones write the same values)
+    const int left = s > 0 ? tl - G : tl, right = s + 1 < sites ? tl + G : tl;
+    const int64_t off = static_cast<int64_t>(win) * wout + s - TS;  // column, not wrapped
+    int64_t col = off % Lc;
+    if (col < 0) col += Lc;
+    const bool writes = s >= TS && s < TS + wout && off < Lc && t / G < sites;
+    const int64_t W = Lc * R;
+    const int64_t at = col * R + (static_cast<int64_t>(grp) * G + g) * V;
+    if constexpr (sizeof(T) == 4) {
+        const float far = walk_strip<T, V, TS, true>(sm, xi + at, xo + at, edge + col, Lr, Lc, W, r0, rows, s, g, tl, left,
+                                                     right, writes, alpha, root);
+        if (__syncthreads_or(!(far < kNear)))
+            walk_again<V, TS>(&sm, xi + at, xo + at, edge + col, Lr, Lc, W, r0, rows, s, g, tl, left, right, writes, alpha,
+                              root);
+    } else {
+        walk_strip<T, V, TS, false>(sm, xi + at, xo + at, edge + col, Lr, Lc, W, r0, rows, s, g, tl, left, right, writes,
+                                    alpha, root);
+    }
 }
 
 __global__ void edge_words(const int8_t *__restrict__ right, const int8_t *__restrict__ down, int64_t Lr, int64_t Lc,

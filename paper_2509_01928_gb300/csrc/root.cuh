@@ -53,13 +53,23 @@ __device__ __forceinline__ typename RootOf<T>::type make_root(double beta) {
 // FP32: one Newton step, the reciprocal 1 / (3 y^2) also from an exponential (2^(-2 l - log2 3)).
 // The residual a - y^3 with a = z / beta carries one rounding of a and one of y^2, each divided
 // by three: the result is within about 0.6 ulp of cbrt of the rounded z / beta (CUDA's cbrtf: 1).
-// Outside [2^-40, 2^40] for y (zero, subnormal quotients, infinities, NaN) y0 is returned.
-__device__ __forceinline__ float root_newton(float z, RootF32 p) {
+// This holds for y in (2^-kNear, 2^kNear). `far` collects the largest |log2 y|: where it reaches kNear (zeros and
+// subnormal z among them, as -infinity) root_near's result is not to be used. NaN passes through.
+constexpr float kNear = 40.f;
+__device__ __forceinline__ float root_near(float z, RootF32 p, float &far) {
     const float l = fmaf(lg2_fast(fabsf(z)), 1.0f / 3.0f, p.c3);
     const float y = copysignf(ex2_fast(l), z);
     const float w = ex2_fast(fmaf(l, -2.0f, -1.5849625007211561f));
     const float e = fmaf(-(y * y), y, z * p.inv_beta);
-    return fabsf(l) < 40.f ? fmaf(e, w, y) : y;
+    far = fmaxf(far, fabsf(l));
+    return fmaf(e, w, y);
+}
+// the same for any z: CUDA's cbrtf outside that range
+static __device__ __noinline__ float root_far(float z, float inv_beta) { return cbrtf(z * inv_beta); }
+__device__ __forceinline__ float root_newton(float z, RootF32 p) {
+    float far = 0.f;
+    const float y = root_near(z, p, far);
+    return far < kNear ? y : root_far(z, p.inv_beta);
 }
 
 // 2^-126 <= |f| < 2^128 as a double, by moving the exponent and mantissa fields (conversions and

@@ -101,3 +101,34 @@ def test_update_of_extreme_values(dtype):
     ok = np.isfinite(ref)
     np.testing.assert_allclose(x[ok], ref[ok], rtol=1e-6 if dtype == np.float32 else 1e-14, atol=1e-6)
     assert np.all(x[ref == 0] == 0)
+
+
+@pytest.mark.parametrize("form", ["lattice", "csr"])
+@pytest.mark.parametrize("lo, hi, beta", [(-149, -100, 2.0 ** -6), (-125, -118, 1.0), (119, 124, 1.0), (-149, 124, 1.0),
+                                          (-10, 10, 2.0)])
+def test_fp32_roots_of_any_size(form, lo, hi, beta):
+    """FP32 updates whose root lies outside 2^-40 .. 2^40, subnormal sums among them, are as exact as the
+    rest. All terms are positive: the five-term sum (six roundings with the division) and the cube root give
+    a relative error of at most (6 / 3 + 1) 2^-24, or half the spacing of subnormal quotients in z."""
+    t = I.torus_pm1(30, 42, seed=17)
+    t.right[:], t.down[:] = 1, 1
+    rng = np.random.default_rng(18)
+    x0 = (np.exp2(rng.uniform(lo, hi, (t.n, 4)))).astype(np.float32)
+    x0[5] = 0.0
+    x = _run(t if form == "lattice" else t.to_csr(), x0, [1.0], beta, 1)
+    z = x0.astype(np.float64).reshape(30, 42, 4)
+    u = sum(np.roll(z, s, a) for s in (1, -1) for a in (0, 1)) + z
+    a = (u / beta).reshape(x.shape)
+    room = np.maximum(np.cbrt(a + 2.0 ** -149) - np.cbrt(a), np.cbrt(a) * 3 * 2.0 ** -24)
+    assert np.all(np.abs(x.astype(np.float64) - np.cbrt(a)) <= room)
+
+
+def test_zero_replica_beside_others():
+    """A replica at zero (a fixed point) leaves the near range in every block; the others keep their values."""
+    t = I.torus_pm1(20, 37, seed=19)
+    x0 = I.x0_uniform(t.n, 4, seed=20)
+    alpha, beta = O.alpha_beta(t, eta=1.0, method="wigner")
+    whole = _run(t, x0, [alpha], beta, 7)
+    x0[:, 2] = 0.0
+    x = _run(t, x0, [alpha], beta, 7)
+    assert np.all(x[:, 2] == 0.0) and np.array_equal(x[:, [0, 1, 3]], whole[:, [0, 1, 3]])
