@@ -569,7 +569,8 @@ ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R
     // one instance whose average share does not fit runs single steps (5000 spins of 100 entries a row, R = 16,
     // FP32, 8 steps and the readout: 1.47 ms here, the couplings read from L2 a row per thread, 0.33 ms so)
     if (c->n_inst == 1 && left / entry_bytes<XT, VT>() < (c->nnz + c->nnz / 16) / K) return ISING_ERR_UNSUPPORTED;
-    const int64_t cap = left <= 0 ? -1 : std::min(left / entry_bytes<XT, VT>(), std::min(c->max_row_nnz * chunk, c->nnz)) / 4 * 4;
+    const int64_t need = std::min(c->max_row_nnz * chunk, c->nnz);
+    const int64_t cap = left <= 0 ? -1 : std::min(left / entry_bytes<XT, VT>() / 4 * 4, (need + 3) / 4 * 4);
     const int smem = static_cast<int>(cap < 0 ? state : optin - left + cap * entry_bytes<XT, VT>());
     auto kern = csr_small<XT, VT, P>;
     DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
