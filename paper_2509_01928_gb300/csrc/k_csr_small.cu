@@ -159,14 +159,20 @@ constexpr int64_t state_bytes(int64_t nb, int64_t rows, bool fix) {
 }
 template <typename XT, typename VT>
 constexpr bool can_fix() { return sizeof(XT) == 8 && sizeof(VT) == 1; }
-// where a launch may take fixed-point steps: rows long enough to repay the integers of the whole iterate
-// (us per step, fixed point / FP64 sums: 300 spins of 3 entries, R = 8 1.93 / 1.49; 400 of 20, R = 1 1.88 / 1.69;
-// 1500 of 30, R = 8 3.21 / 4.18; 800 of 48, R = 8 2.75 / 3.41; 1000 of 50, R = 20 4.24 / 6.44; 1500 of 120, R = 20
-// 8.1 / 11.0)
+// Where a launch may take fixed-point steps. The integers of the whole iterate and the rows' tests cost 0.4 to 1 us
+// per step (400 to 5000 spins); FP64 sums cost more where more than half of the SMs are busy. us per step, fixed
+// point / FP64 sums, by entries a row:
+//   R = 8, K = 16, 800 spins: 6 2.9 / 2.0, 9 2.2 / 2.3, 32 2.6 / 2.9, 48 2.7 / 3.4; 1500 spins: 9 2.6 / 3.2, 32 3.3 / 4.3
+//   R = 20, K = 7, 800 spins: 6 2.7 / 2.3, 9 2.8 / 3.0, 32 3.7 / 4.4; 5000 spins, R = 8: 9 5.8 / 5.2, 20 6.6 / 6.7, 32 7.7 / 8.2
+//   R = 4, K = 16 (64 CTAs), 1200 spins: 32 2.6 / 2.5; 2500 spins: 32 4.5 / 3.8; R = 1, 1200 spins: 72 3.1 / 3.3
+//   shares of 34 rows (400 spins, R = 8, K = 12): 16 1.9 / 1.7, 32 2.0 / 1.9
 template <typename XT, typename VT>
-bool fixed_point(const ising_context *c, const SmallRecord &rec, int K) {
-    return can_fix<XT, VT>() && K > 1 && !rec.base && c->nnz >= 24 * c->n;
+bool fixed_point(const ising_context *c, int R, const SmallRecord &rec, int K) {
+    const int64_t ctas = static_cast<int64_t>(c->n_inst) * R * K, chunk = (c->max_inst_n + K - 1) / K;
+    const int64_t entries = 2 * ctas <= c->num_sms || chunk < 48 ? 40 : chunk <= 256 ? 9 : 20;
+    return can_fix<XT, VT>() && K > 1 && !rec.base && c->nnz >= entries * c->n;
 }
+
 template <typename XT, typename VT>
 constexpr int64_t entry_bytes() { return sizeof(typename Held<XT, VT>::type) + sizeof(uint16_t); }
 
@@ -561,7 +567,7 @@ template <typename XT, typename VT, int P>
 ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R, const XT *h, const ParamTabs &p,
                         int k0, int iters, int K, const SmallRecord &rec, int64_t optin, cudaStream_t st) {
     const int64_t chunk = (c->max_inst_n + K - 1) / K;
-    const bool fix = fixed_point<XT, VT>(c, rec, K);
+    const bool fix = fixed_point<XT, VT>(c, R, rec, K);
     const int64_t state = state_bytes<XT, P>(c->max_inst_n, chunk, fix);
     if (state > optin) return ISING_ERR_UNSUPPORTED;
     // room for the couplings of the fullest share, as far as it goes (shares that need more read the CSR arrays)
@@ -711,7 +717,7 @@ ising_status_t launch_small(const ising_context *c, const XT *x_in, XT *x_out, i
             return launch_k<XT, VT, decltype(p_threads)::value>(c, x_in, x_out, R, h, p, k0, iters, K, rec, optin, st);
         };
         ising_status_t s;
-        if (fixed_point<XT, VT>(c, rec, K))
+        if (fixed_point<XT, VT>(c, R, rec, K))
             s = split && chunk <= 256   ? run(std::integral_constant<int, 8>())
                 : split && chunk <= 512 ? run(std::integral_constant<int, 4>())
                                         : run(std::integral_constant<int, 1>());
