@@ -47,15 +47,16 @@ constexpr int kCsrBatch = 8;  // entries whose loads are issued together
 // FP64; FP32 iterates form the terms in FP32 and sum them per thread with a
 // compensated (Kahan) FP32 sum. Each block writes FP64 partials
 // hpart[block][R][4], summed over threads in a fixed order.
+// A row takes C = R / V <= 256 threads; more replica chunks are taken by further launches, xi and xo moved on (R is the
+// rows' stride throughout).
 template <typename XT, typename VT, int V, bool TRACE>
 __global__ void __launch_bounds__(256)
 csr_step_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col, const VT *__restrict__ val, const XT *__restrict__ h,
-                const int64_t *__restrict__ inst_off, int n_inst, int64_t n, int R,
+                const int64_t *__restrict__ inst_off, int n_inst, int64_t n, int R, int C,
                 const XT *__restrict__ alpha_tab, int alpha_len, int k,
                 const XT *__restrict__ beta_tab, const float *__restrict__ zs_tab,
                 const float *__restrict__ xs_tab, double *__restrict__ hpart) {
-    const int C = R / V;
     const int ak = alpha_len == 1 ? 0 : k;
     // each thread keeps one replica chunk and strides over rows: no division in the loop
     const int rows_per_block = blockDim.x / C;
@@ -264,23 +265,26 @@ cudaError_t launch_step(const ising_context *c, const XT *xi, XT *xo, int R, con
                               dim3(256), st, xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h,
                               static_cast<int>(c->n), R, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc);
     }
-    const int blocks = step_blocks(c, C);
-    const int threads = C <= 256 ? 256 : ((C + 31) / 32) * 32;
-    if (hpart)
-        csr_step_kernel<XT, VT, V, true><<<static_cast<unsigned>(blocks), threads, 0, st>>>(
+    if (hpart)  // C <= 256 (dispatch_val)
+        csr_step_kernel<XT, VT, V, true><<<static_cast<unsigned>(step_blocks(c, C)), 256, 0, st>>>(
             xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, c->inst_off, c->n_inst,
-            c->n, R, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc, hpart);
+            c->n, R, C, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc, hpart);
     else
-        csr_step_kernel<XT, VT, V, false><<<static_cast<unsigned>(blocks), threads, 0, st>>>(
-            xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, c->inst_off, c->n_inst,
-            c->n, R, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc, nullptr);
+        for (int c0 = 0; c0 < C; c0 += 256) {
+            const int cn = std::min(256, C - c0);
+            csr_step_kernel<XT, VT, V, false><<<static_cast<unsigned>(step_blocks(c, cn)), 256, 0, st>>>(
+                xi + c0 * V, xo + c0 * V, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, c->inst_off, c->n_inst,
+                c->n, R, cn, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc, nullptr);
+        }
     return cudaGetLastError();
 }
 
 template <typename XT, int V>
 ising_status_t dispatch_val(const ising_context *c, const XT *xi, XT *xo, int R, const XT *h, const StepTabs<XT> &t,
                             int k, double *hpart, cudaStream_t st) {
-    if (R / V > 1024) return fail(ISING_ERR_UNSUPPORTED, "CSR step: R / vector width must be <= 1024");
+    // instances whose iterate fits shared memory take any R (k_csr_small.cu, or single steps where that declines)
+    if (R / V > 1024 && static_cast<size_t>(c->max_inst_n) > csr_fused_max_spins(sizeof(XT) == 8 ? ISING_F64 : ISING_F32))
+        return fail(ISING_ERR_UNSUPPORTED, "CSR step: R / vector width must be <= 1024");
     if (hpart && R / V > 256) return ISING_ERR_UNSUPPORTED;  // the fused monitor needs one row per 256 threads
     switch (c->jtype) {
         case ISING_I8: DOCH_CUDA((launch_step<XT, int8_t, V>(c, xi, xo, R, h, t, k, hpart, st))); break;

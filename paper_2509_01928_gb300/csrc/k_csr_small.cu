@@ -68,7 +68,7 @@ struct Exchange {
     unsigned long long bar[2];
     int abort_flag;
 };
-constexpr int kStaticSmem = 1024;  // at least the kernels' static shared memory
+constexpr int kStaticSmem = 128;  // at least the kernels' static shared memory
 
 __device__ __forceinline__ void exchange_init(Exchange &x) {  // before the opening cluster barrier
     if (threadIdx.x == 0) {

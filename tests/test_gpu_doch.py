@@ -669,6 +669,38 @@ def test_small_fp64_int8_components(n, R, density, jmax, case):
         N.ising_destroy(hd)
 
 
+@pytest.mark.parametrize("n, per_row, R, dtype", [(1000, 20, 600, np.float64), (1000, 20, 601, np.float64),
+                                                  (2500, 40, 257, np.float32), (1500, 40, 1301, np.float32),
+                                                  ("limit", 3, 513, np.float64), ("limit", 3, 1025, np.float32)])
+def test_many_replicas_of_small_instances(n, per_row, R, dtype):
+    """More replica chunks than a step kernel's block has threads, for instances whose couplings, or
+    whose iterate to the last byte, fill one CTA's shared memory."""
+    if n == "limit":
+        optin = torch.cuda.get_device_properties(0).shared_memory_per_block_optin
+        n = optin // (2 * np.dtype(dtype).itemsize)
+        g = I.regular_pm1(n - n % 2, 3, seed=40)  # (an odd vertex has no edges)
+        g = I.CSR(n, np.concatenate([g.row_ptr, np.full(n % 2, g.row_ptr[-1])]).astype(np.int64), g.col, g.val)
+    else:
+        g = I.erdos_renyi_pm1(n, per_row / n, seed=40)
+    g.val = g.val.astype(dtype)
+    alpha, beta = O.alpha_beta(g, eta=1.0, method="wigner")
+    x0 = I.x0_uniform(n, R, seed=41, dtype=dtype)
+    with Handle(g) as h:
+        x = _dev(x0)
+        N.ising_iterate(h, x, [alpha], [beta], 1)
+        x = x.cpu().numpy().astype(np.float64)
+    x0 = x0.astype(np.float64)
+    ref = O.doch(O.Problem(g), x0, alpha, beta, 1)
+    # z_i is a sum of `terms` products, each addition within 2^-24 (2^-53) of sum |terms|; the FP32 root of
+    # the step kernels adds up to 2^-21 (cbrt.cuh), the FP64 one 4 ulp
+    eps, root = (2.0 ** -24, 2.0 ** -21) if dtype == np.float32 else (2.0 ** -53, 2.0 ** -50)
+    size = np.abs(alpha * x0)
+    np.add.at(size, np.repeat(np.arange(n), np.diff(g.row_ptr)), np.abs(x0[g.col]))  # |J_ij| = 1
+    dz, z = (np.diff(g.row_ptr) + 3)[:, None] * eps * size / beta, ref ** 3
+    room = np.maximum(np.abs(np.cbrt(z + dz) - np.cbrt(z)), np.abs(np.cbrt(z - dz) - np.cbrt(z)))
+    assert np.all(np.abs(x - ref) <= room + root * np.abs(ref))
+
+
 @pytest.mark.parametrize("sizes", [[1000, 17], [1000, 40, 10, 1], [600, 1, 33, 599]])
 @pytest.mark.parametrize("jdtype", [np.int8, np.float64])
 def test_small_fp64_batches_with_short_instances(sizes, jdtype):
