@@ -563,6 +563,20 @@ int cluster_max(const ising_context *c, int R) {
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({16, c->num_sms / pairs, c->max_inst_n / 32})));
 }
 
+// One instance whose average share of couplings does not fit: here, the couplings read from L2 row by row, or
+// single steps? A single step costs about 0.19 us per entry of a row in FP32, 0.26 in FP64 and 0.32 in FP64 with two
+// replicas per thread (even R), nearly whatever the number of rows; here it is about 0.95 ns per entry of a
+// share while few CTAs read (1.3 with 128 of them). us per step, here / single steps, K = 16:
+//   FP64, 3000 spins of 110 entries: R = 1 18.4 / 28.7, R = 4 18.4 / 35.1, R = 8 24.6 / 34.9 (R = 9: 30.0 / 26.7)
+//   FP64, 5000 spins of 80: R = 1 24.8 / 22.7, R = 2 25.0 / 30.5, R = 6 25.1 / 28.8, R = 8 33.6 / 28.7
+//   FP64, 8000 spins of 50: R = 1 28.4 / 16.5, R = 4 28.4 / 22.0
+//   FP32, 5000 spins of 110: R = 1 30.2 / 20.6, R = 4 30.7 / 22.6, R = 8 40.7 / 20.6; 2000 of 110, R = 16, K = 9: 33.3 / 18.5
+template <typename XT>
+bool from_l2(const ising_context *c, int R, int K) {
+    return sizeof(XT) == 8 && static_cast<int64_t>(R) * K <= 128 && c->n * R <= 32768 &&
+           (c->n + K - 1) / K <= (R % 2 == 0 ? 320 : 256);
+}
+
 template <typename XT, typename VT, int P>
 ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R, const XT *h, const ParamTabs &p,
                         int k0, int iters, int K, const SmallRecord &rec, int64_t optin, cudaStream_t st) {
@@ -572,9 +586,8 @@ ising_status_t launch_k(const ising_context *c, const XT *x_in, XT *x_out, int R
     if (state > optin) return ISING_ERR_UNSUPPORTED;
     // room for the couplings of the fullest share, as far as it goes (shares that need more read the CSR arrays)
     const int64_t left = optin - state - static_cast<int64_t>(sizeof(int)) * (chunk + 1);
-    // one instance whose average share does not fit runs single steps (5000 spins of 100 entries a row, R = 16,
-    // FP32, 8 steps and the readout: 1.47 ms here, the couplings read from L2 a row per thread, 0.33 ms so)
-    if (c->n_inst == 1 && left / entry_bytes<XT, VT>() < (c->nnz + c->nnz / 16) / K) return ISING_ERR_UNSUPPORTED;
+    if (c->n_inst == 1 && left / entry_bytes<XT, VT>() < (c->nnz + c->nnz / 16) / K && !from_l2<XT>(c, R, K))
+        return ISING_ERR_UNSUPPORTED;
     const int64_t need = std::min(c->max_row_nnz * chunk, c->nnz);
     const int64_t cap = left <= 0 ? -1 : std::min(left / entry_bytes<XT, VT>() / 4 * 4, (need + 3) / 4 * 4);
     const int smem = static_cast<int>(cap < 0 ? state : optin - left + cap * entry_bytes<XT, VT>());

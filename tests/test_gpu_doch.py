@@ -742,3 +742,20 @@ def test_shares_that_do_not_fit_take_single_steps(n, per_row, R):
         assert err.max() <= 1e-4 and np.median(err) <= 1e-5
     finally:
         N.ising_destroy(hd)
+
+
+@pytest.mark.parametrize("n, per_row, R", [(3000, 110, 1), (3000, 110, 8), (3000, 110, 9), (5000, 60, 1), (5000, 60, 6),
+                                           (5000, 60, 8), (4096, 100, 8)])
+def test_fp64_shares_that_do_not_fit(n, per_row, R):
+    """Both sides of the rule that keeps FP64 instances in one launch with their couplings read from L2."""
+    hd = N.ising_create_s5(n, round(100.0 * per_row / n, 4), 5)
+    try:
+        g = N.ising_csr_export(hd)
+        J = I.CSR(n, g[0], g[1], g[2])
+        alpha, beta = O.alpha_beta(J, eta=1.0, method="wigner")
+        x0 = I.x0_uniform(n, R, seed=6, dtype=np.float64)
+        x = torch.from_numpy(x0.copy()).cuda()
+        N.ising_iterate(hd, x, [alpha], [beta], 3)
+        _close(x.cpu().numpy(), O.doch(O.Problem(J), x0, alpha, beta, 3), TOL64)
+    finally:
+        N.ising_destroy(hd)
