@@ -682,12 +682,13 @@ ising_status_t upload_params(ising_context *c, const double *alpha, int alpha_le
     std::memcpy(host, a.data(), na * 8);
     std::memcpy(host + o1, b.data(), ni * 8);
     for (size_t i = 0; i < na; ++i) reinterpret_cast<float *>(host + o2)[i] = static_cast<float>(a[i]);
-    for (int i = 0; i < ni; ++i) {
+    float zscale0 = 1.f, xscale0 = 1.f;
+    for (int i = ni - 1; i >= 0; --i) {
         const double ib = 1.0 / b[i];
         const int k = cbrt_prescale_exp(ib);
         reinterpret_cast<float *>(host + o3)[i] = static_cast<float>(ib);
-        reinterpret_cast<float *>(host + o4)[i] = static_cast<float>(std::ldexp(ib, 3 * k));
-        reinterpret_cast<float *>(host + o5)[i] = std::ldexp(1.0f, -k);
+        reinterpret_cast<float *>(host + o4)[i] = zscale0 = static_cast<float>(std::ldexp(ib, 3 * k));
+        reinterpret_cast<float *>(host + o5)[i] = xscale0 = std::ldexp(1.0f, -k);
     }
     DOCH_CHECK(c->params.ensure(tot));
     if (small) {
@@ -705,6 +706,11 @@ ising_status_t upload_params(ising_context *c, const double *alpha, int alpha_le
     out.zscale_f = reinterpret_cast<const float *>(base + o4);
     out.xscale_f = reinterpret_cast<const float *>(base + o5);
     out.alpha_len = alpha_len;
+    c->alpha_host = std::move(a);
+    out.alpha_host = c->alpha_host.data();
+    out.beta0 = b[0];
+    out.zscale0 = zscale0;
+    out.xscale0 = xscale0;
     return ISING_OK;
 }
 

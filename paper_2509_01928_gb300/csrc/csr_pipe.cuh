@@ -10,6 +10,7 @@
 #include <cstdint>
 
 #include "cbrt.cuh"
+#include "internal.cuh"
 #include "root.cuh"
 
 namespace doch {
@@ -57,6 +58,7 @@ struct StepRoot;
 template <>
 struct StepRoot<float> {
     float zs, xsc;
+    __device__ __forceinline__ explicit StepRoot(const StepValues<float> &v) : zs(v.zs), xsc(v.xsc) {}
     __device__ __forceinline__ StepRoot(const float *, const float *zs_tab, const float *xs_tab, int b)
         : zs(__ldg(zs_tab + b)), xsc(__ldg(xs_tab + b)) {}
     __device__ __forceinline__ float operator()(float z) const { return cbrt_pow2(z * zs) * xsc; }
@@ -64,6 +66,7 @@ struct StepRoot<float> {
 template <>
 struct StepRoot<double> {
     RootF64 p;
+    __device__ __forceinline__ explicit StepRoot(const StepValues<double> &v) : p(make_root<double>(v.beta)) {}
     __device__ __forceinline__ StepRoot(const double *beta_tab, const float *, const float *, int b)
         : p(make_root<double>(__ldg(beta_tab + b))) {}
     __device__ __forceinline__ double operator()(double z) const { return root_newton(z, p); }

@@ -152,6 +152,7 @@ struct ising_context {
     doch::DevBuf stage_out; // staging of host outputs
     doch::DevBuf partials;  // reduction partials
     doch::DevBuf params;    // alpha/beta tables on the device
+    std::vector<double> alpha_host;  // alpha of the last call
     unsigned char *params_stage = nullptr;  // pinned staging of the tables
     size_t params_stage_bytes = 0;
     cudaEvent_t params_event = nullptr;     // its last copy
@@ -194,11 +195,15 @@ namespace doch {
 // launches that overlap their start with the end of the kernel before them in the stream (a chain of
 // short kernels: 3.1 us per empty launch of 600 blocks, 1.4 us so). The kernel calls pdl_wait() before it
 // reads or writes what other kernels write or read, then pdl_trigger(): at most two kernels overlap.
-// What the kernel before may still have been writing is read past L1 (__ldcg).
+// What the kernel before may still have been writing is read past L1 (__ldcg; parameter tables, which all warps
+// ask for, through it: __ldca), never as read-only data, which may be fetched at any time. To the compiler such a load does not depend on the wait: an index that its
+// address is formed from goes through pdl_after() behind the wait, and then it cannot be moved above it.
 // ---------------------------------------------------------------------------
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ void pdl_after(int &index) { asm volatile("" : "+r"(index) : : "memory"); }
 
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, A &&...args) {
@@ -252,7 +257,23 @@ struct ParamTabs {
     const float *zscale_f = nullptr;
     const float *xscale_f = nullptr;
     int alpha_len = 1;
+    // the host's copy: alpha (the handle's, until its next call) and the values of instance 0
+    const double *alpha_host = nullptr;
+    double beta0 = 1.0;
+    float zscale0 = 1.f, xscale0 = 1.f;
 };
+// One instance's parameters of step k by value, for kernels that overlap the one before them: they may not
+// read the tables ahead of their wait, and behind it all warps asked one L2 line for them (2 us per step).
+template <typename XT>
+struct StepValues {
+    XT alpha;
+    double beta;
+    float zs, xsc;
+};
+template <typename XT>
+StepValues<XT> step_values(const ParamTabs &p, int k) {
+    return {static_cast<XT>(p.alpha_host[p.alpha_len == 1 ? 0 : k]), p.beta0, p.zscale0, p.xscale0};
+}
 
 // CSR, one DOCH step for all instances (alpha of step k), xtype F32 or F64.
 ising_status_t csr_step(const ising_context *c, const void *x_in, void *x_out, int xtype, int R,

@@ -162,9 +162,10 @@ adoch_step(Fn fn, Candidates<XT> x1, Candidates<XT> x0, XT *next_y, XT *next_x, 
     const int Cb = R < kAThreads ? R : kAThreads;
     const int rows = kAThreads / Cb;
     const int rl = threadIdx.x / Cb;
-    const int r = blockIdx.y * Cb + threadIdx.x % Cb;
+    int r = blockIdx.y * Cb + threadIdx.x % Cb;
     const bool active = rl < rows && r < R;
-    const int ch = blockIdx.x, b = blockIdx.z;
+    const int ch = blockIdx.x;
+    int b = blockIdx.z;
     const int64_t lo = inst_off ? inst_off[b] : 0;
     const int64_t hi = inst_off ? inst_off[b + 1] : n;
     const int64_t len = hi - lo;
@@ -172,8 +173,10 @@ adoch_step(Fn fn, Candidates<XT> x1, Candidates<XT> x0, XT *next_y, XT *next_x, 
     SiteSum<XT> acc[kTerms];
     pdl_wait();
     pdl_trigger();
-    const XT a = alpha_tab[b];
-    const AdochRoot<XT> root(beta_tab[b]);
+    pdl_after(r);  // x, u and the decisions
+    pdl_after(b);
+    const XT a = __ldca(alpha_tab + b);
+    const AdochRoot<XT> root(__ldca(beta_tab + b));
     // one load of the decisions per block: all blocks ask one L2 slice for these lines
     __shared__ int dec[2][kAThreads];
     if (active && rl == 0) {
@@ -260,14 +263,15 @@ adoch_decide(const typename SiteSum<XT>::Slot *__restrict__ partials, int n_inst
              const double *__restrict__ alpha_tab, const double *__restrict__ beta_tab, int k, int q,
              double *__restrict__ hist, int *__restrict__ dec, int8_t *__restrict__ acc_out,
              double *__restrict__ H_out) {
-    const int t = blockIdx.x;
-    const int b = t / R;
+    int t = blockIdx.x;
     const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __shared__ double red[kTerms];
-    double *ht = hist + static_cast<int64_t>(t) * (q + 1);
     pdl_wait();
     pdl_trigger();
-    const double a = alpha_tab[b], be = beta_tab[b];
+    pdl_after(t);
+    const int b = t / R;
+    double *ht = hist + static_cast<int64_t>(t) * (q + 1);
+    const double a = __ldca(alpha_tab + b), be = __ldca(beta_tab + b);
     const typename SiteSum<XT>::Slot *p = partials + (static_cast<int64_t>(t) * kTerms + j) * chunks;
     SiteSum<XT> s;
     constexpr int kAhead = 8;  // loads in flight

@@ -212,7 +212,7 @@ adjoint_step_kernel(const float *__restrict__ w_in, const XT *__restrict__ x_cur
     DotSum32 ga32;
     unsigned nz = 0;
     const int rows_per_block = kBThreads / C;
-    const int ch = threadIdx.x % C;
+    int ch = threadIdx.x % C;
     const int rl = threadIdx.x / C;
     const IT S = static_cast<IT>(gridDim.x) * rows_per_block;
     // threads past the block's last full row take no rows
@@ -225,6 +225,7 @@ adjoint_step_kernel(const float *__restrict__ w_in, const XT *__restrict__ x_cur
     pipe_first_batch<kBatchB>(col, val, e0, e1, js, ws);
     pdl_wait();  // the couplings above are never written
     pdl_trigger();
+    pdl_after(ch);
     for (; i < n; i += S) {
         const int cnt = e1 - e0 < kBatchB ? static_cast<int>(e1 - e0) : kBatchB;
         float wj[kBatchB][V];

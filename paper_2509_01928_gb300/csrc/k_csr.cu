@@ -151,12 +151,10 @@ template <typename XT, typename VT, int V>
 __global__ void __launch_bounds__(256, pipe_blocks_per_sm<XT>())
 csr_step_pipe_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__restrict__ row_ptr,
                      const int32_t *__restrict__ col, const VT *__restrict__ val, const XT *__restrict__ h,
-                     int n, int R, const XT *__restrict__ alpha_tab, int alpha_len, int k,
-                     const XT *__restrict__ beta_tab, const float *__restrict__ zs_tab,
-                     const float *__restrict__ xs_tab) {
+                     int n, int R, StepValues<XT> par) {
     const int C = R / V;
     const int rows_per_block = blockDim.x / C;
-    const int ch = threadIdx.x % C;
+    int ch = threadIdx.x % C;
     const int rl = threadIdx.x / C;
     const int S = static_cast<int>(gridDim.x) * rows_per_block;
     int i = rl < rows_per_block ? static_cast<int>(blockIdx.x) * rows_per_block + rl : n;
@@ -168,8 +166,9 @@ csr_step_pipe_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64
     pipe_first_batch<kPipeB>(col, val, e0, e1, js, ws);
     pdl_wait();  // the couplings above are never written
     pdl_trigger();
-    const XT a = __ldg(alpha_tab + (alpha_len == 1 ? 0 : k));
-    const StepRoot<XT> root(beta_tab, zs_tab, xs_tab, 0);
+    pdl_after(ch);
+    const XT a = par.alpha;
+    const StepRoot<XT> root(par);
     for (; i < n; i += S) {
         const int cnt = e1 - e0 < kPipeB ? static_cast<int>(e1 - e0) : kPipeB;
         XT xv[kPipeB][V];
@@ -254,6 +253,7 @@ struct StepTabs {
     const XT *beta;
     const float *zs;
     const float *xsc;
+    StepValues<XT> now;  // one instance: the step's own
 };
 
 template <typename XT, typename VT, int V>
@@ -263,7 +263,7 @@ cudaError_t launch_step(const ising_context *c, const XT *xi, XT *xo, int R, con
     if (use_pipe(c, C, hpart != nullptr)) {
         return launch_chained(csr_step_pipe_kernel<XT, VT, V>, dim3(static_cast<unsigned>(pipe_blocks<XT>(c, C))),
                               dim3(256), st, xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h,
-                              static_cast<int>(c->n), R, t.alpha, t.alpha_len, k, t.beta, t.zs, t.xsc);
+                              static_cast<int>(c->n), R, t.now);
     }
     if (hpart)  // C <= 256 (dispatch_val)
         csr_step_kernel<XT, VT, V, true><<<static_cast<unsigned>(step_blocks(c, C)), 256, 0, st>>>(
@@ -312,7 +312,7 @@ static ising_status_t csr_step_impl(const ising_context *c, const void *xi, void
     if (xtype == ISING_F32) {
         const float *x_in = static_cast<const float *>(xi);
         float *x_out = static_cast<float *>(xo);
-        const StepTabs<float> t{p.alpha_f, p.alpha_len, p.inv_beta_f, p.zscale_f, p.xscale_f};
+        const StepTabs<float> t{p.alpha_f, p.alpha_len, p.inv_beta_f, p.zscale_f, p.xscale_f, step_values<float>(p, k)};
         if (R % 4 == 0 && a % 16 == 0) {
             *blocks = step_blocks(c, R / 4);
             return dispatch_val<float, 4>(c, x_in, x_out, R, c->h_f32, t, k, hpart, st);
@@ -327,7 +327,7 @@ static ising_status_t csr_step_impl(const ising_context *c, const void *xi, void
     if (xtype == ISING_F64) {
         const double *x_in = static_cast<const double *>(xi);
         double *x_out = static_cast<double *>(xo);
-        const StepTabs<double> t{p.alpha_d, p.alpha_len, p.beta_d, nullptr, nullptr};
+        const StepTabs<double> t{p.alpha_d, p.alpha_len, p.beta_d, nullptr, nullptr, step_values<double>(p, k)};
         if (R % 2 == 0 && a % 16 == 0) {
             *blocks = step_blocks(c, R / 2);
             return dispatch_val<double, 2>(c, x_in, x_out, R, c->h_f64, t, k, hpart, st);

@@ -149,15 +149,15 @@ template <typename XT, typename VT, int V>
 __global__ void __launch_bounds__(kUThreads, kUBlocksPerSm)
 until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__restrict__ row_ptr,
              const int32_t *__restrict__ col, const VT *__restrict__ val, const XT *__restrict__ h, int n, int R,
-             const XT *__restrict__ alpha_tab, const XT *__restrict__ beta_tab, const float *__restrict__ zs_tab,
-             const float *__restrict__ xs_tab, int Cp, int dblocks, double eps, int k, typename UntilSum<XT>::Slot *__restrict__ part,
+             StepValues<XT> par, int Cp, int dblocks, double eps, int k, typename UntilSum<XT>::Slot *__restrict__ part,
              const typename UntilSum<XT>::Slot *__restrict__ part_before, int *running, int32_t *__restrict__ steps,
              int *n_running, UntilProgress *progress, int call) {
     const int blocks = static_cast<int>(gridDim.x) - dblocks, blk = static_cast<int>(blockIdx.x) - dblocks;
     if (blk < 0) {
         pdl_wait();
         pdl_trigger();
-        const int t = static_cast<int>(blockIdx.x) * kUWarps + (threadIdx.x >> 5);
+        int t = static_cast<int>(blockIdx.x) * kUWarps + (threadIdx.x >> 5);
+        pdl_after(t);
         if (k > 0 && t < R) until_decide<XT>(part_before, blocks, eps, k - 1, t, running, steps, n_running);
         __syncthreads();
         if (blockIdx.x == 0 && threadIdx.x == 0)  // for the host: launch k runs, and whether any replica still does
@@ -166,7 +166,7 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
     }
     const int C = R / V;
     const int rows_per_block = kUThreads / Cp;
-    const int ch = threadIdx.x % Cp;
+    int ch = threadIdx.x % Cp;
     const int rl = threadIdx.x / Cp;
     const int S = blocks * rows_per_block;
     int i = rl < rows_per_block && ch < C ? blk * rows_per_block + rl : n;
@@ -178,8 +178,9 @@ until_kernel(const XT *__restrict__ xi, XT *__restrict__ xo, const int64_t *__re
     pipe_first_batch<kUBatch>(col, val, e0, e1, js, ws);
     pdl_wait();  // the couplings above are never written
     pdl_trigger();
-    const XT a = alpha_tab[0];
-    const StepRoot<XT> root(beta_tab, zs_tab, xs_tab, 0);
+    pdl_after(ch);  // x and the flags
+    const XT a = par.alpha;
+    const StepRoot<XT> root(par);
     // a flag lowered during this launch may or may not be seen: this launch's writes miss x^k either way
     bool run[V], all = true, any = false;
     int flag[V];  // one load: all warps of the grid ask one L2 slice for this line (V loads a warp: 2 us a step)
@@ -423,17 +424,9 @@ ising_status_t launch_until(const ising_context *c, const XT *xi, XT *xo, int R,
     const int C = R / V;
     const int blocks = until_blocks(c, C);
     const int dblocks = (R + kUWarps - 1) / kUWarps;
-    const XT *alpha = nullptr, *beta = nullptr;
-    if constexpr (sizeof(XT) == 8) {
-        alpha = p.alpha_d;
-        beta = p.beta_d;
-    } else {
-        alpha = p.alpha_f;
-        beta = p.inv_beta_f;
-    }
     DOCH_CUDA(launch_chained(until_kernel<XT, VT, V>, dim3(static_cast<unsigned>(dblocks + blocks)), dim3(kUThreads), st,
                              xi, xo, c->row_ptr, c->col, static_cast<const VT *>(c->val), h, static_cast<int>(c->n), R,
-                             alpha, beta, p.zscale_f, p.xscale_f, row_threads(C), dblocks, eps, k, partials_of<XT>(c, R, k, s),
+                             step_values<XT>(p, 0), row_threads(C), dblocks, eps, k, partials_of<XT>(c, R, k, s),
                              partials_of<XT>(c, R, k + 1, s), s.running, s.steps, s.n_running, s.progress, s.call));
     return ISING_OK;
 }
