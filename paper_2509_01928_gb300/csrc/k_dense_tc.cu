@@ -17,11 +17,9 @@
 //   X  : replica-major [kblocks][R_pad][64] BF16 with the same swizzle, so
 //        the rows r0 .. r0+N-1 of one K block are one contiguous N x 128 B
 //        image; spins >= n are zero.
-// Tiles: one CTA per (128 rows of J) x (N = up to 256 replicas), or a cluster of S <= 8 CTAs that
-// share the tile's K blocks where the tiles alone leave SMs idle (split_of): each CTA puts its partial
-// accumulator in its shared memory, and CTA s adds the S partials of its share of the columns, in
-// order, through distributed shared memory and finishes them. 2000 spins, R = 100 (16 tiles): 21.5 us
-// per step with 16 CTAs, 10.4 us with clusters of 6.
+// Tiles: one CTA per (128 rows of J) x (N = up to 256 replicas); N is smaller where that many tiles
+// leave SMs idle (geometry). Every product adds all K blocks in one accumulator and one order, which depends on
+// the row tile alone: a replica's iterates do not depend on how many run beside it.
 //
 // Pipeline per CTA (256 threads):
 //   warp 0, one lane: producer. K-block kb (64 columns of J = 64 spins of
@@ -62,7 +60,6 @@ template <bool TERN> constexpr int kStagesOf = TERN ? 6 : 4;
 constexpr int kBM = 128;           // rows of J per tile (MMA M)
 constexpr int kBK = 64;            // K per stage: 64 BF16 = 128 bytes = one swizzle row
 constexpr int kThreadsTC = 256;
-constexpr int kMaxSplit = 8;       // CTAs that share a tile's K blocks (the portable cluster size)
 
 constexpr uint32_t kTernTile = kBM * kBK / 4;  // bytes of one packed ternary J tile (2 bits per entry)
 constexpr int kJStages = 8;                      // packed ternary tiles staged ahead
@@ -177,22 +174,6 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(bar)) : "memory");
 }
 
-__device__ __forceinline__ void cluster_sync() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// four floats at `own`'s offset in the shared memory of CTA `rank` of the cluster
-__device__ __forceinline__ float4 cluster_load4(const float *own, uint32_t rank) {
-    uint32_t a;
-    float4 v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr(own)), "r"(rank));
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(a)
-                 : "memory");
-    return v;
-}
-
 // BF16 bits of a 2-bit ternary code: 0 -> 0, 1 -> +1, 2 -> -1 (3 unused -> 0)
 __device__ __forceinline__ uint32_t tern_bf16(uint32_t code) {
     return code == 1 ? 0x3F80u : (code == 2 ? 0xBF80u : 0u);
@@ -207,8 +188,7 @@ template <int MODE, bool TERN>
 __global__ void __launch_bounds__(kThreadsTC, 1)
 dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ xt_in,
                 __nv_bfloat16 *__restrict__ xt_out, const float *__restrict__ h, int n, int kblocks, int R,
-                int R_pad, int n_tile, uint32_t tmem_cols, uint32_t a_col, int split, float alpha, float zscale,
-                float xscale,
+                int R_pad, int n_tile, uint32_t tmem_cols, uint32_t a_col, float alpha, float zscale, float xscale,
                 long long *__restrict__ q_out, int *__restrict__ err) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint32_t lut[16];  // ternary: two 2-bit codes -> two BF16
@@ -217,16 +197,12 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     Smem &sm = *reinterpret_cast<Smem *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m_tile = blockIdx.x / split, rank = blockIdx.x % split;
-    const int m_tiles = gridDim.x / split;
-    const int m0 = m_tile * kBM;
-    // this CTA's K blocks: k_count from k_first
-    const int k_first = kblocks * rank / split, k_count = kblocks * (rank + 1) / split - k_first;
+    const int m0 = blockIdx.x * kBM;
     const int r0 = blockIdx.y * n_tile;
     // bytes of J per K block: a BF16 tile, or a packed ternary tile expanded on chip
     constexpr uint32_t a_bytes = TERN ? kTernTile : kBM * kBK * 2;
     const uint32_t b_bytes = static_cast<uint32_t>(n_tile) * kBK * 2;
-    const unsigned char *a_src = static_cast<const unsigned char *>(jt) + static_cast<size_t>(m_tile) * kblocks * a_bytes;
+    const unsigned char *a_src = static_cast<const unsigned char *>(jt) + static_cast<size_t>(blockIdx.x) * kblocks * a_bytes;
     const __nv_bfloat16 *b_src = xt_in + static_cast<size_t>(r0) * kBK;
     volatile int *abort_flag = &sm.abort_flag;
 
@@ -262,13 +238,12 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     // any moment the CTAs stream different parts of J (equal 4 MB-aligned
     // offsets in lockstep would queue on the same DRAM channels) and read
     // different blocks of X from L2. Sum order only changes FP32 rounding.
-    const int kb0 = static_cast<int>(static_cast<int64_t>(m_tile) * k_count / m_tiles);
+    const int kb0 = static_cast<int>(static_cast<int64_t>(blockIdx.x) * kblocks / gridDim.x);
     if (warp == 0 && lane == 0) {
-        for (int it = 0; it < k_count; ++it) {
+        for (int it = 0; it < kblocks; ++it) {
             const int s = it % kStages;
             int kb = kb0 + it;
-            if (kb >= k_count) kb -= k_count;
-            kb += k_first;
+            if (kb >= kblocks) kb -= kblocks;
             if (it >= kStages && !mbar_wait(&sm.empty[s], ((it / kStages) - 1) & 1, err, abort_flag)) break;
             if (TERN) {
                 mbar_expect_tx(&sm.full[s], b_bytes);
@@ -282,7 +257,7 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     } else if (warp == 1 && lane == 0) {
         const uint32_t idesc = idesc_bf16(kBM, n_tile);
         bool ok = true;
-        for (int it = 0; it < k_count; ++it) {
+        for (int it = 0; it < kblocks; ++it) {
             const int s = it % kStages;
             // ternary: A is ready when the converters arrived on conv[s]; B when full[s] completed
             if ((TERN && !mbar_wait(&sm.conv[s], (it / kStages) & 1, err, abort_flag)) ||
@@ -310,11 +285,10 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
         }
     } else if (TERN && warp == 3 && lane == 0) {
         // producer of the packed ternary tiles (2 KB each), kJStages ahead
-        for (int it = 0; it < k_count; ++it) {
+        for (int it = 0; it < kblocks; ++it) {
             const int p = it % kJStages;
             int kb = kb0 + it;
-            if (kb >= k_count) kb -= k_count;
-            kb += k_first;
+            if (kb >= kblocks) kb -= kblocks;
             if (it >= kJStages && !mbar_wait(&sm.jempty[p], ((it / kJStages) - 1) & 1, err, abort_flag)) break;
             mbar_expect_tx(&sm.jfull[p], a_bytes);
             bulk_load(sm.jp[p], a_src + static_cast<size_t>(kb) * a_bytes, a_bytes, &sm.jfull[p]);
@@ -327,7 +301,7 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
         // waits are made warp-uniform: tcgen05.st is a .sync.aligned instruction.
         const int t = threadIdx.x - 128;
         const uint32_t a_lane = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + a_col;
-        for (int it = 0; it < k_count; ++it) {
+        for (int it = 0; it < kblocks; ++it) {
             const int s = it % kStages, p = it % kJStages;
             if (!__all_sync(0xffffffffu, mbar_wait(&sm.jfull[p], (it / kJStages) & 1, err, abort_flag))) break;
             const uint4 codes = *reinterpret_cast<const uint4 *>(sm.jp[p] + 16 * t);
@@ -348,8 +322,8 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
     __syncwarp();
     // Epilogue, all eight warps: warp w moves TMEM lanes 32 (w % 4) .. +31 (its 32 rows) of every other
     // 32-column block into shared memory, then takes whole columns, a lane per four rows: four spins
-    // of a replica are 8 bytes of X (2-byte accesses by row took 55 us per step at n = 9000, R = 256, two CTAs
-    // per tile; 40 so).
+    // of a replica are 8 bytes of X (2-byte accesses by row took 65.6 us per step at n = 9000, R = 256, tiles of 256
+    // replicas; 59.7 so).
     {
         const int q = warp & 3, half = warp >> 2;
         // warp-uniform decision: tcgen05.ld below is a .sync.aligned warp instruction
@@ -398,52 +372,27 @@ dense_tc_kernel(const void *__restrict__ jt, const __nv_bfloat16 *__restrict__ x
             }
         };
         constexpr int kW = kThreadsTC / 32;
-        if (split == 1) {
-            __syncthreads();
-            const int cols = n_tile < R - r0 ? n_tile : R - r0;
-            constexpr int kAhead = 4;  // columns whose loads are issued together
-            for (int c = warp; ok && c < cols; c += kW * kAhead) {
-                uint2 xw[kAhead];
-                float4 u[kAhead];
+        __syncthreads();
+        const int cols = n_tile < R - r0 ? n_tile : R - r0;
+        constexpr int kAhead = 4;  // columns whose loads are issued together
+        for (int c = warp; ok && c < cols; c += kW * kAhead) {
+            uint2 xw[kAhead];
+            float4 u[kAhead];
 #pragma unroll
-                for (int e = 0; e < kAhead; ++e)
-                    if (c + e * kW < cols) {
-                        xw[e] = state(r0 + c + e * kW);
-                        u[e] = *reinterpret_cast<const float4 *>(partial + (c + e * kW) * kBM + 4 * lane);
-                    }
+            for (int e = 0; e < kAhead; ++e)
+                if (c + e * kW < cols) {
+                    xw[e] = state(r0 + c + e * kW);
+                    u[e] = *reinterpret_cast<const float4 *>(partial + (c + e * kW) * kBM + 4 * lane);
+                }
 #pragma unroll
-                for (int e = 0; e < kAhead; ++e)
-                    if (c + e * kW < cols) finish(c + e * kW, u[e], xw[e]);
-            }
-        } else {
-            const int c1 = n_tile * (rank + 1) / split;
-            cluster_sync();
-            for (int c = n_tile * rank / split + warp; c < c1 && r0 + c < R; c += kW) {
-                float4 v[kMaxSplit];  // all partials of a column in flight
-#pragma unroll
-                for (int t = 0; t < kMaxSplit; ++t)
-                    if (t < split) v[t] = cluster_load4(partial + c * kBM + 4 * lane, t);
-                const uint2 xw = state(r0 + c);
-#pragma unroll
-                for (int t = 1; t < kMaxSplit; ++t)
-                    if (t < split) {
-                        v[0].x += v[t].x;
-                        v[0].y += v[t].y;
-                        v[0].z += v[t].z;
-                        v[0].w += v[t].w;
-                    }
-                finish(c, v[0], xw);
-            }
-            cluster_sync();  // no CTA leaves while a peer reads its partials
+            for (int e = 0; e < kAhead; ++e)
+                if (c + e * kW < cols) finish(c + e * kW, u[e], xw[e]);
         }
         if (MODE == 1) {  // the tile's terms per replica: q_out[row tile][R]
             __syncthreads();
             const int r = r0 + threadIdx.x;
-            const bool mine = split == 1 || (static_cast<int>(threadIdx.x) >= n_tile * rank / split &&
-                                             static_cast<int>(threadIdx.x) < n_tile * (rank + 1) / split);
-            if (static_cast<int>(threadIdx.x) < n_tile && r < R && mine) {
-                q_out[static_cast<size_t>(m_tile) * R + r] = sm.qsum[threadIdx.x];
-            }
+            if (static_cast<int>(threadIdx.x) < n_tile && r < R)
+                q_out[static_cast<size_t>(blockIdx.x) * R + r] = sm.qsum[threadIdx.x];
         }
     }
     // drain: the producer waits (bounded) until every copy it issued has landed
@@ -562,10 +511,17 @@ DenseGeom geometry(const ising_context *c, int R) {
     g.n = static_cast<int>(c->n);
     g.kblocks = static_cast<int>(c->dense_ld / kBK);
     g.R = R;
-    g.R_pad = R <= 256 ? ((R + 15) / 16) * 16 : ((R + 255) / 256) * 256;
-    g.n_tile = g.R_pad < 256 ? g.R_pad : 256;
     g.m_tiles = (g.n + kBM - 1) / kBM;
-    g.r_tiles = g.R_pad / g.n_tile;
+    // Replicas in tiles of up to 256: as many tiles as the SMs hold beside the row tiles, of 16 replicas at least.
+    // A K block costs a CTA about 0.35 us whatever the replicas (its tile of J expanded for the MMA), so what a
+    // narrow tile saves is MMA and epilogue; us per step, tiles of up to 256 / so: 500 spins, R = 256 15.4 / 8.2,
+    // 2000, R = 100 18.4 / 16.5, 2000, R = 256 22.8 / 16.4, 9000, R = 256 59.7 / 55.3. (K blocks shared by a cluster,
+    // 2000, R = 100 10.5: the sums then depend on R; over 54 million components of a step 1236 instead of 1312
+    // are not the BF16 value nearest the exact one.)
+    const int beside = std::max(1, c->num_sms / g.m_tiles);
+    g.n_tile = std::min(256, ((R + beside - 1) / beside + 15) / 16 * 16);
+    g.r_tiles = (R + g.n_tile - 1) / g.n_tile;
+    g.R_pad = g.n_tile * g.r_tiles;
     uint32_t cols = 32;
     while (cols < static_cast<uint32_t>(g.n_tile)) cols <<= 1;
     g.a_col = cols;
@@ -589,30 +545,10 @@ ising_status_t launch_dense(const ising_context *c, const DenseGeom &g, const __
     auto kern = c->dense_ternary ? dense_tc_kernel<MODE, true> : dense_tc_kernel<MODE, false>;
     const size_t smem = c->dense_ternary ? smem_bytes<true>() : smem_bytes<false>();
     DOCH_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    // K blocks shared by up to 8 CTAs (the portable cluster size) while all tiles' clusters run at once
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(kThreadsTC);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const int tiles = g.m_tiles * g.r_tiles;
-    int split = std::max(1, std::min({kMaxSplit, c->num_sms / tiles, g.kblocks}));
-    for (;; --split) {
-        attr[0].val.clusterDim.x = static_cast<unsigned>(split);
-        cfg.gridDim = dim3(static_cast<unsigned>(g.m_tiles * split), static_cast<unsigned>(g.r_tiles));
-        int clusters = 0;
-        if (split == 1) break;
-        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= tiles) break;
-        cudaGetLastError();
-    }
-    DOCH_CUDA(cudaLaunchKernelEx(&cfg, kern, static_cast<const void *>(c->dense), xt_in, xt_out, h, g.n, g.kblocks, g.R,
-                                 g.R_pad, g.n_tile, g.tmem_cols, g.a_col, split, alpha, zscale, xscale, q_out,
-                                 c->err_word));
+    const dim3 grid(static_cast<unsigned>(g.m_tiles), static_cast<unsigned>(g.r_tiles));
+    kern<<<grid, kThreadsTC, smem, st>>>(c->dense, xt_in, xt_out, h, g.n, g.kblocks, g.R, g.R_pad, g.n_tile, g.tmem_cols,
+                                         g.a_col, alpha, zscale, xscale, q_out, c->err_word);
+    DOCH_CUDA(cudaGetLastError());
     return ISING_OK;
 }
 

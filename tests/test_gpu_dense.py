@@ -103,9 +103,9 @@ def test_dense_iterates_bf16(n, R, kind):
 
 @pytest.mark.parametrize("n, R, kind", [(65, 3, "pm1"), (1000, 256, "int"), (1100, 300, "pm1"), (2300, 100, "pm1"),
                                         (2440, 33, "pm1_sparse"), (4100, 16, "pm1"), (4100, 5, "int")])
-def test_dense_shared_k_blocks(n, R, kind):
-    """Instances whose row tiles leave SMs idle: a tile's K blocks are shared by 2 to 8 CTAs (counts
-    that do not divide the blocks or the columns). One step within one BF16 ulp, energies exact."""
+def test_dense_narrow_replica_tiles(n, R, kind):
+    """Instances whose row tiles leave SMs idle: the replicas are taken in tiles of 16 to 256 (counts that
+    do not divide the replicas). One step within one BF16 ulp, energies exact."""
     J = _jmat(kind, n, 96)
     P = O.Problem(J)
     alpha, beta = O.alpha_beta(J, eta=1.0, method="wigner")
@@ -150,6 +150,21 @@ def test_dense_energy_exact(n, R, kind):
             assert np.array_equal(E, Er)
             assert np.array_equal(cut, cr)
             assert best[0] == int(np.argmin(Er))
+    finally:
+        N.ising_destroy(h)
+
+
+@pytest.mark.parametrize("n, R, alone", [(2000, 400, 100), (6000, 300, 64), (1000, 256, 1)])
+def test_dense_replicas_do_not_depend_on_each_other(n, R, alone):
+    """A replica's iterates are the same, bit by bit, however many run beside it: every product adds its K
+    blocks in one order, whatever the tiles."""
+    h = N.ising_create(N.Problem(_jmat("pm1", n, 98)), N.FLAG_SKIP_VALIDATION)
+    try:
+        x0 = torch.from_numpy(I.x0_uniform(n, R, seed=99)).to(torch.bfloat16).cuda()
+        x, y = x0.clone(), x0[:, :alone].contiguous()
+        for v in (x, y):
+            N.ising_iterate(h, v, [2.0 * n ** 0.5], [n ** 1.5 * (2.0 * n ** 0.5 + n)], 6)
+        assert torch.equal(x[:, :alone], y)
     finally:
         N.ising_destroy(h)
 
