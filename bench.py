@@ -746,19 +746,20 @@ class Er800:
         N.ising_energy(self.h, self.x, E_int=self.E, cut_int=self.cut, best=self.best, stream=sid)
 
     def roofline(self, per_launch_s):
-        # FP64 arithmetic of the 1000 steps in the one launch: a multiply-add per stored coupling and
-        # replica, and alpha x, the scale and the cube root's argument per spin and replica (cube root
-        # not counted); against the nominal dense FP64 rate of the part (1.25 TFLOP/s). A cluster of 16 CTAs
-        # per replica (128 of 152 SMs) holds the iterate in shared memory and takes J x in fixed point: the
-        # launch is bound by the latency of a step's chain.
+        # FP64 arithmetic of the 1000 steps in the one launch, against the nominal dense FP64 rate of the part
+        # (1.25 TFLOP/s): per spin and replica alpha x, the scale and sum with J x (3) and the Newton cube root (12).
+        # J x itself is summed in integers (a multiply-add per stored coupling and replica) and not counted.
+        # A cluster of 16 CTAs per replica (128 of 152 SMs) holds the iterate in shared memory: the launch is
+        # bound by the latency of a step's chain.
         nnz = self.nnz
-        flops = self.iters * self.R * (2.0 * nnz + 3.0 * self.n)
+        flops = self.iters * self.R * 15.0 * self.n
         ach = flops / per_launch_s / 1e9
         peak = 1250.0
         return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "GFLOP/s", "frac": ach / peak,
                 "traffic": None, "kernel": self.dominant, "peak_kind": "nominal FP64 (1.25 TFLOP/s)",
                 "algorithmic_flops_per_launch": flops,
-                "note": "a cluster of 16 CTAs per replica (128 of 152 SMs); J x in fixed point; latency-bound"}
+                "integer_products_per_launch": self.iters * self.R * nnz,
+                "note": "a cluster of 16 CTAs per replica (128 of 152 SMs); J x in integers, not counted; latency-bound"}
 
     def e2e(self, n_steps, sid):
         N = self.N

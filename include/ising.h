@@ -242,7 +242,10 @@ ISING_API void ising_destroy(ising_handle_t h);
  * form (FP32 products and accumulation on the CUDA cores, FP32 state, CUDA's
  * cbrtf), the reference the BF16 form is compared with. For PROCEDURAL the iterate is
  * F32 and each step generates the couplings; an H_trace costs one more
- * coupling product per step.
+ * coupling product per step. A TORUS2D lattice with several replicas, F64
+ * iterates, a width that is not a multiple of 4 or x not 16-byte aligned takes
+ * the four couplings of a site as one word: 4 n bytes of device memory, built
+ * at the first such call (which waits for it) and kept by the handle.
  */
 ISING_API ising_status_t ising_iterate(ising_handle_t h, void *x, int32_t xtype, int32_t R,
                              const double *alpha, int32_t alpha_len, const double *beta,
@@ -256,8 +259,10 @@ ISING_API ising_status_t ising_iterate(ising_handle_t h, void *x, int32_t xtype,
  *   v^k = y^k if H(y^k) <= max(H(x^max(0,k-q)), ..., H(x^k)), else x^k,
  *   x^(k+1) = T(v^k)  (Eq. FPE).
  * Each step costs one coupling product (J y^k = (1 + c_k) J x^k - c_k J x^(k-1)),
- * FP64 reductions of H(x^k) and H(y^k) per (instance, replica), and the
- * update; the acceptance test runs per (instance, replica) on the device.
+ * reductions of H(x^k) and H(y^k) per (instance, replica) (FP64 for F64
+ * iterates; FP32 terms in compensated sums, relative error 2^-44 of the sum of
+ * their magnitudes, for F32 ones), and the update; the acceptance test runs in
+ * FP64 per (instance, replica) on the device.
  *   x      [n][R] F32 or F64, x^(0) on entry, x^(iters) on return (in place).
  *   alpha, beta  [max(1,n_instances)] host arrays (constant alpha; beta > 0).
  *   q      window of the non-monotone test (q >= 0; q = 0 compares with
@@ -269,7 +274,8 @@ ISING_API ising_status_t ising_iterate(ising_handle_t h, void *x, int32_t xtype,
  * CSR, TORUS2D and PROCEDURAL (F32) couplings; ISING_ERR_UNSUPPORTED for
  * DENSE. Device scratch: four iterate-sized buffers plus O(R) reduction
  * space, owned by the handle (two for an FP32 lattice with R = 1, whose
- * passes recompute both coupling products instead of storing them).
+ * passes recompute both coupling products instead of storing them; six for
+ * PROCEDURAL).
  */
 ISING_API ising_status_t ising_iterate_adoch(ising_handle_t h, void *x, int32_t xtype, int32_t R,
                                    const double *alpha, const double *beta, int32_t iters, int32_t q,
@@ -278,8 +284,8 @@ ISING_API ising_status_t ising_iterate_adoch(ising_handle_t h, void *x, int32_t 
 /*
  * DOCH (Algorithm 1) with the stopping rule of Remark S2, per (instance,
  * replica) pair: after each step, r^(k) = ||x^(k+1) - x^(k)||_2 / ||x^(k)||_2
- * (compensated FP32 per thread for F32 iterates, FP64 across threads and for
- * F64 iterates); the pair stops at the first k with
+ * (FP64 for F64 iterates; compensated FP32 for F32 ones, relative error about
+ * 2^-44, FP64 across blocks or threads); the pair stops at the first k with
  * r^(k) < eps and keeps x^(k+1). Pairs that never meet the rule run
  * max_iters steps.
  *   x      [n][R] F32 or F64 (in place): each pair's last iterate on return.
@@ -289,9 +295,11 @@ ISING_API ising_status_t ising_iterate_adoch(ising_handle_t h, void *x, int32_t 
  *          steps each pair took.
  * Batched FP32 instances that fit the shared-memory resident kernel apply
  * the rule inside it (FP32 sums per thread and warp, FP64 across warps) and
- * end each instance's replica group once all of its replicas stopped;
- * otherwise the host checks every 8 steps whether any pair still runs and
- * ends the loop when none does. CSR, TORUS2D and PROCEDURAL (F32);
+ * end each instance's replica group once all of its replicas stopped. One CSR
+ * instance of at most 8 entries a row runs a launch per step, which reports its
+ * progress in host memory; the host stays 12 launches ahead and ends the loop
+ * when no replica runs any more. Otherwise the host checks every 8 steps
+ * whether any pair still runs. CSR, TORUS2D and PROCEDURAL (F32);
  * ISING_ERR_UNSUPPORTED for DENSE.
  */
 ISING_API ising_status_t ising_iterate_until(ising_handle_t h, void *x, int32_t xtype, int32_t R,
@@ -354,7 +362,9 @@ ISING_API ising_status_t ising_tune_eta(ising_handle_t h, const void *x0, int32_
  * keeping x^(k) only every ckpt_every steps and recomputing each segment.
  *   x0       [n][R] F32 or F64 (CSR, one instance). The forward iterates
  *            (checkpoints and recomputed segments) run in x0's precision; the
- *            adjoint recursion runs in FP32; its sums (dL/dalpha, the loss)
+ *            adjoint recursion runs in FP32, or in FP64 for F64 iterates of
+ *            at most 2048 spins where R leaves four blocks or more per replica
+ *            and the couplings fit shared memory; its sums (dL/dalpha, the loss)
  *            are compensated FP32 per thread for F32 iterates and FP64 across
  *            threads (FP64 throughout for F64 iterates). d x^(k+1)/d x^k
  *            contains 1/(3 (x^(k+1))^2), so components passing near zero in

@@ -289,7 +289,7 @@ struct SmallRecord {
 };
 ising_status_t csr_small_run(const ising_context *c, const void *x_in, void *x_out, int xtype, int R,
                              const ParamTabs &p, int k0, int iters, const SmallRecord &rec, cudaStream_t st);
-// The same step with the H monitor fused (one instance): H(x^(k)) of Eq. Hamilton
+// csr_step with the H monitor fused (one instance): H(x^(k)) of Eq. Hamilton
 // per replica into H_out [R] (device), alpha_k and beta of the step.
 // ISING_ERR_UNSUPPORTED when the fused form does not apply (batched instances,
 // R / vector width > 256).
@@ -301,9 +301,9 @@ ising_status_t torus_step_f32_traced(ising_context *c, const float *x_in, float 
 // H per replica from fused per-block partials [blocks][R][4] (x^4, x^2, x u, h x)
 ising_status_t ham_fused_finish_launch(const double *hpart, int blocks, int R, double alpha, double beta, double *H,
                                        cudaStream_t st);
-// CSR, all `iters` steps in one launch: one CTA per (instance, replica) with
-// the iterate in shared memory. ISING_ERR_UNSUPPORTED when an instance does
-// not fit (the caller then uses csr_step).
+// CSR, all `iters` steps in one launch, in place: csr_small_run from step 0 (a cluster of 1 to 16 CTAs
+// per (instance, replica), the iterate in shared memory). ISING_ERR_UNSUPPORTED when an instance
+// does not fit or single steps are faster (the caller then uses csr_step).
 ising_status_t csr_fused(const ising_context *c, void *x, int xtype, int R, const ParamTabs &p,
                          int iters, cudaStream_t st);
 size_t csr_fused_max_spins(int xtype);

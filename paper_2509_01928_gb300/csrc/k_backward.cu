@@ -1,7 +1,9 @@
 // Adjoint of N DOCH steps (derived from Eq. FPE; the paper has no gradients).
 //
 // Precision: the forward iterates (checkpoints and recomputed segments) are
-// FP32 or FP64 as the caller's x0; the adjoint recursion (g, w) runs in FP32.
+// FP32 or FP64 as the caller's x0; the adjoint recursion (g, w) runs in FP32 here.
+// (Small instances take their adjoint steps in k_csr_small.cu, in FP64 for FP64
+// iterates; csr_loss_w below serves both.)
 // The FP64 forward exists because d x^(k+1) / d x^k contains
 // 1 / (3 (x^(k+1))^2): components that pass near zero in the transient make
 // the gradient sensitive to the trajectory, and an FP32 trajectory shifts

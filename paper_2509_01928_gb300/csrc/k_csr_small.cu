@@ -11,10 +11,11 @@
 // in the iterate's type (FP64 iterates and 8-bit couplings: the integers, or the upper words of the
 // FP64 values, whose lower words are zero: 6 instead of 10 bytes an entry).
 //
-// Bound by FP64 arithmetic (half a lane per clock and SM partition, about 150 clocks from one operation
-// to the next that needs it; an integer -> FP64 conversion costs as much as an FMA) and the latency of
-// a step's chain: products, tree, cube root, exchange. FP64 iterates with 8-bit couplings take their
-// products in integers (fixed point, below): nine FP64 operations per cube root and five around it are left.
+// Bound by the latency of a step's chain: products, tree, cube root, exchange (29 % of the issue slots and 14 %
+// of the FP64 pipe active for the instance below, 13 warps per SM, bank conflicts on a random gather), in which
+// FP64 operations weigh most (half a lane per clock and SM partition, about 150 clocks from one to the next
+// that needs it; an integer -> FP64 conversion costs as much as an FMA). FP64 iterates with 8-bit couplings take their
+// products in integers (fixed point, below): eight FP64 operations per cube root and four around it are left.
 // 800 spins, 38,000 entries, R = 8, FP64, per step: 10.0 us with one thread per row, the couplings
 // converted at every use and CUDA's cbrt of a quotient; 3.4 us with the couplings held in FP64 and four
 // threads per row (products 2.3, update 0.8, exchange 0.35); 2.75 us in fixed point with eight. The FP64
@@ -399,8 +400,9 @@ csr_small(const XT *x_in, XT *x_out, const int64_t *__restrict__ row_ptr,
 // and the partial sums of dL/dalpha_k = sum w^k x^k / beta of every CTA into part[k][CTA]. Within a
 // gradient the state has the iterate's type, between segments too (the result does not depend on the
 // checkpoint interval): FP64 for FP64 iterates (few rows per CTA, so the latency of the
-// chain counts and not the FP64 rate; the factor 1 / (3 beta x^2) is formed before the wait for the
-// peers' shares); FP32 with compensated row sums for FP32 ones. The products
+// chain counts and not the FP64 rate: 7 % of the issue slots, 22 % of the FP64 pipe active, four warps per
+// SM, 2000 spins, R = 8, 4 us per step; the factor 1 / (3 x^2) is formed before the wait for the peers' shares); FP32
+// with compensated row sums for FP32 ones. The products
 // w x (FP64, or FP32 split exactly) stay in shared memory for up to `hold` steps, and are then added in FP64,
 // a warp per step: added at every step they were a third of it. x^(k0) is x_first and
 // x^(k0 + m) = x_seg + (m - 1) stride, each loaded a step ahead. Every CTA of a cluster owns rows here:
@@ -442,7 +444,7 @@ struct AdjointRow<double> {
     __device__ __forceinline__ void set(double x) {
         const double d = 3.0 * x * x;
         const float df = static_cast<float>(d);
-        if (df > 1e-30f && df < 1e30f) {  // two Newton steps from the FP32 reciprocal
+        if (df > 1e-30f && df < 1e30f) {  // one Newton step from the FP32 reciprocal: within (2^-23)^2 = 1.4e-14
             double r = static_cast<double>(1.0f / df);
             r = fma(r, fma(-d, r, 1.0), r);
             factor = r;
@@ -769,11 +771,13 @@ ising_status_t csr_small_run(const ising_context *c, const void *x_in, void *x_o
 }
 
 // The adjoint's forward steps and adjoint steps run here for instances of at most 2048 spins with at
-// least four CTAs per replica; larger ones take single steps, whose launches overlap. Shared memory
-// against single steps, ms per gradient: FP64, 2000 spins, R = 8, 100 steps 1.43 / 1.49 (relative error of
-// grad_x0 over twelve seeds 0.03 to 0.21 e-6 against 0.46 to 3.9 e-6); 1000 spins, R = 1, 60 steps 0.87 / 0.94;
-// 4000 spins, R = 16, with an FP32 state 1.44 / 1.22; FP32, 60 steps, 1000 spins, R = 16 0.76 / 0.87, 2000 spins,
-// R = 8 0.87 / 0.86, 6000 spins 1.10 / 0.88 (every new value is stored into all CTAs, 13 clocks a warp).
+// least four CTAs per replica; larger ones take single steps, whose launches overlap and whose adjoint state
+// is FP32. Every new value is stored into all CTAs, 13 clocks a warp, so that many rows per CTA lose. Shared
+// memory / single steps, ms per gradient of 100 FP64 steps, checkpoints every 10, degree 3: 2000 spins, R = 8 1.45 / 1.49,
+// 2500 1.53 / 1.51 (R = 1 1.24 / 1.21, R = 16 1.67 / 1.56), 3000 1.63 / 1.53, 4000 1.80 / 1.53 (R = 16 2.06 / 1.65);
+// degree 6: 2500 1.67 / 1.74, 4000 1.82 / 1.75. Relative error of grad_x0: 2e-8 to 1.2e-7 with the FP64 state, 0.7e-6 to
+// 3.7e-6 with the FP32 one. FP32, 60 steps: 1000 spins, R = 16 0.76 / 0.87, 2000 spins, R = 8 0.87 / 0.86, 6000
+// spins 1.10 / 0.88.
 bool backward_small(const ising_context *c, int xtype, int R) {
     return c->n_inst == 1 && c->n <= 2048 && static_cast<size_t>(c->n) <= csr_fused_max_spins(xtype) &&
            cluster_max(c, R) >= 4;

@@ -19,7 +19,8 @@
 // integer pipe). Readout of 128 instances of up to 20,000 spins, R = 16, Gaussian
 // couplings: 1.72 ms with one replica per block and a thread per row, 0.74 ms now (FP64
 // additions); of the 10^5-spin, 10^7-entry integer matrix, R = 16: 1.15 ms and 0.11 ms
-// (gathers from L2); of a lattice of 10^8 sites, R = 1: 0.48 ms and 0.10 ms (HBM). E = -acc0/2 - acc2 and cut = -acc1/2 from the sums over all rows of
+// (gathers from L2); of a lattice of 10^8 sites, R = 1: 0.48 ms and 0.10 ms (HBM).
+// E = -acc0/2 - acc2 and cut = -acc1/2 from the sums over all rows of
 // acc0 = s_i sum_j J_ij s_j, acc1 = sum_j J_ij (1 - s_i s_j), acc2 = h_i s_i.
 #include <cuda_bf16.h>
 

@@ -15,13 +15,16 @@
 // results do not depend on how the steps are grouped.
 //
 // Couplings: one word per site, (right, left, down, up) as bytes offset by 128, built once
-// per handle (the four edges of a site in one 4-byte load instead of two rows and a
-// neighbour of two int8 arrays).
+// per handle, 4 bytes per site kept beside the couplings (the four edges of a site in one 4-byte load
+// instead of two rows and a neighbour of two int8 arrays).
 //
-// Bound by instruction issue (FP32: about 17 instructions per value and step besides the
-// shared-memory traffic of 12 bytes per value) once a pass does three steps. 1000 x 1000
-// lattice, R = 16, FP32: 106 us per step with one thread per value and divisions for its
-// site, 24.6 us per step now.
+// FP32, three steps: 71 % of the issue slots active at 33 lane slots per value and step (halo included),
+// XU, FMA and ALU pipes at 31 to 38 %; the rest are waits of the 16 warps per SM that registers (up to 96)
+// and the ring (47 KB) leave, with a barrier per row. 1000 x 1000 lattice, R = 16: 106 us per step with one
+// thread per value and divisions for its site, 20.5 us now. FP64: its arithmetic.
+//
+// FP32 roots: the walk takes them without a test of their range and walks a strip once more, tests
+// included, where one of its roots left it (zeros do: twice the time for blocks that hold a zero replica).
 #include <algorithm>
 #include <cmath>
 

@@ -585,9 +585,10 @@ def test_fused_hamiltonian_monitor(kind):
                                                  (1500, 20, 0.08, 3), (700, 40, 0.05, 1), (600, 100, 0.05, 1)])
 @pytest.mark.parametrize("start", ["uniform", "wide", "tiny", "huge", "zero"])
 def test_small_fp64_int8_steps(n, R, density, jmax, start):
-    """FP64 iterates of small instances with 8-bit couplings take J x in fixed point; starts outside its
-    range (and one CTA per replica) take FP64 sums. Components over many orders of magnitude, a field and
-    a schedule of alpha included; 1e-12 against the oracle at every size of share and cluster."""
+    """FP64 iterates of small instances with 8-bit couplings take J x in fixed point; short rows, small
+    shares and starts outside its range take FP64 sums. Components over many orders of magnitude, a field and
+    a schedule of alpha included; 1e-12 of the norm of a replica against the oracle at every size of share
+    and cluster (components one by one: test_small_fp64_int8_components)."""
     rng = np.random.default_rng(n + R)
     keep = np.triu(rng.random((n, n)) < density, 1)
     i, j = keep.nonzero()
