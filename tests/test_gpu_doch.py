@@ -624,7 +624,7 @@ def test_small_fp64_int8_steps(n, R, density, jmax, start):
 
 
 @pytest.mark.parametrize("n, R, density, jmax", [(800, 8, 0.06, 1), (300, 8, 0.02, 1), (801, 3, 0.06, 127), (1500, 20, 0.08, 1),
-                                                 (700, 30, 0.05, 3), (64, 1, 0.3, 1)])
+                                                 (700, 30, 0.05, 3), (64, 1, 0.3, 1), (1500, 30, 0.03, 1), (2000, 40, 0.02, 2)])
 @pytest.mark.parametrize("case", ["uniform", "one", "wide", "pinned", "parts", "hub"])
 def test_small_fp64_int8_components(n, R, density, jmax, case):
     """One step of FP64 iterates with 8-bit couplings, component by component, at components of very
